@@ -115,12 +115,13 @@ int fmm_set_timing(fmm_ctx *ctx, int enable);
  * The learned selector's training labels stay those of the unsoftened
  * expansion. */
 int fmm_set_softening(fmm_ctx *ctx, double eps);
-/* Leaf tile of the near field (a8): the number of a leaf's bodies (rows) the
- * mutual P2P kernel stages in shared memory per pass over the leaf's partner
- * columns, 8, 16 (the default) or 32.  Larger tiles take fewer passes over the
- * columns of big leaves; smaller ones fit more warps per SM.  The result is
- * the same sum in another order of the work: FP64 results differ from one
- * tile to another only by rounding.  FMM_EINVAL for other values. */
+/* Leaf tile of the mixed form's near field (a8): the number of a leaf's bodies
+ * (rows) the mutual P2P kernel stages in shared memory per pass over the
+ * leaf's partner columns, 8, 16 (the default) or 32.  Larger tiles take fewer
+ * passes over the columns of big leaves; smaller ones fit more warps per SM.
+ * The result is the same sum in another order of the work.  The FP64 form
+ * sums in fixed point with row blocks of its own and takes no notice of the
+ * tile.  FMM_EINVAL for other values. */
 int fmm_set_tile(fmm_ctx *ctx, int rows);
 
 /* a1-a3 (Sec. 2, first paragraph): bounding cube, 63-bit Morton keys, stable

@@ -21,7 +21,7 @@ FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxe
 # The FP32 interaction kernels flush FP32 subnormals to zero: their pair terms
 # never come near 1e-38, and without it every rsqrtf carries a subnormal
 # fix-up.  (FP64 arithmetic is not affected by the flag.)
-FTZ = {"p2p.cu", "m2l.cu"}
+FTZ = {"p2p.cu", "p2p64.cu", "m2l.cu"}
 
 
 def nvcc() -> str:

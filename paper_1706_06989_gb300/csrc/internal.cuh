@@ -124,7 +124,7 @@ struct fmm_ctx {
   int p2p_rows = 16;  // leaf tile: rows of a leaf staged per pass of the near field (8, 16 or 32)
   amfmm::Sizes sz;
   int m2l_which = 0;  // which of the ekey/eval buffers holds the sorted M2L entries
-  int p2p_order = -1;  // which pval buffer holds the near field's item order (-1: items in index order)
+  int p2p_which = 0;  // which pval buffer holds the FP64 near field's sorted partners
 
   // pinned host scratch for small read-backs
   void *hpin = nullptr;
@@ -145,7 +145,7 @@ struct fmm_ctx {
   // P2P grouping
   amfmm::DBuf pkey[2], pval[2], p2p_A, p2p_offA, p2p_offB, p2p_pos, p2p_poff, p2p_len,
       p2p_slots, p2p_colOff, p2p_cols, p2p_nb, p2p_pre, p2p_bodyf, p2p_items, p2p_itemOff, p2p_extraOff,
-      p2p_extra;
+      p2p_extra, p2p_heavy;
   // scan / sort scratch; `totals` holds small device results (1 KiB):
   // [0,16) scan totals, [64,72) near-field body-pair count, [80,88) selector-scored pairs, [88,92) selector candidates, [96,104) slot total,
   // [128,140) near-field column, work-item and extra-partial totals, [160,168) work queues (near field, gathered far field)
@@ -246,9 +246,15 @@ int m2l_run(fmm_ctx *c);            // m2l.cu: mutual M2L into slots
 int m2l_reduce(fmm_ctx *c);         // m2l.cu: per-cell fixed-order sums
 // the mixed form at order 3 gathers each cell's partners (one-sided, no slots)
 inline bool m2l_gathered(const fmm_ctx *c) { return c->opts.precision == FMM_MIXED && c->opts.order_P == 3; }
-int p2p_prepare(fmm_ctx *c);        // p2p.cu: grouping by leaf, partial slots
-int p2p_run(fmm_ctx *c);            // p2p.cu: mutual near field
-int p2p_reduce(fmm_ctx *c);         // p2p.cu: per-body fixed-order sums
+// every cell's partners over a list of pairs, in the stable order of the list:
+// cell c's are val[*which][off[c] .. off[c + 1])  (m2l.cu)
+int partner_lists(fmm_ctx *c, const int2 *pairs, int64_t K, DBuf key[2], DBuf val[2], int32_t *off, int *which);
+// near field: mixed form (p2p.cu) and FP64 form (p2p64.cu)
+int p2p_prepare(fmm_ctx *c);        // grouping by leaf, partial slots
+int p2p_run(fmm_ctx *c);            // near field
+int p2p_reduce(fmm_ctx *c);         // per-body fixed-order sums of the mixed form's slots
+int p2p64_prepare(fmm_ctx *c);
+int p2p64_run(fmm_ctx *c);
 int downward(fmm_ctx *c);           // down.cu (L2L, L2P into sorted order)
 int forces(fmm_ctx *c, double *ax, double *ay, double *az);  // down.cu (caller order)
 

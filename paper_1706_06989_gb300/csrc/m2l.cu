@@ -827,7 +827,30 @@ int bits_for(int64_t v) {
   return b;
 }
 
+// The entries of K > 0 pairs sorted by cell (stable), and every cell's first
+// position off[cell] (off[ncell] = 2 K).
+int sorted_entries(fmm_ctx *c, const int2 *pairs, int64_t K, int gather, DBuf key[2], DBuf val[2], int32_t *off,
+                   int *which) {
+  const int64_t nc = c->sz.ncell, E = 2 * K;
+  AMFMM_TRY(ensure<uint32_t>(c, key[0], E));
+  AMFMM_TRY(ensure<uint32_t>(c, val[0], E));
+  k_m2l_entries<<<grid_for(K, 256), 256, 0, c->stream>>>(K, pairs, gather, ptr<uint32_t>(key[0]),
+                                                         ptr<uint32_t>(val[0]));
+  AMFMM_TRY(launched(c, "pair_entries"));
+  AMFMM_TRY(radix_sort_u32(c, key, val, E, bits_for(nc), which));
+  k_segment_offsets<<<grid_for((E + 3) / 4, 256), 256, 0, c->stream>>>(E, static_cast<int32_t>(nc),
+                                                                      ptr<uint32_t>(key[*which]), off);
+  return launched(c, "segment_offsets");
+}
+
 }  // namespace
+
+int partner_lists(fmm_ctx *c, const int2 *pairs, int64_t K, DBuf key[2], DBuf val[2], int32_t *off, int *which) {
+  *which = 0;
+  if (K > 0) return sorted_entries(c, pairs, K, 1, key, val, off, which);
+  AMFMM_CUDA(c, cudaMemsetAsync(off, 0, sizeof(int32_t) * (c->sz.ncell + 1), c->stream));
+  return FMM_OK;
+}
 
 int m2l_prepare(fmm_ctx *c) {
   cudaStream_t st = c->stream;
@@ -836,22 +859,15 @@ int m2l_prepare(fmm_ctx *c) {
   AMFMM_TRY(ensure<int32_t>(c, c->m2l_off, nc + 1));
   if (E > 0x7fffffffLL) return set_error(c, FMM_EUNSUPPORTED, "too many M2L pairs (%lld)", (long long)K);
   int32_t *off = ptr<int32_t>(c->m2l_off);
-  AMFMM_CUDA(c, cudaMemsetAsync(off, 0, sizeof(int32_t) * (nc + 1), st));
-  if (K == 0) return FMM_OK;
-  AMFMM_TRY(ensure<uint32_t>(c, c->ekey[0], E));
-  AMFMM_TRY(ensure<uint32_t>(c, c->eval[0], E));
+  if (K == 0) {
+    AMFMM_CUDA(c, cudaMemsetAsync(off, 0, sizeof(int32_t) * (nc + 1), st));
+    return FMM_OK;
+  }
   if (!m2l_gathered(c)) AMFMM_TRY(ensure<int32_t>(c, c->m2l_pos, E));
   const bool fp32 = c->opts.precision == FMM_MIXED;
   const int gather = m2l_gathered(c);
-  k_m2l_entries<<<grid_for(K, 256), 256, 0, st>>>(K, ptr<int2>(c->m2l), gather, ptr<uint32_t>(c->ekey[0]),
-                                                  ptr<uint32_t>(c->eval[0]));
-  AMFMM_TRY(launched(c, "m2l_entries"));
-  int which = 0;
-  AMFMM_TRY(radix_sort_u32(c, c->ekey, c->eval, E, bits_for(nc), &which));
-  c->m2l_which = which;
-  k_segment_offsets<<<grid_for((E + 3) / 4, 256), 256, 0, st>>>(E, static_cast<int32_t>(nc),
-                                                               ptr<uint32_t>(c->ekey[which]), off);
-  AMFMM_TRY(launched(c, "segment_offsets"));
+  AMFMM_TRY(sorted_entries(c, ptr<int2>(c->m2l), K, gather, c->ekey, c->eval, off, &c->m2l_which));
+  const int which = c->m2l_which;
   if (!gather) {
     k_inverse<<<grid_for(E, 256), 256, 0, st>>>(E, ptr<uint32_t>(c->eval[which]), ptr<int32_t>(c->m2l_pos));
     AMFMM_TRY(launched(c, "m2l_inverse"));
