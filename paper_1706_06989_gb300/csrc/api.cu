@@ -155,7 +155,7 @@ void fmm_destroy(fmm_ctx *c) {
   if (c->stream) cudaStreamSynchronize(c->stream);
   else cudaDeviceSynchronize();
   DBuf *all[] = {&c->key[0], &c->key[1], &c->idx[0], &c->idx[1], &c->order, &c->X, &c->Y, &c->Zb, &c->Mb,
-                 &c->cur, &c->flag, &c->incl, &c->lcp, &c->leaf_of, &c->cell_at, &c->near, &c->acc,
+                 &c->flag, &c->incl, &c->lcp, &c->body_lv, &c->leaf_of, &c->cell_at, &c->near, &c->acc,
                  &c->status, &c->bbox_part, &c->bbox, &c->sys_off, &c->sysid, &c->sbox, &c->begin, &c->count, &c->level, &c->parent,
                  &c->first_child, &c->nchild, &c->S, &c->M, &c->Z, &c->invM, &c->Rmax, &c->rmax2, &c->mom,
                  &c->loc, &c->leaves, &c->front[0], &c->front[1],

@@ -69,7 +69,7 @@ GraphKey key_of(const fmm_ctx *c, const double *ax, const double *ay, const doub
 }
 
 // Pass 2: the solve's launches captured into a graph (nothing runs).
-int capture(fmm_ctx *c, int depth0, double *ax, double *ay, double *az) {
+int capture(fmm_ctx *c, double *ax, double *ay, double *az) {
   for (int d = 0; d < kMaxGraphDepth; ++d)
     if (!c->gstream[d]) AMFMM_CUDA(c, cudaStreamCreateWithFlags(&c->gstream[d], cudaStreamNonBlocking));
   if (c->gexec) {
@@ -84,7 +84,6 @@ int capture(fmm_ctx *c, int depth0, double *ax, double *ay, double *az) {
   c->sz.n = n;
   c->sz.nsys = nsys;
   c->launches = 0;
-  c->last_depth = depth0;
   c->gplan_pos = 0;
   c->gdepth = 0;
   c->stream = c->gstream[0];
@@ -242,9 +241,7 @@ int graph_solve(fmm_ctx *c, double *ax, double *ay, double *az) {
   // pass 1: a plain solve that keeps its read-backs.  A solve that had to
   // grow a buffer took a path (a retry) that a capture cannot repeat: the
   // first solve of a context is then planned once more, on grown buffers.
-  int depth0 = c->last_depth;
   for (int attempt = 0; attempt < 2; ++attempt) {
-    depth0 = c->last_depth;
     const int64_t gen0 = c->alloc_gen;
     c->gplan.clear();
     c->gmode = kGraphRecord;
@@ -258,10 +255,9 @@ int graph_solve(fmm_ctx *c, double *ax, double *ay, double *az) {
   c->gkey = key;
   if (c->gwait && !repeat) return FMM_OK;
   const Sizes plan = c->sz;
-  const int depth1 = c->last_depth;
   const int64_t launches = c->launches_last;
   // pass 2: the same solve captured; its results are those of pass 1
-  if (capture(c, depth0, ax, ay, az) == FMM_OK) {
+  if (capture(c, ax, ay, az) == FMM_OK) {
     c->gsz = plan;
     c->gkey = key_of(c, ax, ay, az);
     c->gwait = false;
@@ -274,7 +270,6 @@ int graph_solve(fmm_ctx *c, double *ax, double *ay, double *az) {
     c->errbuf[0] = 0;
   }
   c->sz = plan;
-  c->last_depth = depth1;
   c->stage = kDown;
   c->launches_last = launches;
   return FMM_OK;

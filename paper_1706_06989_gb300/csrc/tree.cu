@@ -209,34 +209,12 @@ __global__ void k_gather_sorted(int64_t n, const uint32_t *__restrict__ perm, co
   i2[t] = i1[perm[t]];
 }
 
-// level 0: one root per system
-__global__ void k_roots(int32_t nsys, const int64_t *__restrict__ off, int32_t *__restrict__ begin,
-                        int32_t *__restrict__ count, int32_t *__restrict__ level, int32_t *__restrict__ parent,
-                        int32_t *__restrict__ first_child, int32_t *__restrict__ nchild, int32_t *__restrict__ lvl,
-                        int *__restrict__ ovf) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s == 0) {
-    lvl[0] = 0;
-    lvl[1] = nsys;
-    *ovf = 0;
-  }
-  if (s >= nsys) return;
-  begin[s] = static_cast<int32_t>(off[s]);
-  count[s] = static_cast<int32_t>(off[s + 1] - off[s]);
-  level[s] = 0;
-  parent[s] = -1;
-  first_child[s] = -1;
-  nchild[s] = 0;
-}
-
-// Gather the bodies into key order; lcp[s] = octal digits shared by keys s-1, s.
+// Gather the bodies into key order.
 __global__ void k_permute(const double *__restrict__ x, const double *__restrict__ y,
                           const double *__restrict__ z, const double *__restrict__ m,
-                          const uint64_t *__restrict__ key, const uint32_t *__restrict__ idx,
-                          int64_t n, double *__restrict__ X, double *__restrict__ Y,
-                          double *__restrict__ Zb, double *__restrict__ Mb,
-                          int32_t *__restrict__ order, int32_t *__restrict__ lcp,
-                          int32_t *__restrict__ cur, const int32_t *__restrict__ sysid) {
+                          const uint32_t *__restrict__ idx, int64_t n, double *__restrict__ X,
+                          double *__restrict__ Y, double *__restrict__ Zb, double *__restrict__ Mb,
+                          int32_t *__restrict__ order) {
   int64_t s = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (s >= n) return;
   const uint32_t o = idx[s];
@@ -245,97 +223,190 @@ __global__ void k_permute(const double *__restrict__ x, const double *__restrict
   Zb[s] = z[o];
   Mb[s] = m[o];
   order[s] = static_cast<int32_t>(o);
-  int l = 0;
-  if (s > 0) {
-    uint64_t d = key[s - 1] ^ key[s];
-    l = d == 0 ? kMaxLevel : (__clzll(static_cast<long long>(d)) - 1) / 3;
-  }
-  lcp[s] = l;
-  cur[s] = sysid ? sysid[o] : 0;  // root of the body's system
 }
 
 // ---------------------------------------------------------------------------
-// a3: octree, one level per pass
+// a3: octree, all levels at once
 // ---------------------------------------------------------------------------
-// A body starts a child cell at level lev+1 when its cell at level lev is split
-// and it is the cell's first body or its key differs from its predecessor's
-// in digit lev+1.
-// The level kernels read the level's first new cell id from lvl[lev + 1]
-// (device-resident, so that several levels are enqueued before the host
-// looks) and do nothing once a level has run out of cell capacity (*ovf).
-// From the second level on it first moves every body to its cell of this
-// level: -1 for a body of a leaf of the previous level (retired), else the
-// child of its previous cell that starts at the last flagged body at or
-// before it (same cell), from that level's flags and their exclusive sums.
-__global__ void k_level_flags(int64_t n, int lev, int n_crit, const int32_t *__restrict__ lcp,
-                              const int32_t *__restrict__ begin, const int32_t *__restrict__ count,
-                              int32_t *__restrict__ cur, int32_t *__restrict__ flag,
-                              const int32_t *__restrict__ excl, const int32_t *__restrict__ lvl,
-                              int32_t *__restrict__ cell_at_lev, int32_t *__restrict__ leaf_of,
-                              const int *__restrict__ ovf) {
-  int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
-  if (i >= n || *ovf) return;
-  int c = cur[i];
-  if (lev > 0 && c >= 0) {
-    c = count[c] <= n_crit ? -1 : lvl[lev] + excl[i] + flag[i] - 1;
-    cur[i] = c;
-  }
-  cell_at_lev[i] = c;
-  int f = 0;
-  if (c >= 0) {
-    const bool leaf = count[c] <= n_crit || lev == kMaxLevel;
-    if (leaf) leaf_of[i] = c;
-    else f = (i == begin[c]) || (lcp[i] == lev);
-  }
-  flag[i] = f;
+// The sorted keys fix the tree without a pass per level.  A run of bodies that
+// share l octal digits is a cell of level l if the run at level l - 1 is
+// split, that is, holds more than n_crit bodies (and l <= 21).  A body's run
+// holds more than n_crit bodies at level l exactly when some window of
+// n_crit + 1 consecutive bodies around it shares l digits, and a window shares
+// as many as its first and last key do.  So its leaf lies at level
+//     D = min(21, 1 + max over its windows of the digits shared by their ends)
+// (0 without a window), and the cells that start at the body are those of the
+// levels (digits shared with its predecessor) + 1 .. D.  Counting the starts
+// per level and block, one scan over (level, block) gives every cell its id
+// in breadth-first order; a body's cell at any level up to D is the last
+// start at or before it.  (One pass per level, five launches each: 0.45 of the
+// 0.79 ms of the tree at N = 1,048,576, 0.26 of 0.50 ms at 65,536.)
+constexpr int kLevels = kMaxLevel + 1;
+// largest n_crit whose windows a block keeps in shared memory and each body
+// scans; wider ones take the maximum by doubling, a launch per step
+constexpr int kWindowMax = 2048;
+
+// octal digits that two keys share
+__device__ __forceinline__ int shared_digits(uint64_t a, uint64_t b) {
+  const uint64_t d = a ^ b;
+  return d == 0 ? kMaxLevel : (__clzll(static_cast<long long>(d)) - 1) / 3;
+}
+// system of the body at sorted position s
+__device__ __forceinline__ int system_of(const int32_t *__restrict__ sysid, const uint32_t *__restrict__ idx,
+                                         int64_t s) {
+  return sysid ? sysid[idx[s]] : 0;
+}
+// digits shared by the ends of the window [j, j + w], -1 if there is none
+__device__ __forceinline__ int window_digits(const uint64_t *__restrict__ key, const uint32_t *__restrict__ idx,
+                                             const int32_t *__restrict__ sysid, int64_t n, int64_t j, int w) {
+  if (j < 0 || j + w >= n || system_of(sysid, idx, j) != system_of(sysid, idx, j + w)) return -1;
+  return shared_digits(key[j], key[j + w]);
 }
 
-// Also closes the level: lvl[lev + 2] = lvl[lev + 1] + (new cells).
-__global__ void k_make_cells(int64_t n, int lev, int32_t *__restrict__ lvl, const int32_t *__restrict__ ntot,
-                             int64_t cap, const int32_t *__restrict__ flag, const int32_t *__restrict__ excl,
-                             const int32_t *__restrict__ cur, int32_t *__restrict__ begin,
-                             int32_t *__restrict__ level, int32_t *__restrict__ parent,
-                             int32_t *__restrict__ first_child, int32_t *__restrict__ nchild, int *__restrict__ ovf) {
-  int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
-  const int off = lvl[lev + 1];
-  if (i == 0) {
-    lvl[lev + 2] = off + *ntot;
-    if (static_cast<int64_t>(off) + *ntot > cap) atomicOr(ovf, 1);
+// For n_crit beyond kWindowMax: the windows' digits, and their running maximum
+// over the last 2^k window starts by doubling (out = max of in at j and at
+// j - step).
+__global__ void k_window_digits(const uint64_t *__restrict__ key, const uint32_t *__restrict__ idx,
+                                const int32_t *__restrict__ sysid, int64_t n, int w, int8_t *__restrict__ out) {
+  const int64_t j = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
+  if (j < n) out[j] = static_cast<int8_t>(window_digits(key, idx, sysid, n, j, w));
+}
+__global__ void k_window_max(int64_t n, int64_t step, const int8_t *__restrict__ in, int8_t *__restrict__ out) {
+  const int64_t j = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
+  if (j < n) out[j] = j >= step ? max(in[j], in[j - step]) : in[j];
+}
+
+// Per body: the digits shared with its predecessor (-1 for the first of a
+// system) and its leaf's level; per block and level: cells and leaves that
+// start there.  wmax (n_crit > kWindowMax): the maximum over the body's
+// windows.
+__global__ void k_cell_levels(const uint64_t *__restrict__ key, const uint32_t *__restrict__ idx,
+                              const int32_t *__restrict__ sysid, int64_t n, int n_crit,
+                              const int8_t *__restrict__ wmax, char2 *__restrict__ lv, int32_t *__restrict__ cnt) {
+  extern __shared__ int8_t win[];  // kBlock + n_crit window starts
+  __shared__ int32_t tot[2][kLevels];
+  const int t = threadIdx.x, lane = t & 31;
+  const int64_t i0 = blockIdx.x * static_cast<int64_t>(kBlock), i = i0 + t;
+  if (t < 2 * kLevels) tot[t / kLevels][t % kLevels] = 0;
+  if (!wmax)
+    for (int q = t; q < kBlock + n_crit; q += kBlock)
+      win[q] = static_cast<int8_t>(window_digits(key, idx, sysid, n, i0 - n_crit + q, n_crit));
+  __syncthreads();
+  int lcp = kMaxLevel, D = -1;
+  if (i < n) {
+    int m = -1;
+    if (wmax) m = wmax[i];
+    else
+      for (int q = 0; q <= n_crit; ++q) m = max(m, static_cast<int>(win[t + q]));
+    D = min(kMaxLevel, 1 + m);
+    lcp = i == 0 || system_of(sysid, idx, i) != system_of(sysid, idx, i - 1) ? -1 : shared_digits(key[i - 1], key[i]);
+    lv[i] = make_char2(static_cast<signed char>(lcp), static_cast<signed char>(D));
   }
-  if (i >= n || !flag[i] || *ovf) return;
-  const int c = cur[i];
-  const int id = off + excl[i];
-  if (id >= cap) return;  // flagged above; the tree is built again with more room
-  begin[id] = static_cast<int32_t>(i);
-  level[id] = lev + 1;
-  parent[id] = c;
-  first_child[id] = -1;
-  nchild[id] = 0;
-  if (i == begin[c]) first_child[c] = id;
+#pragma unroll
+  for (int l = 0; l < kLevels; ++l) {
+    const unsigned c = __ballot_sync(0xffffffffu, l > lcp && l <= D);
+    const unsigned f = __ballot_sync(0xffffffffu, l > lcp && l == D);
+    if (lane == 0 && c) atomicAdd(&tot[0][l], __popc(c));
+    if (lane == 0 && f) atomicAdd(&tot[1][l], __popc(f));
+  }
+  __syncthreads();
+  if (t < 2 * kLevels) cnt[static_cast<int64_t>(t) * gridDim.x + blockIdx.x] = tot[t / kLevels][t % kLevels];
+  if (blockIdx.x == 0 && t == 0) cnt[2 * kLevels * static_cast<int64_t>(gridDim.x)] = 0;  // closes the scan
 }
 
-__global__ void k_cell_counts(int lev, const int32_t *__restrict__ lvl, int32_t *__restrict__ begin,
-                              int32_t *__restrict__ count, const int32_t *__restrict__ parent,
-                              int32_t *__restrict__ nchild, const int *__restrict__ ovf) {
-  int k = blockIdx.x * blockDim.x + threadIdx.x;
-  const int off = lvl[lev + 1], nnew = lvl[lev + 2] - off;
-  if (k >= nnew || *ovf) return;
-  const int id = off + k;
-  const int p = parent[id];
-  int end = begin[p] + count[p];
-  if (k + 1 < nnew) end = min(end, begin[id + 1]);
-  count[id] = end - begin[id];
-  atomicAdd(&nchild[p], 1);
+// Emits the cells: begin, level, parent; every body's cell per level (-1 below
+// its leaf), its leaf, and the leaves in id order.  lvl: first id of every
+// level (23 entries) and the number of leaves.
+__global__ void k_emit_cells(int64_t n, const char2 *__restrict__ lv, const int32_t *__restrict__ offs, int64_t cap,
+                             int32_t *__restrict__ begin, int32_t *__restrict__ level, int32_t *__restrict__ parent,
+                             int32_t *__restrict__ cell_at, int32_t *__restrict__ leaf_of,
+                             int32_t *__restrict__ leaves, int32_t *__restrict__ lvl) {
+  __shared__ int32_t base[2][kLevels][kBlock / 32];
+  __shared__ int32_t first[kLevels + 1];
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+  const int64_t nb = gridDim.x, i = blockIdx.x * static_cast<int64_t>(kBlock) + t;
+  int lcp = kMaxLevel, D = -1;
+  if (i < n) {
+    const char2 v = lv[i];
+    lcp = v.x;
+    D = v.y;
+  }
+  if (t <= kLevels) first[t] = offs[t * nb];
+#pragma unroll
+  for (int l = 0; l < kLevels; ++l) {
+    const unsigned c = __ballot_sync(0xffffffffu, l > lcp && l <= D);
+    const unsigned f = __ballot_sync(0xffffffffu, l > lcp && l == D);
+    if (lane == 0) {
+      base[0][l][w] = __popc(c);
+      base[1][l][w] = __popc(f);
+    }
+  }
+  __syncthreads();
+  if (t < 2 * kLevels) {
+    int run = offs[static_cast<int64_t>(t) * nb + blockIdx.x];
+    int32_t *b = base[t / kLevels][t % kLevels];
+    for (int q = 0; q < kBlock / 32; ++q) {
+      const int v = b[q];
+      b[q] = run;
+      run += v;
+    }
+  }
+  __syncthreads();
+  const int ncell = first[kLevels];
+  if (blockIdx.x == 0 && t <= kLevels) lvl[t] = first[t];
+  if (blockIdx.x == 0 && t == 0) lvl[kLevels + 1] = offs[2 * kLevels * nb] - ncell;
+  const unsigned lt = (1u << lane) - 1;
+  int up = -1;  // the body's cell of the level above
+  for (int l = 0; l < kLevels && first[l] < ncell; ++l) {
+    const bool starts = l > lcp && l <= D;
+    const unsigned c = __ballot_sync(0xffffffffu, starts);
+    const unsigned f = __ballot_sync(0xffffffffu, starts && l == D);
+    if (i >= n) continue;
+    const int id = l <= D ? base[0][l][w] + __popc(c & lt) + (starts ? 1 : 0) - 1 : -1;
+    cell_at[static_cast<int64_t>(l) * n + i] = id;
+    if (starts && id < cap) {
+      begin[id] = static_cast<int32_t>(i);
+      level[id] = l;
+      parent[id] = up;
+    }
+    if (l == D) {
+      leaf_of[i] = id;
+      if (starts) leaves[base[1][l][w] + __popc(f & lt) - ncell] = id;
+    }
+    up = id;
+  }
 }
 
-__global__ void k_leaf_flags(int32_t ncell, const int32_t *__restrict__ nchild, int32_t *__restrict__ f) {
-  int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c < ncell) f[c] = nchild[c] == 0;
-}
-__global__ void k_leaf_compact(int32_t ncell, const int32_t *__restrict__ nchild,
-                               const int32_t *__restrict__ excl, int32_t *__restrict__ leaves) {
-  int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c < ncell && nchild[c] == 0) leaves[excl[c]] = c;
+// Ends and children of the cells.  A cell ends where its next sibling begins,
+// or with its parent; the children of a split cell are the cells of its first
+// to its last body on the next level.
+__global__ void k_finish_cells(int64_t n, int n_crit, int nsys, int64_t cap, const int64_t *__restrict__ sys_off,
+                               const int32_t *__restrict__ lvl, const int32_t *__restrict__ begin,
+                               const int32_t *__restrict__ level, const int32_t *__restrict__ parent,
+                               const int32_t *__restrict__ cell_at, int32_t *__restrict__ count,
+                               int32_t *__restrict__ first_child, int32_t *__restrict__ nchild) {
+  const int ncell = lvl[kLevels];
+  if (ncell > cap) return;  // built again with more room
+  for (int64_t id = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; id < ncell;
+       id += static_cast<int64_t>(gridDim.x) * blockDim.x) {
+    int64_t q = id, e = -1;
+    while (e < 0) {
+      const int p = parent[q];
+      if (p < 0) e = sys_off[q + 1];  // the roots are the first cells
+      else if (q + 1 < ncell && parent[q + 1] == p) e = begin[q + 1];
+      else q = p;
+    }
+    const int b = begin[id], l = level[id], c = static_cast<int>(e) - b;
+    int f = -1, k = 0;
+    if (c > n_crit && l < kMaxLevel) {
+      const int32_t *next = cell_at + static_cast<int64_t>(l + 1) * n;
+      f = next[b];
+      k = next[b + c - 1] - f + 1;
+    }
+    count[id] = c;
+    first_child[id] = f;
+    nchild[id] = k;
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -578,11 +649,16 @@ __global__ void k_rmax_final(int32_t ncell, const unsigned long long *__restrict
   if (c < ncell) Rmax[c] = __dsqrt_rn(__longlong_as_double(static_cast<long long>(rmax2[c])));
 }
 
-int ensure_cells(fmm_ctx *c, int64_t need, int64_t used) {
+int ensure_cells(fmm_ctx *c, int64_t need) {
   DBuf *ib[] = {&c->begin, &c->count, &c->level, &c->parent, &c->first_child, &c->nchild};
-  for (DBuf *b : ib) AMFMM_TRY(ensure_keep_bytes(c, *b, need * sizeof(int32_t), used * sizeof(int32_t)));
+  for (DBuf *b : ib) AMFMM_TRY(ensure<int32_t>(c, *b, need));
   return FMM_OK;
 }
+
+// device words of the tree stage: [0] bad input, [8, 32) the levels' first
+// cell ids, the number of cells and of leaves
+constexpr int kStatusLvl = 8;
+constexpr int kStatusWords = kStatusLvl + kLevels + 2;
 
 }  // namespace
 
@@ -597,19 +673,17 @@ int build_tree(fmm_ctx *c) {
   AMFMM_TRY(ensure<double>(c, c->Zb, n));
   AMFMM_TRY(ensure<double>(c, c->Mb, n));
   AMFMM_TRY(ensure<int32_t>(c, c->order, n));
-  AMFMM_TRY(ensure<int32_t>(c, c->cur, n));
-  AMFMM_TRY(ensure<int32_t>(c, c->flag, n));
-  AMFMM_TRY(ensure<int32_t>(c, c->incl, n + 1));
+  AMFMM_TRY(ensure<int32_t>(c, c->leaves, n + 1));
   AMFMM_TRY(ensure<int32_t>(c, c->leaf_of, n));
   AMFMM_TRY(ensure<int32_t>(c, c->cell_at, static_cast<size_t>(kMaxLevel + 1) * n));
-  AMFMM_TRY(ensure<int>(c, c->status, 8 + kMaxLevel + 3));
+  AMFMM_TRY(ensure<int>(c, c->status, kStatusWords));
   const int nbb = std::max(1, std::min<int>(c->num_sms * 4, static_cast<int>((n + kBlock - 1) / kBlock)));
   AMFMM_TRY(ensure<double>(c, c->bbox_part, 6 * nbb));
   AMFMM_TRY(ensure<double>(c, c->bbox, 8));
   
 
   int *status = ptr<int>(c->status);
-  AMFMM_CUDA(c, cudaMemsetAsync(status, 0, sizeof(int) * (8 + kMaxLevel + 3), st));
+  AMFMM_CUDA(c, cudaMemsetAsync(status, 0, sizeof(int) * kStatusWords, st));
   const int nsys = c->sz.nsys;
   int which = 0;
   if (nsys == 1) {
@@ -649,131 +723,89 @@ int build_tree(fmm_ctx *c) {
   }
   const uint64_t *skey = ptr<uint64_t>(c->key[which]);
   const uint32_t *sidx = ptr<uint32_t>(c->idx[which]);
-  AMFMM_TRY(ensure<int32_t>(c, c->lcp, n));
-  int32_t *lcp = ptr<int32_t>(c->lcp);
   c->sz.key_which = which;
+  k_permute<<<grid_for(n, kBlock), kBlock, 0, st>>>(c->x, c->y, c->z, c->m, sidx, n, ptr<double>(c->X),
+                                                    ptr<double>(c->Y), ptr<double>(c->Zb), ptr<double>(c->Mb),
+                                                    ptr<int32_t>(c->order));
+  AMFMM_TRY(launched(c, "permute"));
 
-  // Octree level by level, from one root per system.  The levels' first cell
-  // ids live on the device (lvl), so levels are enqueued in batches and the
-  // host reads the counts once per batch: the first batch runs as many
-  // levels as the previous tree had (a repeated or slowly changing system
-  // needs one round trip), later ones two at a time.  Levels past the last
-  // find no body left and do nothing.  A level that runs out of cell room
-  // stops the batch; the tree is then built again with twice the room.
-  int *ovf = status + 1;
-  int32_t *lvl = reinterpret_cast<int32_t *>(status + 8);  // kMaxLevel + 3 entries
-  int32_t *flag = ptr<int32_t>(c->flag);
-  int32_t *excl = ptr<int32_t>(c->incl);
-  int32_t *total = ptr<int32_t>(c->totals);
+  // octree: levels of every body, ids by one scan, cells
+  const int n_crit = static_cast<int>(std::min<int64_t>(c->opts.n_crit, n));
+  const int32_t *sysid = nsys == 1 ? nullptr : ptr<int32_t>(c->sysid);
+  const unsigned nb = grid_for(n, kBlock);
+  const int64_t ncnt = 2 * kLevels * static_cast<int64_t>(nb) + 1;
+  AMFMM_TRY(ensure<char2>(c, c->body_lv, n));
+  AMFMM_TRY(ensure<int32_t>(c, c->flag, std::max(n, ncnt) + 1));
+  AMFMM_TRY(ensure<int32_t>(c, c->incl, std::max(n, ncnt) + 1));
+  int32_t *cnt = ptr<int32_t>(c->flag), *offs = ptr<int32_t>(c->incl);
+  const int8_t *wmax = nullptr;
+  if (n_crit > kWindowMax) {
+    // windows wider than a block: maximum over the last n_crit + 1 starts by
+    // doubling, then once more over the two halves that cover them
+    AMFMM_TRY(ensure<int8_t>(c, c->lcp, 2 * n));
+    int8_t *a = ptr<int8_t>(c->lcp), *o = a + n;
+    k_window_digits<<<nb, kBlock, 0, st>>>(skey, sidx, sysid, n, n_crit, a);
+    AMFMM_TRY(launched(c, "window_digits"));
+    int64_t have = 1;
+    while (have < n_crit + 1) {
+      const int64_t step = std::min<int64_t>(have, n_crit + 1 - have);
+      k_window_max<<<nb, kBlock, 0, st>>>(n, step, a, o);
+      AMFMM_TRY(launched(c, "window_max"));
+      std::swap(a, o);
+      have += step;
+    }
+    wmax = a;
+  }
+  k_cell_levels<<<nb, kBlock, wmax ? 0 : kBlock + n_crit, st>>>(skey, sidx, sysid, n, n_crit, wmax,
+                                                              ptr<char2>(c->body_lv), cnt);
+  AMFMM_TRY(launched(c, "cell_levels"));
+  AMFMM_TRY(exclusive_scan_i32(c, cnt, offs, ncnt, nullptr));
+  int32_t *lvl = reinterpret_cast<int32_t *>(status + kStatusLvl);
   int64_t cap_cells = std::max<int64_t>(std::max<int64_t>(1024, n / 2 + 64), 2 * static_cast<int64_t>(nsys));
-  int lev = 0;
+  int32_t *h = static_cast<int32_t *>(c->hpin);
+  double *hb = reinterpret_cast<double *>(h + kStatusWords);
+  const double *bbox = nsys == 1 ? ptr<double>(c->bbox) : ptr<double>(c->sbox);
   for (int attempt = 0;; ++attempt) {
-    if (attempt > 16) return set_error(c, FMM_EINVAL, "octree: cell room still short after growing");
-    AMFMM_TRY(ensure_cells(c, cap_cells, 0));
+    AMFMM_TRY(ensure_cells(c, cap_cells));
     const int64_t cap = static_cast<int64_t>(std::min({c->begin.cap, c->count.cap, c->level.cap, c->parent.cap,
                                                        c->first_child.cap, c->nchild.cap}) /
                                              sizeof(int32_t));
-    k_permute<<<grid_for(n, kBlock), kBlock, 0, st>>>(c->x, c->y, c->z, c->m, skey, sidx, n,
-                                                      ptr<double>(c->X), ptr<double>(c->Y),
-                                                      ptr<double>(c->Zb), ptr<double>(c->Mb),
-                                                      ptr<int32_t>(c->order), lcp, ptr<int32_t>(c->cur),
-                                                      nsys == 1 ? nullptr : ptr<int32_t>(c->sysid));
-    AMFMM_TRY(launched(c, "permute"));
-    k_roots<<<grid_for(nsys, kBlock), kBlock, 0, st>>>(nsys, ptr<int64_t>(c->sys_off), ptr<int32_t>(c->begin),
-                                                       ptr<int32_t>(c->count), ptr<int32_t>(c->level),
-                                                       ptr<int32_t>(c->parent), ptr<int32_t>(c->first_child),
-                                                       ptr<int32_t>(c->nchild), lvl, ovf);
-    AMFMM_TRY(launched(c, "roots"));
-    bool done = false, over = false;
-    int32_t *h = static_cast<int32_t *>(c->hpin);
-    for (lev = 0; !done;) {
-      const int batch = lev == 0 ? std::max(1, c->last_depth + 1) : 2;
-      const int lev_end = std::min(lev + batch, kMaxLevel + 1);
-      for (int l = lev; l < lev_end; ++l) {
-        k_level_flags<<<grid_for(n, kBlock), kBlock, 0, st>>>(
-            n, l, c->opts.n_crit, lcp, ptr<int32_t>(c->begin), ptr<int32_t>(c->count), ptr<int32_t>(c->cur),
-            flag, excl, lvl, ptr<int32_t>(c->cell_at) + static_cast<int64_t>(l) * n, ptr<int32_t>(c->leaf_of), ovf);
-        AMFMM_TRY(launched(c, "level_flags"));
-        AMFMM_TRY(exclusive_scan_i32(c, flag, excl, n, total));
-        k_make_cells<<<grid_for(n, kBlock), kBlock, 0, st>>>(
-            n, l, lvl, total, cap, flag, excl, ptr<int32_t>(c->cur), ptr<int32_t>(c->begin),
-            ptr<int32_t>(c->level), ptr<int32_t>(c->parent), ptr<int32_t>(c->first_child),
-            ptr<int32_t>(c->nchild), ovf);
-        AMFMM_TRY(launched(c, "make_cells"));
-        // no more new cells than bodies
-        k_cell_counts<<<grid_for(n, kBlock), kBlock, 0, st>>>(l, lvl, ptr<int32_t>(c->begin), ptr<int32_t>(c->count),
-                                                             ptr<int32_t>(c->parent), ptr<int32_t>(c->nchild), ovf);
-        AMFMM_TRY(launched(c, "cell_counts"));
-      }
-      const HostRead rb{h, status, sizeof(int) * (8 + kMaxLevel + 3)};
-      AMFMM_TRY(read_back(c, &rb, 1));
-      if (capturing(c)) {
-        // a captured solve keeps the planned cell room
-        if (h[1]) return set_error(c, FMM_ECUDA, "graph capture: the planning solve grew the cell room");
-        Expect e;
-        for (int k = 0; k < 8 + kMaxLevel + 3; ++k) e.add(status + k, static_cast<uint32_t>(h[k]));
-        AMFMM_TRY(graph_expect(c, e));
-        st = c->stream;
-      }
-      const int32_t *hl = h + 8;
-      if (h[1]) {  // out of cell room: grow beyond what the levels so far asked for
-        int64_t need = cap;
-        for (int l = 0; l < lev_end; ++l) need = std::max<int64_t>(need, hl[l + 2]);
-        cap_cells = std::max<int64_t>(2 * cap, need + n / 2 + 64);
-        over = true;
-        break;
-      }
-      for (int l = lev; l < lev_end && !done; ++l)
-        if (hl[l + 2] == hl[l + 1]) {  // level l made no new cells: the tree is complete
-          done = true;
-          lev = l;
-        }
-      if (!done) {
-        if (lev_end > kMaxLevel) return set_error(c, FMM_EINVAL, "octree: cells below the deepest level");
-        lev = lev_end;
-      }
-    }
-    if (over) continue;
-    c->sz.lvl_off.assign(h + 8, h + 8 + lev + 2);
-    break;
+    k_emit_cells<<<nb, kBlock, 0, st>>>(n, ptr<char2>(c->body_lv), offs, cap, ptr<int32_t>(c->begin),
+                                        ptr<int32_t>(c->level), ptr<int32_t>(c->parent), ptr<int32_t>(c->cell_at),
+                                        ptr<int32_t>(c->leaf_of), ptr<int32_t>(c->leaves), lvl);
+    AMFMM_TRY(launched(c, "emit_cells"));
+    k_finish_cells<<<static_cast<unsigned>(std::min<int64_t>(grid_for(std::min(cap, n), kBlock), 8 * c->num_sms)),
+                     kBlock, 0, st>>>(n, n_crit, nsys, cap, ptr<int64_t>(c->sys_off), lvl, ptr<int32_t>(c->begin),
+                                      ptr<int32_t>(c->level), ptr<int32_t>(c->parent), ptr<int32_t>(c->cell_at),
+                                      ptr<int32_t>(c->count), ptr<int32_t>(c->first_child), ptr<int32_t>(c->nchild));
+    AMFMM_TRY(launched(c, "finish_cells"));
+    const HostRead rb[2] = {{h, status, sizeof(int) * kStatusWords}, {hb, bbox, 4 * sizeof(double)}};
+    AMFMM_TRY(read_back(c, rb, 2));
+    if (h[kStatusLvl + kLevels] <= cap) break;
+    // a tree of single-child chains can have more cells than bodies
+    if (capturing(c) || attempt > 0) return set_error(c, FMM_EINVAL, "octree: cell room still short after growing");
+    cap_cells = h[kStatusLvl + kLevels];
   }
-  c->last_depth = lev;
-  c->sz.depth = lev;
-  c->sz.ncell = c->sz.lvl_off.back();
-  // leaves in id order
-  const int64_t nc = c->sz.ncell;
-  AMFMM_TRY(ensure<int32_t>(c, c->leaves, nc + 1));
-  // a tree of single-child chains can have more cells than bodies
+  if (capturing(c)) {
+    AMFMM_TRY(graph_record_bbox(c, bbox));
+    Expect e;
+    for (int k = 0; k < kStatusWords; ++k) e.add(status + k, static_cast<uint32_t>(h[k]));
+    AMFMM_TRY(graph_expect(c, e));
+  }
+  const int32_t *hl = h + kStatusLvl;
+  const int64_t nc = hl[kLevels];
+  int depth = 0;
+  while (depth + 1 < kLevels && hl[depth + 1] < nc) ++depth;
+  c->sz.depth = depth;
+  c->sz.ncell = nc;
+  c->sz.lvl_off.assign(hl, hl + depth + 2);
+  c->sz.nleaf = hl[kLevels + 1];
+  for (int d = 0; d < 3; ++d) c->sz.lo[d] = hb[d];
+  c->sz.scale = hb[3];
+  if (h[0] != 0)
+    return set_error(c, FMM_EINVAL, "a body has a non-finite coordinate or a mass that is not positive and finite");
   AMFMM_TRY(ensure<int32_t>(c, c->flag, std::max(n, nc) + 1));
   AMFMM_TRY(ensure<int32_t>(c, c->incl, std::max(n, nc) + 1));
-  flag = ptr<int32_t>(c->flag);
-  excl = ptr<int32_t>(c->incl);
-  k_leaf_flags<<<grid_for(nc, kBlock), kBlock, 0, st>>>(static_cast<int32_t>(nc), ptr<int32_t>(c->nchild), flag);
-  AMFMM_TRY(launched(c, "leaf_flags"));
-  AMFMM_TRY(exclusive_scan_i32(c, flag, excl, nc, total));
-  k_leaf_compact<<<grid_for(nc, kBlock), kBlock, 0, st>>>(static_cast<int32_t>(nc), ptr<int32_t>(c->nchild),
-                                                          excl, ptr<int32_t>(c->leaves));
-  AMFMM_TRY(launched(c, "leaf_compact"));
-  {
-    int32_t *h = static_cast<int32_t *>(c->hpin);
-    double *hb = reinterpret_cast<double *>(h + 4);
-    const double *bbox = c->sz.nsys == 1 ? ptr<double>(c->bbox) : ptr<double>(c->sbox);
-    const HostRead rb[3] = {{h, total, sizeof(int32_t)}, {h + 1, status, sizeof(int32_t)},
-                            {hb, bbox, 4 * sizeof(double)}};
-    AMFMM_TRY(read_back(c, rb, 3));
-    if (capturing(c)) {
-      AMFMM_TRY(graph_record_bbox(c, bbox));
-      Expect e;
-      e.add(total, static_cast<uint32_t>(h[0]));
-      e.add(status, static_cast<uint32_t>(h[1]));
-      AMFMM_TRY(graph_expect(c, e));
-    }
-    c->sz.nleaf = h[0];
-    for (int d = 0; d < 3; ++d) c->sz.lo[d] = hb[d];
-    c->sz.scale = hb[3];
-    if (h[1] != 0)
-      return set_error(c, FMM_EINVAL, "a body has a non-finite coordinate or a mass that is not positive and finite");
-  }
   return FMM_OK;
 }
 
