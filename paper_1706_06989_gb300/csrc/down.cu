@@ -34,6 +34,12 @@ __device__ __forceinline__ int i3(int i, int j, int k) {
   return 9;                               // zzz
 }
 
+// With h_ij = C_ijk s_k:  C_i' = C_i + (C_ij + h_ij / 2) s_j.
+//
+// A thread per child where a level fills the GPU: 58 FP64 instructions for 32
+// children.  An FP64 instruction holds its pipe for 64 cycles whatever number
+// of lanes work, so on a small level those 58 are a chain of 2 us; there a
+// warp takes one child, a lane per coefficient, with a chain of 9.
 __global__ void k_l2l(int32_t c0, int32_t c1, const int32_t *__restrict__ parent,
                       const double *__restrict__ Z, double *__restrict__ loc) {
   const int c = c0 + blockIdx.x * blockDim.x + threadIdx.x;
@@ -42,34 +48,55 @@ __global__ void k_l2l(int32_t c0, int32_t c1, const int32_t *__restrict__ parent
   const double s[3] = {Z[3 * c] - Z[3 * p], Z[3 * c + 1] - Z[3 * p + 1], Z[3 * c + 2] - Z[3 * p + 2]};
   const double *P = loc + static_cast<int64_t>(p) * kLocStride;
   double *C = loc + static_cast<int64_t>(c) * kLocStride;
-  double Pl[19];
+  double Pl[19], h[6];
 #pragma unroll
   for (int q = 0; q < 19; ++q) Pl[q] = P[q];
-  // C_ijk' = C_ijk (shift adds nothing new)
 #pragma unroll
   for (int q = 0; q < 10; ++q) C[9 + q] += Pl[9 + q];
-  // C_ij' = C_ij + C_ijk s_k
 #pragma unroll
   for (int i = 0; i < 3; ++i)
 #pragma unroll
     for (int j = i; j < 3; ++j) {
-      double v = Pl[3 + i2(i, j)];
-#pragma unroll
-      for (int k = 0; k < 3; ++k) v += Pl[9 + i3(i, j, k)] * s[k];
-      C[3 + i2(i, j)] += v;
+      const int q = i2(i, j);
+      h[q] = Pl[9 + i3(i, j, 0)] * s[0] + Pl[9 + i3(i, j, 1)] * s[1] + Pl[9 + i3(i, j, 2)] * s[2];
+      C[3 + q] += Pl[3 + q] + h[q];
+      h[q] = fma(0.5, h[q], Pl[3 + q]);
     }
-  // C_i' = C_i + C_ij s_j + C_ijk s_j s_k / 2
 #pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    double v = Pl[i], w = 0.0;
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      v += Pl[3 + i2(i, j)] * s[j];
-#pragma unroll
-      for (int k = 0; k < 3; ++k) w += Pl[9 + i3(i, j, k)] * s[j] * s[k];
-    }
-    C[i] += v + 0.5 * w;
+  for (int i = 0; i < 3; ++i) C[i] += Pl[i] + (h[i2(i, 0)] * s[0] + h[i2(i, 1)] * s[1] + h[i2(i, 2)] * s[2]);
+}
+
+constexpr int kL2LWarps = 4;
+
+__global__ void __launch_bounds__(kL2LWarps * 32) k_l2l_warp(int32_t c0, int32_t c1,
+                                                             const int32_t *__restrict__ parent,
+                                                             const double *__restrict__ Z, double *__restrict__ loc) {
+  __shared__ double sp[kL2LWarps][kLocStride], sh[kL2LWarps][6];
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+  const int c = c0 + blockIdx.x * kL2LWarps + w;
+  if (c >= c1) return;  // whole warp
+  const int p = parent[c];
+  double own = 0.0, up = 0.0;
+  if (l < 19) {
+    own = loc[static_cast<int64_t>(c) * kLocStride + l];
+    sp[w][l] = up = loc[static_cast<int64_t>(p) * kLocStride + l];
   }
+  double s = 0.0;
+  if (l < 3) s = Z[3 * c + l] - Z[3 * p + l];
+  const double s0 = __shfl_sync(0xffffffffu, s, 0), s1 = __shfl_sync(0xffffffffu, s, 1),
+               s2 = __shfl_sync(0xffffffffu, s, 2);
+  __syncwarp();
+  const int q = l - 3;                             // this lane's C_ij
+  const int i = q < 3 ? 0 : q < 5 ? 1 : 2;
+  const int j = q < 3 ? q : q < 5 ? q - 2 : 2;
+  if (q >= 0 && q < 6) {
+    const double h = sp[w][9 + i3(i, j, 0)] * s0 + sp[w][9 + i3(i, j, 1)] * s1 + sp[w][9 + i3(i, j, 2)] * s2;
+    sh[w][q] = fma(0.5, h, up);
+    up += h;
+  }
+  __syncwarp();
+  if (l < 3) up += sh[w][i2(l, 0)] * s0 + sh[w][i2(l, 1)] * s1 + sh[w][i2(l, 2)] * s2;
+  if (l < 19) loc[static_cast<int64_t>(c) * kLocStride + l] = own + up;
 }
 
 __global__ void k_l2p(int64_t n, const int32_t *__restrict__ leaf_of, const double *__restrict__ Z,
@@ -112,12 +139,16 @@ int downward(fmm_ctx *c) {
   const int64_t n = c->sz.n;
   AMFMM_TRY(ensure<double>(c, c->acc, 3 * n));
   if (c->opts.order_P != 3) return downward_general(c);
+  const int64_t fill = std::max(1, c->num_sms);
   for (int lev = 1; lev <= c->sz.depth; ++lev) {
     const int64_t c0 = c->sz.lvl_off[lev], c1 = c->sz.lvl_off[lev + 1];
     if (c1 <= c0) continue;
-    k_l2l<<<grid_for(c1 - c0, 128), 128, 0, st>>>(static_cast<int32_t>(c0), static_cast<int32_t>(c1),
-                                                   ptr<int32_t>(c->parent), ptr<double>(c->Z),
-                                                   ptr<double>(c->loc));
+    const bool many = c1 - c0 >= 16 * fill;  // then a thread per child has fewer instructions in all
+    const auto down = many ? k_l2l : k_l2l_warp;
+    const int threads = many ? 128 : kL2LWarps * 32;
+    down<<<grid_for(c1 - c0, many ? 128 : kL2LWarps), threads, 0, st>>>(
+        static_cast<int32_t>(c0), static_cast<int32_t>(c1), ptr<int32_t>(c->parent), ptr<double>(c->Z),
+        ptr<double>(c->loc));
     AMFMM_TRY(launched(c, "l2l"));
   }
   k_l2p<<<grid_for(n, 256), 256, 0, st>>>(n, ptr<int32_t>(c->leaf_of), ptr<double>(c->Z), ptr<double>(c->loc),

@@ -29,6 +29,22 @@ struct Err {
   std::string msg;
 };
 
+// A body as hi + lo floats: differences formed from them keep FP32 relative
+// accuracy for close positions too.
+struct BodyF {
+  float4 h;  // x, y, z hi; mass
+  float4 l;  // x, y, z lo
+};
+#ifdef __CUDACC__
+__device__ __forceinline__ BodyF split_body(double x, double y, double z, double m) {
+  const float hx = static_cast<float>(x), hy = static_cast<float>(y), hz = static_cast<float>(z);
+  BodyF b;
+  b.h = make_float4(hx, hy, hz, static_cast<float>(m));
+  b.l = make_float4(static_cast<float>(x - hx), static_cast<float>(y - hy), static_cast<float>(z - hz), 0.f);
+  return b;
+}
+#endif
+
 // Per-solve sizes read back to the host.
 struct Sizes {
   int64_t n = 0, ncell = 0, nleaf = 0, n_m2l = 0, n_p2p = 0, n_self = 0;
@@ -131,11 +147,11 @@ struct fmm_ctx {
 
   // ---- device buffers ----
   // bodies
-  amfmm::DBuf key[2], idx[2], order, X, Y, Zb, Mb, flag, incl, lcp, body_lv, leaf_of, cell_at,
+  amfmm::DBuf key[2], idx[2], order, X, Y, Zb, Mb, bodyf, flag, incl, lcp, body_lv, leaf_of, cell_at,
       near, acc, status, bbox_part, bbox, sys_off, sysid, sbox;
   // cells
   amfmm::DBuf begin, count, level, parent, first_child, nchild, S, M, Z, invM, Rmax,
-      rmax2, mom, loc, leaves;
+      rmax2, cellzf, mom, loc, leaves;
   // walk
   amfmm::DBuf front[2], m2l, p2p, self_list, walk_zr, walk_zf, walk_nl, walk_state, walk_lb;
   unsigned walk_epoch = 0;  // epochs of the single-pass walk generations
@@ -143,7 +159,7 @@ struct fmm_ctx {
   amfmm::DBuf ekey[2], eval[2], m2l_pos, m2l_off, m2l_slots, cell32, qoh;
   // P2P grouping
   amfmm::DBuf pkey[2], pval[2], p2p_A, p2p_offA, p2p_offB, p2p_pos, p2p_poff, p2p_len,
-      p2p_slots, p2p_colOff, p2p_cols, p2p_nb, p2p_pre, p2p_bodyf, p2p_items, p2p_itemOff, p2p_extraOff,
+      p2p_slots, p2p_colOff, p2p_cols, p2p_nb, p2p_pre, p2p_rec, p2p_items, p2p_itemOff, p2p_extraOff,
       p2p_extra, p2p_heavy;
   // scan / sort scratch; `totals` holds small device results (1 KiB):
   // [0,16) scan totals, [64,72) near-field body-pair count, [80,88) selector-scored pairs, [88,92) selector candidates, [96,104) slot total,

@@ -88,26 +88,9 @@ __device__ __forceinline__ void rows32(P2PSmem<ROWS> &sm, int i, int l, bool val
   }
 }
 
-// Mixed form: bodies and the leaf centre as hi + lo floats, so an offset
+// Bodies and the leaf centre are hi + lo floats, so an offset
 // (x_hi - z_hi) + (x_lo - z_lo) is formed with FP32 operations only (FP64
 // costs 64 FP32 operations on this GPU) and keeps FP32 relative accuracy.
-struct BodyF {
-  float4 h;  // x, y, z hi; mass
-  float4 l;  // x, y, z lo
-};
-
-__global__ void k_body32(int64_t n, const double *__restrict__ X, const double *__restrict__ Y,
-                         const double *__restrict__ Zb, const double *__restrict__ Mb, BodyF *__restrict__ out) {
-  const int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
-  if (i >= n) return;
-  const double x = X[i], y = Y[i], z = Zb[i];
-  const float hx = static_cast<float>(x), hy = static_cast<float>(y), hz = static_cast<float>(z);
-  BodyF b;
-  b.h = make_float4(hx, hy, hz, static_cast<float>(Mb[i]));
-  b.l = make_float4(static_cast<float>(x - hx), static_cast<float>(y - hy), static_cast<float>(z - hz), 0.f);
-  out[i] = b;
-}
-
 __device__ __forceinline__ float3 offset32(const BodyF &b, const float4 zh, const float4 zl) {
   return make_float3((b.h.x - zh.x) + (b.l.x - zl.x), (b.h.y - zh.y) + (b.l.y - zl.y),
                      (b.h.z - zh.z) + (b.l.z - zl.z));
@@ -497,7 +480,7 @@ int launch_p2p_rows(fmm_ctx *c) {
   k_p2p<ROWS><<<grid, kWarps * 32, shm, c->stream>>>(
       nitem, n, ptr<int4>(c->p2p_items), ptr<int32_t>(c->begin), ptr<int32_t>(c->count),
       ptr<double>(c->Z), ptr<int2>(c->p2p_cols), ptr<double>(c->near), ptr<double>(c->p2p_extra),
-      static_cast<float *>(c->p2p_slots.p), ptr<BodyF>(c->p2p_bodyf), static_cast<float>(c->eps2), queue);
+      static_cast<float *>(c->p2p_slots.p), ptr<BodyF>(c->bodyf), static_cast<float>(c->eps2), queue);
   AMFMM_TRY(launched(c, "p2p"));
   if (nitem > nleaf) {
     k_p2p_chunks<<<grid_for(static_cast<int64_t>(nleaf) * 32, 256), 256, 0, c->stream>>>(
@@ -528,10 +511,6 @@ int p2p_prepare(fmm_ctx *c) {
   unsigned long long *stat = ptr<unsigned long long>(c->totals) + 8;
   int32_t *ctot = ptr<int32_t>(c->totals) + 32;
   AMFMM_CUDA(c, cudaMemsetAsync(stat, 0, sizeof(unsigned long long), st));
-  AMFMM_TRY(ensure<BodyF>(c, c->p2p_bodyf, n));
-  k_body32<<<grid_for(n, 256), 256, 0, st>>>(n, ptr<double>(c->X), ptr<double>(c->Y), ptr<double>(c->Zb),
-                                             ptr<double>(c->Mb), ptr<BodyF>(c->p2p_bodyf));
-  AMFMM_TRY(launched(c, "p2p_body32"));
   AMFMM_TRY(ensure<int32_t>(c, c->p2p_nb, K + 1));
   AMFMM_TRY(ensure<int32_t>(c, c->p2p_pre, K + 1));
   int32_t *nb = ptr<int32_t>(c->p2p_nb), *pre = ptr<int32_t>(c->p2p_pre);

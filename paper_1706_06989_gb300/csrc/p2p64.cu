@@ -437,16 +437,16 @@ int p2p64_prepare(fmm_ctx *c) {
   AMFMM_TRY(ensure<int32_t>(c, c->p2p_itemOff, nleaf + 1));
   AMFMM_TRY(ensure<int32_t>(c, c->p2p_extraOff, nleaf + 1));
   AMFMM_TRY(ensure<int32_t>(c, c->incl, std::max<int64_t>(nc + 1, n + 1)));
-  AMFMM_TRY(ensure<Rec>(c, c->p2p_bodyf, n));
+  AMFMM_TRY(ensure<Rec>(c, c->p2p_rec, n));
   const bool forest = c->sz.nsys > 1;
   k_body_fixed<<<grid_for(n, 256), 256, 0, st>>>(
       n, ptr<double>(c->X), ptr<double>(c->Y), ptr<double>(c->Zb), ptr<double>(c->Mb),
       forest ? ptr<double>(c->sbox) : ptr<double>(c->bbox), ptr<int32_t>(c->order),
-      forest ? ptr<int32_t>(c->sysid) : nullptr, ptr<Rec>(c->p2p_bodyf));
+      forest ? ptr<int32_t>(c->sysid) : nullptr, ptr<Rec>(c->p2p_rec));
   AMFMM_TRY(launched(c, "p2p_body_fixed"));
   AMFMM_TRY(ensure<int2>(c, c->p2p_heavy, nc));
   k_leaf_heavy<<<grid_for(32 * static_cast<int64_t>(nleaf), 256), 256, 0, st>>>(
-      nleaf, ptr<int32_t>(c->leaves), ptr<int32_t>(c->begin), ptr<int32_t>(c->count), ptr<Rec>(c->p2p_bodyf),
+      nleaf, ptr<int32_t>(c->leaves), ptr<int32_t>(c->begin), ptr<int32_t>(c->count), ptr<Rec>(c->p2p_rec),
       ptr<int2>(c->p2p_heavy));
   AMFMM_TRY(launched(c, "p2p_leaf_heavy"));
   // every leaf's partners, in the stable order of the pair list
@@ -500,7 +500,7 @@ int p2p64_run(fmm_ctx *c) {
   kern<<<grid, kWarps * 32, 0, c->stream>>>(
       nitem, c->sz.n, ptr<int4>(c->p2p_items), ptr<int32_t>(c->begin), ptr<int32_t>(c->count),
       ptr<int32_t>(c->p2p_offA), c->sz.n_p2p > 0 ? ptr<uint32_t>(c->pval[c->p2p_which]) : nullptr,
-      ptr<int2>(c->p2p_heavy), ptr<Rec>(c->p2p_bodyf), ptr<double>(c->X), ptr<double>(c->Y), ptr<double>(c->Zb),
+      ptr<int2>(c->p2p_heavy), ptr<Rec>(c->p2p_rec), ptr<double>(c->X), ptr<double>(c->Y), ptr<double>(c->Zb),
       ptr<double>(c->Mb), c->eps2, ptr<double>(c->near), ptr<double>(c->p2p_extra), queue);
   AMFMM_TRY(launched(c, "p2p"));
   if (c->sz.n_p2p == 0) return FMM_OK;

@@ -209,20 +209,23 @@ __global__ void k_gather_sorted(int64_t n, const uint32_t *__restrict__ perm, co
   i2[t] = i1[perm[t]];
 }
 
-// Gather the bodies into key order.
+// Gather the bodies into key order, also as hi + lo floats (R_max, and the
+// mixed form's near field).
 __global__ void k_permute(const double *__restrict__ x, const double *__restrict__ y,
                           const double *__restrict__ z, const double *__restrict__ m,
                           const uint32_t *__restrict__ idx, int64_t n, double *__restrict__ X,
                           double *__restrict__ Y, double *__restrict__ Zb, double *__restrict__ Mb,
-                          int32_t *__restrict__ order) {
+                          int32_t *__restrict__ order, BodyF *__restrict__ bodyf) {
   int64_t s = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (s >= n) return;
   const uint32_t o = idx[s];
-  X[s] = x[o];
-  Y[s] = y[o];
-  Zb[s] = z[o];
-  Mb[s] = m[o];
+  const double xs = x[o], ys = y[o], zs = z[o], ms = m[o];
+  X[s] = xs;
+  Y[s] = ys;
+  Zb[s] = zs;
+  Mb[s] = ms;
   order[s] = static_cast<int32_t>(o);
+  bodyf[s] = split_body(xs, ys, zs, ms);
 }
 
 // ---------------------------------------------------------------------------
@@ -414,52 +417,131 @@ __global__ void k_finish_cells(int64_t n, int n_crit, int nsys, int64_t cap, con
 // ---------------------------------------------------------------------------
 // Moments about Z in the order M, x, y, z, xx, xy, xz, yy, yz, zz, xxx, xxy,
 // xxz, xyy, xyz, xzz, yyy, yyz, yzz, zzz.
-__device__ __forceinline__ void add_body_moments(double *mo, double mu, double x, double y, double z) {
-  const double mx = mu * x, my = mu * y, mz = mu * z;
-  mo[0] += mu;
-  mo[1] += mx;
-  mo[2] += my;
-  mo[3] += mz;
-  const double mxx = mx * x, mxy = mx * y, mxz = mx * z, myy = my * y, myz = my * z, mzz = mz * z;
-  mo[4] += mxx;
-  mo[5] += mxy;
-  mo[6] += mxz;
-  mo[7] += myy;
-  mo[8] += myz;
-  mo[9] += mzz;
-  mo[10] += mxx * x;
-  mo[11] += mxx * y;
-  mo[12] += mxx * z;
-  mo[13] += myy * x;
-  mo[14] += mxy * z;
-  mo[15] += mzz * x;
-  mo[16] += myy * y;
-  mo[17] += myy * z;
-  mo[18] += mzz * y;
-  mo[19] += mzz * z;
-}
+//
+// An FP64 instruction holds its pipe for 64 cycles per warp, however many of
+// its lanes work, so what counts here is the number of FP64 warp instructions:
+// their total where a level fills the GPU, their chain where it does not.
+//
+// Leaves: a warp takes G leaves and 32 of their bodies at a time.  The centre
+// of mass is summed in body order (as its definition here demands), one lane
+// per (leaf, component); then each lane forms its body's offset and the ten
+// products of up to second order, and one lane per (leaf, moment) sums in body
+// order with one FMA per body.  About 17 FP64 warp instructions per leaf at
+// G = 8 against 27 with a thread per leaf (leaves differ in size), and a chain
+// of about 75 instead of 1,100 for a leaf of 25 bodies.
+// A moment as (base product of up to second order) x coordinate: base 0..9 =
+// mu, mx, my, mz, mxx, mxy, mxz, myy, myz, mzz; coordinate 0..2, 3: one.
+__constant__ signed char c_mom_base[kMomStride] = {0, 0, 0, 0, 1, 1, 1, 2, 2, 3, 4, 4, 4, 7, 5, 9, 7, 7, 9, 9};
+__constant__ signed char c_mom_coord[kMomStride] = {3, 0, 1, 2, 0, 1, 2, 1, 2, 2, 0, 1, 2, 0, 2, 0, 1, 2, 1, 2};
+constexpr int kUpWarps = 4;
 
-__global__ void k_leaf_upward(int32_t nleaf, const int32_t *__restrict__ leaves,
-                              const int32_t *__restrict__ begin, const int32_t *__restrict__ count,
-                              const double *__restrict__ X, const double *__restrict__ Y,
-                              const double *__restrict__ Zb, const double *__restrict__ Mb,
-                              double *__restrict__ S, double *__restrict__ M, double *__restrict__ Z,
-                              double *__restrict__ invM, double *__restrict__ mom) {
-  int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= nleaf) return;
-  const int c = leaves[q];
-  const int b = begin[c], e = b + count[c];
-  double zc[3];
-  leaf_com(c, b, e, X, Y, Zb, Mb, S, M, Z, invM, zc);
-  const double zx = zc[0], zy = zc[1], zz = zc[2], mm = M[c];
-  double mo[kMomStride];
+template <int G>
+__global__ void __launch_bounds__(kUpWarps * 32) k_leaf_upward(
+    int32_t nleaf, const int32_t *__restrict__ leaves, const int32_t *__restrict__ begin,
+    const int32_t *__restrict__ count, const double *__restrict__ X, const double *__restrict__ Y,
+    const double *__restrict__ Zb, const double *__restrict__ Mb, double *__restrict__ S, double *__restrict__ M,
+    double *__restrict__ Z, double *__restrict__ invM, double *__restrict__ mom) {
+  constexpr int kRounds = (G * kMomStride + 31) / 32;
+  __shared__ double sh[kUpWarps][14][33];  // per body: ten products, x, y, z, 1 (first: mu x, mu y, mu z, mu)
+  __shared__ double com[kUpWarps][G][4];
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+  const int q0 = (blockIdx.x * kUpWarps + w) * G;
+  if (q0 >= nleaf) return;  // whole warp
+  const int ng = min(G, nleaf - q0);
+  const int c = l < ng ? leaves[q0 + l] : 0;
+  const int b = l < ng ? begin[c] : 0, cnt = l < ng ? count[c] : 0;
+  int end = cnt;  // inclusive prefix: leaf g owns concatenated bodies [end - cnt, end)
 #pragma unroll
-  for (int k = 0; k < kMomStride; ++k) mo[k] = 0.0;
-  for (int i = b; i < e; ++i) add_body_moments(mo, Mb[i], X[i] - zx, Y[i] - zy, Zb[i] - zz);
-  mo[0] = mm;
-  double *out = mom + static_cast<int64_t>(c) * kMomStride;
+  for (int o = 1; o < G; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, end, o);
+    if (l >= o) end += y;
+  }
+  const int total = __shfl_sync(0xffffffffu, end, ng - 1);
+  // body of lane l in the tile at t0, and its leaf
+  const auto locate = [&](int t0, int &g) {
+    const int t = t0 + l;
+    g = 0;
 #pragma unroll
-  for (int k = 0; k < kMomStride; ++k) out[k] = mo[k];
+    for (int k = 0; k < G - 1; ++k) g += t >= __shfl_sync(0xffffffffu, end, k) ? 1 : 0;
+    g = min(g, ng - 1);
+    const int bg = __shfl_sync(0xffffffffu, b, g), eg = __shfl_sync(0xffffffffu, end, g),
+              cg = __shfl_sync(0xffffffffu, cnt, g);
+    return bg + (t - (eg - cg));
+  };
+  // bodies of leaf g in the tile at t0: lanes [lo, hi)
+  const int cg4 = l >> 2;  // leaf of this lane's centre-of-mass component
+  const int ce = __shfl_sync(0xffffffffu, end, cg4 < G ? cg4 : 0), cc = __shfl_sync(0xffffffffu, cnt, cg4 < G ? cg4 : 0);
+  double s = 0.0;
+  for (int t0 = 0; t0 < total; t0 += 32) {
+    int g;
+    const int i = locate(t0, g);
+    if (t0 + l < total) {
+      const double mu = Mb[i];
+      sh[w][0][l] = __dmul_rn(mu, X[i]);
+      sh[w][1][l] = __dmul_rn(mu, Y[i]);
+      sh[w][2][l] = __dmul_rn(mu, Zb[i]);
+      sh[w][3][l] = mu;
+    }
+    __syncwarp();
+    if (cg4 < ng)
+      for (int k = max(ce - cc - t0, 0); k < min(ce - t0, 32); ++k) s = __dadd_rn(s, sh[w][l & 3][k]);
+    __syncwarp();
+  }
+  const double mm = __shfl_sync(0xffffffffu, s, (l & ~3) + 3);
+  const double z = __ddiv_rn((l & 3) == 3 ? 1.0 : s, mm);
+  if (cg4 < ng) {
+    const int cell = leaves[q0 + cg4];
+    com[w][cg4][l & 3] = (l & 3) == 3 ? mm : z;
+    if ((l & 3) == 3) {
+      M[cell] = mm;
+      invM[cell] = z;
+    } else {
+      S[3 * cell + (l & 3)] = s;
+      Z[3 * cell + (l & 3)] = z;
+    }
+  }
+  __syncwarp();
+  double acc[kRounds];
+#pragma unroll
+  for (int r = 0; r < kRounds; ++r) acc[r] = 0.0;
+  for (int t0 = 0; t0 < total; t0 += 32) {
+    int g;
+    const int i = locate(t0, g);
+    if (t0 + l < total) {
+      const double mu = Mb[i], x = X[i] - com[w][g][0], y = Y[i] - com[w][g][1], zz = Zb[i] - com[w][g][2];
+      const double mx = mu * x, my = mu * y, mz = mu * zz;
+      sh[w][0][l] = mu;
+      sh[w][1][l] = mx;
+      sh[w][2][l] = my;
+      sh[w][3][l] = mz;
+      sh[w][4][l] = mx * x;
+      sh[w][5][l] = mx * y;
+      sh[w][6][l] = mx * zz;
+      sh[w][7][l] = my * y;
+      sh[w][8][l] = my * zz;
+      sh[w][9][l] = mz * zz;
+      sh[w][10][l] = x;
+      sh[w][11][l] = y;
+      sh[w][12][l] = zz;
+      sh[w][13][l] = 1.0;
+    }
+    __syncwarp();
+#pragma unroll
+    for (int r = 0; r < kRounds; ++r) {
+      const int task = l + 32 * r, tg = task / kMomStride, q = task - tg * kMomStride;
+      const int te = __shfl_sync(0xffffffffu, end, tg < G ? tg : 0), tc = __shfl_sync(0xffffffffu, cnt, tg < G ? tg : 0);
+      if (tg < ng) {
+        const double *p = sh[w][c_mom_base[q]], *x = sh[w][10 + c_mom_coord[q]];
+        for (int k = max(te - tc - t0, 0); k < min(te - t0, 32); ++k) acc[r] = fma(p[k], x[k], acc[r]);
+      }
+    }
+    __syncwarp();
+  }
+#pragma unroll
+  for (int r = 0; r < kRounds; ++r) {
+    const int task = l + 32 * r, tg = task / kMomStride, q = task - tg * kMomStride;
+    if (tg < ng) mom[static_cast<int64_t>(leaves[q0 + tg]) * kMomStride + q] = q == 0 ? com[w][tg][3] : acc[r];
+  }
 }
 
 // One level of internal cells: S, M from the children in octant order, then
@@ -470,177 +552,178 @@ __global__ void k_leaf_upward(int32_t nleaf, const int32_t *__restrict__ leaves,
 // The child dipoles D' (zero about a centre of mass up to rounding, Sec. 2)
 // are left out of the shift; the parent's dipole is the shift of the child
 // monopoles, D_i = Sum M' s_i.
-__global__ void k_internal_upward(int32_t c0, int32_t c1, const int32_t *__restrict__ first_child,
-                                  const int32_t *__restrict__ nchild, double *__restrict__ S,
-                                  double *__restrict__ M, double *__restrict__ Z,
-                                  double *__restrict__ invM, double *__restrict__ mom) {
-  const int c = c0 + blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= c1) return;
-  const int nch = nchild[c];
-  if (nch == 0) return;
-  const int f = first_child[c];
-  double zc[3];
-  parent_com(c, f, nch, S, M, Z, invM, zc);
-  const double zx = zc[0], zy = zc[1], zz = zc[2], mm = M[c];
-  double p[kMomStride];
+// A warp takes CELLS parents, eight lanes each, one per child: a lane shifts its
+// child's moments, and one lane per (parent, moment) adds the shifted ones in
+// octant order.  About 120 FP64 warp instructions whatever the number of
+// parents in the warp; a thread per parent had a chain of 600 (52 us per level
+// of 4,000 to 16,000 cells), a warp per parent one of 170 (14 to 21 us).
+template <int CELLS>
+__global__ void __launch_bounds__(kUpWarps * 32) k_internal_upward(
+    int32_t c0, int32_t c1, const int32_t *__restrict__ first_child, const int32_t *__restrict__ nchild,
+    double *__restrict__ S, double *__restrict__ M, double *__restrict__ Z, double *__restrict__ invM,
+    double *__restrict__ mom) {
+  constexpr int kRounds = (CELLS * kMomStride + 31) / 32;
+  __shared__ double sh[kUpWarps][kMomStride][33];
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+  const int64_t first = c0 + static_cast<int64_t>(blockIdx.x * kUpWarps + w) * CELLS;
+  if (first >= c1) return;  // whole warp
+  const int g = l >> 3, k = l & 7;
+  const int64_t cc = first + g;
+  const int c = static_cast<int>(cc);
+  const int nch = g < CELLS && cc < c1 ? nchild[c] : 0;
+  const int f = nch > 0 ? first_child[c] : 0;
+  const bool child = k < nch;
+  double zk[3] = {0.0, 0.0, 0.0}, q[kMomStride];
 #pragma unroll
-  for (int k = 0; k < kMomStride; ++k) p[k] = 0.0;
-  for (int k = f; k < f + nch; ++k) {
-    const double *q = mom + static_cast<int64_t>(k) * kMomStride;
-    const double s[3] = {Z[3 * k] - zx, Z[3 * k + 1] - zy, Z[3 * k + 2] - zz};
-    const double Mc = q[0];
-    const double Ms[3] = {Mc * s[0], Mc * s[1], Mc * s[2]};
-    // symmetric Q' as a full matrix
+  for (int t = 0; t < kMomStride; ++t) q[t] = 0.0;
+  if (child) {
+    const double *qk = mom + static_cast<int64_t>(f + k) * kMomStride;
+#pragma unroll
+    for (int t = 0; t < kMomStride; ++t) q[t] = qk[t];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      zk[d] = Z[3 * (f + k) + d];
+      sh[w][d][l] = S[3 * (f + k) + d];
+    }
+    sh[w][3][l] = M[f + k];
+  }
+  __syncwarp();
+  // lane d of a group sums component d (lane 3: the mass)
+  double s = 0.0;
+  if (k < 4)
+    for (int j = 0; j < nch; ++j) s = __dadd_rn(s, sh[w][k][8 * g + j]);
+  const double mm = __shfl_sync(0xffffffffu, s, 8 * g + 3);
+  const double z = __ddiv_rn(k == 3 ? 1.0 : s, mm);
+  if (nch > 0 && k < 4) {
+    if (k == 3) {
+      M[c] = mm;
+      invM[c] = z;
+    } else {
+      S[3 * c + k] = s;
+      Z[3 * c + k] = z;
+    }
+  }
+  double sv[3];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) sv[d] = zk[d] - __shfl_sync(0xffffffffu, z, 8 * g + d);
+  __syncwarp();
+  if (child) {
+    const double Ms[3] = {q[0] * sv[0], q[0] * sv[1], q[0] * sv[2]};
     const double Q[3][3] = {{q[4], q[5], q[6]}, {q[5], q[7], q[8]}, {q[6], q[8], q[9]}};
 #pragma unroll
-    for (int i = 0; i < 3; ++i) p[1 + i] += Ms[i];
-    // Q: xx xy xz yy yz zz
+    for (int d = 0; d < 3; ++d) sh[w][1 + d][l] = Ms[d];
     const int qi[6] = {0, 0, 0, 1, 1, 2}, qj[6] = {0, 1, 2, 1, 2, 2};
 #pragma unroll
-    for (int t = 0; t < 6; ++t) p[4 + t] += Q[qi[t]][qj[t]] + Ms[qi[t]] * s[qj[t]];
-    // O: xxx xxy xxz xyy xyz xzz yyy yyz yzz zzz
+    for (int t = 0; t < 6; ++t) sh[w][4 + t][l] = q[4 + t] + Ms[qi[t]] * sv[qj[t]];
     const int oi[10] = {0, 0, 0, 0, 0, 0, 1, 1, 1, 2};
     const int oj[10] = {0, 0, 0, 1, 1, 2, 1, 1, 2, 2};
     const int ok[10] = {0, 1, 2, 1, 2, 2, 1, 2, 2, 2};
 #pragma unroll
     for (int t = 0; t < 10; ++t) {
-      const int i = oi[t], j = oj[t], l = ok[t];
-      p[10 + t] += q[10 + t] + (Q[i][j] * s[l] + Q[i][l] * s[j] + Q[j][l] * s[i]) + Ms[i] * s[j] * s[l];
+      const int a = oi[t], b = oj[t], e = ok[t];
+      sh[w][10 + t][l] = q[10 + t] + (Q[a][b] * sv[e] + Q[a][e] * sv[b] + Q[b][e] * sv[a]) + Ms[a] * sv[b] * sv[e];
     }
   }
-  p[0] = mm;
-  double *out = mom + static_cast<int64_t>(c) * kMomStride;
+  __syncwarp();
 #pragma unroll
-  for (int k = 0; k < kMomStride; ++k) out[k] = p[k];
-}
-
-// index tables of the symmetric moments: Q in the order xx xy xz yy yz zz,
-// O in the order xxx xxy xxz xyy xyz xzz yyy yyz yzz zzz
-__constant__ int c_q2i[6] = {0, 0, 0, 1, 1, 2}, c_q2j[6] = {0, 1, 2, 1, 2, 2};
-__constant__ int c_o3i[10] = {0, 0, 0, 0, 0, 0, 1, 1, 1, 2};
-__constant__ int c_o3j[10] = {0, 0, 0, 1, 1, 2, 1, 1, 2, 2};
-__constant__ int c_o3k[10] = {0, 1, 2, 1, 2, 2, 1, 2, 2, 2};
-// position of Q_ab in that order
-__device__ __forceinline__ int sym2(int a, int b) {
-  const int lo = min(a, b), hi = max(a, b);
-  return lo * 3 - lo * (lo - 1) / 2 + (hi - lo);
-}
-
-// The same level with one warp per cell, for levels of few cells.  With one
-// thread per cell a small level is a single warp's chain of FP64 operations,
-// and an FP64 warp instruction takes many cycles on this GPU (the top
-// levels took 30-40 us each).  Here lane k loads child k, every lane forms
-// the same octant-order sums of S and M from the shuffled child values (so Z
-// is bit-identical to the one-thread form), and lane q then adds moment
-// component q over the children in child order.
-__global__ void k_internal_upward_warp(int32_t c0, int32_t c1, const int32_t *__restrict__ first_child,
-                                       const int32_t *__restrict__ nchild, double *__restrict__ S,
-                                       double *__restrict__ M, double *__restrict__ Z,
-                                       double *__restrict__ invM, double *__restrict__ mom) {
-  const int64_t wg = (blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  const int64_t cc = c0 + wg;
-  if (cc >= c1) return;  // whole warp
-  const int c = static_cast<int>(cc);
-  const int nch = nchild[c];
-  if (nch == 0) return;  // whole warp
-  const int f = first_child[c];
-  double sx = 0.0, sy = 0.0, sz = 0.0, mc = 0.0;
-  if (lane < nch) {
-    sx = S[3 * (f + lane)];
-    sy = S[3 * (f + lane) + 1];
-    sz = S[3 * (f + lane) + 2];
-    mc = M[f + lane];
-  }
-  double tx = 0.0, ty = 0.0, tz = 0.0, tm = 0.0;
-#pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    const double vx = __shfl_sync(0xffffffffu, sx, j), vy = __shfl_sync(0xffffffffu, sy, j);
-    const double vz = __shfl_sync(0xffffffffu, sz, j), vm = __shfl_sync(0xffffffffu, mc, j);
-    if (j < nch) {
-      tx = __dadd_rn(tx, vx);
-      ty = __dadd_rn(ty, vy);
-      tz = __dadd_rn(tz, vz);
-      tm = __dadd_rn(tm, vm);
+  for (int r = 0; r < kRounds; ++r) {
+    const int task = l + 32 * r, tg = task / kMomStride, t = task - tg * kMomStride;
+    const int n = __shfl_sync(0xffffffffu, nch, tg < CELLS ? 8 * tg : 0);
+    const double total = __shfl_sync(0xffffffffu, mm, tg < CELLS ? 8 * tg : 0);
+    if (tg < CELLS && n > 0) {
+      double a = 0.0;
+      if (t > 0)
+        for (int j = 0; j < n; ++j) a += sh[w][t][8 * tg + j];
+      mom[(first + tg) * kMomStride + t] = t == 0 ? total : a;
     }
   }
-  const double zx = __ddiv_rn(tx, tm), zy = __ddiv_rn(ty, tm), zz = __ddiv_rn(tz, tm);
-  if (lane == 0) {
-    S[3 * c] = tx;
-    S[3 * c + 1] = ty;
-    S[3 * c + 2] = tz;
-    M[c] = tm;
-    Z[3 * c] = zx;
-    Z[3 * c + 1] = zy;
-    Z[3 * c + 2] = zz;
-    invM[c] = 1.0 / tm;
-    mom[static_cast<int64_t>(c) * kMomStride] = tm;
-  }
-  const int q = lane;
-  if (q < 1 || q >= kMomStride) return;
-  // component q: 1..3 dipole (i), 4..9 Q (i, j), 10..19 O (i, j, l); the
-  // indices of this lane, and the slots of the Q entries it needs
-  int i = 0, j = 0, l = 0;
-  if (q < 4) {
-    i = q - 1;
-  } else if (q < 10) {
-    i = c_q2i[q - 4];
-    j = c_q2j[q - 4];
-  } else {
-    i = c_o3i[q - 10];
-    j = c_o3j[q - 10];
-    l = c_o3k[q - 10];
-  }
-  const int qij = 4 + sym2(i, j), qil = 4 + sym2(i, l), qjl = 4 + sym2(j, l);
-  double acc = 0.0;
-  for (int k = f; k < f + nch; ++k) {
-    const double *cq = mom + static_cast<int64_t>(k) * kMomStride;
-    const double s0 = Z[3 * k] - zx, s1 = Z[3 * k + 1] - zy, s2 = Z[3 * k + 2] - zz;
-    const double si = i == 0 ? s0 : (i == 1 ? s1 : s2);
-    const double sj = j == 0 ? s0 : (j == 1 ? s1 : s2);
-    const double sl = l == 0 ? s0 : (l == 1 ? s1 : s2);
-    const double Msi = cq[0] * si;
-    if (q < 4) acc += Msi;
-    else if (q < 10) acc += cq[q] + Msi * sj;
-    else acc += cq[q] + (cq[qij] * sl + cq[qil] * sj + cq[qjl] * si) + Msi * sj * sl;
-  }
-  mom[static_cast<int64_t>(c) * kMomStride + q] = acc;
 }
 
-// R_max^2 of every cell: for each level, each body's squared distance to the
-// centre of its cell at that level; a segmented warp maximum (bodies of one
-// cell are contiguous) and one atomicMax per segment, both on the bit pattern
-// (monotone for non-negative doubles, and integer work, which keeps the
-// maximum off the FP64 pipe).  max is exact, so the order of combination
-// does not matter.
-__global__ void k_rmax_bodies(int64_t n, const int32_t *__restrict__ cell_at,
-                              const double *__restrict__ X, const double *__restrict__ Y,
-                              const double *__restrict__ Zb, const double *__restrict__ Z,
-                              unsigned long long *__restrict__ rmax2) {
-  const int lev = blockIdx.y;
+// Centres as hi + lo floats for the filter of R_max.
+__global__ void k_split_centres(int32_t ncell, const double *__restrict__ Z, float4 *__restrict__ zf) {
+  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  if (c >= ncell) return;
+  const double x = Z[3 * c], y = Z[3 * c + 1], z = Z[3 * c + 2];
+  const float hx = static_cast<float>(x), hy = static_cast<float>(y), hz = static_cast<float>(z);
+  zf[2 * c] = make_float4(hx, hy, hz, 0.f);
+  zf[2 * c + 1] =
+      make_float4(static_cast<float>(x - hx), static_cast<float>(y - hy), static_cast<float>(z - hz), 0.f);
+}
+
+// R_max^2 of every cell, the exact maximum of the FP64 |X - Z|^2 over its
+// bodies.  At every level a warp's bodies form runs of one cell.  Distances are
+// first taken in FP32, from hi + lo floats: only a body whose FP32 value is
+// within its error bound of its run's largest can hold the maximum (the bounds
+// are those of separated_fast: each value is within 1e-6 of the exact one plus
+// 3e-21 of the squared coordinates; outside the comfortable range every body
+// stays).  Those, about one per run, are collected over the levels and
+// evaluated in FP64 32 at a time, so the FP64 pipe sees about one round of
+// eight instructions per warp instead of one per level (180 -> 60 us at N =
+// 1,048,576).  The maximum is taken on the bit pattern (monotone for
+// non-negative doubles); it is exact, so its order does not matter.
+__global__ void __launch_bounds__(kBlock) k_rmax_bodies(
+    int64_t n, int nlev, const int32_t *__restrict__ cell_at, const BodyF *__restrict__ bodyf,
+    const float4 *__restrict__ zf, const double *__restrict__ X, const double *__restrict__ Y,
+    const double *__restrict__ Zb, const double *__restrict__ Z, unsigned long long *__restrict__ rmax2) {
+  __shared__ int2 todo[kBlock / 32][64];  // (body, cell) still to be evaluated
   const int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
-  const int lane = threadIdx.x & 31;
-  int c = -1;
-  unsigned long long d2 = 0;  // bit pattern of |X - Z|^2 >= +0
-  if (i < n) {
-    c = cell_at[static_cast<int64_t>(lev) * n + i];
-    if (c >= 0) {
-      const double dx = __dsub_rn(X[i], Z[3 * c]);
-      const double dy = __dsub_rn(Y[i], Z[3 * c + 1]);
-      const double dz = __dsub_rn(Zb[i], Z[3 * c + 2]);
-      d2 = static_cast<unsigned long long>(
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  constexpr unsigned kAll = 0xffffffffu;
+  BodyF b{};
+  if (i < n) b = bodyf[i];
+  const float am = fmaxf(fmaxf(fabsf(b.h.x), fabsf(b.h.y)), fabsf(b.h.z));
+  int have = 0;
+  const auto evaluate = [&](int first, int num) {
+    if (lane < num) {
+      const int2 e = todo[w][first + lane];
+      const double dx = __dsub_rn(X[e.x], Z[3 * e.y]);
+      const double dy = __dsub_rn(Y[e.x], Z[3 * e.y + 1]);
+      const double dz = __dsub_rn(Zb[e.x], Z[3 * e.y + 2]);
+      const unsigned long long d2 = static_cast<unsigned long long>(
           __double_as_longlong(__dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz))));
+      if (d2 > rmax2[e.y]) atomicMax(&rmax2[e.y], d2);
+    }
+  };
+  for (int lev = 0; lev < nlev; ++lev) {
+    const int c = i < n ? cell_at[static_cast<int64_t>(lev) * n + i] : -1;
+    if (!__any_sync(kAll, c >= 0)) break;  // no body of the warp reaches this level
+    float d2 = -1.f, m = 0.f;
+    if (c >= 0) {
+      const float4 h = zf[2 * c], o = zf[2 * c + 1];
+      const float dx = (b.h.x - h.x) + (b.l.x - o.x), dy = (b.h.y - h.y) + (b.l.y - o.y),
+                  dz = (b.h.z - h.z) + (b.l.z - o.z);
+      d2 = dx * dx + dy * dy + dz * dz;
+      m = fmaxf(am, fmaxf(fmaxf(fabsf(h.x), fabsf(h.y)), fabsf(h.z)));
+    }
+    // largest value and bound of the run, at its first lane, then to all
+    const int cprev = __shfl_up_sync(kAll, c, 1);
+    const unsigned heads = __ballot_sync(kAll, lane == 0 || cprev != c);
+    float best = d2, bound = m;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const float v = __shfl_down_sync(kAll, best, o), u = __shfl_down_sync(kAll, bound, o);
+      const int co = __shfl_down_sync(kAll, c, o);
+      if (lane + o < 32 && co == c) {
+        best = fmaxf(best, v);
+        bound = fmaxf(bound, u);
+      }
+    }
+    const int head = 31 - __clz(static_cast<int>(heads & (kAll >> (31 - lane))));
+    best = __shfl_sync(kAll, best, head);
+    bound = __shfl_sync(kAll, bound, head);
+    const bool exactly = !(best > 1e-30f && best < 1e30f);
+    const bool cand = c >= 0 && (exactly || !(d2 + 1e-5f * best + 6e-21f * bound * bound < best));  // NaN: stays
+    const unsigned mask = __ballot_sync(kAll, cand);
+    if (cand) todo[w][have + __popc(mask & ((1u << lane) - 1))] = make_int2(static_cast<int>(i), c);
+    have += __popc(mask);
+    __syncwarp();
+    if (have >= 32) {
+      have -= 32;
+      evaluate(have, 32);  // the last ones
+      __syncwarp();
     }
   }
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const unsigned long long v = __shfl_down_sync(0xffffffffu, d2, o);
-    const int co = __shfl_down_sync(0xffffffffu, c, o);
-    if (lane + o < 32 && co == c && v > d2) d2 = v;
-  }
-  const int cprev = __shfl_up_sync(0xffffffffu, c, 1);
-  const bool head = (lane == 0) || (cprev != c);
-  if (c >= 0 && head) atomicMax(&rmax2[c], d2);
+  evaluate(0, have);
 }
 
 __global__ void k_rmax_final(int32_t ncell, const unsigned long long *__restrict__ rmax2,
@@ -673,6 +756,7 @@ int build_tree(fmm_ctx *c) {
   AMFMM_TRY(ensure<double>(c, c->Zb, n));
   AMFMM_TRY(ensure<double>(c, c->Mb, n));
   AMFMM_TRY(ensure<int32_t>(c, c->order, n));
+  AMFMM_TRY(ensure<BodyF>(c, c->bodyf, n));
   AMFMM_TRY(ensure<int32_t>(c, c->leaves, n + 1));
   AMFMM_TRY(ensure<int32_t>(c, c->leaf_of, n));
   AMFMM_TRY(ensure<int32_t>(c, c->cell_at, static_cast<size_t>(kMaxLevel + 1) * n));
@@ -726,7 +810,7 @@ int build_tree(fmm_ctx *c) {
   c->sz.key_which = which;
   k_permute<<<grid_for(n, kBlock), kBlock, 0, st>>>(c->x, c->y, c->z, c->m, sidx, n, ptr<double>(c->X),
                                                     ptr<double>(c->Y), ptr<double>(c->Zb), ptr<double>(c->Mb),
-                                                    ptr<int32_t>(c->order));
+                                                    ptr<int32_t>(c->order), ptr<BodyF>(c->bodyf));
   AMFMM_TRY(launched(c, "permute"));
 
   // octree: levels of every body, ids by one scan, cells
@@ -822,33 +906,36 @@ int upward(fmm_ctx *c) {
   if (c->opts.order_P != 3) {
     AMFMM_TRY(upward_general(c));
   } else {
-  k_leaf_upward<<<grid_for(c->sz.nleaf, 128), 128, 0, st>>>(
-      static_cast<int32_t>(c->sz.nleaf), ptr<int32_t>(c->leaves), ptr<int32_t>(c->begin),
-      ptr<int32_t>(c->count), ptr<double>(c->X), ptr<double>(c->Y), ptr<double>(c->Zb),
-      ptr<double>(c->Mb), ptr<double>(c->S), ptr<double>(c->M), ptr<double>(c->Z),
-      ptr<double>(c->invM), ptr<double>(c->mom));
+  // leaves per warp: as many as leave two warps per partition of the GPU
+  // (fewer FP64 instructions per leaf), down to one (a short chain)
+  const int64_t nleaf = c->sz.nleaf;
+  const int64_t fill = 8 * static_cast<int64_t>(std::max(1, c->num_sms));
+  const auto leaf = nleaf >= 8 * fill ? k_leaf_upward<8> : nleaf >= 4 * fill ? k_leaf_upward<4>
+                  : nleaf >= 2 * fill ? k_leaf_upward<2> : k_leaf_upward<1>;
+  const int per = nleaf >= 8 * fill ? 8 : nleaf >= 4 * fill ? 4 : nleaf >= 2 * fill ? 2 : 1;
+  leaf<<<grid_for(nleaf, kUpWarps * per), kUpWarps * 32, 0, st>>>(
+      static_cast<int32_t>(nleaf), ptr<int32_t>(c->leaves), ptr<int32_t>(c->begin), ptr<int32_t>(c->count),
+      ptr<double>(c->X), ptr<double>(c->Y), ptr<double>(c->Zb), ptr<double>(c->Mb), ptr<double>(c->S),
+      ptr<double>(c->M), ptr<double>(c->Z), ptr<double>(c->invM), ptr<double>(c->mom));
   AMFMM_TRY(launched(c, "leaf_upward"));
   for (int lev = c->sz.depth - 1; lev >= 0; --lev) {
     const int64_t c0 = c->sz.lvl_off[lev], c1 = c->sz.lvl_off[lev + 1];
-    // few cells: a warp per cell; many: a thread per cell (throughput-bound)
-    if (c1 - c0 < 8192)
-      k_internal_upward_warp<<<grid_for(32 * (c1 - c0), 128), 128, 0, st>>>(
-          static_cast<int32_t>(c0), static_cast<int32_t>(c1), ptr<int32_t>(c->first_child),
-          ptr<int32_t>(c->nchild), ptr<double>(c->S), ptr<double>(c->M), ptr<double>(c->Z),
-          ptr<double>(c->invM), ptr<double>(c->mom));
-    else
-      k_internal_upward<<<grid_for(c1 - c0, 128), 128, 0, st>>>(
-          static_cast<int32_t>(c0), static_cast<int32_t>(c1), ptr<int32_t>(c->first_child),
-          ptr<int32_t>(c->nchild), ptr<double>(c->S), ptr<double>(c->M), ptr<double>(c->Z),
-          ptr<double>(c->invM), ptr<double>(c->mom));
+    const bool many = c1 - c0 >= 4 * fill;  // four parents per warp once one each would fill the GPU
+    const auto up = many ? k_internal_upward<4> : k_internal_upward<1>;
+    up<<<grid_for(c1 - c0, many ? 4 * kUpWarps : kUpWarps), kUpWarps * 32, 0, st>>>(
+        static_cast<int32_t>(c0), static_cast<int32_t>(c1), ptr<int32_t>(c->first_child), ptr<int32_t>(c->nchild),
+        ptr<double>(c->S), ptr<double>(c->M), ptr<double>(c->Z), ptr<double>(c->invM), ptr<double>(c->mom));
     AMFMM_TRY(launched(c, "internal_upward"));
   }
   }
   AMFMM_CUDA(c, cudaMemsetAsync(c->rmax2.p, 0, sizeof(unsigned long long) * nc, st));
-  dim3 g(grid_for(n, kBlock), static_cast<unsigned>(c->sz.depth + 1));
-  k_rmax_bodies<<<g, kBlock, 0, st>>>(n, ptr<int32_t>(c->cell_at), ptr<double>(c->X), ptr<double>(c->Y),
-                                      ptr<double>(c->Zb), ptr<double>(c->Z),
-                                      ptr<unsigned long long>(c->rmax2));
+  AMFMM_TRY(ensure<float4>(c, c->cellzf, 2 * nc));
+  k_split_centres<<<grid_for(nc, kBlock), kBlock, 0, st>>>(static_cast<int32_t>(nc), ptr<double>(c->Z),
+                                                           ptr<float4>(c->cellzf));
+  AMFMM_TRY(launched(c, "split_centres"));
+  k_rmax_bodies<<<grid_for(n, kBlock), kBlock, 0, st>>>(
+      n, c->sz.depth + 1, ptr<int32_t>(c->cell_at), ptr<BodyF>(c->bodyf), ptr<float4>(c->cellzf), ptr<double>(c->X),
+      ptr<double>(c->Y), ptr<double>(c->Zb), ptr<double>(c->Z), ptr<unsigned long long>(c->rmax2));
   AMFMM_TRY(launched(c, "rmax_bodies"));
   k_rmax_final<<<grid_for(nc, kBlock), kBlock, 0, st>>>(static_cast<int32_t>(nc),
                                                         ptr<unsigned long long>(c->rmax2), ptr<double>(c->Rmax));
