@@ -316,6 +316,11 @@ int fmm_selector_train(fmm_ctx *ctx, float *params, float *adam, const float *X,
  * context stays usable (the next call must be fmm_build_tree or fmm_solve).
  * Synchronises the stream. */
 int fmm_debug_walk_wait_timeout(fmm_ctx *ctx);
+/* Test hook: the radix sort of n (key, value) pairs on the device (keys of 4 or
+ * 8 bytes, their low `bits` bits), with at most `spins` polls per wait of a tile
+ * for the tiles before it. */
+int fmm_debug_sort(fmm_ctx *ctx, int key_bytes, const void *key, const uint32_t *val, int64_t n, int bits, int spins,
+                   void *okey, uint32_t *oval);
 
 /* ---- a10 diagnostics (Sec. 3) ---------------------------------------------- */
 

@@ -248,6 +248,13 @@ int exclusive_scan_i4(fmm_ctx *c, const int4 *in, int4 *out, int64_t n, int4 *to
 // Sorted data ends in buffer index *which (0 or 1) of the ping-pong pairs.
 int radix_sort_u64(fmm_ctx *c, DBuf key[2], DBuf val[2], int64_t n, int bits, int *which);
 int radix_sort_u32(fmm_ctx *c, DBuf key[2], DBuf val[2], int64_t n, int bits, int *which);
+// Stable sorts of what a list of K > 0 pairs holds (buffers only receive):
+// both cells of every pair, valued with the other cell of the pair or with the
+// position 2 k + side; pairs by their first cell, valued with the second, or by
+// their second, valued with the position k.
+int sort_pair_sides(fmm_ctx *c, const int2 *pairs, int64_t K, bool partner, DBuf key[2], DBuf val[2], int bits,
+                    int *which);
+int sort_pairs(fmm_ctx *c, const int2 *pairs, int64_t K, bool second, DBuf key[2], DBuf val[2], int bits, int *which);
 
 // ---------------------------------------------------------------------------
 // stages
@@ -261,6 +268,8 @@ int m2l_run(fmm_ctx *c);            // m2l.cu: mutual M2L into slots
 int m2l_reduce(fmm_ctx *c);         // m2l.cu: per-cell fixed-order sums
 // the mixed form at order 3 gathers each cell's partners (one-sided, no slots)
 inline bool m2l_gathered(const fmm_ctx *c) { return c->opts.precision == FMM_MIXED && c->opts.order_P == 3; }
+// first position of every cell among E > 0 sorted keys (off[ncell] = E)  (m2l.cu)
+int segment_offsets(fmm_ctx *c, int64_t E, const uint32_t *key, int32_t *off);
 // every cell's partners over a list of pairs, in the stable order of the list:
 // cell c's are val[*which][off[c] .. off[c + 1])  (m2l.cu)
 int partner_lists(fmm_ctx *c, const int2 *pairs, int64_t K, DBuf key[2], DBuf val[2], int32_t *off, int *which);

@@ -619,19 +619,6 @@ __global__ void k_pair_locals(int64_t K, const int2 *__restrict__ pairs, const d
   }
 }
 
-// entries for the stable sort by cell: (cell, 2k + side) for the slot form,
-// (cell, partner) for the gather form
-__global__ void k_m2l_entries(int64_t K, const int2 *__restrict__ pairs, int gather, uint32_t *__restrict__ key,
-                              uint32_t *__restrict__ val) {
-  const int64_t k = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
-  if (k >= K) return;
-  const int2 p = pairs[k];
-  key[2 * k] = static_cast<uint32_t>(p.x);
-  val[2 * k] = gather ? static_cast<uint32_t>(p.y) : static_cast<uint32_t>(2 * k);
-  key[2 * k + 1] = static_cast<uint32_t>(p.y);
-  val[2 * k + 1] = gather ? static_cast<uint32_t>(p.x) : static_cast<uint32_t>(2 * k + 1);
-}
-
 // off[c] = first sorted position of cell c (cells without entries get the
 // position of the next cell): every position s starts the cells
 // (key[s-1], key[s]], and the last entry closes the cells after it.
@@ -832,18 +819,16 @@ int bits_for(int64_t v) {
 int sorted_entries(fmm_ctx *c, const int2 *pairs, int64_t K, int gather, DBuf key[2], DBuf val[2], int32_t *off,
                    int *which) {
   const int64_t nc = c->sz.ncell, E = 2 * K;
-  AMFMM_TRY(ensure<uint32_t>(c, key[0], E));
-  AMFMM_TRY(ensure<uint32_t>(c, val[0], E));
-  k_m2l_entries<<<grid_for(K, 256), 256, 0, c->stream>>>(K, pairs, gather, ptr<uint32_t>(key[0]),
-                                                         ptr<uint32_t>(val[0]));
-  AMFMM_TRY(launched(c, "pair_entries"));
-  AMFMM_TRY(radix_sort_u32(c, key, val, E, bits_for(nc), which));
-  k_segment_offsets<<<grid_for((E + 3) / 4, 256), 256, 0, c->stream>>>(E, static_cast<int32_t>(nc),
-                                                                      ptr<uint32_t>(key[*which]), off);
-  return launched(c, "segment_offsets");
+  AMFMM_TRY(sort_pair_sides(c, pairs, K, gather != 0, key, val, bits_for(nc), which));
+  return segment_offsets(c, E, ptr<uint32_t>(key[*which]), off);
 }
 
 }  // namespace
+
+int segment_offsets(fmm_ctx *c, int64_t E, const uint32_t *key, int32_t *off) {
+  k_segment_offsets<<<grid_for((E + 3) / 4, 256), 256, 0, c->stream>>>(E, static_cast<int32_t>(c->sz.ncell), key, off);
+  return launched(c, "segment_offsets");
+}
 
 int partner_lists(fmm_ctx *c, const int2 *pairs, int64_t K, DBuf key[2], DBuf val[2], int32_t *off, int *which) {
   *which = 0;

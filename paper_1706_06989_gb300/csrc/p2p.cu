@@ -342,36 +342,24 @@ __global__ void k_p2p_reduce(int64_t n, const int32_t *__restrict__ leaf_of, con
   near[2 * n + i] = a2;
 }
 
-// Sort keys of the pairs by one side, the per-cell pair counts, and (if nb is
-// given) every pair's column count n_B.
-__global__ void k_pair_keys(int64_t K, const int2 *__restrict__ pairs, int side, uint32_t *__restrict__ key,
-                            uint32_t *__restrict__ val, int32_t *__restrict__ cnt,
-                            const int32_t *__restrict__ count, int32_t *__restrict__ nb) {
-  const int64_t k = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
-  if (k >= K) return;
-  const int2 p = pairs[k];
-  const int c = side == 0 ? p.x : p.y;
-  key[k] = static_cast<uint32_t>(c);
-  val[k] = static_cast<uint32_t>(k);
-  atomicAdd(&cnt[c], 1);
-  if (nb) nb[k] = count[p.y];
-}
-
-__global__ void k_gather_pairs(int64_t K, const int2 *__restrict__ in, const uint32_t *__restrict__ sval,
-                               int2 *__restrict__ out) {
+// the sorted (A, B) as pairs, and every pair's column count n_B
+__global__ void k_sorted_pairs(int64_t K, const uint32_t *__restrict__ key, const uint32_t *__restrict__ val,
+                               const int32_t *__restrict__ count, int2 *__restrict__ out, int32_t *__restrict__ nb) {
   const int64_t s = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
-  if (s < K) out[s] = in[sval[s]];
+  if (s >= K) return;
+  const int2 p = make_int2(static_cast<int>(key[s]), static_cast<int>(val[s]));
+  out[s] = p;
+  nb[s] = count[p.y];
 }
 
 // pos[s] = CSR position of sorted pair s on its B side; len[e] = 3 n_B
-__global__ void k_b_positions(int64_t K, const uint32_t *__restrict__ sval, const int2 *__restrict__ pairs,
+__global__ void k_b_positions(int64_t K, const uint32_t *__restrict__ key, const uint32_t *__restrict__ sval,
                               const int32_t *__restrict__ count, int32_t *__restrict__ pos,
                               int64_t *__restrict__ len) {
   const int64_t e = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (e >= K) return;
-  const uint32_t s = sval[e];
-  pos[s] = static_cast<int32_t>(e);
-  len[e] = 3 * static_cast<int64_t>(count[pairs[s].y]);
+  pos[sval[e]] = static_cast<int32_t>(e);
+  len[e] = 3 * static_cast<int64_t>(count[key[e]]);
 }
 
 int bits_for(int64_t v) {
@@ -517,30 +505,19 @@ int p2p_prepare(fmm_ctx *c) {
   int64_t *h = static_cast<int64_t *>(c->hpin);
   h[0] = 0;
   if (K > 0) {
-    AMFMM_TRY(ensure<uint32_t>(c, c->pkey[0], K));
-    AMFMM_TRY(ensure<uint32_t>(c, c->pval[0], K));
-    // group by A (stable)
-    AMFMM_CUDA(c, cudaMemsetAsync(cnt, 0, sizeof(int32_t) * (nc + 1), st));
-    k_pair_keys<<<grid_for(K, 256), 256, 0, st>>>(K, ptr<int2>(c->p2p), 0, ptr<uint32_t>(c->pkey[0]),
-                                                  ptr<uint32_t>(c->pval[0]), cnt, nullptr, nullptr);
-    AMFMM_TRY(launched(c, "p2p_keysA"));
-    AMFMM_TRY(exclusive_scan_i32(c, cnt, offA, nc + 1, nullptr));
+    // group by A (stable), with the column counts n_B
     int which = 0;
-    AMFMM_TRY(radix_sort_u32(c, c->pkey, c->pval, K, bits_for(nc), &which));
-    k_gather_pairs<<<grid_for(K, 256), 256, 0, st>>>(K, ptr<int2>(c->p2p), ptr<uint32_t>(c->pval[which]),
-                                                     ptr<int2>(c->p2p_A));
-    AMFMM_TRY(launched(c, "p2p_gather"));
-    // CSR on the B side; column counts n_B in A-sorted order
-    AMFMM_CUDA(c, cudaMemsetAsync(cnt, 0, sizeof(int32_t) * (nc + 1), st));
-    k_pair_keys<<<grid_for(K, 256), 256, 0, st>>>(K, ptr<int2>(c->p2p_A), 1, ptr<uint32_t>(c->pkey[0]),
-                                                  ptr<uint32_t>(c->pval[0]), cnt, ptr<int32_t>(c->count), nb);
-    AMFMM_TRY(launched(c, "p2p_keysB"));
-    AMFMM_TRY(exclusive_scan_i32(c, cnt, offB, nc + 1, nullptr));
-    AMFMM_TRY(radix_sort_u32(c, c->pkey, c->pval, K, bits_for(nc), &which));
-    // B-side slot offsets: 3 n_B doubles per pair, in B-CSR order
+    AMFMM_TRY(sort_pairs(c, ptr<int2>(c->p2p), K, false, c->pkey, c->pval, bits_for(nc), &which));
+    AMFMM_TRY(segment_offsets(c, K, ptr<uint32_t>(c->pkey[which]), offA));
+    k_sorted_pairs<<<grid_for(K, 256), 256, 0, st>>>(K, ptr<uint32_t>(c->pkey[which]), ptr<uint32_t>(c->pval[which]),
+                                                     ptr<int32_t>(c->count), ptr<int2>(c->p2p_A), nb);
+    AMFMM_TRY(launched(c, "p2p_sorted_pairs"));
+    // CSR on the B side; slot offsets: 3 n_B floats per pair, in that order
+    AMFMM_TRY(sort_pairs(c, ptr<int2>(c->p2p_A), K, true, c->pkey, c->pval, bits_for(nc), &which));
+    AMFMM_TRY(segment_offsets(c, K, ptr<uint32_t>(c->pkey[which]), offB));
     AMFMM_TRY(ensure<int64_t>(c, c->p2p_len, K + 1));
     int64_t *len = ptr<int64_t>(c->p2p_len);
-    k_b_positions<<<grid_for(K, 256), 256, 0, st>>>(K, ptr<uint32_t>(c->pval[which]), ptr<int2>(c->p2p_A),
+    k_b_positions<<<grid_for(K, 256), 256, 0, st>>>(K, ptr<uint32_t>(c->pkey[which]), ptr<uint32_t>(c->pval[which]),
                                                     ptr<int32_t>(c->count), ptr<int32_t>(c->p2p_pos), len);
     AMFMM_TRY(launched(c, "p2p_bpos"));
     int64_t *ptot = ptr<int64_t>(c->totals) + 12;
