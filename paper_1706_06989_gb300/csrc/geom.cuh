@@ -8,54 +8,6 @@
 
 namespace amfmm {
 
-__device__ __forceinline__ void leaf_com(int c, int b, int e, const double *__restrict__ X,
-                                         const double *__restrict__ Y, const double *__restrict__ Zb,
-                                         const double *__restrict__ Mb, double *__restrict__ S,
-                                         double *__restrict__ M, double *__restrict__ Z,
-                                         double *__restrict__ invM, double z[3]) {
-  double sx = 0.0, sy = 0.0, sz = 0.0, mm = 0.0;
-  for (int i = b; i < e; ++i) {
-    const double mu = Mb[i];
-    sx = __dadd_rn(sx, __dmul_rn(mu, X[i]));
-    sy = __dadd_rn(sy, __dmul_rn(mu, Y[i]));
-    sz = __dadd_rn(sz, __dmul_rn(mu, Zb[i]));
-    mm = __dadd_rn(mm, mu);
-  }
-  z[0] = __ddiv_rn(sx, mm);
-  z[1] = __ddiv_rn(sy, mm);
-  z[2] = __ddiv_rn(sz, mm);
-  S[3 * c] = sx;
-  S[3 * c + 1] = sy;
-  S[3 * c + 2] = sz;
-  M[c] = mm;
-  Z[3 * c] = z[0];
-  Z[3 * c + 1] = z[1];
-  Z[3 * c + 2] = z[2];
-  invM[c] = 1.0 / mm;
-}
-
-__device__ __forceinline__ void parent_com(int c, int f, int nch, double *__restrict__ S, double *__restrict__ M,
-                                           double *__restrict__ Z, double *__restrict__ invM, double z[3]) {
-  double sx = 0.0, sy = 0.0, sz = 0.0, mm = 0.0;
-  for (int k = f; k < f + nch; ++k) {
-    sx = __dadd_rn(sx, S[3 * k]);
-    sy = __dadd_rn(sy, S[3 * k + 1]);
-    sz = __dadd_rn(sz, S[3 * k + 2]);
-    mm = __dadd_rn(mm, M[k]);
-  }
-  z[0] = __ddiv_rn(sx, mm);
-  z[1] = __ddiv_rn(sy, mm);
-  z[2] = __ddiv_rn(sz, mm);
-  S[3 * c] = sx;
-  S[3 * c + 1] = sy;
-  S[3 * c + 2] = sz;
-  M[c] = mm;
-  Z[3 * c] = z[0];
-  Z[3 * c + 1] = z[1];
-  Z[3 * c + 2] = z[2];
-  invM[c] = 1.0 / mm;
-}
-
 // ---- opening criterion (Sec. 2), shared by the walk and the learned selector ----
 // per cell {Z_x, Z_y, Z_z, R_max}, one 32-byte load
 __device__ __forceinline__ bool well_separated(const double4_32a a, const double4_32a b, double theta) {

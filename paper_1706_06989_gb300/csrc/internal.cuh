@@ -173,7 +173,7 @@ struct fmm_ctx {
   int64_t sel_min_work = 256;  // pairs with n_A n_B below this are left to the floor
   int sel_rule = FMM_SEL_RELATIVE;  // acceptance rule of the learned selector
   // index tables of the table-driven general order (P = 6 .. 8)
-  amfmm::DBuf gen_tab;
+  amfmm::DBuf gen_fold;
   // host-solve staging
   amfmm::DBuf hx, hy, hz, hm, hax, hay, haz;
   // graph-captured solves
@@ -282,17 +282,14 @@ int p2p64_run(fmm_ctx *c);
 int downward(fmm_ctx *c);           // down.cu (L2L, L2P into sorted order)
 int forces(fmm_ctx *c, double *ax, double *ay, double *az);  // down.cu (caller order)
 
-// general order P (expansion.cu)
+// general order P = 4 .. 8 (expansion.cu, expansion_m2l.cu)
 int mom_stride(int P);  // moments of order 0..P per cell
 int loc_stride(int P);  // local coefficients per cell (order 3: 20 with padding)
+int slot_stride_general(int P);  // doubles per M2L slot
 int upward_general(fmm_ctx *c);
 int m2l_general(fmm_ctx *c);
 int reduce_general(fmm_ctx *c);
 int downward_general(fmm_ctx *c);
-// the same stages at P = 6 .. 8, table-driven (expansion_table.cu)
-int upward_table(fmm_ctx *c);
-int m2l_table(fmm_ctx *c);
-int downward_table(fmm_ctx *c);
 
 // learned selector (selector.cu, m2l.cu)
 int cell_features(fmm_ctx *c);  // per-cell parts of the selector's features

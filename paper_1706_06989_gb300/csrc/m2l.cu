@@ -857,7 +857,7 @@ int m2l_prepare(fmm_ctx *c) {
     k_inverse<<<grid_for(E, 256), 256, 0, st>>>(E, ptr<uint32_t>(c->eval[which]), ptr<int32_t>(c->m2l_pos));
     AMFMM_TRY(launched(c, "m2l_inverse"));
     const size_t esz = fp32 ? sizeof(float) : sizeof(double);
-    const int stride = c->opts.order_P == 3 ? kSlot64 : loc_stride(c->opts.order_P);
+    const int stride = c->opts.order_P == 3 ? kSlot64 : slot_stride_general(c->opts.order_P);
     AMFMM_TRY(ensure_bytes(c, c->m2l_slots, static_cast<size_t>(E) * stride * esz));
   }
   if (fp32) {
