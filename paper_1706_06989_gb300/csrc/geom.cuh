@@ -33,7 +33,7 @@ __device__ __forceinline__ bool well_separated(const double4_32a a, const double
 // the comfortable FP32 range, return -1 and are decided in FP64.
 struct CellF {
   float4 h;  // Z hi (x, y, z), R_max rounded to FP32
-  float4 l;  // Z - hi (x, y, z), unused
+  float4 l;  // Z - hi (x, y, z), bits of nchild | level << 8
 };
 
 __device__ __forceinline__ int separated_fast(const CellF &a, const CellF &b, float th2) {
@@ -51,6 +51,34 @@ __device__ __forceinline__ int separated_fast(const CellF &a, const CellF &b, fl
   if (diff > tol) return 1;
   if (diff < -tol) return 0;
   return -1;
+}
+
+// ---- records of the walk's frontier ----
+// Up to eight pairs: {first varying cell, fixed cell, n | side << 4} stands for
+// (v + a, fixed), a < n (side 1: (fixed, v + a)); the pairs of a cell's children
+// f .. f + k - 1 with themselves, (f, f) .. (f+k-1, f+k-1), (f, f+1), (f, f+2) ..,
+// from the q-th on, are {f, k, n | 32 | q << 8}.
+__device__ __forceinline__ int4 split_record(int first, int n, int fixed, bool second) {
+  return make_int4(first, fixed, n | (second ? 16 : 0), 0);
+}
+__device__ __forceinline__ int4 self_record(int first, int k, int q, int n) {
+  return make_int4(first, k, n | 32 | (q << 8), 0);
+}
+__device__ __forceinline__ bool front_pair(int4 rec, int a, int2 &pr) {
+  if (a >= (rec.z & 15)) return false;
+  if (rec.z & 32) {
+    int q = (rec.z >> 8) + a, i = 0;
+    if (q < rec.y) {
+      pr = make_int2(rec.x + q, rec.x + q);
+    } else {
+      q -= rec.y;
+      while (q >= rec.y - 1 - i) q -= rec.y - 1 - i++;
+      pr = make_int2(rec.x + i, rec.x + i + 1 + q);
+    }
+  } else {
+    pr = rec.z & 16 ? make_int2(rec.y, rec.x + a) : make_int2(rec.x + a, rec.y);
+  }
+  return true;
 }
 
 }  // namespace amfmm

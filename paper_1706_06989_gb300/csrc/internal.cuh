@@ -294,7 +294,7 @@ int downward_general(fmm_ctx *c);
 // learned selector (selector.cu, m2l.cu)
 int cell_features(fmm_ctx *c);  // per-cell parts of the selector's features
 int field_estimate(fmm_ctx *c);  // per-cell log10 |a| estimate of the selector's relative rule
-int walk_scores(fmm_ctx *c, const long long *nf_dev, int64_t cap, const int2 *front, float *score);
+int walk_scores(fmm_ctx *c, const long long *nf_dev, int64_t cap, const int4 *front, float *score);
 int pair_locals_tc(fmm_ctx *c, const int2 *pairs, int64_t K, double *out);
 
 void timer(fmm_ctx *c, int slot);

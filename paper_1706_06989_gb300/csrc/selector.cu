@@ -687,13 +687,13 @@ __global__ void k_adam(float *__restrict__ p, float *__restrict__ m, float *__re
 // list's order varies from run to run, but a pair's score depends only on the
 // pair (the rows of a tensor-core product are independent), so the walk does
 // not.  k_walk_scores then runs the network on the candidates only.
-__global__ void k_band_select(const long long *__restrict__ nf_dev, int64_t cap, const int2 *__restrict__ front,
+__global__ void k_band_select(const long long *__restrict__ nf_dev, int64_t cap, const int4 *__restrict__ front,
                               const double4_32a *__restrict__ zr, const CellF *__restrict__ zf,
                               const int32_t *__restrict__ count, int64_t min_work, double th_lo, double th_hi,
                               float *__restrict__ score, int32_t *__restrict__ cand, unsigned *__restrict__ ncand) {
   // the frontier size comes from the walk's generation record; a frontier
   // beyond the buffers (the walk then stops and runs again) is not scored
-  const int64_t nf = min(static_cast<int64_t>(*nf_dev), cap);
+  const int64_t nf = 8 * min(static_cast<int64_t>(*nf_dev), cap);  // places of its records
   const int lane = threadIdx.x & 31;
   for (int64_t base = blockIdx.x * static_cast<int64_t>(blockDim.x); base < nf;
        base += static_cast<int64_t>(gridDim.x) * blockDim.x) {
@@ -701,9 +701,11 @@ __global__ void k_band_select(const long long *__restrict__ nf_dev, int64_t cap,
   bool ok = false;
   if (t < nf) {
     score[t] = INFINITY;
-    const int A = front[t].x, B = front[t].y;
+    int2 pr = make_int2(0, 0);
+    const bool there = front_pair(front[t >> 3], static_cast<int>(t & 7), pr);
+    const int A = pr.x, B = pr.y;
     // a pair of few bodies costs less to open than to score
-    if (A != B && static_cast<int64_t>(count[A]) * count[B] >= min_work) {
+    if (there && A != B && static_cast<int64_t>(count[A]) * count[B] >= min_work) {
       const float th2f_lo = static_cast<float>(th_lo) * static_cast<float>(th_lo);
       const float th2f_hi = static_cast<float>(th_hi) * static_cast<float>(th_hi);
       const CellF fa = zf[A], fb = zf[B];
@@ -734,7 +736,7 @@ __global__ void k_band_select(const long long *__restrict__ nf_dev, int64_t cap,
 // side A's error is at most 10^pred M_B/r^2, side B's 10^pred M_A/r^2, and
 //   score = pred + log10 max(M_B / (r^2 |a_A|), M_A / (r^2 |a_B|)),
 // compared by the walk with log10 of the relative target.
-__global__ void __launch_bounds__(128) k_walk_scores(const int2 *__restrict__ front,
+__global__ void __launch_bounds__(128) k_walk_scores(const int4 *__restrict__ front,
                                                      const int32_t *__restrict__ cand,
                                                      const unsigned *__restrict__ ncand,
                                                      const float *__restrict__ params,
@@ -762,7 +764,9 @@ __global__ void __launch_bounds__(128) k_walk_scores(const int2 *__restrict__ fr
       float f[kF] = {0, 0, 0, 0, 0, 0, 0, 0};
       float ad = 0.f;
       if (base + lane < K) {
-        const int2 pr = front[cand[base + lane]];
+        const int slot = cand[base + lane];
+        int2 pr = make_int2(0, 0);
+        front_pair(front[slot >> 3], slot & 7, pr);
         pair_features(pr.x, pr.y, zf, cf, f);
         const float l2r = 2.f * f[0];
         ad = lga ? fmaxf(cf[pr.y].y - l2r - lga[pr.x], cf[pr.x].y - l2r - lga[pr.y])
@@ -822,7 +826,7 @@ int field_estimate(fmm_ctx *c) {
   return launched(c, "field_estimate");
 }
 
-int walk_scores(fmm_ctx *c, const long long *nf_dev, int64_t cap, const int2 *front, float *score) {
+int walk_scores(fmm_ctx *c, const long long *nf_dev, int64_t cap, const int4 *front, float *score) {
   cudaStream_t st = c->stream;
   unsigned *ncand = reinterpret_cast<unsigned *>(ptr<int64_t>(c->totals) + 11);
   AMFMM_CUDA(c, cudaMemsetAsync(ncand, 0, sizeof(unsigned), st));

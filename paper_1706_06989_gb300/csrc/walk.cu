@@ -16,7 +16,8 @@
 // The set of emitted pairs depends only on these per-pair decisions, so it is
 // independent of the traversal order.  The walk proceeds one generation of
 // pairs at a time; an exclusive scan of the per-pair output counts places
-// every output, which makes the list order deterministic.
+// every output, which makes the list order deterministic.  The pairs of a
+// generation are kept as records of up to eight pairs that share a cell.
 #include <cmath>
 #include <cstring>
 
@@ -31,10 +32,10 @@ constexpr int kBlock = 256;
 enum Action : int32_t { kSelfLeaf = 0, kSelfSplit = 1, kAccept = 2, kNear = 3, kSplitA = 4, kSplitB = 5 };
 
 // packs the walk's per-cell inputs: {Z, R_max} (FP64 and the FP32 filter's
-// copy) and {nchild, level}
+// copy, with nchild | level << 8) and {first child, nchild}
 __global__ void k_pack_cells(int32_t ncell, const double *__restrict__ Z, const double *__restrict__ Rmax,
                              const int32_t *__restrict__ nchild, const int32_t *__restrict__ level,
-                             double4_32a *__restrict__ zr, CellF *__restrict__ zf, int2 *__restrict__ nl) {
+                             const int32_t *__restrict__ first_child, double4_32a *__restrict__ zr, CellF *__restrict__ zf, int2 *__restrict__ nl) {
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= ncell) return;
   const double x = Z[3 * c], y = Z[3 * c + 1], z = Z[3 * c + 2], R = Rmax[c];
@@ -42,65 +43,45 @@ __global__ void k_pack_cells(int32_t ncell, const double *__restrict__ Z, const 
   const float hx = static_cast<float>(x), hy = static_cast<float>(y), hz = static_cast<float>(z);
   CellF f;
   f.h = make_float4(hx, hy, hz, static_cast<float>(R));
-  f.l = make_float4(static_cast<float>(x - hx), static_cast<float>(y - hy), static_cast<float>(z - hz), 0.f);
+  f.l = make_float4(static_cast<float>(x - hx), static_cast<float>(y - hy), static_cast<float>(z - hz),
+                    __int_as_float(nchild[c] | (level[c] << 8)));
   zf[c] = f;
-  nl[c] = make_int2(nchild[c], level[c]);
+  nl[c] = make_int2(first_child[c], nchild[c]);
 }
 
-// score (may be NULL): the learned selector's prediction for every frontier
-// pair (+inf where the safety bound fails); with it, a pair is accepted when
-// the opening criterion accepts it (theta is then a floor on the accepted
-// set, which bounds the work of a strict target) or when score < target.
-// Output counts: x = next-generation pairs, y = M2L, z = P2P, w = leaf self.
-__device__ __forceinline__ int classify(int A, int B, const int2 *__restrict__ nl,
-                                        const double4_32a *__restrict__ zr, const CellF *__restrict__ zf,
-                                        double theta, float th2f, bool accept_hint, int4 &cnt) {
-  cnt = make_int4(0, 0, 0, 0);
-  const int2 nlA = nl[A];
-  if (A == B) {
-    const int k = nlA.x;
-    if (k == 0) {
-      cnt.w = 1;
-      return kSelfLeaf;
-    }
-    cnt.x = k + k * (k - 1) / 2;
-    return kSelfSplit;
-  }
-  int sep = 1;
-  float rA = 0.f, rB = 0.f;  // FP32 R_max, kept for the split choice
-  if (!accept_hint) {
-    const CellF fA = zf[A], fB = zf[B];
-    sep = separated_fast(fA, fB, th2f);
-    rA = fA.h.w;
-    rB = fB.h.w;
-  }
+// What becomes of the pair (A, B).  accept_hint: the learned selector accepts
+// the pair (then the criterion is a floor on the accepted set, which bounds the
+// work of a strict target).  Everything a decision usually needs is loaded
+// before the first branch.
+__device__ __forceinline__ int classify(int A, int B, const double4_32a *__restrict__ zr,
+                                        const CellF *__restrict__ zf, double theta, float th2f, bool accept_hint,
+                                        int &children) {
+  const CellF fA = zf[A], fB = zf[B];
+  const int nlA = __float_as_int(fA.l.w), nlB = __float_as_int(fB.l.w), ka = nlA & 255, kb = nlB & 255;
+  children = ka;
+  if (A == B) return ka == 0 ? kSelfLeaf : kSelfSplit;
+  int sep = accept_hint ? 1 : separated_fast(fA, fB, th2f);
   if (sep < 0) sep = well_separated(zr[A], zr[B], theta);
-  if (sep) {
-    cnt.y = 1;
-    return kAccept;
-  }
-  const int2 nlB = nl[B];
-  const int ka = nlA.x, kb = nlB.x;
-  if (ka == 0 && kb == 0) {
-    cnt.z = 1;
-    return kNear;
-  }
+  if (sep) return kAccept;
+  if (ka == 0 && kb == 0) return kNear;
   bool pickA;
   if (kb == 0) pickA = true;
   else if (ka == 0) pickA = false;
-  else if (rA != rB) {
+  else if (fA.h.w != fB.h.w) {
     // R_max rounded to FP32 (monotone rounding): unequal FP32 values order
     // the FP64 values the same way, strictly
-    pickA = rA > rB;
+    pickA = fA.h.w > fB.h.w;
   } else {
     const double ra = zr[A].w, rb = zr[B].w;
     if (ra != rb) pickA = ra > rb;
-    else if (nlA.y != nlB.y) pickA = nlA.y < nlB.y;
+    else if (nlA >> 8 != nlB >> 8) pickA = nlA >> 8 < nlB >> 8;
     else pickA = A < B;
   }
-  cnt.x = pickA ? ka : kb;
   return pickA ? kSplitA : kSplitB;
 }
+
+// records of a cell's pairs with itself
+__device__ __forceinline__ int self_records(int k) { return (k + k * (k - 1) / 2 + 7) / 8; }
 
 __device__ __forceinline__ int4 add4(int4 a, int4 b) { return make_int4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
 
@@ -130,10 +111,16 @@ struct GenState {
   GenIn in;
 };
 
-constexpr int kGenItems = 4;
-constexpr int kGenBlock = 256;  // threads of a generation block (128: 1.29 ms, 512: 1.21 ms, 256: 1.16 ms per 1M solve)
-constexpr int kGenTile = kGenBlock * kGenItems;
+constexpr int kGenBlock = 256;  // threads of a generation block
+constexpr int kGenRounds = 16;  // at most, each of four records per warp
+constexpr int kGenWave = kGenBlock / 8;           // records of a block in one round
+constexpr int kGenTile = kGenWave * kGenRounds;   // largest tile
 constexpr int kGenBlocksPerSM = 5;  // resident blocks per SM the registers are limited for
+// rounds per tile: one while that gives every block at most one tile
+__device__ __forceinline__ int gen_rounds(int64_t nf, int64_t blocks) {
+  const int64_t r = (nf + kGenWave * blocks - 1) / (kGenWave * blocks);
+  return r < 1 ? 1 : r > kGenRounds ? kGenRounds : static_cast<int>(r);
+}
 constexpr long long kSpinLimit = 1LL << 22;
 
 __device__ __forceinline__ int4 ld_volatile4(const int4 *p) {
@@ -151,6 +138,17 @@ __device__ __forceinline__ void st_volatile4(int4 *p, int4 v) {
 // One generation of the walk: every pair of the frontier is classified, the
 // output counts are scanned across the block and then across tiles (single
 // pass, decoupled look-back), and the outputs are written in frontier order.
+// Eight lanes take a record, so a warp's loads touch four runs of neighbouring
+// cells and four shared ones, its counts are votes, and a split pair becomes one
+// 16-byte record instead of up to eight pairs written one by one.  A record has
+// 5 to 6 pairs on average, so about 30% of the lanes idle.
+// Between its two passes over a tile the kernel keeps votes only (lane r those of
+// round r) and forms the pairs again, so a tile can have 16 rounds and its
+// look-back, which cost as many instructions as the pairs at four, is shared by
+// more of them.  All generations at N = 1,048,576: 0.71 ms, and 1.97 at 4,194,304
+// (1.04 and 3.10 with eight pairs per split and four consecutive pairs per
+// thread; 0.85 and 2.61 with four rounds per tile); 0.24 ms at 65,536 (0.33).
+// A generation of one tile is a chain of loads of about 6 us.
 // The grid is persistent: blocks draw tiles until the frontier is done.  The
 // frontier size and the list offsets come from the generation's record, so
 // the host launches all generations without waiting.  Writes beyond a
@@ -158,9 +156,9 @@ __device__ __forceinline__ void st_volatile4(int4 *p, int4 v) {
 // walk and flags it, and the host grows the buffers (keeping what earlier
 // generations wrote) and resumes the walk at the flagged generation.
 __global__ void __launch_bounds__(kGenBlock, kGenBlocksPerSM) k_walk_gen(
-    GenState *__restrict__ gs, int g, const int2 *__restrict__ front, const int2 *__restrict__ nl,
+    GenState *__restrict__ gs, int g, const int4 *__restrict__ front, const int2 *__restrict__ nl,
     const double4_32a *__restrict__ zr, const CellF *__restrict__ zf, double theta, const float *__restrict__ score,
-    float target, const int32_t *__restrict__ first_child, int2 *__restrict__ next, int64_t cap_next,
+    float target, int4 *__restrict__ next, int64_t cap_next,
     int2 *__restrict__ m2l, int64_t cap_m2l, int2 *__restrict__ p2p, int64_t cap_p2p, int32_t *__restrict__ self,
     int64_t cap_self, unsigned epoch, int64_t max_places, int *__restrict__ flag, int4 *__restrict__ agg,
     int4 *__restrict__ inc) {
@@ -168,12 +166,14 @@ __global__ void __launch_bounds__(kGenBlock, kGenBlocksPerSM) k_walk_gen(
   __shared__ int4 s_warp[kGenBlock / 32];
   __shared__ int4 s_red[kGenBlock / 32];
   __shared__ int s_stop[kGenBlock / 32];
+  constexpr unsigned kAll = 0xffffffffu;
   const float th2f = static_cast<float>(theta) * static_cast<float>(theta);
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
   GenState &G = gs[g];
   const GenIn in = G.in;
   const int64_t nf = in.nf;
-  const int64_t nb = (nf + kGenTile - 1) / kGenTile;
+  const int rounds = gen_rounds(nf, gridDim.x), tile = kGenWave * rounds;
+  const int64_t nb = (nf + tile - 1) / tile;
   if (nb == 0 || nb > max_places) {
     if (blockIdx.x == 0 && t == 0) {
       if (nb > max_places) atomicOr(&G.status, 4);
@@ -192,33 +192,42 @@ __global__ void __launch_bounds__(kGenBlock, kGenBlocksPerSM) k_walk_gen(
   __syncthreads();
   const unsigned place = s_place;
   if (place >= nb) break;
-  const int64_t i0 = static_cast<int64_t>(place) * kGenTile + static_cast<int64_t>(t) * kGenItems;
-  int act[kGenItems];
-  int2 pr[kGenItems];
-  int4 mine = make_int4(0, 0, 0, 0);
-#pragma unroll
-  for (int k = 0; k < kGenItems; ++k) {
-    const int64_t i = i0 + k;
-    act[k] = -1;
-    if (i < nf) {
-      pr[k] = front[i];
-      int4 cnt;
-      const bool hint = score != nullptr && score[i] < target;
-      act[k] = classify(pr[k].x, pr[k].y, nl, zr, zf, theta, th2f, hint, cnt);
-      mine = add4(mine, cnt);
+  const int64_t i0 = static_cast<int64_t>(place) * tile + w * 4 * rounds + (lane >> 3);
+  // lane r keeps the votes of round r
+  unsigned v_acc = 0, v_near = 0, v_splA = 0, v_splB = 0, v_leaf = 0, v_self = 0;
+  int4 mine = make_int4(0, 0, 0, 0);  // the warp's
+  for (int r = 0; r < rounds; ++r) {
+    int act = -1, children = 0;
+    int2 pr;
+    const int64_t i = i0 + 4 * r;
+    if (i < nf && front_pair(front[i], lane & 7, pr)) {
+      const bool hint = score != nullptr && score[8 * i + (lane & 7)] < target;
+      act = classify(pr.x, pr.y, zr, zf, theta, th2f, hint, children);
+    }
+    const unsigned acc = __ballot_sync(kAll, act == kAccept), near = __ballot_sync(kAll, act == kNear),
+                   splA = __ballot_sync(kAll, act == kSplitA), splB = __ballot_sync(kAll, act == kSplitB);
+    mine.y += __popc(acc);
+    mine.z += __popc(near);
+    mine.x += __popc(splA | splB);
+    unsigned leaf = 0, own = 0;
+    if (__any_sync(kAll, act >= 0 && act < kAccept)) {
+      leaf = __ballot_sync(kAll, act == kSelfLeaf);
+      own = __ballot_sync(kAll, act == kSelfSplit);
+      mine.w += __popc(leaf);
+      mine.x += __reduce_add_sync(kAll, act == kSelfSplit ? self_records(children) : 0);
+    }
+    if (lane == r) {
+      v_acc = acc;
+      v_near = near;
+      v_splA = splA;
+      v_splB = splB;
+      v_leaf = leaf;
+      v_self = own;
     }
   }
-  // block-wide exclusive scan of the per-thread counts
-  int4 incl = mine;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int4 y = make_int4(__shfl_up_sync(0xffffffffu, incl.x, o), __shfl_up_sync(0xffffffffu, incl.y, o),
-                             __shfl_up_sync(0xffffffffu, incl.z, o), __shfl_up_sync(0xffffffffu, incl.w, o));
-    if (lane >= o) incl = add4(incl, y);
-  }
-  if (lane == 31) s_warp[w] = incl;
+  if (lane == 0) s_warp[w] = mine;
   __syncthreads();
-  int4 before = make_int4(incl.x - mine.x, incl.y - mine.y, incl.z - mine.z, incl.w - mine.w);
+  int4 before = make_int4(0, 0, 0, 0);
   int4 block_total = make_int4(0, 0, 0, 0);
 #pragma unroll
   for (int q = 0; q < kGenBlock / 32; ++q) {
@@ -271,10 +280,8 @@ __global__ void __launch_bounds__(kGenBlock, kGenBlocksPerSM) k_walk_gen(
       int4 v = make_int4(0, 0, 0, 0);
       if (j >= 0 && t < stop) v = ld_volatile4(&agg[j]);
       if (j >= 0 && t == stop) v = ld_volatile4(&inc[j]);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1)
-        v = add4(v, make_int4(__shfl_xor_sync(0xffffffffu, v.x, o), __shfl_xor_sync(0xffffffffu, v.y, o),
-                              __shfl_xor_sync(0xffffffffu, v.z, o), __shfl_xor_sync(0xffffffffu, v.w, o)));
+      v = make_int4(__reduce_add_sync(kAll, v.x), __reduce_add_sync(kAll, v.y), __reduce_add_sync(kAll, v.z),
+                    __reduce_add_sync(kAll, v.w));
       if (lane == 0) s_red[w] = v;
       __syncthreads();
 #pragma unroll
@@ -300,71 +307,62 @@ __global__ void __launch_bounds__(kGenBlock, kGenBlocksPerSM) k_walk_gen(
   }
   const int4 base = add4(pre, before);
   int64_t ox = base.x, oy = m2l_base + base.y, oz = p2p_base + base.z, ow = self_base + base.w;
-  bool over = false;
+  // (outputs beyond a capacity are dropped: the block of the last tile judges
+  // overflow from the totals)
+  const unsigned lt = (1u << lane) - 1;
+  for (int r = 0; r < rounds; ++r) {
+    const unsigned acc = __shfl_sync(kAll, v_acc, r), near = __shfl_sync(kAll, v_near, r),
+                   splA = __shfl_sync(kAll, v_splA, r), splB = __shfl_sync(kAll, v_splB, r),
+                   leaf = __shfl_sync(kAll, v_leaf, r), own = __shfl_sync(kAll, v_self, r), spl = splA | splB;
+    const unsigned bit = 1u << lane;
+    int2 pr = make_int2(0, 0);
+    if ((acc | near | spl | leaf | own) & bit) front_pair(front[i0 + 4 * r], lane & 7, pr);
+    const int A = pr.x, B = pr.y;
+    if (acc & bit) {
+      const int64_t o = oy + __popc(acc & lt);
+      if (o < cap_m2l) m2l[o] = make_int2(min(A, B), max(A, B));
+    } else if (near & bit) {
+      const int64_t o = oz + __popc(near & lt);
+      if (o < cap_p2p) p2p[o] = make_int2(min(A, B), max(A, B));
+    }
+    oy += __popc(acc);
+    oz += __popc(near);
+    int2 sc = make_int2(0, 0);  // first child and number of children of the cell to split
+    if ((spl | own) & bit) sc = nl[splB & bit ? B : A];
+    int at = __popc(spl & lt), num = __popc(spl);
+    if (leaf | own) {
+      if (leaf & bit) {
+        const int64_t o = ow + __popc(leaf & lt);
+        if (o < cap_self) self[o] = A;
+      }
+      ow += __popc(leaf);
+      // records of self pairs vary in number: a scan of all records
+      const int e = own & bit ? self_records(sc.y) : spl & bit ? 1 : 0;
+      int incl = e;
 #pragma unroll
-  for (int k = 0; k < kGenItems; ++k) {
-    if (act[k] < 0) continue;
-    const int A = pr[k].x, B = pr[k].y;
-    switch (act[k]) {
-      case kSelfLeaf:
-        if (ow < cap_self) self[ow] = A;
-        else over = true;
-        ++ow;
-        break;
-      case kSelfSplit: {
-        const int f = first_child[A], kk = nl[A].x;
-        for (int a = 0; a < kk; ++a) {
-          if (ox < cap_next) next[ox] = make_int2(f + a, f + a);
-          else over = true;
-          ++ox;
-        }
-        for (int a = 0; a < kk; ++a)
-          for (int b = a + 1; b < kk; ++b) {
-            if (ox < cap_next) next[ox] = make_int2(f + a, f + b);
-            else over = true;
-            ++ox;
-          }
-        break;
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(kAll, incl, o);
+        if (lane >= o) incl += y;
       }
-      case kAccept:
-        if (oy < cap_m2l) m2l[oy] = make_int2(min(A, B), max(A, B));
-        else over = true;
-        ++oy;
-        break;
-      case kNear:
-        if (oz < cap_p2p) p2p[oz] = make_int2(min(A, B), max(A, B));
-        else over = true;
-        ++oz;
-        break;
-      case kSplitA: {
-        const int f = first_child[A], kk = nl[A].x;
-        for (int a = 0; a < kk; ++a) {
-          if (ox < cap_next) next[ox] = make_int2(f + a, B);
-          else over = true;
-          ++ox;
-        }
-        break;
-      }
-      default: {
-        const int f = first_child[B], kk = nl[B].x;
-        for (int a = 0; a < kk; ++a) {
-          if (ox < cap_next) next[ox] = make_int2(A, f + a);
-          else over = true;
-          ++ox;
-        }
-        break;
+      at = incl - e;
+      num = __shfl_sync(kAll, incl, 31);
+      if (own & bit) {
+        const int all = sc.y + sc.y * (sc.y - 1) / 2;
+        for (int q = 0; q < e; ++q)
+          if (ox + at + q < cap_next) next[ox + at + q] = self_record(sc.x, sc.y, 8 * q, min(8, all - 8 * q));
       }
     }
+    if ((spl & bit) && ox + at < cap_next) next[ox + at] = split_record(sc.x, sc.y, splB & bit ? A : B, splB & bit);
+    ox += num;
   }
-  (void)over;  // the block of the last tile judges overflow from the totals
   __syncthreads();  // shared memory is reused by the next tile
   }
 }
 
 // one self pair per root, and the first generation's inputs
-__global__ void k_roots_front(int32_t nsys, int2 *__restrict__ front, GenState *__restrict__ gs) {
+__global__ void k_roots_front(int32_t nsys, int4 *__restrict__ front, GenState *__restrict__ gs) {
   const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s < nsys) front[s] = make_int2(s, s);
+  if (s < nsys) front[s] = split_record(s, 1, s, false);
   if (s == 0) gs[0].in = GenIn{nsys, 0, 0, 0};
 }
 
@@ -377,7 +375,7 @@ int pack_walk_cells(fmm_ctx *c) {
   AMFMM_TRY(ensure<CellF>(c, c->walk_zf, nc));
   k_pack_cells<<<grid_for(nc, kBlock), kBlock, 0, c->stream>>>(
       static_cast<int32_t>(nc), ptr<double>(c->Z), ptr<double>(c->Rmax), ptr<int32_t>(c->nchild),
-      ptr<int32_t>(c->level), ptr<double4_32a>(c->walk_zr), ptr<CellF>(c->walk_zf), ptr<int2>(c->walk_nl));
+      ptr<int32_t>(c->level), ptr<int32_t>(c->first_child), ptr<double4_32a>(c->walk_zr), ptr<CellF>(c->walk_zf), ptr<int2>(c->walk_nl));
   return launched(c, "walk_pack");
 }
 
@@ -392,9 +390,11 @@ int walk(fmm_ctx *c) {
   const auto per_body = [&](double lo, double k, double hi) {
     return static_cast<int64_t>(static_cast<double>(n) * std::min(hi, std::max(lo, k * s3)));
   };
-  int64_t cap_front = std::max<int64_t>(4096, per_body(0.25, 8.0, 32.0));
-  AMFMM_TRY(ensure<int2>(c, c->front[0], cap_front));
-  AMFMM_TRY(ensure<int2>(c, c->front[1], cap_front));
+  // (the largest frontier of a Plummer sphere at theta = 0.5 has about seven
+  // pairs per body, in 1.3 records)
+  int64_t cap_front = std::max<int64_t>(4096, per_body(0.1, 2.0, 8.0));
+  AMFMM_TRY(ensure<int4>(c, c->front[0], cap_front));
+  AMFMM_TRY(ensure<int4>(c, c->front[1], cap_front));
   int64_t cap_m2l = c->m2l.cap / sizeof(int2), cap_p2p = c->p2p.cap / sizeof(int2),
           cap_self = c->self_list.cap / sizeof(int32_t);
   if (cap_m2l < 1024) {
@@ -420,7 +420,7 @@ int walk(fmm_ctx *c) {
   }
   // one self pair per root: systems of a forest never interact
   const int64_t nsys = c->sz.nsys;
-  if (nsys > static_cast<int64_t>(c->front[0].cap / sizeof(int2))) AMFMM_TRY(ensure<int2>(c, c->front[0], nsys));
+  if (nsys > static_cast<int64_t>(c->front[0].cap / sizeof(int4))) AMFMM_TRY(ensure<int4>(c, c->front[0], nsys));
   // The walk lasts at most 2 depth + 1 generations with pairs (a generation
   // raises the sum of the two cells' levels by one, or by two for a pair of
   // a cell with itself); one more finds the frontier empty.
@@ -432,18 +432,19 @@ int walk(fmm_ctx *c) {
   const unsigned grid = static_cast<unsigned>(std::max(1, c->num_sms * kGenBlocksPerSM));
   // generation records: zero, then the first generation's inputs (the roots)
   AMFMM_CUDA(c, cudaMemsetAsync(gs, 0, sizeof(GenState) * (ngen + 1), st));
-  k_roots_front<<<grid_for(nsys, kBlock), kBlock, 0, st>>>(static_cast<int32_t>(nsys), ptr<int2>(c->front[0]), gs);
+  k_roots_front<<<grid_for(nsys, kBlock), kBlock, 0, st>>>(static_cast<int32_t>(nsys), ptr<int4>(c->front[0]), gs);
   AMFMM_TRY(launched(c, "walk_roots"));
   int gstart = 0;  // first generation to (re)run
   for (int attempt = 0;; ++attempt) {
     if (attempt > 16) return set_error(c, FMM_EINVAL, "walk: outputs still overflow after growing the buffers");
-    const int64_t cap_next = std::min(c->front[0].cap, c->front[1].cap) / sizeof(int2);
+    const int64_t cap_next = std::min(c->front[0].cap, c->front[1].cap) / sizeof(int4);
     cap_front = cap_next;
-    if (c->sel_enabled) {  // one score and one candidate slot per frontier pair
-      AMFMM_TRY(ensure<float>(c, c->sel_score, cap_front));
-      AMFMM_TRY(ensure<int32_t>(c, c->sel_cand, cap_front));
+    if (c->sel_enabled) {  // one score and one candidate slot per place of a record
+      AMFMM_TRY(ensure<float>(c, c->sel_score, 8 * cap_front));
+      AMFMM_TRY(ensure<int32_t>(c, c->sel_cand, 8 * cap_front));
     }
-    const int64_t max_places = (cap_next + kGenTile - 1) / kGenTile + 1;
+    // tiles are full-sized as soon as there are more of them than blocks
+    const int64_t max_places = std::max<int64_t>(grid, (cap_next + kGenTile - 1) / kGenTile) + 1;
     // look-back records; fresh memory is zeroed so no stale flag matches an epoch
     const size_t lb_bytes = static_cast<size_t>(max_places) * (sizeof(int) + 2 * sizeof(int4)) + 64;
     if (c->walk_lb.cap < lb_bytes) {
@@ -463,15 +464,15 @@ int walk(fmm_ctx *c) {
     for (int g = gstart; g < ngen; ++g) {
       const float *score = nullptr;
       if (c->sel_enabled) {
-        AMFMM_TRY(walk_scores(c, &gs[g].in.nf, cap_front, ptr<int2>(c->front[g & 1]), ptr<float>(c->sel_score)));
+        AMFMM_TRY(walk_scores(c, &gs[g].in.nf, cap_front, ptr<int4>(c->front[g & 1]), ptr<float>(c->sel_score)));
         score = ptr<float>(c->sel_score);
       }
       unsigned ep = (epoch0 + g) & 0x3fffffffu;
       if (ep == 0) ep = 1;
       k_walk_gen<<<grid, kGenBlock, 0, st>>>(
-          gs, g, ptr<int2>(c->front[g & 1]), ptr<int2>(c->walk_nl), ptr<double4_32a>(c->walk_zr),
+          gs, g, ptr<int4>(c->front[g & 1]), ptr<int2>(c->walk_nl), ptr<double4_32a>(c->walk_zr),
           ptr<CellF>(c->walk_zf), c->theta, score, static_cast<float>(c->sel_log10_target),
-          ptr<int32_t>(c->first_child), ptr<int2>(c->front[(g + 1) & 1]), cap_next, ptr<int2>(c->m2l), cap_m2l,
+          ptr<int4>(c->front[(g + 1) & 1]), cap_next, ptr<int2>(c->m2l), cap_m2l,
           ptr<int2>(c->p2p), cap_p2p, ptr<int32_t>(c->self_list), cap_self, ep, std::min(max_places, nbc), flg,
           agg, inc);
       AMFMM_TRY(launched(c, "walk_gen"));
@@ -511,8 +512,8 @@ int walk(fmm_ctx *c) {
     const GenState hb = h[b];
     if ((hb.status & 4) || hb.total.x > cap_next) {
       const int64_t want = std::max<int64_t>(2 * cap_next, hb.total.x);
-      AMFMM_TRY(ensure_keep_bytes(c, c->front[b & 1], want * sizeof(int2), hb.in.nf * sizeof(int2)));
-      AMFMM_TRY(ensure<int2>(c, c->front[(b + 1) & 1], want));
+      AMFMM_TRY(ensure_keep_bytes(c, c->front[b & 1], want * sizeof(int4), hb.in.nf * sizeof(int4)));
+      AMFMM_TRY(ensure<int4>(c, c->front[(b + 1) & 1], want));
     }
     if (hb.in.m2l + hb.total.y > cap_m2l) {
       AMFMM_TRY(ensure_keep_bytes(c, c->m2l, std::max<int64_t>(2 * cap_m2l, hb.in.m2l + hb.total.y) * sizeof(int2),
@@ -557,7 +558,7 @@ using namespace amfmm;
 extern "C" int fmm_debug_walk_wait_timeout(fmm_ctx *c) {
   if (!c) return FMM_EINVAL;
   cudaStream_t st = c->stream;
-  const int64_t nf = kGenTile + 1;  // two tiles
+  const int64_t nf = kGenTile + 1;  // two tiles of empty records
   AMFMM_TRY(ensure_bytes(c, c->walk_state, 2 * sizeof(GenState)));
   const size_t lb_bytes = 2 * (sizeof(int) + 2 * sizeof(int4)) + 64;
   if (c->walk_lb.cap < lb_bytes) {
@@ -568,13 +569,12 @@ extern "C" int fmm_debug_walk_wait_timeout(fmm_ctx *c) {
   int4 *agg = static_cast<int4 *>(c->walk_lb.p);
   int4 *inc = agg + nbc;
   int *flg = reinterpret_cast<int *>(inc + nbc);
-  AMFMM_TRY(ensure<int2>(c, c->front[0], nf));
-  AMFMM_TRY(ensure<int2>(c, c->front[1], 1));
+  AMFMM_TRY(ensure<int4>(c, c->front[0], nf));
+  AMFMM_TRY(ensure<int4>(c, c->front[1], 1));
   AMFMM_TRY(ensure<int2>(c, c->walk_nl, 1));
   AMFMM_TRY(ensure<double4_32a>(c, c->walk_zr, 1));
   AMFMM_TRY(ensure<CellF>(c, c->walk_zf, 1));
-  AMFMM_TRY(ensure<int32_t>(c, c->first_child, 1));
-  AMFMM_CUDA(c, cudaMemsetAsync(c->front[0].p, 0, sizeof(int2) * nf, st));
+  AMFMM_CUDA(c, cudaMemsetAsync(c->front[0].p, 0, sizeof(int4) * nf, st));
   AMFMM_CUDA(c, cudaMemsetAsync(c->walk_nl.p, 0, sizeof(int2), st));
   AMFMM_CUDA(c, cudaMemsetAsync(c->walk_zr.p, 0, sizeof(double4_32a), st));
   AMFMM_CUDA(c, cudaMemsetAsync(c->walk_zf.p, 0, sizeof(CellF), st));
@@ -587,9 +587,9 @@ extern "C" int fmm_debug_walk_wait_timeout(fmm_ctx *c) {
   AMFMM_CUDA(c, cudaMemcpyAsync(gs, hs, 2 * sizeof(GenState), cudaMemcpyHostToDevice, st));
   c->walk_epoch = (c->walk_epoch + 1) & 0x3fffffffu;
   if (c->walk_epoch == 0) c->walk_epoch = 1;
-  k_walk_gen<<<1, kGenBlock, 0, st>>>(gs, 0, ptr<int2>(c->front[0]), ptr<int2>(c->walk_nl),
+  k_walk_gen<<<1, kGenBlock, 0, st>>>(gs, 0, ptr<int4>(c->front[0]), ptr<int2>(c->walk_nl),
                                       ptr<double4_32a>(c->walk_zr), ptr<CellF>(c->walk_zf), 0.5, nullptr, 0.f,
-                                      ptr<int32_t>(c->first_child), ptr<int2>(c->front[1]), 0, nullptr, 0, nullptr,
+                                      ptr<int4>(c->front[1]), 0, nullptr, 0, nullptr,
                                       0, nullptr, 0, c->walk_epoch, std::min<int64_t>(2, nbc), flg, agg, inc);
   AMFMM_TRY(launched(c, "walk_gen_wait_test"));
   GenState *h = static_cast<GenState *>(c->hpin);
