@@ -42,6 +42,7 @@ __device__ __forceinline__ int i3(int i, int j, int k) {
 // warp takes one child, a lane per coefficient, with a chain of 9.
 __global__ void k_l2l(int32_t c0, int32_t c1, const int32_t *__restrict__ parent,
                       const double *__restrict__ Z, double *__restrict__ loc) {
+  pdl_wait();
   const int c = c0 + blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= c1) return;
   const int p = parent[c];
@@ -71,6 +72,7 @@ constexpr int kL2LWarps = 4;
 __global__ void __launch_bounds__(kL2LWarps * 32) k_l2l_warp(int32_t c0, int32_t c1,
                                                              const int32_t *__restrict__ parent,
                                                              const double *__restrict__ Z, double *__restrict__ loc) {
+  pdl_wait();
   __shared__ double sp[kL2LWarps][kLocStride], sh[kL2LWarps][6];
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
   const int c = c0 + blockIdx.x * kL2LWarps + w;
@@ -103,6 +105,7 @@ __global__ void k_l2p(int64_t n, const int32_t *__restrict__ leaf_of, const doub
                       const double *__restrict__ loc, const double *__restrict__ X,
                       const double *__restrict__ Y, const double *__restrict__ Zb,
                       const double *__restrict__ near, double *__restrict__ acc) {
+  pdl_wait();
   const int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (i >= n) return;
   const int L = leaf_of[i];
@@ -124,6 +127,7 @@ __global__ void k_l2p(int64_t n, const int32_t *__restrict__ leaf_of, const doub
 __global__ void k_unpermute(int64_t n, const int32_t *__restrict__ order, const double *__restrict__ acc,
                             double G, double *__restrict__ ax, double *__restrict__ ay,
                             double *__restrict__ az) {
+  pdl_wait();
   const int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (i >= n) return;
   const int o = order[i];
@@ -135,7 +139,6 @@ __global__ void k_unpermute(int64_t n, const int32_t *__restrict__ order, const 
 }  // namespace
 
 int downward(fmm_ctx *c) {
-  cudaStream_t st = c->stream;
   const int64_t n = c->sz.n;
   AMFMM_TRY(ensure<double>(c, c->acc, 3 * n));
   if (c->opts.order_P != 3) return downward_general(c);
@@ -146,21 +149,19 @@ int downward(fmm_ctx *c) {
     const bool many = c1 - c0 >= 16 * fill;  // then a thread per child has fewer instructions in all
     const auto down = many ? k_l2l : k_l2l_warp;
     const int threads = many ? 128 : kL2LWarps * 32;
-    down<<<grid_for(c1 - c0, many ? 128 : kL2LWarps), threads, 0, st>>>(
-        static_cast<int32_t>(c0), static_cast<int32_t>(c1), ptr<int32_t>(c->parent), ptr<double>(c->Z),
-        ptr<double>(c->loc));
+    launch(c, down, grid_for(c1 - c0, many ? 128 : kL2LWarps), threads, 0, static_cast<int32_t>(c0),
+           static_cast<int32_t>(c1), ptr<int32_t>(c->parent), ptr<double>(c->Z), ptr<double>(c->loc));
     AMFMM_TRY(launched(c, "l2l"));
   }
-  k_l2p<<<grid_for(n, 256), 256, 0, st>>>(n, ptr<int32_t>(c->leaf_of), ptr<double>(c->Z), ptr<double>(c->loc),
-                                          ptr<double>(c->X), ptr<double>(c->Y), ptr<double>(c->Zb),
-                                          ptr<double>(c->near), ptr<double>(c->acc));
+  launch(c, k_l2p, grid_for(n, 256), 256, 0, n, ptr<int32_t>(c->leaf_of), ptr<double>(c->Z), ptr<double>(c->loc),
+         ptr<double>(c->X), ptr<double>(c->Y), ptr<double>(c->Zb), ptr<double>(c->near), ptr<double>(c->acc));
   return launched(c, "l2p");
 }
 
 int forces(fmm_ctx *c, double *ax, double *ay, double *az) {
   const int64_t n = c->sz.n;
-  k_unpermute<<<grid_for(n, 256), 256, 0, c->stream>>>(n, ptr<int32_t>(c->order), ptr<double>(c->acc),
-                                                       c->opts.G, ax, ay, az);
+  launch(c, k_unpermute, grid_for(n, 256), 256, 0, n, ptr<int32_t>(c->order), ptr<double>(c->acc), c->opts.G, ax, ay,
+         az);
   return launched(c, "unpermute");
 }
 

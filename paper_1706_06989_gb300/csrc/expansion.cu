@@ -39,6 +39,7 @@ __global__ void __launch_bounds__(kWarps * 32) k_p2m(
     const int32_t *__restrict__ count, const double *__restrict__ X, const double *__restrict__ Y,
     const double *__restrict__ Zb, const double *__restrict__ Mb, double *__restrict__ S, double *__restrict__ M,
     double *__restrict__ Z, double *__restrict__ invM, double *__restrict__ mom) {
+  pdl_wait();
   constexpr int NM = mi_off(P + 1), kRounds = (NM + 31) / 32, kRows = kP2MRows<P>;
   extern __shared__ double rows_all[];  // [kWarps][kRows][33]
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
@@ -125,6 +126,7 @@ __global__ void __launch_bounds__(kWarps * 32) k_m2m(int32_t c0, const int32_t *
                                                      const int32_t *__restrict__ nchild, double *__restrict__ S,
                                                      double *__restrict__ M, double *__restrict__ Z,
                                                      double *__restrict__ invM, double *__restrict__ mom) {
+  pdl_wait();
   constexpr int NM = mi_off(P + 1);
   __shared__ double buf[2][8 * NM], sf[8][3][P + 1];
   const int t = threadIdx.x, l = t & 31;
@@ -190,6 +192,7 @@ template <int P>
 __global__ void __launch_bounds__(kWarps * 32) k_l2l_general(int32_t c0, int32_t c1,
                                                              const int32_t *__restrict__ parent,
                                                              const double *__restrict__ Z, double *__restrict__ loc) {
+  pdl_wait();
   constexpr int NM = mi_off(P + 1), NL = NM - 1;
   __shared__ double buf_all[kWarps][2][NM], sf_all[kWarps][3][P + 1];
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
@@ -231,6 +234,7 @@ __global__ void k_l2p_general(int64_t n, const int32_t *__restrict__ leaf_of, co
                               const double *__restrict__ loc, const double *__restrict__ X,
                               const double *__restrict__ Y, const double *__restrict__ Zb,
                               const double *__restrict__ near, double *__restrict__ acc) {
+  pdl_wait();
   const int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (i >= n) return;
   const int L = leaf_of[i];
@@ -243,21 +247,20 @@ __global__ void k_l2p_general(int64_t n, const int32_t *__restrict__ leaf_of, co
 
 template <int P>
 int upward_p(fmm_ctx *c) {
-  cudaStream_t st = c->stream;
   constexpr int kShared = static_cast<int>(sizeof(double)) * kWarps * kP2MRows<P> * 33;
   if (kShared > 48 * 1024)
     AMFMM_CUDA(c, cudaFuncSetAttribute(k_p2m<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, kShared));
-  k_p2m<P><<<grid_for(c->sz.nleaf, kWarps), kWarps * 32, kShared, st>>>(
-      static_cast<int32_t>(c->sz.nleaf), ptr<int32_t>(c->leaves), ptr<int32_t>(c->begin), ptr<int32_t>(c->count),
-      ptr<double>(c->X), ptr<double>(c->Y), ptr<double>(c->Zb), ptr<double>(c->Mb), ptr<double>(c->S),
-      ptr<double>(c->M), ptr<double>(c->Z), ptr<double>(c->invM), ptr<double>(c->mom));
+  launch(c, k_p2m<P>, grid_for(c->sz.nleaf, kWarps), kWarps * 32, kShared, static_cast<int32_t>(c->sz.nleaf),
+         ptr<int32_t>(c->leaves), ptr<int32_t>(c->begin), ptr<int32_t>(c->count), ptr<double>(c->X), ptr<double>(c->Y),
+         ptr<double>(c->Zb), ptr<double>(c->Mb), ptr<double>(c->S), ptr<double>(c->M), ptr<double>(c->Z),
+         ptr<double>(c->invM), ptr<double>(c->mom));
   AMFMM_TRY(launched(c, "p2m"));
   for (int lev = c->sz.depth - 1; lev >= 0; --lev) {
     const int64_t c0 = c->sz.lvl_off[lev], c1 = c->sz.lvl_off[lev + 1];
     if (c1 <= c0) continue;
-    k_m2m<P><<<static_cast<unsigned>(c1 - c0), kWarps * 32, 0, st>>>(
-        static_cast<int32_t>(c0), ptr<int32_t>(c->first_child), ptr<int32_t>(c->nchild), ptr<double>(c->S),
-        ptr<double>(c->M), ptr<double>(c->Z), ptr<double>(c->invM), ptr<double>(c->mom));
+    launch(c, k_m2m<P>, static_cast<unsigned>(c1 - c0), kWarps * 32, 0, static_cast<int32_t>(c0),
+           ptr<int32_t>(c->first_child), ptr<int32_t>(c->nchild), ptr<double>(c->S), ptr<double>(c->M),
+           ptr<double>(c->Z), ptr<double>(c->invM), ptr<double>(c->mom));
     AMFMM_TRY(launched(c, "m2m"));
   }
   return FMM_OK;
@@ -265,19 +268,17 @@ int upward_p(fmm_ctx *c) {
 
 template <int P>
 int downward_p(fmm_ctx *c) {
-  cudaStream_t st = c->stream;
   const int64_t n = c->sz.n;
   for (int lev = 1; lev <= c->sz.depth; ++lev) {
     const int64_t c0 = c->sz.lvl_off[lev], c1 = c->sz.lvl_off[lev + 1];
     if (c1 <= c0) continue;
-    k_l2l_general<P><<<grid_for(c1 - c0, kWarps), kWarps * 32, 0, st>>>(
-        static_cast<int32_t>(c0), static_cast<int32_t>(c1), ptr<int32_t>(c->parent), ptr<double>(c->Z),
-        ptr<double>(c->loc));
+    launch(c, k_l2l_general<P>, grid_for(c1 - c0, kWarps), kWarps * 32, 0, static_cast<int32_t>(c0),
+           static_cast<int32_t>(c1), ptr<int32_t>(c->parent), ptr<double>(c->Z), ptr<double>(c->loc));
     AMFMM_TRY(launched(c, "l2l_general"));
   }
-  k_l2p_general<P><<<grid_for(n, 128), 128, 0, st>>>(n, ptr<int32_t>(c->leaf_of), ptr<double>(c->Z),
-                                                     ptr<double>(c->loc), ptr<double>(c->X), ptr<double>(c->Y),
-                                                     ptr<double>(c->Zb), ptr<double>(c->near), ptr<double>(c->acc));
+  launch(c, k_l2p_general<P>, grid_for(n, 128), 128, 0, n, ptr<int32_t>(c->leaf_of), ptr<double>(c->Z),
+         ptr<double>(c->loc), ptr<double>(c->X), ptr<double>(c->Y), ptr<double>(c->Zb), ptr<double>(c->near),
+         ptr<double>(c->acc));
   return launched(c, "l2p_general");
 }
 

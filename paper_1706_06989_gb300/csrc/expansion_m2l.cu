@@ -116,6 +116,7 @@ struct UnitDerivs {
 template <int P>
 __global__ void __launch_bounds__(128) k_fold_moments(int32_t ncell, const double *__restrict__ mom,
                                                       double *__restrict__ out) {
+  pdl_wait();
   constexpr int NM = mi_off(P + 1), NR = (P + 1) * (P + 1), NS = red_mom_stride(P);
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= ncell) return;
@@ -145,6 +146,7 @@ __global__ void __launch_bounds__(128, 2) k_m2l_general(int64_t K, int variant, 
                                                         const double *__restrict__ Z, const double *__restrict__ invM,
                                                         const double *__restrict__ fold,
                                                         const int32_t *__restrict__ pos, double *__restrict__ slots) {
+  pdl_wait();
   constexpr int NR = (P + 1) * (P + 1), NL = red_loc_stride(P), NS = red_mom_stride(P);
   const int64_t k = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (k >= K) return;
@@ -240,6 +242,7 @@ template <int P>
 __global__ void __launch_bounds__(kSumBlock) k_reduce_general(const int32_t *__restrict__ off,
                                                               const double *__restrict__ slots,
                                                               double *__restrict__ loc) {
+  pdl_wait();
   constexpr int NS = red_loc_stride(P), NR = (P + 1) * (P + 1) - 1, NL = mi_off(P + 1) - 1;
   constexpr int kGroups = kSumBlock / NS;
   __shared__ double part[kGroups][NS];
@@ -276,21 +279,19 @@ __global__ void __launch_bounds__(kSumBlock) k_reduce_general(const int32_t *__r
 template <int P>
 int m2l_p(fmm_ctx *c) {
   const int64_t K = c->sz.n_m2l, nc = c->sz.ncell;
-  cudaStream_t st = c->stream;
   AMFMM_TRY(ensure<double>(c, c->gen_fold, static_cast<size_t>(red_mom_stride(P)) * nc));
-  k_fold_moments<P><<<grid_for(nc, 128), 128, 0, st>>>(static_cast<int32_t>(nc), ptr<double>(c->mom),
-                                                       ptr<double>(c->gen_fold));
+  launch(c, k_fold_moments<P>, grid_for(nc, 128), 128, 0, static_cast<int32_t>(nc), ptr<double>(c->mom),
+         ptr<double>(c->gen_fold));
   AMFMM_TRY(launched(c, "fold_moments"));
-  k_m2l_general<P><<<grid_for(K, 128), 128, 0, st>>>(K, c->opts.variant, ptr<int2>(c->m2l), ptr<double>(c->Z),
-                                                     ptr<double>(c->invM), ptr<double>(c->gen_fold),
-                                                     ptr<int32_t>(c->m2l_pos), ptr<double>(c->m2l_slots));
+  launch(c, k_m2l_general<P>, grid_for(K, 128), 128, 0, K, c->opts.variant, ptr<int2>(c->m2l), ptr<double>(c->Z),
+         ptr<double>(c->invM), ptr<double>(c->gen_fold), ptr<int32_t>(c->m2l_pos), ptr<double>(c->m2l_slots));
   return launched(c, "m2l_general");
 }
 
 template <int P>
 int reduce_p(fmm_ctx *c) {
-  k_reduce_general<P><<<static_cast<unsigned>(c->sz.ncell), kSumBlock, 0, c->stream>>>(
-      ptr<int32_t>(c->m2l_off), ptr<double>(c->m2l_slots), ptr<double>(c->loc));
+  launch(c, k_reduce_general<P>, static_cast<unsigned>(c->sz.ncell), kSumBlock, 0, ptr<int32_t>(c->m2l_off),
+         ptr<double>(c->m2l_slots), ptr<double>(c->loc));
   return launched(c, "reduce_general");
 }
 

@@ -18,6 +18,7 @@ constexpr int kBlock = 256;
 __global__ void k_kick(int64_t n, double h, const double *__restrict__ ax, const double *__restrict__ ay,
                        const double *__restrict__ az, double *__restrict__ vx, double *__restrict__ vy,
                        double *__restrict__ vz) {
+  pdl_wait();
   const int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (i >= n) return;
   vx[i] += h * ax[i];
@@ -28,6 +29,7 @@ __global__ void k_kick(int64_t n, double h, const double *__restrict__ ax, const
 __global__ void k_drift(int64_t n, double dt, const double *__restrict__ vx, const double *__restrict__ vy,
                         const double *__restrict__ vz, double *__restrict__ x, double *__restrict__ y,
                         double *__restrict__ z) {
+  pdl_wait();
   const int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (i >= n) return;
   x[i] += dt * vx[i];
@@ -54,6 +56,7 @@ __global__ void __launch_bounds__(kBlock) k_momentum_partial(int64_t n, const do
                                                              const double *__restrict__ vz,
                                                              const double *__restrict__ m,
                                                              double *__restrict__ part) {
+  pdl_wait();
   Comp v[6];
 #pragma unroll
   for (int k = 0; k < 6; ++k) v[k] = Comp{0, 0};
@@ -88,6 +91,7 @@ __global__ void __launch_bounds__(kBlock) k_momentum_partial(int64_t n, const do
 }
 
 __global__ void k_momentum_final(int nb, const double *__restrict__ part, double *__restrict__ out) {
+  pdl_wait();
   if (threadIdx.x >= 6 || blockIdx.x != 0) return;
   const int k = threadIdx.x;
   Comp a{0, 0};
@@ -103,9 +107,9 @@ int momentum(fmm_ctx *c, const double *x, const double *y, const double *z, cons
   const int nb = static_cast<int>(std::min<int64_t>(c->num_sms * 2, (n + kBlock - 1) / kBlock));
   AMFMM_TRY(ensure<double>(c, c->diag, static_cast<size_t>(nb) * 12 + 8));
   double *part = ptr<double>(c->diag);
-  k_momentum_partial<<<nb, kBlock, 0, c->stream>>>(n, x, y, z, vx, vy, vz, m, part);
+  launch(c, k_momentum_partial, nb, kBlock, 0, n, x, y, z, vx, vy, vz, m, part);
   AMFMM_TRY(launched(c, "momentum_partial"));
-  k_momentum_final<<<1, 32, 0, c->stream>>>(nb, part, out);
+  launch(c, k_momentum_final, 1, 32, 0, nb, part, out);
   return launched(c, "momentum_final");
 }
 
@@ -121,18 +125,17 @@ extern "C" int fmm_leapfrog(fmm_ctx *c, double *x, double *y, double *z, double 
   if (n < 1 || nsteps < 0 || !(dt == dt)) return set_error(c, FMM_EINVAL, "bad leapfrog arguments");
   if (!x || !y || !z || !vx || !vy || !vz || !m || !ax || !ay || !az)
     return set_error(c, FMM_EINVAL, "NULL array");
-  cudaStream_t st = c->stream;
   const unsigned g = grid_for(n, kBlock);
   const double h = 0.5 * dt;
   if (mom) AMFMM_TRY(momentum(c, x, y, z, vx, vy, vz, m, n, mom));
   AMFMM_TRY(fmm_solve(c, x, y, z, m, n, ax, ay, az));
   for (int s = 0; s < nsteps; ++s) {
-    k_kick<<<g, kBlock, 0, st>>>(n, h, ax, ay, az, vx, vy, vz);
+    launch(c, k_kick, g, kBlock, 0, n, h, ax, ay, az, vx, vy, vz);
     AMFMM_TRY(launched(c, "kick"));
-    k_drift<<<g, kBlock, 0, st>>>(n, dt, vx, vy, vz, x, y, z);
+    launch(c, k_drift, g, kBlock, 0, n, dt, vx, vy, vz, x, y, z);
     AMFMM_TRY(launched(c, "drift"));
     AMFMM_TRY(fmm_solve(c, x, y, z, m, n, ax, ay, az));
-    k_kick<<<g, kBlock, 0, st>>>(n, h, ax, ay, az, vx, vy, vz);
+    launch(c, k_kick, g, kBlock, 0, n, h, ax, ay, az, vx, vy, vz);
     AMFMM_TRY(launched(c, "kick"));
     if (mom) AMFMM_TRY(momentum(c, x, y, z, vx, vy, vz, m, n, mom + 6 * static_cast<int64_t>(s + 1)));
   }

@@ -232,6 +232,7 @@ __global__ void __launch_bounds__(kBlock) k_m2l64(int64_t K, const int2 *__restr
                                                    const double *__restrict__ qoh,
                                                    const int32_t *__restrict__ pos, double eps2,
                                                    double *__restrict__ slots) {
+  pdl_wait();
   const int64_t k = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (k >= K) return;
   const int A = pairs[k].x, B = pairs[k].y;
@@ -415,6 +416,7 @@ __global__ void __launch_bounds__(kGatherWarps * 32) k_m2l32_gather(int32_t ncel
                                                                     const float *__restrict__ cell32,
                                                                     double *__restrict__ loc, float eps2,
                                                                     int *__restrict__ queue) {
+  pdl_wait();
   // per warp, per coefficient, per lane: the lane's sum and (negated) error
   __shared__ float sh[kGatherWarps][19][33];
   __shared__ float sl[kGatherWarps][19][33];
@@ -496,6 +498,7 @@ __global__ void __launch_bounds__(kGatherWarps * 32) k_m2l32_gather(int32_t ncel
 // t_i = Oh_ijj (both trace-free).
 __global__ void k_qoh(int32_t ncell, const double *__restrict__ invM, const double *__restrict__ mom, int tf_q,
                       int tf_o, double *__restrict__ qoh) {
+  pdl_wait();
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= ncell) return;
   const double *m = mom + static_cast<int64_t>(c) * kMomStride;
@@ -535,6 +538,7 @@ __global__ void k_qoh(int32_t ncell, const double *__restrict__ invM, const doub
 __global__ void k_cell32(int32_t ncell, const double *__restrict__ Z, const double *__restrict__ M,
                          const double *__restrict__ invM, const double *__restrict__ mom,
                          float *__restrict__ cell32) {
+  pdl_wait();
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= ncell) return;
   float *o = cell32 + static_cast<int64_t>(c) * kCell32;
@@ -558,6 +562,7 @@ __global__ void k_cell32(int32_t ncell, const double *__restrict__ Z, const doub
 __global__ void k_cell32_tf(int32_t ncell, const double *__restrict__ Z, const double *__restrict__ M,
                             const double *__restrict__ invM, const double *__restrict__ mom,
                             float *__restrict__ cell32) {
+  pdl_wait();
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= ncell) return;
   float *o = cell32 + static_cast<int64_t>(c) * kCell32TF;
@@ -596,6 +601,7 @@ __global__ void k_cell32_tf(int32_t ncell, const double *__restrict__ Z, const d
 __global__ void k_pair_locals(int64_t K, const int2 *__restrict__ pairs, const double *__restrict__ Z,
                               const double *__restrict__ M, const double *__restrict__ invM,
                               const double *__restrict__ mom, double *__restrict__ out) {
+  pdl_wait();
   const int64_t k = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (k >= K) return;
   const int A = pairs[k].x, B = pairs[k].y;
@@ -625,6 +631,7 @@ __global__ void k_pair_locals(int64_t K, const int2 *__restrict__ pairs, const d
 // Four positions per thread, read as one 16-byte load (key is 16-byte aligned).
 __global__ void k_segment_offsets(int64_t E, int32_t ncell, const uint32_t *__restrict__ key,
                                   int32_t *__restrict__ off) {
+  pdl_wait();
   const int64_t s0 = 4 * (blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x);
   if (s0 >= E) return;
   int k[4];
@@ -650,6 +657,7 @@ __global__ void k_segment_offsets(int64_t E, int32_t ncell, const uint32_t *__re
 }
 
 __global__ void k_inverse(int64_t E, const uint32_t *__restrict__ sval, int32_t *__restrict__ pos) {
+  pdl_wait();
   const int64_t s = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (s < E) pos[sval[s]] = static_cast<int32_t>(s);
 }
@@ -698,6 +706,7 @@ static_assert((kRedPhases * 32) % kSlot64 == 0, "a period of loads covers whole 
 __global__ void __launch_bounds__(kRedWarps * 32) k_m2l_reduce(int32_t ncell, const int32_t *__restrict__ off,
                                                                const double *__restrict__ slots,
                                                                double *__restrict__ loc) {
+  pdl_wait();
   __shared__ double part[kRedWarps][kRedPhases][32];
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
   const int c = blockIdx.x * kRedWarps + w;
@@ -761,22 +770,21 @@ int launch_m2l64(fmm_ctx *c, int64_t K) {
   const double *Z = ptr<double>(c->Z), *M = ptr<double>(c->M), *qoh = ptr<double>(c->qoh);
   const int32_t *pos = ptr<int32_t>(c->m2l_pos);
   double *slots = ptr<double>(c->m2l_slots);
-  cudaStream_t st = c->stream;
   const double e2 = c->eps2;
   // the trace-free forms hold for the unsoftened 1/R (k_qoh wrote them)
   const bool harm = e2 == 0.0;
   switch (c->opts.variant) {
     case FMM_UC:
-      if (harm) k_m2l64<FMM_UC, true><<<g, kBlock, 0, st>>>(K, pairs, Z, M, qoh, pos, e2, slots);
-      else k_m2l64<FMM_UC, false><<<g, kBlock, 0, st>>>(K, pairs, Z, M, qoh, pos, e2, slots);
+      if (harm) launch(c, k_m2l64<FMM_UC, true>, g, kBlock, 0, K, pairs, Z, M, qoh, pos, e2, slots);
+      else launch(c, k_m2l64<FMM_UC, false>, g, kBlock, 0, K, pairs, Z, M, qoh, pos, e2, slots);
       break;
     case FMM_TC:
-      if (harm) k_m2l64<FMM_TC, true><<<g, kBlock, 0, st>>>(K, pairs, Z, M, qoh, pos, e2, slots);
-      else k_m2l64<FMM_TC, false><<<g, kBlock, 0, st>>>(K, pairs, Z, M, qoh, pos, e2, slots);
+      if (harm) launch(c, k_m2l64<FMM_TC, true>, g, kBlock, 0, K, pairs, Z, M, qoh, pos, e2, slots);
+      else launch(c, k_m2l64<FMM_TC, false>, g, kBlock, 0, K, pairs, Z, M, qoh, pos, e2, slots);
       break;
     default:
-      if (harm) k_m2l64<FMM_TCO, true><<<g, kBlock, 0, st>>>(K, pairs, Z, M, qoh, pos, e2, slots);
-      else k_m2l64<FMM_TCO, false><<<g, kBlock, 0, st>>>(K, pairs, Z, M, qoh, pos, e2, slots);
+      if (harm) launch(c, k_m2l64<FMM_TCO, true>, g, kBlock, 0, K, pairs, Z, M, qoh, pos, e2, slots);
+      else launch(c, k_m2l64<FMM_TCO, false>, g, kBlock, 0, K, pairs, Z, M, qoh, pos, e2, slots);
       break;
   }
   return launched(c, "m2l");
@@ -804,7 +812,7 @@ int launch_m2l32_gather(fmm_ctx *c) {
   const int64_t resident = static_cast<int64_t>(std::max(1, per_sm)) * std::max(1, c->num_sms);
   const unsigned g =
       static_cast<unsigned>(std::min<int64_t>(grid_for(static_cast<int64_t>(nc) * 32, kGatherWarps * 32), resident));
-  kern<<<g, kGatherWarps * 32, 0, st>>>(nc, off, partner, c32, loc, static_cast<float>(c->eps2), queue);
+  launch(c, kern, g, kGatherWarps * 32, 0, nc, off, partner, c32, loc, static_cast<float>(c->eps2), queue);
   return launched(c, "m2l");
 }
 
@@ -826,7 +834,7 @@ int sorted_entries(fmm_ctx *c, const int2 *pairs, int64_t K, int gather, DBuf ke
 }  // namespace
 
 int segment_offsets(fmm_ctx *c, int64_t E, const uint32_t *key, int32_t *off) {
-  k_segment_offsets<<<grid_for((E + 3) / 4, 256), 256, 0, c->stream>>>(E, static_cast<int32_t>(c->sz.ncell), key, off);
+  launch(c, k_segment_offsets, grid_for((E + 3) / 4, 256), 256, 0, E, static_cast<int32_t>(c->sz.ncell), key, off);
   return launched(c, "segment_offsets");
 }
 
@@ -854,7 +862,7 @@ int m2l_prepare(fmm_ctx *c) {
   AMFMM_TRY(sorted_entries(c, ptr<int2>(c->m2l), K, gather, c->ekey, c->eval, off, &c->m2l_which));
   const int which = c->m2l_which;
   if (!gather) {
-    k_inverse<<<grid_for(E, 256), 256, 0, st>>>(E, ptr<uint32_t>(c->eval[which]), ptr<int32_t>(c->m2l_pos));
+    launch(c, k_inverse, grid_for(E, 256), 256, 0, E, ptr<uint32_t>(c->eval[which]), ptr<int32_t>(c->m2l_pos));
     AMFMM_TRY(launched(c, "m2l_inverse"));
     const size_t esz = fp32 ? sizeof(float) : sizeof(double);
     const int stride = c->opts.order_P == 3 ? kSlot64 : slot_stride_general(c->opts.order_P);
@@ -863,25 +871,25 @@ int m2l_prepare(fmm_ctx *c) {
   if (fp32) {
     AMFMM_TRY(ensure<float>(c, c->cell32, static_cast<size_t>(kCell32) * nc));
     if (cell32_tf(c))
-      k_cell32_tf<<<grid_for(nc, 256), 256, 0, st>>>(static_cast<int32_t>(nc), ptr<double>(c->Z), ptr<double>(c->M),
-                                                     ptr<double>(c->invM), ptr<double>(c->mom), ptr<float>(c->cell32));
+      launch(c, k_cell32_tf, grid_for(nc, 256), 256, 0, static_cast<int32_t>(nc), ptr<double>(c->Z), ptr<double>(c->M),
+             ptr<double>(c->invM), ptr<double>(c->mom), ptr<float>(c->cell32));
     else
-      k_cell32<<<grid_for(nc, 256), 256, 0, st>>>(static_cast<int32_t>(nc), ptr<double>(c->Z), ptr<double>(c->M),
-                                                  ptr<double>(c->invM), ptr<double>(c->mom), ptr<float>(c->cell32));
+      launch(c, k_cell32, grid_for(nc, 256), 256, 0, static_cast<int32_t>(nc), ptr<double>(c->Z), ptr<double>(c->M),
+             ptr<double>(c->invM), ptr<double>(c->mom), ptr<float>(c->cell32));
     AMFMM_TRY(launched(c, "cell32"));
   } else if (c->opts.order_P == 3) {
     AMFMM_TRY(ensure<double>(c, c->qoh, static_cast<size_t>(kQOh) * nc));
     const int harm = c->eps2 == 0.0;
-    k_qoh<<<grid_for(nc, 128), 128, 0, st>>>(static_cast<int32_t>(nc), ptr<double>(c->invM), ptr<double>(c->mom),
-                                             harm, harm && c->opts.variant == FMM_TC, ptr<double>(c->qoh));
+    launch(c, k_qoh, grid_for(nc, 128), 128, 0, static_cast<int32_t>(nc), ptr<double>(c->invM), ptr<double>(c->mom),
+           harm, harm && c->opts.variant == FMM_TC, ptr<double>(c->qoh));
     AMFMM_TRY(launched(c, "qoh"));
   }
   return FMM_OK;
 }
 
 int pair_locals_tc(fmm_ctx *c, const int2 *pairs, int64_t K, double *out) {
-  k_pair_locals<<<grid_for(K, 128), 128, 0, c->stream>>>(K, pairs, ptr<double>(c->Z), ptr<double>(c->M),
-                                                        ptr<double>(c->invM), ptr<double>(c->mom), out);
+  launch(c, k_pair_locals, grid_for(K, 128), 128, 0, K, pairs, ptr<double>(c->Z), ptr<double>(c->M),
+         ptr<double>(c->invM), ptr<double>(c->mom), out);
   return launched(c, "pair_locals");
 }
 
@@ -905,8 +913,8 @@ int m2l_reduce(fmm_ctx *c) {
   int32_t *off = ptr<int32_t>(c->m2l_off);
   // (warps drawing cells from a queue, as the gather does, measured 2.44 ms
   // against 2.39 ms for one warp per cell at N = 1M)
-  k_m2l_reduce<<<grid_for(nc * 32, kRedWarps * 32), kRedWarps * 32, 0, st>>>(
-      static_cast<int32_t>(nc), off, ptr<double>(c->m2l_slots), ptr<double>(c->loc));
+  launch(c, k_m2l_reduce, grid_for(nc * 32, kRedWarps * 32), kRedWarps * 32, 0, static_cast<int32_t>(nc), off,
+         ptr<double>(c->m2l_slots), ptr<double>(c->loc));
   return launched(c, "m2l_reduce");
 }
 

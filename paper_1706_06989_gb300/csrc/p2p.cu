@@ -102,6 +102,7 @@ __global__ void __launch_bounds__(kWarps * 32) k_p2p(
     const int32_t *__restrict__ count, const double *__restrict__ Zc, const int2 *__restrict__ cols,
     double *__restrict__ near, double *__restrict__ extra, float *__restrict__ slots,
     const BodyF *__restrict__ bodyf, float eps2, int *__restrict__ queue) {
+  pdl_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
   P2PSmem<ROWS> &sm = reinterpret_cast<P2PSmem<ROWS> *>(smem_raw)[w];
@@ -243,6 +244,7 @@ __global__ void k_p2p_chunks(int32_t nleaf, int64_t n, const int32_t *__restrict
                              const int32_t *__restrict__ begin, const int32_t *__restrict__ count,
                              const int32_t *__restrict__ itemOff, const int4 *__restrict__ items,
                              const double *__restrict__ extra, double *__restrict__ near) {
+  pdl_wait();
   const int q = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int l = threadIdx.x & 31;
   if (q >= nleaf) return;
@@ -280,6 +282,7 @@ __device__ __forceinline__ int chunks_of(int ncol, int nself) {
 __global__ void k_item_counts(int32_t nleaf, const int32_t *__restrict__ leaves, const int32_t *__restrict__ count,
                               const int32_t *__restrict__ colOff, int32_t *__restrict__ nitems,
                               int32_t *__restrict__ nextra) {
+  pdl_wait();
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= nleaf) return;
   const int L = leaves[q];
@@ -291,6 +294,7 @@ __global__ void k_item_counts(int32_t nleaf, const int32_t *__restrict__ leaves,
 __global__ void k_item_fill(int32_t nleaf, const int32_t *__restrict__ leaves, const int32_t *__restrict__ count,
                             const int32_t *__restrict__ colOff, const int32_t *__restrict__ itemOff,
                             const int32_t *__restrict__ extraOff, int4 *__restrict__ items) {
+  pdl_wait();
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= nleaf) return;
   const int L = leaves[q];
@@ -310,6 +314,7 @@ __global__ void k_item_fill(int32_t nleaf, const int32_t *__restrict__ leaves, c
 __global__ void k_p2p_reduce(int64_t n, const int32_t *__restrict__ leaf_of, const int32_t *__restrict__ begin,
                              const int32_t *__restrict__ offB, const int64_t *__restrict__ poff,
                              const float *__restrict__ slots, double *__restrict__ near) {
+  pdl_wait();
   const int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (i >= n) return;
   const int L = leaf_of[i];
@@ -345,6 +350,7 @@ __global__ void k_p2p_reduce(int64_t n, const int32_t *__restrict__ leaf_of, con
 // the sorted (A, B) as pairs, and every pair's column count n_B
 __global__ void k_sorted_pairs(int64_t K, const uint32_t *__restrict__ key, const uint32_t *__restrict__ val,
                                const int32_t *__restrict__ count, int2 *__restrict__ out, int32_t *__restrict__ nb) {
+  pdl_wait();
   const int64_t s = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (s >= K) return;
   const int2 p = make_int2(static_cast<int>(key[s]), static_cast<int>(val[s]));
@@ -356,6 +362,7 @@ __global__ void k_sorted_pairs(int64_t K, const uint32_t *__restrict__ key, cons
 __global__ void k_b_positions(int64_t K, const uint32_t *__restrict__ key, const uint32_t *__restrict__ sval,
                               const int32_t *__restrict__ count, int32_t *__restrict__ pos,
                               int64_t *__restrict__ len) {
+  pdl_wait();
   const int64_t e = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (e >= K) return;
   pos[sval[e]] = static_cast<int32_t>(e);
@@ -378,6 +385,7 @@ int bits_for(int64_t v) {
 __global__ void k_leaf_cols(int32_t nleaf, const int32_t *__restrict__ leaves, const int32_t *__restrict__ count,
                             const int32_t *__restrict__ offA, const int32_t *__restrict__ pre,
                             int32_t *__restrict__ ccount, unsigned long long *__restrict__ work) {
+  pdl_wait();
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
   unsigned long long v = 0;
   if (q < nleaf) {
@@ -395,6 +403,7 @@ __global__ void k_leaf_cols(int32_t nleaf, const int32_t *__restrict__ leaves, c
 __global__ void k_cols_self(int32_t nleaf, const int32_t *__restrict__ leaves, const int32_t *__restrict__ begin,
                             const int32_t *__restrict__ count, const int32_t *__restrict__ colOff,
                             int2 *__restrict__ cols) {
+  pdl_wait();
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= nleaf) return;
   const int L = leaves[q];
@@ -407,6 +416,7 @@ __global__ void k_cols_pairs(int64_t K, const int2 *__restrict__ pairs, const in
                              const int32_t *__restrict__ offA, const int32_t *__restrict__ pre,
                              const int32_t *__restrict__ pos, const int64_t *__restrict__ poff,
                              int2 *__restrict__ cols) {
+  pdl_wait();
   // A warp writes the runs of its 32 pairs together: entry j of the warp's
   // concatenated runs goes to lane j mod 32, which finds the pair owning it
   // by a binary search over the warp's prefix sums, so consecutive lanes
@@ -465,15 +475,15 @@ int launch_p2p_rows(fmm_ctx *c) {
   const unsigned grid = static_cast<unsigned>(std::min<int64_t>(grid_for(nitem, kWarps), resident));
   int *queue = ptr<int32_t>(c->totals) + 40;
   AMFMM_CUDA(c, cudaMemsetAsync(queue, 0, sizeof(int), c->stream));
-  k_p2p<ROWS><<<grid, kWarps * 32, shm, c->stream>>>(
-      nitem, n, ptr<int4>(c->p2p_items), ptr<int32_t>(c->begin), ptr<int32_t>(c->count),
-      ptr<double>(c->Z), ptr<int2>(c->p2p_cols), ptr<double>(c->near), ptr<double>(c->p2p_extra),
-      static_cast<float *>(c->p2p_slots.p), ptr<BodyF>(c->bodyf), static_cast<float>(c->eps2), queue);
+  launch(c, k_p2p<ROWS>, grid, kWarps * 32, shm, nitem, n, ptr<int4>(c->p2p_items), ptr<int32_t>(c->begin),
+         ptr<int32_t>(c->count), ptr<double>(c->Z), ptr<int2>(c->p2p_cols), ptr<double>(c->near),
+         ptr<double>(c->p2p_extra), static_cast<float *>(c->p2p_slots.p), ptr<BodyF>(c->bodyf),
+         static_cast<float>(c->eps2), queue);
   AMFMM_TRY(launched(c, "p2p"));
   if (nitem > nleaf) {
-    k_p2p_chunks<<<grid_for(static_cast<int64_t>(nleaf) * 32, 256), 256, 0, c->stream>>>(
-        nleaf, n, ptr<int32_t>(c->leaves), ptr<int32_t>(c->begin), ptr<int32_t>(c->count),
-        ptr<int32_t>(c->p2p_itemOff), ptr<int4>(c->p2p_items), ptr<double>(c->p2p_extra), ptr<double>(c->near));
+    launch(c, k_p2p_chunks, grid_for(static_cast<int64_t>(nleaf) * 32, 256), 256, 0, nleaf, n, ptr<int32_t>(c->leaves),
+           ptr<int32_t>(c->begin), ptr<int32_t>(c->count), ptr<int32_t>(c->p2p_itemOff), ptr<int4>(c->p2p_items),
+           ptr<double>(c->p2p_extra), ptr<double>(c->near));
     AMFMM_TRY(launched(c, "p2p_chunks"));
   }
   return FMM_OK;
@@ -509,16 +519,16 @@ int p2p_prepare(fmm_ctx *c) {
     int which = 0;
     AMFMM_TRY(sort_pairs(c, ptr<int2>(c->p2p), K, false, c->pkey, c->pval, bits_for(nc), &which));
     AMFMM_TRY(segment_offsets(c, K, ptr<uint32_t>(c->pkey[which]), offA));
-    k_sorted_pairs<<<grid_for(K, 256), 256, 0, st>>>(K, ptr<uint32_t>(c->pkey[which]), ptr<uint32_t>(c->pval[which]),
-                                                     ptr<int32_t>(c->count), ptr<int2>(c->p2p_A), nb);
+    launch(c, k_sorted_pairs, grid_for(K, 256), 256, 0, K, ptr<uint32_t>(c->pkey[which]),
+           ptr<uint32_t>(c->pval[which]), ptr<int32_t>(c->count), ptr<int2>(c->p2p_A), nb);
     AMFMM_TRY(launched(c, "p2p_sorted_pairs"));
     // CSR on the B side; slot offsets: 3 n_B floats per pair, in that order
     AMFMM_TRY(sort_pairs(c, ptr<int2>(c->p2p_A), K, true, c->pkey, c->pval, bits_for(nc), &which));
     AMFMM_TRY(segment_offsets(c, K, ptr<uint32_t>(c->pkey[which]), offB));
     AMFMM_TRY(ensure<int64_t>(c, c->p2p_len, K + 1));
     int64_t *len = ptr<int64_t>(c->p2p_len);
-    k_b_positions<<<grid_for(K, 256), 256, 0, st>>>(K, ptr<uint32_t>(c->pkey[which]), ptr<uint32_t>(c->pval[which]),
-                                                    ptr<int32_t>(c->count), ptr<int32_t>(c->p2p_pos), len);
+    launch(c, k_b_positions, grid_for(K, 256), 256, 0, K, ptr<uint32_t>(c->pkey[which]), ptr<uint32_t>(c->pval[which]),
+           ptr<int32_t>(c->count), ptr<int32_t>(c->p2p_pos), len);
     AMFMM_TRY(launched(c, "p2p_bpos"));
     int64_t *ptot = ptr<int64_t>(c->totals) + 12;
     AMFMM_TRY(exclusive_scan_i64(c, len, ptr<int64_t>(c->p2p_poff), K, ptot));
@@ -530,8 +540,8 @@ int p2p_prepare(fmm_ctx *c) {
     AMFMM_TRY(exclusive_scan_i32(c, nb, pre, K + 1, nullptr));
   }
   AMFMM_CUDA(c, cudaMemsetAsync(cnt, 0, sizeof(int32_t) * (nc + 1), st));
-  k_leaf_cols<<<grid_for(nleaf, 256), 256, 0, st>>>(nleaf, ptr<int32_t>(c->leaves), ptr<int32_t>(c->count), offA,
-                                                    K > 0 ? pre : nullptr, cnt, stat);
+  launch(c, k_leaf_cols, grid_for(nleaf, 256), 256, 0, nleaf, ptr<int32_t>(c->leaves), ptr<int32_t>(c->count), offA,
+         K > 0 ? pre : nullptr, cnt, stat);
   AMFMM_TRY(launched(c, "p2p_leaf_cols"));
   AMFMM_TRY(exclusive_scan_i32(c, cnt, colOff, nc + 1, ctot));
   // work items: chunks of the column streams
@@ -543,8 +553,8 @@ int p2p_prepare(fmm_ctx *c) {
   int32_t *icnt = cnt, *ecnt = ptr<int32_t>(c->flag);  // free scratch of >= nleaf + 1
   AMFMM_CUDA(c, cudaMemsetAsync(icnt + nleaf, 0, sizeof(int32_t), st));
   AMFMM_CUDA(c, cudaMemsetAsync(ecnt + nleaf, 0, sizeof(int32_t), st));
-  k_item_counts<<<grid_for(nleaf, 256), 256, 0, st>>>(nleaf, ptr<int32_t>(c->leaves), ptr<int32_t>(c->count),
-                                                      colOff, icnt, ecnt);
+  launch(c, k_item_counts, grid_for(nleaf, 256), 256, 0, nleaf, ptr<int32_t>(c->leaves), ptr<int32_t>(c->count),
+         colOff, icnt, ecnt);
   AMFMM_TRY(launched(c, "p2p_item_counts"));
   AMFMM_TRY(exclusive_scan_i32(c, icnt, itemOff, nleaf + 1, itot));
   AMFMM_TRY(exclusive_scan_i32(c, ecnt, extraOff, nleaf + 1, etot));
@@ -575,19 +585,18 @@ int p2p_prepare(fmm_ctx *c) {
   c->sz.p2p_items = nitem;
   AMFMM_TRY(ensure<int4>(c, c->p2p_items, nitem + 1));
   AMFMM_TRY(ensure<double>(c, c->p2p_extra, nextra + 1));
-  k_item_fill<<<grid_for(nleaf, 256), 256, 0, st>>>(nleaf, ptr<int32_t>(c->leaves), ptr<int32_t>(c->count), colOff,
-                                                    itemOff, extraOff, ptr<int4>(c->p2p_items));
+  launch(c, k_item_fill, grid_for(nleaf, 256), 256, 0, nleaf, ptr<int32_t>(c->leaves), ptr<int32_t>(c->count), colOff,
+         itemOff, extraOff, ptr<int4>(c->p2p_items));
   AMFMM_TRY(launched(c, "p2p_item_fill"));
   AMFMM_TRY(ensure_bytes(c, c->p2p_slots, static_cast<size_t>(nslot + 3) * sizeof(float)));
   AMFMM_TRY(ensure<int2>(c, c->p2p_cols, ncol + 1));
-  k_cols_self<<<grid_for(nleaf, 256), 256, 0, st>>>(nleaf, ptr<int32_t>(c->leaves), ptr<int32_t>(c->begin),
-                                                    ptr<int32_t>(c->count), colOff, ptr<int2>(c->p2p_cols));
+  launch(c, k_cols_self, grid_for(nleaf, 256), 256, 0, nleaf, ptr<int32_t>(c->leaves), ptr<int32_t>(c->begin),
+         ptr<int32_t>(c->count), colOff, ptr<int2>(c->p2p_cols));
   AMFMM_TRY(launched(c, "p2p_cols_self"));
   if (K > 0) {
-    k_cols_pairs<<<grid_for(K, 256), 256, 0, st>>>(K, ptr<int2>(c->p2p_A), ptr<int32_t>(c->begin),
-                                                   ptr<int32_t>(c->count), colOff, offA, pre,
-                                                   ptr<int32_t>(c->p2p_pos), ptr<int64_t>(c->p2p_poff),
-                                                   ptr<int2>(c->p2p_cols));
+    launch(c, k_cols_pairs, grid_for(K, 256), 256, 0, K, ptr<int2>(c->p2p_A), ptr<int32_t>(c->begin),
+           ptr<int32_t>(c->count), colOff, offA, pre, ptr<int32_t>(c->p2p_pos), ptr<int64_t>(c->p2p_poff),
+           ptr<int2>(c->p2p_cols));
     AMFMM_TRY(launched(c, "p2p_cols_pairs"));
   }
   return FMM_OK;
@@ -604,9 +613,9 @@ int p2p_run(fmm_ctx *c) {
 int p2p_reduce(fmm_ctx *c) {
   if (c->sz.n_p2p == 0) return FMM_OK;
   const int64_t n = c->sz.n;
-  k_p2p_reduce<<<grid_for(n, 256), 256, 0, c->stream>>>(n, ptr<int32_t>(c->leaf_of), ptr<int32_t>(c->begin),
-                                                        ptr<int32_t>(c->p2p_offB), ptr<int64_t>(c->p2p_poff),
-                                                        static_cast<float *>(c->p2p_slots.p), ptr<double>(c->near));
+  launch(c, k_p2p_reduce, grid_for(n, 256), 256, 0, n, ptr<int32_t>(c->leaf_of), ptr<int32_t>(c->begin),
+         ptr<int32_t>(c->p2p_offB), ptr<int64_t>(c->p2p_poff), static_cast<float *>(c->p2p_slots.p),
+         ptr<double>(c->near));
   return launched(c, "p2p_reduce");
 }
 

@@ -50,6 +50,7 @@ __global__ void k_body_fixed(int64_t n, const double *__restrict__ X, const doub
                              const double *__restrict__ Zb, const double *__restrict__ Mb,
                              const double *__restrict__ box, const int32_t *__restrict__ order,
                              const int32_t *__restrict__ sysid, Rec *__restrict__ rec) {
+  pdl_wait();
   const int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (i >= n) return;
   const int ex = fix::extent_exponent(box[(sysid ? 4 * sysid[order[i]] : 0) + 3]);
@@ -121,6 +122,7 @@ __global__ void __launch_bounds__(kWarps * 32, 4) k_p2p64(
     const int2 *__restrict__ heavy, const Rec *__restrict__ rec, const double *__restrict__ X,
     const double *__restrict__ Y, const double *__restrict__ Zb, const double *__restrict__ Mb, double eps2, double *__restrict__ near,
     double *__restrict__ extra, int *__restrict__ queue) {
+  pdl_wait();
   __shared__ WarpSmem smem[kWarps];
   const int l = threadIdx.x & 31;
   WarpSmem &sm = smem[threadIdx.x >> 5];
@@ -338,6 +340,7 @@ __global__ void __launch_bounds__(kWarps * 32, 4) k_p2p64(
 __global__ void k_leaf_heavy(int32_t nleaf, const int32_t *__restrict__ leaves, const int32_t *__restrict__ begin,
                              const int32_t *__restrict__ count, const Rec *__restrict__ rec,
                              int2 *__restrict__ heavy) {
+  pdl_wait();
   const int q = static_cast<int>((blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x) >> 5);
   const int l = threadIdx.x & 31;
   if (q >= nleaf) return;  // a warp per leaf
@@ -364,6 +367,7 @@ __global__ void k_items64_count(int32_t nleaf, const int32_t *__restrict__ leave
                                 const int32_t *__restrict__ off, const uint32_t *__restrict__ partner,
                                 int32_t *__restrict__ nitems, int32_t *__restrict__ nextra,
                                 unsigned long long *__restrict__ work, unsigned long long *__restrict__ extot) {
+  pdl_wait();
   // one warp per leaf
   const int q = static_cast<int>((blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x) >> 5);
   const int l = threadIdx.x & 31;
@@ -393,6 +397,7 @@ __global__ void k_items64_count(int32_t nleaf, const int32_t *__restrict__ leave
 __global__ void k_items64_fill(int32_t nleaf, const int32_t *__restrict__ leaves, const int32_t *__restrict__ count,
                                const int32_t *__restrict__ off, const int32_t *__restrict__ itemOff,
                                const int32_t *__restrict__ extraOff, int4 *__restrict__ items) {
+  pdl_wait();
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= nleaf) return;
   const int L = leaves[q], a = count[L];
@@ -409,6 +414,7 @@ __global__ void k_p2p64_groups(int32_t nleaf, int64_t n, const int32_t *__restri
                                const int32_t *__restrict__ begin, const int32_t *__restrict__ count,
                                const int32_t *__restrict__ off, const int32_t *__restrict__ extraOff,
                                const double *__restrict__ extra, double *__restrict__ near) {
+  pdl_wait();
   const int q = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int l = threadIdx.x & 31;
   if (q >= nleaf) return;
@@ -439,15 +445,13 @@ int p2p64_prepare(fmm_ctx *c) {
   AMFMM_TRY(ensure<int32_t>(c, c->incl, std::max<int64_t>(nc + 1, n + 1)));
   AMFMM_TRY(ensure<Rec>(c, c->p2p_rec, n));
   const bool forest = c->sz.nsys > 1;
-  k_body_fixed<<<grid_for(n, 256), 256, 0, st>>>(
-      n, ptr<double>(c->X), ptr<double>(c->Y), ptr<double>(c->Zb), ptr<double>(c->Mb),
-      forest ? ptr<double>(c->sbox) : ptr<double>(c->bbox), ptr<int32_t>(c->order),
-      forest ? ptr<int32_t>(c->sysid) : nullptr, ptr<Rec>(c->p2p_rec));
+  launch(c, k_body_fixed, grid_for(n, 256), 256, 0, n, ptr<double>(c->X), ptr<double>(c->Y), ptr<double>(c->Zb),
+         ptr<double>(c->Mb), forest ? ptr<double>(c->sbox) : ptr<double>(c->bbox), ptr<int32_t>(c->order),
+         forest ? ptr<int32_t>(c->sysid) : nullptr, ptr<Rec>(c->p2p_rec));
   AMFMM_TRY(launched(c, "p2p_body_fixed"));
   AMFMM_TRY(ensure<int2>(c, c->p2p_heavy, nc));
-  k_leaf_heavy<<<grid_for(32 * static_cast<int64_t>(nleaf), 256), 256, 0, st>>>(
-      nleaf, ptr<int32_t>(c->leaves), ptr<int32_t>(c->begin), ptr<int32_t>(c->count), ptr<Rec>(c->p2p_rec),
-      ptr<int2>(c->p2p_heavy));
+  launch(c, k_leaf_heavy, grid_for(32 * static_cast<int64_t>(nleaf), 256), 256, 0, nleaf, ptr<int32_t>(c->leaves),
+         ptr<int32_t>(c->begin), ptr<int32_t>(c->count), ptr<Rec>(c->p2p_rec), ptr<int2>(c->p2p_heavy));
   AMFMM_TRY(launched(c, "p2p_leaf_heavy"));
   // every leaf's partners, in the stable order of the pair list
   int32_t *off = ptr<int32_t>(c->p2p_offA);
@@ -460,9 +464,9 @@ int p2p64_prepare(fmm_ctx *c) {
   int32_t *itemOff = ptr<int32_t>(c->p2p_itemOff), *extraOff = ptr<int32_t>(c->p2p_extraOff);
   AMFMM_CUDA(c, cudaMemsetAsync(stat, 0, sizeof(unsigned long long), st));
   AMFMM_CUDA(c, cudaMemsetAsync(ext64, 0, sizeof(unsigned long long), st));
-  k_items64_count<<<grid_for(32 * (static_cast<int64_t>(nleaf) + 1), 256), 256, 0, st>>>(
-      nleaf, ptr<int32_t>(c->leaves), ptr<int32_t>(c->count), off, K > 0 ? ptr<uint32_t>(c->pval[c->p2p_which]) : nullptr,
-      icnt, ecnt, stat, ext64);
+  launch(c, k_items64_count, grid_for(32 * (static_cast<int64_t>(nleaf) + 1), 256), 256, 0, nleaf,
+         ptr<int32_t>(c->leaves), ptr<int32_t>(c->count), off, K > 0 ? ptr<uint32_t>(c->pval[c->p2p_which]) : nullptr,
+         icnt, ecnt, stat, ext64);
   AMFMM_TRY(launched(c, "p2p64_item_counts"));
   AMFMM_TRY(exclusive_scan_i32(c, icnt, itemOff, nleaf + 1, itot));
   AMFMM_TRY(exclusive_scan_i32(c, ecnt, extraOff, nleaf + 1, etot));
@@ -483,8 +487,8 @@ int p2p64_prepare(fmm_ctx *c) {
   c->sz.p2p_items = nitem;
   AMFMM_TRY(ensure<int4>(c, c->p2p_items, nitem + 1));
   AMFMM_TRY(ensure<double>(c, c->p2p_extra, nextra + 1));
-  k_items64_fill<<<grid_for(nleaf, 256), 256, 0, st>>>(nleaf, ptr<int32_t>(c->leaves), ptr<int32_t>(c->count), off,
-                                                       itemOff, extraOff, ptr<int4>(c->p2p_items));
+  launch(c, k_items64_fill, grid_for(nleaf, 256), 256, 0, nleaf, ptr<int32_t>(c->leaves), ptr<int32_t>(c->count), off,
+         itemOff, extraOff, ptr<int4>(c->p2p_items));
   return launched(c, "p2p64_item_fill");
 }
 
@@ -497,16 +501,16 @@ int p2p64_run(fmm_ctx *c) {
   const unsigned grid = static_cast<unsigned>(std::min<int64_t>(grid_for(nitem, kWarps), resident));
   int *queue = ptr<int32_t>(c->totals) + 40;
   AMFMM_CUDA(c, cudaMemsetAsync(queue, 0, sizeof(int), c->stream));
-  kern<<<grid, kWarps * 32, 0, c->stream>>>(
-      nitem, c->sz.n, ptr<int4>(c->p2p_items), ptr<int32_t>(c->begin), ptr<int32_t>(c->count),
-      ptr<int32_t>(c->p2p_offA), c->sz.n_p2p > 0 ? ptr<uint32_t>(c->pval[c->p2p_which]) : nullptr,
-      ptr<int2>(c->p2p_heavy), ptr<Rec>(c->p2p_rec), ptr<double>(c->X), ptr<double>(c->Y), ptr<double>(c->Zb),
-      ptr<double>(c->Mb), c->eps2, ptr<double>(c->near), ptr<double>(c->p2p_extra), queue);
+  launch(c, kern, grid, kWarps * 32, 0, nitem, c->sz.n, ptr<int4>(c->p2p_items), ptr<int32_t>(c->begin),
+         ptr<int32_t>(c->count), ptr<int32_t>(c->p2p_offA),
+         c->sz.n_p2p > 0 ? ptr<uint32_t>(c->pval[c->p2p_which]) : nullptr, ptr<int2>(c->p2p_heavy),
+         ptr<Rec>(c->p2p_rec), ptr<double>(c->X), ptr<double>(c->Y), ptr<double>(c->Zb), ptr<double>(c->Mb), c->eps2,
+         ptr<double>(c->near), ptr<double>(c->p2p_extra), queue);
   AMFMM_TRY(launched(c, "p2p"));
   if (c->sz.n_p2p == 0) return FMM_OK;
-  k_p2p64_groups<<<grid_for(static_cast<int64_t>(nleaf) * 32, 256), 256, 0, c->stream>>>(
-      nleaf, c->sz.n, ptr<int32_t>(c->leaves), ptr<int32_t>(c->begin), ptr<int32_t>(c->count),
-      ptr<int32_t>(c->p2p_offA), ptr<int32_t>(c->p2p_extraOff), ptr<double>(c->p2p_extra), ptr<double>(c->near));
+  launch(c, k_p2p64_groups, grid_for(static_cast<int64_t>(nleaf) * 32, 256), 256, 0, nleaf, c->sz.n,
+         ptr<int32_t>(c->leaves), ptr<int32_t>(c->begin), ptr<int32_t>(c->count), ptr<int32_t>(c->p2p_offA),
+         ptr<int32_t>(c->p2p_extraOff), ptr<double>(c->p2p_extra), ptr<double>(c->near));
   return launched(c, "p2p_groups");
 }
 

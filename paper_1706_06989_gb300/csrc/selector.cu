@@ -57,6 +57,7 @@ __device__ __forceinline__ float lg(float v) { return __log2f(v) * 0.30102999566
 __global__ void k_cell_features(int32_t ncell, const double *__restrict__ Rmax, const double *__restrict__ M,
                                 const double *__restrict__ mom, int mstride, const int32_t *__restrict__ count,
                                 float4 *__restrict__ cf) {
+  pdl_wait();
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= ncell) return;
   const double *q = mom + static_cast<int64_t>(c) * mstride + 4;
@@ -101,6 +102,7 @@ __device__ __forceinline__ void pair_features(int A, int B, const CellF *__restr
 
 __global__ void k_features(int64_t K, const int2 *__restrict__ pairs, const CellF *__restrict__ zf,
                            const float4 *__restrict__ cf, float *__restrict__ feat) {
+  pdl_wait();
   const int64_t k = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (k >= K) return;
   float f[kF];
@@ -119,6 +121,7 @@ constexpr int kFieldTile = 256;
 __global__ void __launch_bounds__(kFieldTile) k_field_estimate(int32_t ncell, const CellF *__restrict__ zf,
                                                               const double *__restrict__ M, int32_t k0,
                                                               int32_t k1, float *__restrict__ lga) {
+  pdl_wait();
   __shared__ float4 src[kFieldTile];
   __shared__ float eps2[kFieldTile];
   const int c = blockIdx.x * kFieldTile + threadIdx.x;
@@ -173,6 +176,7 @@ __global__ void __launch_bounds__(128) k_labels(int64_t K, const int2 *__restric
                                                 const double *__restrict__ Zb, const double *__restrict__ Mb,
                                                 const double *__restrict__ Z, const double *__restrict__ loc_pair,
                                                 float *__restrict__ label) {
+  pdl_wait();
   const int64_t k = blockIdx.x;
   if (k >= K) return;
   int A = pairs[k].x, B = pairs[k].y;
@@ -474,6 +478,7 @@ __device__ __forceinline__ void infer16(const NetSmem &s, const NetRegs &r, cons
 // inference over K samples of raw features
 __global__ void __launch_bounds__(128) k_mlp_infer(int64_t K, const float *__restrict__ params,
                                                    const float *__restrict__ feat, float *__restrict__ out) {
+  pdl_wait();
   __shared__ NetSmem s;
   __shared__ float xs[4][16][kF];
   load_net(s, params);
@@ -508,6 +513,7 @@ struct TrainSmem {
 __global__ void __launch_bounds__(128) k_mlp_grad(int64_t B, const float *__restrict__ params,
                                                   const float *__restrict__ feat, const float *__restrict__ lab,
                                                   float *__restrict__ part, float *__restrict__ loss_part) {
+  pdl_wait();
   extern __shared__ __align__(16) unsigned char raw[];
   TrainSmem &s = *reinterpret_cast<TrainSmem *>(raw);
   load_net(s.net, params);
@@ -648,6 +654,7 @@ __global__ void __launch_bounds__(128) k_mlp_grad(int64_t B, const float *__rest
 // gradient = sum of the block partials in block order; loss likewise
 __global__ void k_grad_reduce(int nblk, const float *__restrict__ part, const float *__restrict__ loss_part,
                               int64_t B, float *__restrict__ grad, float *__restrict__ loss) {
+  pdl_wait();
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q < kNWeights) {
     float acc = 0.f;
@@ -663,6 +670,7 @@ __global__ void k_grad_reduce(int nblk, const float *__restrict__ part, const fl
 
 __global__ void k_adam(float *__restrict__ p, float *__restrict__ m, float *__restrict__ v,
                        const float *__restrict__ g, float lr, float b1, float b2, float eps, int step) {
+  pdl_wait();
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= kNWeights) return;
   const float gg = g[q];
@@ -691,6 +699,7 @@ __global__ void k_band_select(const long long *__restrict__ nf_dev, int64_t cap,
                               const double4_32a *__restrict__ zr, const CellF *__restrict__ zf,
                               const int32_t *__restrict__ count, int64_t min_work, double th_lo, double th_hi,
                               float *__restrict__ score, int32_t *__restrict__ cand, unsigned *__restrict__ ncand) {
+  pdl_wait();
   // the frontier size comes from the walk's generation record; a frontier
   // beyond the buffers (the walk then stops and runs again) is not scored
   const int64_t nf = 8 * min(static_cast<int64_t>(*nf_dev), cap);  // places of its records
@@ -743,6 +752,7 @@ __global__ void __launch_bounds__(128) k_walk_scores(const int4 *__restrict__ fr
                                                      const CellF *__restrict__ zf, const float4 *__restrict__ cf,
                                                      const float *__restrict__ lga, float *__restrict__ score,
                                                      unsigned long long *__restrict__ scored) {
+  pdl_wait();
   __shared__ NetSmem s;
   __shared__ float xs[4][16][kF];
   __shared__ float adj[4][16];
@@ -790,6 +800,7 @@ __global__ void __launch_bounds__(128) k_walk_scores(const int4 *__restrict__ fr
 __global__ void k_gather_batch(int64_t B, const int64_t *__restrict__ perm, int64_t start, int64_t n,
                                const float *__restrict__ X, const float *__restrict__ y, float *__restrict__ xb,
                                float *__restrict__ yb) {
+  pdl_wait();
   const int64_t b = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (b >= B) return;
   const int64_t i = perm[(start + b) % n];
@@ -803,10 +814,9 @@ __global__ void k_gather_batch(int64_t B, const int64_t *__restrict__ perm, int6
 int cell_features(fmm_ctx *c) {
   const int64_t nc = c->sz.ncell;
   AMFMM_TRY(ensure<float4>(c, c->sel_cellfeat, nc));
-  k_cell_features<<<grid_for(nc, 256), 256, 0, c->stream>>>(static_cast<int32_t>(nc), ptr<double>(c->Rmax),
-                                                           ptr<double>(c->M), ptr<double>(c->mom),
-                                                           mom_stride(c->opts.order_P), ptr<int32_t>(c->count),
-                                                           ptr<float4>(c->sel_cellfeat));
+  launch(c, k_cell_features, grid_for(nc, 256), 256, 0, static_cast<int32_t>(nc), ptr<double>(c->Rmax),
+         ptr<double>(c->M), ptr<double>(c->mom), mom_stride(c->opts.order_P), ptr<int32_t>(c->count),
+         ptr<float4>(c->sel_cellfeat));
   return launched(c, "cell_features");
 }
 
@@ -820,9 +830,9 @@ int field_estimate(fmm_ctx *c) {
     L = l;
   }
   AMFMM_TRY(ensure<float>(c, c->sel_lga, nc));
-  k_field_estimate<<<grid_for(nc, kFieldTile), kFieldTile, 0, c->stream>>>(
-      static_cast<int32_t>(nc), ptr<CellF>(c->walk_zf), ptr<double>(c->M), static_cast<int32_t>(c->sz.lvl_off[L]),
-      static_cast<int32_t>(c->sz.lvl_off[L + 1]), ptr<float>(c->sel_lga));
+  launch(c, k_field_estimate, grid_for(nc, kFieldTile), kFieldTile, 0, static_cast<int32_t>(nc),
+         ptr<CellF>(c->walk_zf), ptr<double>(c->M), static_cast<int32_t>(c->sz.lvl_off[L]),
+         static_cast<int32_t>(c->sz.lvl_off[L + 1]), ptr<float>(c->sel_lga));
   return launched(c, "field_estimate");
 }
 
@@ -832,15 +842,15 @@ int walk_scores(fmm_ctx *c, const long long *nf_dev, int64_t cap, const int4 *fr
   AMFMM_CUDA(c, cudaMemsetAsync(ncand, 0, sizeof(unsigned), st));
   const double lo = c->opts.theta, hi = c->sel_theta_max;
   // persistent grids: the frontier size is only known on the device
-  k_band_select<<<static_cast<unsigned>(c->num_sms * 8), 256, 0, st>>>(
-      nf_dev, cap, front, ptr<double4_32a>(c->walk_zr), ptr<CellF>(c->walk_zf), ptr<int32_t>(c->count),
-      c->sel_min_work, lo, hi, score, ptr<int32_t>(c->sel_cand), ncand);
+  launch(c, k_band_select, static_cast<unsigned>(c->num_sms * 8), 256, 0, nf_dev, cap, front,
+         ptr<double4_32a>(c->walk_zr), ptr<CellF>(c->walk_zf), ptr<int32_t>(c->count), c->sel_min_work, lo, hi, score,
+         ptr<int32_t>(c->sel_cand), ncand);
   AMFMM_TRY(launched(c, "band_select"));
   const unsigned g = static_cast<unsigned>(c->num_sms * 4);
-  k_walk_scores<<<g, 128, 0, st>>>(front, ptr<int32_t>(c->sel_cand), ncand, ptr<float>(c->sel_params),
-                                   ptr<CellF>(c->walk_zf), ptr<float4>(c->sel_cellfeat),
-                                   c->sel_rule == FMM_SEL_RELATIVE ? ptr<float>(c->sel_lga) : nullptr,
-                                   score, ptr<unsigned long long>(c->totals) + 10);
+  launch(c, k_walk_scores, g, 128, 0, front, ptr<int32_t>(c->sel_cand), ncand, ptr<float>(c->sel_params),
+         ptr<CellF>(c->walk_zf), ptr<float4>(c->sel_cellfeat),
+         c->sel_rule == FMM_SEL_RELATIVE ? ptr<float>(c->sel_lga) : nullptr, score,
+         ptr<unsigned long long>(c->totals) + 10);
   return launched(c, "walk_scores");
 }
 
@@ -883,20 +893,18 @@ int fmm_selector_samples(fmm_ctx *c, const int32_t *pairs, int64_t K, float *fea
   if (c->opts.order_P != 3) return set_error(c, FMM_EUNSUPPORTED, "samples are built at order 3");
   if (K < 0 || (K > 0 && (!pairs || !feat))) return set_error(c, FMM_EINVAL, "bad sample arguments");
   if (K == 0) return FMM_OK;
-  cudaStream_t st = c->stream;
   const int2 *pp = reinterpret_cast<const int2 *>(pairs);
   AMFMM_TRY(pack_walk_cells(c));
   AMFMM_TRY(cell_features(c));
-  k_features<<<grid_for(K, 256), 256, 0, st>>>(K, pp, ptr<CellF>(c->walk_zf), ptr<float4>(c->sel_cellfeat), feat);
+  launch(c, k_features, grid_for(K, 256), 256, 0, K, pp, ptr<CellF>(c->walk_zf), ptr<float4>(c->sel_cellfeat), feat);
   AMFMM_TRY(launched(c, "features"));
   if (label) {
     // the pairs' order-3 TC locals, then the per-pair errors
     AMFMM_TRY(ensure<double>(c, c->sel_scratch, static_cast<size_t>(K) * 40));
     AMFMM_TRY(pair_locals_tc(c, pp, K, ptr<double>(c->sel_scratch)));
-    k_labels<<<static_cast<unsigned>(K), 128, 0, st>>>(K, pp, ptr<int32_t>(c->begin), ptr<int32_t>(c->count),
-                                                         ptr<double>(c->X), ptr<double>(c->Y), ptr<double>(c->Zb),
-                                                         ptr<double>(c->Mb), ptr<double>(c->Z),
-                                                         ptr<double>(c->sel_scratch), label);
+    launch(c, k_labels, static_cast<unsigned>(K), 128, 0, K, pp, ptr<int32_t>(c->begin), ptr<int32_t>(c->count),
+           ptr<double>(c->X), ptr<double>(c->Y), ptr<double>(c->Zb), ptr<double>(c->Mb), ptr<double>(c->Z),
+           ptr<double>(c->sel_scratch), label);
     AMFMM_TRY(launched(c, "labels"));
   }
   return FMM_OK;
@@ -905,7 +913,7 @@ int fmm_selector_samples(fmm_ctx *c, const int32_t *pairs, int64_t K, float *fea
 int fmm_mlp_forward(fmm_ctx *c, const float *params, const float *feat, int64_t K, float *out) {
   if (!c || !params || K < 0) return FMM_EINVAL;
   if (K == 0) return FMM_OK;
-  k_mlp_infer<<<grid_for(K, 64), 128, 0, c->stream>>>(K, params, feat, out);
+  launch(c, k_mlp_infer, grid_for(K, 64), 128, 0, K, params, feat, out);
   return launched(c, "mlp_infer");
 }
 
@@ -919,15 +927,15 @@ int fmm_mlp_grad(fmm_ctx *c, const float *params, const float *feat, const float
   const size_t shm = sizeof(TrainSmem);
   // per function and device, so set on every launch (a host-side call)
   AMFMM_CUDA(c, cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(shm)));
-  k_mlp_grad<<<nblk, 128, shm, c->stream>>>(B, params, feat, label, part, lpart);
+  launch(c, k_mlp_grad, nblk, 128, shm, B, params, feat, label, part, lpart);
   AMFMM_TRY(launched(c, "mlp_grad"));
-  k_grad_reduce<<<grid_for(kNWeights, 256), 256, 0, c->stream>>>(nblk, part, lpart, B, grad, loss);
+  launch(c, k_grad_reduce, grid_for(kNWeights, 256), 256, 0, nblk, part, lpart, B, grad, loss);
   return launched(c, "grad_reduce");
 }
 
 int fmm_mlp_adam(fmm_ctx *c, float *params, float *m, float *v, const float *grad, float lr, int step) {
   if (!c || !params || !m || !v || !grad || step < 1) return FMM_EINVAL;
-  k_adam<<<grid_for(kNWeights, 256), 256, 0, c->stream>>>(params, m, v, grad, lr, 0.9f, 0.999f, 1e-8f, step);
+  launch(c, k_adam, grid_for(kNWeights, 256), 256, 0, params, m, v, grad, lr, 0.9f, 0.999f, 1e-8f, step);
   return launched(c, "adam");
 }
 
@@ -951,9 +959,8 @@ int fmm_selector_train(fmm_ctx *c, float *params, float *adam, const float *X, c
   float *grad = ptr<float>(c->sel_grad);
   float *losses = grad + kNWeights + 1;
   for (int s = 0; s < steps; ++s) {
-    k_gather_batch<<<grid_for(batch, 256), 256, 0, c->stream>>>(batch, ptr<int64_t>(c->sel_perm),
-                                                                static_cast<int64_t>(s) * batch, n, X, y,
-                                                                ptr<float>(c->sel_xb), ptr<float>(c->sel_yb));
+    launch(c, k_gather_batch, grid_for(batch, 256), 256, 0, batch, ptr<int64_t>(c->sel_perm),
+           static_cast<int64_t>(s) * batch, n, X, y, ptr<float>(c->sel_xb), ptr<float>(c->sel_yb));
     AMFMM_TRY(launched(c, "gather_batch"));
     AMFMM_TRY(fmm_mlp_grad(c, params, ptr<float>(c->sel_xb), ptr<float>(c->sel_yb), batch, grad, losses + s));
     AMFMM_TRY(fmm_mlp_adam(c, params, adam, adam + kNWeights, grad, lr, s + 1));

@@ -70,6 +70,7 @@ __device__ __forceinline__ T block_exclusive(T v, T *excl) {
 
 template <class T>
 __global__ void k_tile_reduce(const T *__restrict__ in, int64_t n, T *__restrict__ sums) {
+  pdl_wait();
   const int64_t base = static_cast<int64_t>(blockIdx.x) * kScanTile;
   T s = vzero<T>();
 #pragma unroll
@@ -89,7 +90,8 @@ __global__ void k_tile_reduce(const T *__restrict__ in, int64_t n, T *__restrict
 template <class T>
 __global__ void k_tile_scan(const T *__restrict__ in, T *__restrict__ out, int64_t n,
                             const T *__restrict__ offs, T *__restrict__ total,
-                            const T *__restrict__ sums = nullptr) {
+                            const T *__restrict__ sums) {
+  pdl_wait();
   const int64_t base = static_cast<int64_t>(blockIdx.x) * kScanTile;
   T pre = vzero<T>();
   if (!offs && sums) {
@@ -128,7 +130,7 @@ int scan_impl(fmm_ctx *c, const T *in, T *out, int64_t n, T *total, size_t tmp_o
   }
   const int64_t nt = (n + kScanTile - 1) / kScanTile;
   if (nt == 1) {
-    k_tile_scan<T><<<1, kScanBlock, 0, c->stream>>>(in, out, n, nullptr, total);
+    launch(c, k_tile_scan<T>, 1, kScanBlock, 0, in, out, n, nullptr, total, nullptr);
     return launched(c, "tile_scan");
   }
   // scratch: sums[nt], offs[nt], then the recursion's scratch
@@ -140,16 +142,16 @@ int scan_impl(fmm_ctx *c, const T *in, T *out, int64_t n, T *total, size_t tmp_o
   T *sums = reinterpret_cast<T *>(base);
   T *offs = sums + nt;
   size_t next = tmp_off + ((2 * static_cast<size_t>(nt) * sizeof(T) + 255) / 256) * 256;
-  k_tile_reduce<T><<<static_cast<unsigned>(nt), kScanBlock, 0, c->stream>>>(in, n, sums);
+  launch(c, k_tile_reduce<T>, static_cast<unsigned>(nt), kScanBlock, 0, in, n, sums);
   AMFMM_TRY(launched(c, "tile_reduce"));
   if (nt <= kRedundantTiles) {
     // few tiles: every block adds up the sums of the tiles before it (at
     // most kRedundantTiles reads, from L2) instead of a separate scan of them
-    k_tile_scan<T><<<static_cast<unsigned>(nt), kScanBlock, 0, c->stream>>>(in, out, n, nullptr, total, sums);
+    launch(c, k_tile_scan<T>, static_cast<unsigned>(nt), kScanBlock, 0, in, out, n, nullptr, total, sums);
     return launched(c, "tile_scan");
   }
   AMFMM_TRY(scan_impl<T>(c, sums, offs, nt, nullptr, next));
-  k_tile_scan<T><<<static_cast<unsigned>(nt), kScanBlock, 0, c->stream>>>(in, out, n, offs, total);
+  launch(c, k_tile_scan<T>, static_cast<unsigned>(nt), kScanBlock, 0, in, out, n, offs, total, nullptr);
   return launched(c, "tile_scan");
 }
 
@@ -264,6 +266,7 @@ __device__ __forceinline__ void count_digits(const K *__restrict__ key, int src,
 template <class K, int R>
 __global__ void __launch_bounds__(kHistBlock) k_sort_hist(const K *__restrict__ key, int src, int64_t n, int passes,
                                                           int width, SortCtl<R> *__restrict__ ctl) {
+  pdl_wait();
   extern __shared__ int cnt[];  // [passes][R]
   __shared__ bool last;
   const int t = threadIdx.x, lane = t & 31;
@@ -300,6 +303,7 @@ template <class K, int R>
 __global__ void __launch_bounds__(kHistBlock) k_group_hist(const K *__restrict__ key, int src, int64_t n, int ktile,
                                                            int tiles, int pass, int width, SortCtl<R> *__restrict__ ctl,
                                                            WaveRows wave, int64_t ntiles) {
+  pdl_wait();
   __shared__ int cnt[R];
   const int t = threadIdx.x, nd = 1 << width, shift = pass * width;
   const unsigned dmask = nd - 1;
@@ -343,6 +347,7 @@ __global__ void __launch_bounds__(kHistBlock) k_group_hist(const K *__restrict__
 template <int R>
 __global__ void __launch_bounds__(1024) k_group_scan(int ngroup, int pass, const SortCtl<R> *__restrict__ ctl,
                                                      int32_t *__restrict__ rows) {
+  pdl_wait();
   __shared__ int part[32][33], wsum[32];
   const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
   const int d0 = 32 * blockIdx.x;
@@ -398,6 +403,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) k_radix_pass(
     const K *__restrict__ key, const uint32_t *__restrict__ val, int src, int64_t n, int pass, int width,
     SortCtl<(1 << RB)> *__restrict__ ctl, const int32_t *__restrict__ rows, WaveRows wave, int spins,
     K *__restrict__ okey, uint32_t *__restrict__ oval) {
+  pdl_wait();
   constexpr int kGroup = ::amfmm::kGroup<WAVE>;
   constexpr int R = 1 << RB, kW = THREADS / 32, kTile = THREADS * ITEMS, kWarpKeys = 32 * ITEMS;
   constexpr int kD = (R + THREADS - 1) / THREADS;  // digits per thread
@@ -607,7 +613,7 @@ int radix_sort_with(fmm_ctx *c, const K *src_key, int src, DBuf key[2], DBuf val
   if (WAVE) {
     const unsigned hg = static_cast<unsigned>(std::min<int64_t>((n + 2 * kHistBlock - 1) / (2 * kHistBlock),
                                                                 2 * static_cast<int64_t>(std::max(1, c->num_sms))));
-    k_sort_hist<K, R><<<hg, kHistBlock, sizeof(int) * passes * R, st>>>(src_key, src, n, passes, width, ctl);
+    launch(c, k_sort_hist<K, R>, hg, kHistBlock, sizeof(int) * passes * R, src_key, src, n, passes, width, ctl);
     AMFMM_TRY(launched(c, "sort_hist"));
   }
   // keys given as arrays are in buffer 0; others are first written there
@@ -624,14 +630,14 @@ int radix_sort_with(fmm_ctx *c, const K *src_key, int src, DBuf key[2], DBuf val
       // tiles per block: a whole group only where the groups fill the GPU
       const int tiles = ngroups >= 2 * std::max(1, c->num_sms) ? kGroup : 1;
       AMFMM_CUDA(c, cudaMemsetAsync(wave.group, 0, sizeof(int32_t) * ngroups * R, st));
-      k_group_hist<K, R><<<static_cast<unsigned>((ntiles + tiles - 1) / tiles), kHistBlock, 0, st>>>(
-          in_key, from, n, kTile, tiles, p, width, ctl, wave, ntiles);
+      launch(c, k_group_hist<K, R>, static_cast<unsigned>((ntiles + tiles - 1) / tiles), kHistBlock, 0, in_key, from,
+             n, kTile, tiles, p, width, ctl, wave, ntiles);
       AMFMM_TRY(launched(c, "group_hist"));
-      k_group_scan<R><<<((1 << width) + 31) / 32, 1024, 0, st>>>(static_cast<int>(ngroups), p, ctl, wave.group);
+      launch(c, k_group_scan<R>, ((1 << width) + 31) / 32, 1024, 0, static_cast<int>(ngroups), p, ctl, wave.group);
       AMFMM_TRY(launched(c, "group_scan"));
     }
-    kern<<<static_cast<unsigned>(ntiles), THREADS, kPool, st>>>(in_key, in_val, from, n, p, width, ctl, wave.group, wave,
-                                                                spins, ptr<K>(key[out]), ptr<uint32_t>(val[out]));
+    launch(c, kern, static_cast<unsigned>(ntiles), THREADS, kPool, in_key, in_val, from, n, p, width, ctl, wave.group,
+           wave, spins, ptr<K>(key[out]), ptr<uint32_t>(val[out]));
     AMFMM_TRY(launched(c, "radix_pass"));
     in_key = ptr<K>(key[out]);
     in_val = ptr<uint32_t>(val[out]);

@@ -23,6 +23,7 @@ constexpr int kBlock = 256;
 __global__ void k_bbox_partial(const double *__restrict__ x, const double *__restrict__ y,
                                const double *__restrict__ z, const double *__restrict__ m,
                                int64_t n, double *__restrict__ part, int *__restrict__ status) {
+  pdl_wait();
   double lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
   bool bad = false;
   for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n;
@@ -63,6 +64,7 @@ __global__ void k_bbox_partial(const double *__restrict__ x, const double *__res
 // bbox[0..2] = lo, bbox[3] = scale = 2^21 / ext (0 when ext == 0).  One block;
 // min and max are exact, so the order of combination does not matter.
 __global__ void k_bbox_final(const double *__restrict__ part, int nb, double *__restrict__ bbox) {
+  pdl_wait();
   __shared__ double sh[6][kBlock / 32];
   double v[6] = {INFINITY, INFINITY, INFINITY, -INFINITY, -INFINITY, -INFINITY};
   for (int b = threadIdx.x; b < nb; b += blockDim.x)
@@ -114,6 +116,7 @@ __device__ __forceinline__ uint64_t spread3(uint64_t q) {
 __global__ void k_keys(const double *__restrict__ x, const double *__restrict__ y,
                        const double *__restrict__ z, int64_t n, const double *__restrict__ bbox,
                        uint64_t *__restrict__ key, uint32_t *__restrict__ idx) {
+  pdl_wait();
   int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (i >= n) return;
   const double s = bbox[3];
@@ -135,6 +138,7 @@ __global__ void k_bbox_sys(const double *__restrict__ x, const double *__restric
                            const double *__restrict__ z, const double *__restrict__ m,
                            const int64_t *__restrict__ off, double *__restrict__ sbox,
                            int32_t *__restrict__ sysid, int *__restrict__ status) {
+  pdl_wait();
   const int s = blockIdx.x;
   const int64_t b = off[s], e = off[s + 1];
   double lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
@@ -183,6 +187,7 @@ __global__ void k_keys_sys(const double *__restrict__ x, const double *__restric
                            const double *__restrict__ z, int64_t n, const double *__restrict__ sbox,
                            const int32_t *__restrict__ sysid, uint64_t *__restrict__ key,
                            uint32_t *__restrict__ idx) {
+  pdl_wait();
   int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (i >= n) return;
   const double *b = sbox + 4 * sysid[i];
@@ -194,6 +199,7 @@ __global__ void k_keys_sys(const double *__restrict__ x, const double *__restric
 // second pass: (system of the body at sorted position s, s)
 __global__ void k_sys_keys(int64_t n, const uint32_t *__restrict__ idx, const int32_t *__restrict__ sysid,
                            uint32_t *__restrict__ skey, uint32_t *__restrict__ sval) {
+  pdl_wait();
   int64_t s = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (s >= n) return;
   skey[s] = static_cast<uint32_t>(sysid[idx[s]]);
@@ -203,6 +209,7 @@ __global__ void k_sys_keys(int64_t n, const uint32_t *__restrict__ idx, const in
 __global__ void k_gather_sorted(int64_t n, const uint32_t *__restrict__ perm, const uint64_t *__restrict__ k1,
                                 const uint32_t *__restrict__ i1, uint64_t *__restrict__ k2,
                                 uint32_t *__restrict__ i2) {
+  pdl_wait();
   int64_t t = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (t >= n) return;
   k2[t] = k1[perm[t]];
@@ -216,6 +223,7 @@ __global__ void k_permute(const double *__restrict__ x, const double *__restrict
                           const uint32_t *__restrict__ idx, int64_t n, double *__restrict__ X,
                           double *__restrict__ Y, double *__restrict__ Zb, double *__restrict__ Mb,
                           int32_t *__restrict__ order, BodyF *__restrict__ bodyf) {
+  pdl_wait();
   int64_t s = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (s >= n) return;
   const uint32_t o = idx[s];
@@ -271,10 +279,12 @@ __device__ __forceinline__ int window_digits(const uint64_t *__restrict__ key, c
 // j - step).
 __global__ void k_window_digits(const uint64_t *__restrict__ key, const uint32_t *__restrict__ idx,
                                 const int32_t *__restrict__ sysid, int64_t n, int w, int8_t *__restrict__ out) {
+  pdl_wait();
   const int64_t j = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (j < n) out[j] = static_cast<int8_t>(window_digits(key, idx, sysid, n, j, w));
 }
 __global__ void k_window_max(int64_t n, int64_t step, const int8_t *__restrict__ in, int8_t *__restrict__ out) {
+  pdl_wait();
   const int64_t j = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (j < n) out[j] = j >= step ? max(in[j], in[j - step]) : in[j];
 }
@@ -286,6 +296,7 @@ __global__ void k_window_max(int64_t n, int64_t step, const int8_t *__restrict__
 __global__ void k_cell_levels(const uint64_t *__restrict__ key, const uint32_t *__restrict__ idx,
                               const int32_t *__restrict__ sysid, int64_t n, int n_crit,
                               const int8_t *__restrict__ wmax, char2 *__restrict__ lv, int32_t *__restrict__ cnt) {
+  pdl_wait();
   extern __shared__ int8_t win[];  // kBlock + n_crit window starts
   __shared__ int32_t tot[2][kLevels];
   const int t = threadIdx.x, lane = t & 31;
@@ -324,6 +335,7 @@ __global__ void k_emit_cells(int64_t n, const char2 *__restrict__ lv, const int3
                              int32_t *__restrict__ begin, int32_t *__restrict__ level, int32_t *__restrict__ parent,
                              int32_t *__restrict__ cell_at, int32_t *__restrict__ leaf_of,
                              int32_t *__restrict__ leaves, int32_t *__restrict__ lvl) {
+  pdl_wait();
   __shared__ int32_t base[2][kLevels][kBlock / 32];
   __shared__ int32_t first[kLevels + 1];
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
@@ -388,6 +400,7 @@ __global__ void k_finish_cells(int64_t n, int n_crit, int nsys, int64_t cap, con
                                const int32_t *__restrict__ level, const int32_t *__restrict__ parent,
                                const int32_t *__restrict__ cell_at, int32_t *__restrict__ count,
                                int32_t *__restrict__ first_child, int32_t *__restrict__ nchild) {
+  pdl_wait();
   const int ncell = lvl[kLevels];
   if (ncell > cap) return;  // built again with more room
   for (int64_t id = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; id < ncell;
@@ -441,6 +454,7 @@ __global__ void __launch_bounds__(kUpWarps * 32) k_leaf_upward(
     const int32_t *__restrict__ count, const double *__restrict__ X, const double *__restrict__ Y,
     const double *__restrict__ Zb, const double *__restrict__ Mb, double *__restrict__ S, double *__restrict__ M,
     double *__restrict__ Z, double *__restrict__ invM, double *__restrict__ mom) {
+  pdl_wait();
   constexpr int kRounds = (G * kMomStride + 31) / 32;
   __shared__ double sh[kUpWarps][14][33];  // per body: ten products, x, y, z, 1 (first: mu x, mu y, mu z, mu)
   __shared__ double com[kUpWarps][G][4];
@@ -562,6 +576,7 @@ __global__ void __launch_bounds__(kUpWarps * 32) k_internal_upward(
     int32_t c0, int32_t c1, const int32_t *__restrict__ first_child, const int32_t *__restrict__ nchild,
     double *__restrict__ S, double *__restrict__ M, double *__restrict__ Z, double *__restrict__ invM,
     double *__restrict__ mom) {
+  pdl_wait();
   constexpr int kRounds = (CELLS * kMomStride + 31) / 32;
   __shared__ double sh[kUpWarps][kMomStride][33];
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
@@ -641,6 +656,7 @@ __global__ void __launch_bounds__(kUpWarps * 32) k_internal_upward(
 
 // Centres as hi + lo floats for the filter of R_max.
 __global__ void k_split_centres(int32_t ncell, const double *__restrict__ Z, float4 *__restrict__ zf) {
+  pdl_wait();
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= ncell) return;
   const double x = Z[3 * c], y = Z[3 * c + 1], z = Z[3 * c + 2];
@@ -665,6 +681,7 @@ __global__ void __launch_bounds__(kBlock) k_rmax_bodies(
     int64_t n, int nlev, const int32_t *__restrict__ cell_at, const BodyF *__restrict__ bodyf,
     const float4 *__restrict__ zf, const double *__restrict__ X, const double *__restrict__ Y,
     const double *__restrict__ Zb, const double *__restrict__ Z, unsigned long long *__restrict__ rmax2) {
+  pdl_wait();
   __shared__ int2 todo[kBlock / 32][64];  // (body, cell) still to be evaluated
   const int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -728,6 +745,7 @@ __global__ void __launch_bounds__(kBlock) k_rmax_bodies(
 
 __global__ void k_rmax_final(int32_t ncell, const unsigned long long *__restrict__ rmax2,
                              double *__restrict__ Rmax) {
+  pdl_wait();
   int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c < ncell) Rmax[c] = __dsqrt_rn(__longlong_as_double(static_cast<long long>(rmax2[c])));
 }
@@ -771,46 +789,44 @@ int build_tree(fmm_ctx *c) {
   const int nsys = c->sz.nsys;
   int which = 0;
   if (nsys == 1) {
-    k_bbox_partial<<<nbb, kBlock, 0, st>>>(c->x, c->y, c->z, c->m, n, ptr<double>(c->bbox_part), status);
+    launch(c, k_bbox_partial, nbb, kBlock, 0, c->x, c->y, c->z, c->m, n, ptr<double>(c->bbox_part), status);
     AMFMM_TRY(launched(c, "bbox_partial"));
-    k_bbox_final<<<1, kBlock, 0, st>>>(ptr<double>(c->bbox_part), nbb, ptr<double>(c->bbox));
+    launch(c, k_bbox_final, 1, kBlock, 0, ptr<double>(c->bbox_part), nbb, ptr<double>(c->bbox));
     AMFMM_TRY(launched(c, "bbox_final"));
-    k_keys<<<grid_for(n, kBlock), kBlock, 0, st>>>(c->x, c->y, c->z, n, ptr<double>(c->bbox),
-                                                   ptr<uint64_t>(c->key[0]), ptr<uint32_t>(c->idx[0]));
+    launch(c, k_keys, grid_for(n, kBlock), kBlock, 0, c->x, c->y, c->z, n, ptr<double>(c->bbox),
+           ptr<uint64_t>(c->key[0]), ptr<uint32_t>(c->idx[0]));
     AMFMM_TRY(launched(c, "keys"));
     AMFMM_TRY(radix_sort_u64(c, c->key, c->idx, n, 63, &which));
   } else {
     AMFMM_TRY(ensure<double>(c, c->sbox, 4 * static_cast<size_t>(nsys)));
     AMFMM_TRY(ensure<int32_t>(c, c->sysid, n));
-    k_bbox_sys<<<nsys, kBlock, 0, st>>>(c->x, c->y, c->z, c->m, ptr<int64_t>(c->sys_off), ptr<double>(c->sbox),
-                                        ptr<int32_t>(c->sysid), status);
+    launch(c, k_bbox_sys, nsys, kBlock, 0, c->x, c->y, c->z, c->m, ptr<int64_t>(c->sys_off), ptr<double>(c->sbox),
+           ptr<int32_t>(c->sysid), status);
     AMFMM_TRY(launched(c, "bbox_sys"));
-    k_keys_sys<<<grid_for(n, kBlock), kBlock, 0, st>>>(c->x, c->y, c->z, n, ptr<double>(c->sbox),
-                                                       ptr<int32_t>(c->sysid), ptr<uint64_t>(c->key[0]),
-                                                       ptr<uint32_t>(c->idx[0]));
+    launch(c, k_keys_sys, grid_for(n, kBlock), kBlock, 0, c->x, c->y, c->z, n, ptr<double>(c->sbox),
+           ptr<int32_t>(c->sysid), ptr<uint64_t>(c->key[0]), ptr<uint32_t>(c->idx[0]));
     AMFMM_TRY(launched(c, "keys_sys"));
     int w1 = 0;
     AMFMM_TRY(radix_sort_u64(c, c->key, c->idx, n, 63, &w1));
     AMFMM_TRY(ensure<uint32_t>(c, c->ekey[0], n));
     AMFMM_TRY(ensure<uint32_t>(c, c->eval[0], n));
-    k_sys_keys<<<grid_for(n, kBlock), kBlock, 0, st>>>(n, ptr<uint32_t>(c->idx[w1]), ptr<int32_t>(c->sysid),
-                                                       ptr<uint32_t>(c->ekey[0]), ptr<uint32_t>(c->eval[0]));
+    launch(c, k_sys_keys, grid_for(n, kBlock), kBlock, 0, n, ptr<uint32_t>(c->idx[w1]), ptr<int32_t>(c->sysid),
+           ptr<uint32_t>(c->ekey[0]), ptr<uint32_t>(c->eval[0]));
     AMFMM_TRY(launched(c, "sys_keys"));
     int w2 = 0, sbits = 1;
     while ((int64_t(1) << sbits) <= nsys) ++sbits;
     AMFMM_TRY(radix_sort_u32(c, c->ekey, c->eval, n, sbits, &w2));
-    k_gather_sorted<<<grid_for(n, kBlock), kBlock, 0, st>>>(n, ptr<uint32_t>(c->eval[w2]), ptr<uint64_t>(c->key[w1]),
-                                                            ptr<uint32_t>(c->idx[w1]), ptr<uint64_t>(c->key[w1 ^ 1]),
-                                                            ptr<uint32_t>(c->idx[w1 ^ 1]));
+    launch(c, k_gather_sorted, grid_for(n, kBlock), kBlock, 0, n, ptr<uint32_t>(c->eval[w2]),
+           ptr<uint64_t>(c->key[w1]), ptr<uint32_t>(c->idx[w1]), ptr<uint64_t>(c->key[w1 ^ 1]),
+           ptr<uint32_t>(c->idx[w1 ^ 1]));
     AMFMM_TRY(launched(c, "gather_sorted"));
     which = w1 ^ 1;
   }
   const uint64_t *skey = ptr<uint64_t>(c->key[which]);
   const uint32_t *sidx = ptr<uint32_t>(c->idx[which]);
   c->sz.key_which = which;
-  k_permute<<<grid_for(n, kBlock), kBlock, 0, st>>>(c->x, c->y, c->z, c->m, sidx, n, ptr<double>(c->X),
-                                                    ptr<double>(c->Y), ptr<double>(c->Zb), ptr<double>(c->Mb),
-                                                    ptr<int32_t>(c->order), ptr<BodyF>(c->bodyf));
+  launch(c, k_permute, grid_for(n, kBlock), kBlock, 0, c->x, c->y, c->z, c->m, sidx, n, ptr<double>(c->X),
+         ptr<double>(c->Y), ptr<double>(c->Zb), ptr<double>(c->Mb), ptr<int32_t>(c->order), ptr<BodyF>(c->bodyf));
   AMFMM_TRY(launched(c, "permute"));
 
   // octree: levels of every body, ids by one scan, cells
@@ -828,20 +844,20 @@ int build_tree(fmm_ctx *c) {
     // doubling, then once more over the two halves that cover them
     AMFMM_TRY(ensure<int8_t>(c, c->lcp, 2 * n));
     int8_t *a = ptr<int8_t>(c->lcp), *o = a + n;
-    k_window_digits<<<nb, kBlock, 0, st>>>(skey, sidx, sysid, n, n_crit, a);
+    launch(c, k_window_digits, nb, kBlock, 0, skey, sidx, sysid, n, n_crit, a);
     AMFMM_TRY(launched(c, "window_digits"));
     int64_t have = 1;
     while (have < n_crit + 1) {
       const int64_t step = std::min<int64_t>(have, n_crit + 1 - have);
-      k_window_max<<<nb, kBlock, 0, st>>>(n, step, a, o);
+      launch(c, k_window_max, nb, kBlock, 0, n, step, a, o);
       AMFMM_TRY(launched(c, "window_max"));
       std::swap(a, o);
       have += step;
     }
     wmax = a;
   }
-  k_cell_levels<<<nb, kBlock, wmax ? 0 : kBlock + n_crit, st>>>(skey, sidx, sysid, n, n_crit, wmax,
-                                                              ptr<char2>(c->body_lv), cnt);
+  launch(c, k_cell_levels, nb, kBlock, wmax ? 0 : kBlock + n_crit, skey, sidx, sysid, n, n_crit, wmax,
+         ptr<char2>(c->body_lv), cnt);
   AMFMM_TRY(launched(c, "cell_levels"));
   AMFMM_TRY(exclusive_scan_i32(c, cnt, offs, ncnt, nullptr));
   int32_t *lvl = reinterpret_cast<int32_t *>(status + kStatusLvl);
@@ -854,14 +870,15 @@ int build_tree(fmm_ctx *c) {
     const int64_t cap = static_cast<int64_t>(std::min({c->begin.cap, c->count.cap, c->level.cap, c->parent.cap,
                                                        c->first_child.cap, c->nchild.cap}) /
                                              sizeof(int32_t));
-    k_emit_cells<<<nb, kBlock, 0, st>>>(n, ptr<char2>(c->body_lv), offs, cap, ptr<int32_t>(c->begin),
-                                        ptr<int32_t>(c->level), ptr<int32_t>(c->parent), ptr<int32_t>(c->cell_at),
-                                        ptr<int32_t>(c->leaf_of), ptr<int32_t>(c->leaves), lvl);
+    launch(c, k_emit_cells, nb, kBlock, 0, n, ptr<char2>(c->body_lv), offs, cap, ptr<int32_t>(c->begin),
+           ptr<int32_t>(c->level), ptr<int32_t>(c->parent), ptr<int32_t>(c->cell_at), ptr<int32_t>(c->leaf_of),
+           ptr<int32_t>(c->leaves), lvl);
     AMFMM_TRY(launched(c, "emit_cells"));
-    k_finish_cells<<<static_cast<unsigned>(std::min<int64_t>(grid_for(std::min(cap, n), kBlock), 8 * c->num_sms)),
-                     kBlock, 0, st>>>(n, n_crit, nsys, cap, ptr<int64_t>(c->sys_off), lvl, ptr<int32_t>(c->begin),
-                                      ptr<int32_t>(c->level), ptr<int32_t>(c->parent), ptr<int32_t>(c->cell_at),
-                                      ptr<int32_t>(c->count), ptr<int32_t>(c->first_child), ptr<int32_t>(c->nchild));
+    launch(c, k_finish_cells,
+           static_cast<unsigned>(std::min<int64_t>(grid_for(std::min(cap, n), kBlock), 8 * c->num_sms)), kBlock, 0, n,
+           n_crit, nsys, cap, ptr<int64_t>(c->sys_off), lvl, ptr<int32_t>(c->begin), ptr<int32_t>(c->level),
+           ptr<int32_t>(c->parent), ptr<int32_t>(c->cell_at), ptr<int32_t>(c->count), ptr<int32_t>(c->first_child),
+           ptr<int32_t>(c->nchild));
     AMFMM_TRY(launched(c, "finish_cells"));
     const HostRead rb[2] = {{h, status, sizeof(int) * kStatusWords}, {hb, bbox, 4 * sizeof(double)}};
     AMFMM_TRY(read_back(c, rb, 2));
@@ -913,32 +930,32 @@ int upward(fmm_ctx *c) {
   const auto leaf = nleaf >= 8 * fill ? k_leaf_upward<8> : nleaf >= 4 * fill ? k_leaf_upward<4>
                   : nleaf >= 2 * fill ? k_leaf_upward<2> : k_leaf_upward<1>;
   const int per = nleaf >= 8 * fill ? 8 : nleaf >= 4 * fill ? 4 : nleaf >= 2 * fill ? 2 : 1;
-  leaf<<<grid_for(nleaf, kUpWarps * per), kUpWarps * 32, 0, st>>>(
-      static_cast<int32_t>(nleaf), ptr<int32_t>(c->leaves), ptr<int32_t>(c->begin), ptr<int32_t>(c->count),
-      ptr<double>(c->X), ptr<double>(c->Y), ptr<double>(c->Zb), ptr<double>(c->Mb), ptr<double>(c->S),
-      ptr<double>(c->M), ptr<double>(c->Z), ptr<double>(c->invM), ptr<double>(c->mom));
+  launch(c, leaf, grid_for(nleaf, kUpWarps * per), kUpWarps * 32, 0, static_cast<int32_t>(nleaf),
+         ptr<int32_t>(c->leaves), ptr<int32_t>(c->begin), ptr<int32_t>(c->count), ptr<double>(c->X), ptr<double>(c->Y),
+         ptr<double>(c->Zb), ptr<double>(c->Mb), ptr<double>(c->S), ptr<double>(c->M), ptr<double>(c->Z),
+         ptr<double>(c->invM), ptr<double>(c->mom));
   AMFMM_TRY(launched(c, "leaf_upward"));
   for (int lev = c->sz.depth - 1; lev >= 0; --lev) {
     const int64_t c0 = c->sz.lvl_off[lev], c1 = c->sz.lvl_off[lev + 1];
     const bool many = c1 - c0 >= 4 * fill;  // four parents per warp once one each would fill the GPU
     const auto up = many ? k_internal_upward<4> : k_internal_upward<1>;
-    up<<<grid_for(c1 - c0, many ? 4 * kUpWarps : kUpWarps), kUpWarps * 32, 0, st>>>(
-        static_cast<int32_t>(c0), static_cast<int32_t>(c1), ptr<int32_t>(c->first_child), ptr<int32_t>(c->nchild),
-        ptr<double>(c->S), ptr<double>(c->M), ptr<double>(c->Z), ptr<double>(c->invM), ptr<double>(c->mom));
+    launch(c, up, grid_for(c1 - c0, many ? 4 * kUpWarps : kUpWarps), kUpWarps * 32, 0, static_cast<int32_t>(c0),
+           static_cast<int32_t>(c1), ptr<int32_t>(c->first_child), ptr<int32_t>(c->nchild), ptr<double>(c->S),
+           ptr<double>(c->M), ptr<double>(c->Z), ptr<double>(c->invM), ptr<double>(c->mom));
     AMFMM_TRY(launched(c, "internal_upward"));
   }
   }
   AMFMM_CUDA(c, cudaMemsetAsync(c->rmax2.p, 0, sizeof(unsigned long long) * nc, st));
   AMFMM_TRY(ensure<float4>(c, c->cellzf, 2 * nc));
-  k_split_centres<<<grid_for(nc, kBlock), kBlock, 0, st>>>(static_cast<int32_t>(nc), ptr<double>(c->Z),
-                                                           ptr<float4>(c->cellzf));
+  launch(c, k_split_centres, grid_for(nc, kBlock), kBlock, 0, static_cast<int32_t>(nc), ptr<double>(c->Z),
+         ptr<float4>(c->cellzf));
   AMFMM_TRY(launched(c, "split_centres"));
-  k_rmax_bodies<<<grid_for(n, kBlock), kBlock, 0, st>>>(
-      n, c->sz.depth + 1, ptr<int32_t>(c->cell_at), ptr<BodyF>(c->bodyf), ptr<float4>(c->cellzf), ptr<double>(c->X),
-      ptr<double>(c->Y), ptr<double>(c->Zb), ptr<double>(c->Z), ptr<unsigned long long>(c->rmax2));
+  launch(c, k_rmax_bodies, grid_for(n, kBlock), kBlock, 0, n, c->sz.depth + 1, ptr<int32_t>(c->cell_at),
+         ptr<BodyF>(c->bodyf), ptr<float4>(c->cellzf), ptr<double>(c->X), ptr<double>(c->Y), ptr<double>(c->Zb),
+         ptr<double>(c->Z), ptr<unsigned long long>(c->rmax2));
   AMFMM_TRY(launched(c, "rmax_bodies"));
-  k_rmax_final<<<grid_for(nc, kBlock), kBlock, 0, st>>>(static_cast<int32_t>(nc),
-                                                        ptr<unsigned long long>(c->rmax2), ptr<double>(c->Rmax));
+  launch(c, k_rmax_final, grid_for(nc, kBlock), kBlock, 0, static_cast<int32_t>(nc), ptr<unsigned long long>(c->rmax2),
+         ptr<double>(c->Rmax));
   return launched(c, "rmax_final");
 }
 

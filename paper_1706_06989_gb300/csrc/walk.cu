@@ -36,6 +36,7 @@ enum Action : int32_t { kSelfLeaf = 0, kSelfSplit = 1, kAccept = 2, kNear = 3, k
 __global__ void k_pack_cells(int32_t ncell, const double *__restrict__ Z, const double *__restrict__ Rmax,
                              const int32_t *__restrict__ nchild, const int32_t *__restrict__ level,
                              const int32_t *__restrict__ first_child, double4_32a *__restrict__ zr, CellF *__restrict__ zf, int2 *__restrict__ nl) {
+  pdl_wait();
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= ncell) return;
   const double x = Z[3 * c], y = Z[3 * c + 1], z = Z[3 * c + 2], R = Rmax[c];
@@ -162,6 +163,7 @@ __global__ void __launch_bounds__(kGenBlock, kGenBlocksPerSM) k_walk_gen(
     int2 *__restrict__ m2l, int64_t cap_m2l, int2 *__restrict__ p2p, int64_t cap_p2p, int32_t *__restrict__ self,
     int64_t cap_self, unsigned epoch, int64_t max_places, int *__restrict__ flag, int4 *__restrict__ agg,
     int4 *__restrict__ inc) {
+  pdl_wait();
   __shared__ unsigned s_place;
   __shared__ int4 s_warp[kGenBlock / 32];
   __shared__ int4 s_red[kGenBlock / 32];
@@ -361,6 +363,7 @@ __global__ void __launch_bounds__(kGenBlock, kGenBlocksPerSM) k_walk_gen(
 
 // one self pair per root, and the first generation's inputs
 __global__ void k_roots_front(int32_t nsys, int4 *__restrict__ front, GenState *__restrict__ gs) {
+  pdl_wait();
   const int s = blockIdx.x * blockDim.x + threadIdx.x;
   if (s < nsys) front[s] = split_record(s, 1, s, false);
   if (s == 0) gs[0].in = GenIn{nsys, 0, 0, 0};
@@ -373,9 +376,9 @@ int pack_walk_cells(fmm_ctx *c) {
   AMFMM_TRY(ensure<double4_32a>(c, c->walk_zr, nc));
   AMFMM_TRY(ensure<int2>(c, c->walk_nl, nc));
   AMFMM_TRY(ensure<CellF>(c, c->walk_zf, nc));
-  k_pack_cells<<<grid_for(nc, kBlock), kBlock, 0, c->stream>>>(
-      static_cast<int32_t>(nc), ptr<double>(c->Z), ptr<double>(c->Rmax), ptr<int32_t>(c->nchild),
-      ptr<int32_t>(c->level), ptr<int32_t>(c->first_child), ptr<double4_32a>(c->walk_zr), ptr<CellF>(c->walk_zf), ptr<int2>(c->walk_nl));
+  launch(c, k_pack_cells, grid_for(nc, kBlock), kBlock, 0, static_cast<int32_t>(nc), ptr<double>(c->Z),
+         ptr<double>(c->Rmax), ptr<int32_t>(c->nchild), ptr<int32_t>(c->level), ptr<int32_t>(c->first_child),
+         ptr<double4_32a>(c->walk_zr), ptr<CellF>(c->walk_zf), ptr<int2>(c->walk_nl));
   return launched(c, "walk_pack");
 }
 
@@ -432,7 +435,7 @@ int walk(fmm_ctx *c) {
   const unsigned grid = static_cast<unsigned>(std::max(1, c->num_sms * kGenBlocksPerSM));
   // generation records: zero, then the first generation's inputs (the roots)
   AMFMM_CUDA(c, cudaMemsetAsync(gs, 0, sizeof(GenState) * (ngen + 1), st));
-  k_roots_front<<<grid_for(nsys, kBlock), kBlock, 0, st>>>(static_cast<int32_t>(nsys), ptr<int4>(c->front[0]), gs);
+  launch(c, k_roots_front, grid_for(nsys, kBlock), kBlock, 0, static_cast<int32_t>(nsys), ptr<int4>(c->front[0]), gs);
   AMFMM_TRY(launched(c, "walk_roots"));
   int gstart = 0;  // first generation to (re)run
   for (int attempt = 0;; ++attempt) {
@@ -469,12 +472,11 @@ int walk(fmm_ctx *c) {
       }
       unsigned ep = (epoch0 + g) & 0x3fffffffu;
       if (ep == 0) ep = 1;
-      k_walk_gen<<<grid, kGenBlock, 0, st>>>(
-          gs, g, ptr<int4>(c->front[g & 1]), ptr<int2>(c->walk_nl), ptr<double4_32a>(c->walk_zr),
-          ptr<CellF>(c->walk_zf), c->theta, score, static_cast<float>(c->sel_log10_target),
-          ptr<int4>(c->front[(g + 1) & 1]), cap_next, ptr<int2>(c->m2l), cap_m2l,
-          ptr<int2>(c->p2p), cap_p2p, ptr<int32_t>(c->self_list), cap_self, ep, std::min(max_places, nbc), flg,
-          agg, inc);
+      launch(c, k_walk_gen, grid, kGenBlock, 0, gs, g, ptr<int4>(c->front[g & 1]), ptr<int2>(c->walk_nl),
+             ptr<double4_32a>(c->walk_zr), ptr<CellF>(c->walk_zf), c->theta, score,
+             static_cast<float>(c->sel_log10_target), ptr<int4>(c->front[(g + 1) & 1]), cap_next, ptr<int2>(c->m2l),
+             cap_m2l, ptr<int2>(c->p2p), cap_p2p, ptr<int32_t>(c->self_list), cap_self, ep, std::min(max_places, nbc),
+             flg, agg, inc);
       AMFMM_TRY(launched(c, "walk_gen"));
     }
     GenState *h = static_cast<GenState *>(c->hpin);
@@ -587,10 +589,9 @@ extern "C" int fmm_debug_walk_wait_timeout(fmm_ctx *c) {
   AMFMM_CUDA(c, cudaMemcpyAsync(gs, hs, 2 * sizeof(GenState), cudaMemcpyHostToDevice, st));
   c->walk_epoch = (c->walk_epoch + 1) & 0x3fffffffu;
   if (c->walk_epoch == 0) c->walk_epoch = 1;
-  k_walk_gen<<<1, kGenBlock, 0, st>>>(gs, 0, ptr<int4>(c->front[0]), ptr<int2>(c->walk_nl),
-                                      ptr<double4_32a>(c->walk_zr), ptr<CellF>(c->walk_zf), 0.5, nullptr, 0.f,
-                                      ptr<int4>(c->front[1]), 0, nullptr, 0, nullptr,
-                                      0, nullptr, 0, c->walk_epoch, std::min<int64_t>(2, nbc), flg, agg, inc);
+  launch(c, k_walk_gen, 1, kGenBlock, 0, gs, 0, ptr<int4>(c->front[0]), ptr<int2>(c->walk_nl),
+         ptr<double4_32a>(c->walk_zr), ptr<CellF>(c->walk_zf), 0.5, nullptr, 0.f, ptr<int4>(c->front[1]), 0, nullptr,
+         0, nullptr, 0, nullptr, 0, c->walk_epoch, std::min<int64_t>(2, nbc), flg, agg, inc);
   AMFMM_TRY(launched(c, "walk_gen_wait_test"));
   GenState *h = static_cast<GenState *>(c->hpin);
   AMFMM_CUDA(c, cudaMemcpyAsync(h, gs, sizeof(GenState), cudaMemcpyDeviceToHost, st));
