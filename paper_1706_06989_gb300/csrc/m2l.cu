@@ -49,7 +49,8 @@ constexpr int kBlock = 256;
 constexpr int kCell32 = 24;    // floats per cell in the mixed form's copy (raw moments)
 constexpr int kCell32TF = 20;  // the same with trace-free moments (unsoftened UC and TC)
 constexpr int kQOh = 16;     // doubles per cell of the FP64 form's quadrupole and octupole per mass
-constexpr int kSlot64 = 24;  // doubles per slot of the FP64 order-3 M2L (21 used: m2l_pair's SLOT form)
+constexpr int kSlot64 = 24;  // doubles per slot of the FP64 order-3 M2L, softened (21 used: m2l_pair's SLOT form)
+constexpr int kSlotTF = 18;  // unsoftened (m2l_slot_tf)
 
 __device__ __forceinline__ double rsqrt_t(double v) { return rsqrt(v); }
 __device__ __forceinline__ float rsqrt_t(float v) { return rsqrtf(v); }
@@ -78,22 +79,12 @@ __device__ __forceinline__ float min_r2<float>() { return 1e-30f; }
 // no divisions.  (The FP64 form runs at the FP64 pipe's rate: every
 // operation per pair counts.)
 //
-// HARM: the unsoftened 1/R is harmonic away from R = 0, so every D tensor is
-// trace-free in any two indices and its contraction with the trace part of a
-// moment vanishes.  With HARM the caller passes trace-free quadrupoles
-// (Q - tr Q / 3 I), which drops the trace term of h, and for TC trace-free
-// octupoles per unit mass (t = 0 for their difference), which drops every
-// t term of the correction: F = R^-5 [7.5 u - 17.5 n (n.u)].  Same sums up
-// to rounding, about 24 fewer FP64 operations per pair.  (Softened
-// derivatives are not trace-free, and TCO's correction is not a contraction
-// with the full D: both keep the raw moments.)
-//
-// SLOT: the pair's slot form for the FP64 reduction (kSlot64 values per
+// SLOT: the softened pair's slot form for the FP64 reduction (kSlot64 values per
 // side): C_i as above, then the unit tensors U2 and U3 themselves, then the
 // side's scale factors of the two (C^A: M_B R^-3, M_B R^-4; C^B: M_A R^-3,
 // -M_A R^-4), which the reduction applies with one FMA per value where it
 // would otherwise add (32 products fewer per pair).
-template <class T, int VARIANT, bool HARM = false, bool SLOT = false>
+template <class T, int VARIANT, bool SLOT = false>
 __device__ __forceinline__ void m2l_pair(const T r[3], T MA, T MB, const T *QA, const T *QB, const T *OhA,
                                          const T *OhB, T eps2, T *CA, T *CB) {
   const T r2 = r[0] * r[0] + r[1] * r[1] + r[2] * r[2];
@@ -118,15 +109,13 @@ __device__ __forceinline__ void m2l_pair(const T r[3], T MA, T MB, const T *QA, 
   const T Ri4 = Ri2 * Ri2;
   // h = Q_jk D_ijk / 2 = R^-4 [n_i (15 n.Q.n - 3 trQ) - 6 (Q n)_i] / 2
   const T v = T(-3) * Ri4;
-  const T c75 = T(7.5) * Ri4;
   T hA[3], hB[3];
   {
     const T *Q = QB;
     const T qx = Q[0] * x + Q[1] * y + Q[2] * z;
     const T qy = Q[1] * x + Q[3] * y + Q[4] * z;
     const T qz = Q[2] * x + Q[4] * y + Q[5] * z;
-    const T w = HARM ? c75 * (x * qx + y * qy + z * qz)
-                     : (T(7.5) * (x * qx + y * qy + z * qz) - T(1.5) * (Q[0] + Q[3] + Q[5])) * Ri4;
+    const T w = (T(7.5) * (x * qx + y * qy + z * qz) - T(1.5) * (Q[0] + Q[3] + Q[5])) * Ri4;
     hB[0] = w * x + v * qx;
     hB[1] = w * y + v * qy;
     hB[2] = w * z + v * qz;
@@ -136,8 +125,7 @@ __device__ __forceinline__ void m2l_pair(const T r[3], T MA, T MB, const T *QA, 
     const T qx = Q[0] * x + Q[1] * y + Q[2] * z;
     const T qy = Q[1] * x + Q[3] * y + Q[4] * z;
     const T qz = Q[2] * x + Q[4] * y + Q[5] * z;
-    const T w = HARM ? c75 * (x * qx + y * qy + z * qz)
-                     : (T(7.5) * (x * qx + y * qy + z * qz) - T(1.5) * (Q[0] + Q[3] + Q[5])) * Ri4;
+    const T w = (T(7.5) * (x * qx + y * qy + z * qz) - T(1.5) * (Q[0] + Q[3] + Q[5])) * Ri4;
     hA[0] = w * x + v * qx;
     hA[1] = w * y + v * qy;
     hA[2] = w * z + v * qz;
@@ -169,26 +157,7 @@ __device__ __forceinline__ void m2l_pair(const T r[3], T MA, T MB, const T *QA, 
       CB[9 + k] = -(MA4 * U3[k]);
     }
   }
-  if (VARIANT == FMM_TC && HARM) {
-    // trace-free Sh: F = 7.5 R^-5 [u + (-7/3) n (n.u)], the 7.5 R^-5 folded
-    // into the scale factors
-    T S[10];
-#pragma unroll
-    for (int k = 0; k < 10; ++k) S[k] = OhB[k] - OhA[k];
-    const T xy2 = T(2) * xy, xz2 = T(2) * xz, yz2 = T(2) * yz;
-    const T ux = S[0] * xx + S[3] * yy + S[5] * zz + S[1] * xy2 + S[2] * xz2 + S[4] * yz2;
-    const T uy = S[1] * xx + S[6] * yy + S[8] * zz + S[3] * xy2 + S[4] * xz2 + S[7] * yz2;
-    const T uz = S[2] * xx + S[7] * yy + S[9] * zz + S[4] * xy2 + S[5] * xz2 + S[8] * yz2;
-    const T w = T(-7.0 / 3.0) * (x * ux + y * uy + z * uz);
-    const T F[3] = {ux + w * x, uy + w * y, uz + w * z};
-    const T c5 = c75 * Ri;
-    const T sA = MB * c5, sB = MA * c5;
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      CA[i] -= F[i] * sA;
-      CB[i] += F[i] * sB;
-    }
-  } else if (VARIANT != FMM_UC) {
+  if (VARIANT != FMM_UC) {
     // Sh = Oh_B - Oh_A = S / (M_A M_B) (xxx xxy xxz xyy xyz xzz yyy yyz yzz zzz)
     T S[10];
 #pragma unroll
@@ -220,12 +189,102 @@ __device__ __forceinline__ void m2l_pair(const T r[3], T MA, T MB, const T *QA, 
   }
 }
 
-// One thread per accepted pair.  Slots are kSlot64 wide (m2l_pair's SLOT
-// form, 21 used).
-// FP64 form: reads the FP64 cell data.
-// qoh: per cell the quadrupole (6) and the octupole per unit mass (10) the
-// pair function takes, trace-free where HARM allows (k_qoh).
-template <int VARIANT, bool HARM>
+// The unsoftened pair's slot form (kSlotTF values per side).  The unsoftened
+// 1/R is harmonic away from R = 0, so every D tensor is trace-free in any two
+// indices: its contraction with the trace part of a moment vanishes, so the
+// caller passes trace-free quadrupoles (Q - tr Q / 3 I) and, for TC, trace-free
+// octupoles per unit mass, and 7 of the 10 components of D_ijk carry the others.  (TCO's correction is not a contraction with the
+// full D: its octupoles are raw.)  With q = Q n, S = Oh_B - Oh_A, u_i = S_ikl n_k n_l,
+//   C^A_i = n_i (M_B R^-2 + 7.5 R^-4 n.q_B - sigma_B w) - 3 R^-4 q_B,i - sigma_B u_i,
+//   sigma_B = 7.5 M_B R^-5, w = -(7/3) n.u for TC,
+// and C^B_i the negative of the same with A's moments and -sigma_A.  A slot
+// holds C_i, then n_i n_j (xx xy xz yy yz zz) and D_ijk R^4 / 3 (xxx xxy xxz xyy
+// xyz yyy yyz), then the side's factors of the two; the sums form d_ij tr - 3
+// n_i n_j, multiply by 3 and restore the traces.  126 FP64 operations per pair
+// against 160 with all components of the tensors themselves (the FP64 pipe
+// bounds this kernel: 25.0M pairs in 5.7 ms against 6.9).  Subtracted constants
+// are exact: a rounded 1/3 or 1/5 errs the same way in every pair.
+template <int VARIANT>
+__device__ __forceinline__ void m2l_slot_tf(const double r[3], double MA, double MB, const double *QA,
+                                            const double *QB, const double *OhA, const double *OhB, double *CA,
+                                            double *CB) {
+  const double r2 = r[0] * r[0] + r[1] * r[1] + r[2] * r[2];
+  if (!(r2 > min_r2<double>())) {
+#pragma unroll
+    for (int q = 0; q < kSlotTF; ++q) CA[q] = CB[q] = 0.0;
+    return;
+  }
+  const double Ri = rsqrt_t(r2);
+  const double x = r[0] * Ri, y = r[1] * Ri, z = r[2] * Ri;
+  const double xx = x * x, yy = y * y, zz = z * z, xy = x * y, xz = x * z, yz = y * z;
+  const double fx = fma(5.0, xx, -1.0), fy = fma(5.0, yy, -1.0);
+  const double U[13] = {xx, xy, xz, yy, yz, zz, (fx - 2.0) * x, fx * y, fx * z, fy * x, 5.0 * xy * z,
+                        (fy - 2.0) * y, fy * z};
+#pragma unroll
+  for (int q = 0; q < 13; ++q) CA[3 + q] = CB[3 + q] = U[q];
+  const double Ri2 = Ri * Ri, Ri4 = Ri2 * Ri2, c75 = 7.5 * Ri4, v = -3.0 * Ri4;
+  const double MA2 = MA * Ri2, MB2 = MB * Ri2, MA3 = MA2 * Ri, MB3 = MB2 * Ri;
+  CA[16] = MB3;
+  CA[17] = MB3 * Ri;
+  CB[16] = MA3;
+  CB[17] = -(MA3 * Ri);
+  const double n[3] = {x, y, z};
+  // q = Q n of B and of A
+  double qB[3], qA[3];
+  qB[0] = QB[0] * x + QB[1] * y + QB[2] * z;
+  qB[1] = QB[1] * x + QB[3] * y + QB[4] * z;
+  qB[2] = QB[2] * x + QB[4] * y + QB[5] * z;
+  qA[0] = QA[0] * x + QA[1] * y + QA[2] * z;
+  qA[1] = QA[1] * x + QA[3] * y + QA[4] * z;
+  qA[2] = QA[2] * x + QA[4] * y + QA[5] * z;
+  double sA = fma(c75, x * qB[0] + y * qB[1] + z * qB[2], MB2);
+  double sB = fma(c75, x * qA[0] + y * qA[1] + z * qA[2], MA2);
+  if (VARIANT == FMM_UC) {
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      CA[i] = fma(v, qB[i], sA * n[i]);
+      CB[i] = -fma(v, qA[i], sB * n[i]);
+    }
+    return;
+  }
+  const double c5 = c75 * Ri, xy2 = 2.0 * xy, xz2 = 2.0 * xz, yz2 = 2.0 * yz;
+  double u[3], tauA, tauB;  // C^A_i -= tauA u_i, C^B_i += tauB u_i
+  if (VARIANT == FMM_TC) {
+    // S in the order xxx xxy xxz xyy xyz yyy yyz; xzz = -xxx - xyy, yzz = -xxy
+    // - yyy, zzz = -xxz - yyz
+    const double S0 = OhB[0] - OhA[0], S1 = OhB[1] - OhA[1], S2 = OhB[2] - OhA[2], S3 = OhB[3] - OhA[3],
+                 S4 = OhB[4] - OhA[4], S6 = OhB[6] - OhA[6], S7 = OhB[7] - OhA[7];
+    const double a = xx - zz, b = yy - zz;
+    u[0] = S0 * a + S3 * b + S1 * xy2 + S2 * xz2 + S4 * yz2;
+    u[1] = S1 * a + S6 * b + S3 * xy2 + S4 * xz2 + S7 * yz2;
+    u[2] = S2 * a + S7 * b + S4 * xy2 - (S0 + S3) * xz2 - (S1 + S6) * yz2;
+    tauA = MB * c5;
+    tauB = MA * c5;
+    const double w = (-7.0 / 3.0) * (x * u[0] + y * u[1] + z * u[2]);
+    sA = fma(-tauA, w, sA);
+    sB = fma(-tauB, w, sB);
+  } else {
+    double S[10];
+#pragma unroll
+    for (int k = 0; k < 10; ++k) S[k] = OhB[k] - OhA[k];
+    // F = R^-5 [7.5 u - 1.5 t], t_i = S_ijj: 7.5 R^-5 (u - t / 5)
+    u[0] = S[0] * xx + S[3] * yy + S[5] * zz + S[1] * xy2 + S[2] * xz2 + S[4] * yz2 - 0.2 * (S[0] + S[3] + S[5]);
+    u[1] = S[1] * xx + S[6] * yy + S[8] * zz + S[3] * xy2 + S[4] * xz2 + S[7] * yz2 - 0.2 * (S[1] + S[6] + S[8]);
+    u[2] = S[2] * xx + S[7] * yy + S[9] * zz + S[4] * xy2 + S[5] * xz2 + S[8] * yz2 - 0.2 * (S[2] + S[7] + S[9]);
+    tauA = MB * c5;
+    tauB = MA * c5;
+  }
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    CA[i] = fma(-tauA, u[i], fma(v, qB[i], sA * n[i]));
+    CB[i] = fma(tauB, u[i], -fma(v, qA[i], sB * n[i]));
+  }
+}
+
+// One thread per accepted pair, FP64.  qoh: per cell the quadrupole (6) and the
+// octupole per unit mass (10), trace-free where the slot form takes them so
+// (k_qoh).
+template <int VARIANT, bool TF>
 __global__ void __launch_bounds__(kBlock) k_m2l64(int64_t K, const int2 *__restrict__ pairs,
                                                    const double *__restrict__ Z,
                                                    const double *__restrict__ M,
@@ -233,19 +292,24 @@ __global__ void __launch_bounds__(kBlock) k_m2l64(int64_t K, const int2 *__restr
                                                    const int32_t *__restrict__ pos, double eps2,
                                                    double *__restrict__ slots) {
   pdl_wait();
+  constexpr int kSlot = TF ? kSlotTF : kSlot64;
   const int64_t k = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (k >= K) return;
   const int A = pairs[k].x, B = pairs[k].y;
-  double CA[kSlot64], CB[kSlot64];
+  double CA[kSlot], CB[kSlot];
   const double r[3] = {Z[3 * A] - Z[3 * B], Z[3 * A + 1] - Z[3 * B + 1], Z[3 * A + 2] - Z[3 * B + 2]};
   const double *qA = qoh + static_cast<int64_t>(A) * kQOh;
   const double *qB = qoh + static_cast<int64_t>(B) * kQOh;
-  m2l_pair<double, VARIANT, HARM, true>(r, M[A], M[B], qA, qB, qA + 6, qB + 6, eps2, CA, CB);
-  CA[21] = CB[21] = CA[22] = CB[22] = CA[23] = CB[23] = 0.0;
-  double *sa = slots + static_cast<int64_t>(pos[2 * k]) * kSlot64;
-  double *sb = slots + static_cast<int64_t>(pos[2 * k + 1]) * kSlot64;
+  if constexpr (TF) {
+    m2l_slot_tf<VARIANT>(r, M[A], M[B], qA, qB, qA + 6, qB + 6, CA, CB);
+  } else {
+    m2l_pair<double, VARIANT, true>(r, M[A], M[B], qA, qB, qA + 6, qB + 6, eps2, CA, CB);
+    CA[21] = CB[21] = CA[22] = CB[22] = CA[23] = CB[23] = 0.0;
+  }
+  double *sa = slots + static_cast<int64_t>(pos[2 * k]) * kSlot;
+  double *sb = slots + static_cast<int64_t>(pos[2 * k + 1]) * kSlot;
 #pragma unroll
-  for (int q = 0; q < kSlot64; q += 2) {
+  for (int q = 0; q < kSlot; q += 2) {
     *reinterpret_cast<double2 *>(sa + q) = make_double2(CA[q], CA[q + 1]);
     *reinterpret_cast<double2 *>(sb + q) = make_double2(CB[q], CB[q + 1]);
   }
@@ -662,7 +726,7 @@ __global__ void k_inverse(int64_t E, const uint32_t *__restrict__ sval, int32_t 
   if (s < E) pos[sval[s]] = static_cast<int32_t>(s);
 }
 
-// Every cell sums its FP64 slots (kSlot64 = 24 doubles per slot, in the
+// Every cell sums its softened FP64 slots (kSlot64 = 24 doubles per slot, in the
 // stable order of the sort): one warp per cell reads the cell's slot rows as
 // one flat array, 32 consecutive doubles per load, so every lane is busy and
 // every load is two full 128-byte lines.  Element e of the block is value
@@ -762,6 +826,51 @@ __global__ void __launch_bounds__(kRedWarps * 32) k_m2l_reduce(int32_t ncell, co
   } else if (l == 19) {
     loc[static_cast<int64_t>(c) * kLocStride + 19] = 0.0;
   }
+}
+
+// The same for unsoftened slots (kSlotTF = 18 doubles): a warp per cell takes two
+// slots per step, every lane of a half a value of its slot and the factor it
+// needs, one FMA each; the FP64 pipe bounds it (50M slots of N = 1M: 1.38 ms
+// against 2.18 with 24 values on 32 lanes).  The halves' sums are added, and the
+// trace relations give the components that the slots leave out.
+__global__ void __launch_bounds__(kRedWarps * 32) k_m2l_reduce_tf(int32_t ncell, const int32_t *__restrict__ off,
+                                                                  const double *__restrict__ slots,
+                                                                  double *__restrict__ loc) {
+  pdl_wait();
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31, q = l & 15;
+  const int c = blockIdx.x * kRedWarps + w;
+  if (c >= ncell) return;  // whole warp
+  const int s0 = off[c], s1 = off[c + 1];
+  const int f = q < 9 ? 16 : 17;  // place of the value's factor
+  constexpr int kFlight = 4;      // steps in flight
+  const double *p = slots + (static_cast<int64_t>(s0) + (l >> 4)) * kSlotTF;
+  double sum[kFlight] = {};  // eight sums per coefficient: short sums round less
+  for (int s = s0 + (l >> 4); s - (l >> 4) < s1; s += 2 * kFlight, p += 2 * kFlight * kSlotTF) {
+    double v[kFlight], g[kFlight];
+#pragma unroll
+    for (int u = 0; u < kFlight; ++u) {
+      const bool in = s + 2 * u < s1;
+      v[u] = in ? p[2 * u * kSlotTF + q] : 0.0;
+      g[u] = in && q >= 3 ? p[2 * u * kSlotTF + f] : 1.0;
+    }
+#pragma unroll
+    for (int u = 0; u < kFlight; ++u) sum[u] = fma(v[u], g[u], sum[u]);
+  }
+  static_assert(kFlight == 4, "the sums are added in pairs");
+  double acc = (sum[0] + sum[1]) + (sum[2] + sum[3]);
+  acc += __shfl_down_sync(0xffffffffu, acc, 16);
+  // C_ij = d_ij tr(S) - 3 S_ij, S the sums of n_i n_j; C_ijk = 3 x its sum
+  const double sxx = __shfl_sync(0xffffffffu, acc, 3), syy = __shfl_sync(0xffffffffu, acc, 6),
+               szz = __shfl_sync(0xffffffffu, acc, 8);
+  if (q >= 3) acc *= q < 9 ? -3.0 : 3.0;
+  if (q == 3 || q == 6 || q == 8) acc += sxx + syy + szz;
+  // lane of each coefficient, or the two whose negative sum it is
+  // (xx xy xz yy yz zz | xxx xxy xxz xyy xyz xzz yyy yyz yzz zzz)
+  const int a = l < 14 ? l : l == 14 ? 9 : l < 17 ? l - 1 : l == 17 ? 10 : 11;
+  const int b = l == 14 ? 12 : l == 17 ? 14 : 15;
+  const double va = __shfl_sync(0xffffffffu, acc, a), vb = __shfl_sync(0xffffffffu, acc, b);
+  const bool trace = l == 14 || l >= 17;
+  if (l < kLocStride) loc[static_cast<int64_t>(c) * kLocStride + l] = l == 19 ? 0.0 : trace ? -(va + vb) : va;
 }
 
 int launch_m2l64(fmm_ctx *c, int64_t K) {
@@ -865,7 +974,7 @@ int m2l_prepare(fmm_ctx *c) {
     launch(c, k_inverse, grid_for(E, 256), 256, 0, E, ptr<uint32_t>(c->eval[which]), ptr<int32_t>(c->m2l_pos));
     AMFMM_TRY(launched(c, "m2l_inverse"));
     const size_t esz = fp32 ? sizeof(float) : sizeof(double);
-    const int stride = c->opts.order_P == 3 ? kSlot64 : slot_stride_general(c->opts.order_P);
+    const int stride = c->opts.order_P != 3 ? slot_stride_general(c->opts.order_P) : c->eps2 == 0.0 ? kSlotTF : kSlot64;
     AMFMM_TRY(ensure_bytes(c, c->m2l_slots, static_cast<size_t>(E) * stride * esz));
   }
   if (fp32) {
@@ -913,7 +1022,8 @@ int m2l_reduce(fmm_ctx *c) {
   int32_t *off = ptr<int32_t>(c->m2l_off);
   // (warps drawing cells from a queue, as the gather does, measured 2.44 ms
   // against 2.39 ms for one warp per cell at N = 1M)
-  launch(c, k_m2l_reduce, grid_for(nc * 32, kRedWarps * 32), kRedWarps * 32, 0, static_cast<int32_t>(nc), off,
+  const auto kern = c->eps2 == 0.0 ? k_m2l_reduce_tf : k_m2l_reduce;
+  launch(c, kern, grid_for(nc * 32, kRedWarps * 32), kRedWarps * 32, 0, static_cast<int32_t>(nc), off,
          ptr<double>(c->m2l_slots), ptr<double>(c->loc));
   return launched(c, "m2l_reduce");
 }
