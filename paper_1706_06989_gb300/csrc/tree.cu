@@ -20,86 +20,113 @@ constexpr int kBlock = 256;
 // ---------------------------------------------------------------------------
 // a1: bounding cube and keys
 // ---------------------------------------------------------------------------
-__global__ void k_bbox_partial(const double *__restrict__ x, const double *__restrict__ y,
-                               const double *__restrict__ z, const double *__restrict__ m,
-                               int64_t n, double *__restrict__ part, int *__restrict__ status) {
-  pdl_wait();
-  double lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
+// Finite doubles as integers of the same order: minima and maxima then need no
+// FP64 instruction (64 cycles of their pipe per warp).
+__device__ __forceinline__ long long ordered(double v) {
+  const long long b = __double_as_longlong(v);
+  return b < 0 ? b ^ 0x7fffffffffffffffll : b;
+}
+__device__ __forceinline__ double from_ordered(long long k) {
+  return __longlong_as_double(k < 0 ? k ^ 0x7fffffffffffffffll : k);
+}
+__device__ __forceinline__ bool finite_bits(double v) { return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000; }
+
+// Extremes of coordinates, in thread 0 those of the whole block.  body_extremes
+// sets bit 0 of status for a coordinate that is not finite or a mass that is not
+// finite and positive.
+struct Extremes {
+  long long lo[3], hi[3];
+  __device__ __forceinline__ void combine(int d, long long l, long long h) {
+    lo[d] = min(lo[d], l);
+    hi[d] = max(hi[d], h);
+  }
+};
+__device__ __forceinline__ void block_extremes(Extremes &v) {
+  __shared__ long long sh[6][kBlock / 32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    for (int o = 16; o > 0; o >>= 1)
+      v.combine(d, __shfl_xor_sync(0xffffffffu, v.lo[d], o), __shfl_xor_sync(0xffffffffu, v.hi[d], o));
+    if (lane == 0) {
+      sh[d][w] = v.lo[d];
+      sh[3 + d][w] = v.hi[d];
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x == 0)
+    for (int d = 0; d < 3; ++d)
+      for (int q = 1; q < kBlock / 32; ++q) v.combine(d, sh[d][q], sh[3 + d][q]);
+}
+__device__ __forceinline__ Extremes no_extremes() {
+  Extremes v;
+  for (int d = 0; d < 3; ++d) {
+    v.lo[d] = 0x7fffffffffffffffll;
+    v.hi[d] = -0x7fffffffffffffffll - 1;
+  }
+  return v;
+}
+__device__ __forceinline__ Extremes body_extremes(const double *__restrict__ x, const double *__restrict__ y,
+                                                  const double *__restrict__ z, const double *__restrict__ m,
+                                                  int64_t first, int64_t end, int64_t stride, int *status) {
+  Extremes v = no_extremes();
   bool bad = false;
-  for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n;
-       i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    const double p[3] = {x[i], y[i], z[i]};
-    const double mi = m[i];
+  for (int64_t i = first; i < end; i += stride) {
+    const double p[3] = {x[i], y[i], z[i]}, mi = m[i];
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-      bad |= !isfinite(p[d]);
-      lo[d] = fmin(lo[d], p[d]);
-      hi[d] = fmax(hi[d], p[d]);
+      bad |= !finite_bits(p[d]);
+      v.combine(d, ordered(p[d]), ordered(p[d]));
     }
-    bad |= !(mi > 0.0) || !isfinite(mi);
+    bad |= __double_as_longlong(mi) <= 0 || !finite_bits(mi);
   }
   if (bad) atomicOr(status, 1);
-  __shared__ double sh[6][kBlock / 32];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-#pragma unroll
+  block_extremes(v);
+  return v;
+}
+// box[0..2] = lo, box[3] = scale = 2^21 / ext (0 when ext == 0)
+__device__ __forceinline__ void write_box(const Extremes &v, double *__restrict__ box) {
+  double ext = 0.0;
   for (int d = 0; d < 3; ++d) {
-    for (int o = 16; o > 0; o >>= 1) {
-      lo[d] = fmin(lo[d], __shfl_xor_sync(0xffffffffu, lo[d], o));
-      hi[d] = fmax(hi[d], __shfl_xor_sync(0xffffffffu, hi[d], o));
-    }
-    if (lane == 0) {
-      sh[d][w] = lo[d];
-      sh[3 + d][w] = hi[d];
-    }
+    const double lo = from_ordered(v.lo[d]), e = __dsub_rn(from_ordered(v.hi[d]), lo);
+    ext = d == 0 ? e : fmax(ext, e);
+    box[d] = lo;
   }
-  __syncthreads();
-  if (threadIdx.x < 6) {
-    const int k = threadIdx.x;
-    double v = sh[k][0];
-    for (int q = 1; q < kBlock / 32; ++q) v = k < 3 ? fmin(v, sh[k][q]) : fmax(v, sh[k][q]);
-    part[blockIdx.x * 6 + k] = v;
-  }
+  box[3] = ext > 0.0 ? __ddiv_rn(2097152.0, ext) : 0.0;
 }
 
-// bbox[0..2] = lo, bbox[3] = scale = 2^21 / ext (0 when ext == 0).  One block;
-// min and max are exact, so the order of combination does not matter.
-__global__ void k_bbox_final(const double *__restrict__ part, int nb, double *__restrict__ bbox) {
+// Bounding cube: every block its part, the last one to finish the whole (minima
+// and maxima are exact, so their order does not matter).  14 us at N = 1M; two
+// launches with FP64 comparisons took 45.6 + 10.1.
+__global__ void k_bbox(const double *__restrict__ x, const double *__restrict__ y, const double *__restrict__ z,
+                       const double *__restrict__ m, int64_t n, long long *__restrict__ part,
+                       int *__restrict__ status, unsigned *__restrict__ done, double *__restrict__ bbox) {
   pdl_wait();
-  __shared__ double sh[6][kBlock / 32];
-  double v[6] = {INFINITY, INFINITY, INFINITY, -INFINITY, -INFINITY, -INFINITY};
-  for (int b = threadIdx.x; b < nb; b += blockDim.x)
-    for (int k = 0; k < 6; ++k) v[k] = k < 3 ? fmin(v[k], part[b * 6 + k]) : fmax(v[k], part[b * 6 + k]);
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  for (int k = 0; k < 6; ++k) {
-    for (int o = 16; o > 0; o >>= 1) {
-      const double u = __shfl_xor_sync(0xffffffffu, v[k], o);
-      v[k] = k < 3 ? fmin(v[k], u) : fmax(v[k], u);
+  __shared__ bool last;
+  Extremes v = body_extremes(x, y, z, m, blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x, n,
+                             static_cast<int64_t>(gridDim.x) * blockDim.x, status);
+  if (threadIdx.x == 0) {
+    for (int d = 0; d < 3; ++d) {
+      part[6 * blockIdx.x + d] = v.lo[d];
+      part[6 * blockIdx.x + 3 + d] = v.hi[d];
     }
-    if (lane == 0) sh[k][w] = v[k];
+    __threadfence();
+    last = atomicAdd(done, 1u) == gridDim.x - 1;
   }
   __syncthreads();
-  if (threadIdx.x != 0) return;
-  double lo[3], hi[3];
-  for (int d = 0; d < 3; ++d) {
-    lo[d] = sh[d][0];
-    hi[d] = sh[3 + d][0];
-    for (int q = 1; q < kBlock / 32; ++q) {
-      lo[d] = fmin(lo[d], sh[d][q]);
-      hi[d] = fmax(hi[d], sh[3 + d][q]);
-    }
-  }
-  double ext = __dsub_rn(hi[0], lo[0]);
-  ext = fmax(ext, __dsub_rn(hi[1], lo[1]));
-  ext = fmax(ext, __dsub_rn(hi[2], lo[2]));
-  for (int d = 0; d < 3; ++d) bbox[d] = lo[d];
-  bbox[3] = ext > 0.0 ? __ddiv_rn(2097152.0, ext) : 0.0;
+  if (!last) return;
+  __threadfence();
+  v = no_extremes();
+  for (unsigned b = threadIdx.x; b < gridDim.x; b += blockDim.x)
+    for (int d = 0; d < 3; ++d)
+      v.combine(d, *const_cast<volatile long long *>(&part[6 * b + d]),
+                *const_cast<volatile long long *>(&part[6 * b + 3 + d]));
+  block_extremes(v);
+  if (threadIdx.x == 0) write_box(v, bbox);
 }
 
 __device__ __forceinline__ uint64_t quantise(double v, double lo, double scale) {
-  double t = __dmul_rn(__dsub_rn(v, lo), scale);
-  double f = floor(t);
-  f = fmin(f, 2097151.0);
-  return static_cast<uint64_t>(f);
+  return static_cast<uint64_t>(min(__double2int_rd(__dmul_rn(__dsub_rn(v, lo), scale)), 2097151));
 }
 
 // bit b of q -> bit 3b
@@ -141,46 +168,9 @@ __global__ void k_bbox_sys(const double *__restrict__ x, const double *__restric
   pdl_wait();
   const int s = blockIdx.x;
   const int64_t b = off[s], e = off[s + 1];
-  double lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
-  bool bad = false;
-  for (int64_t i = b + threadIdx.x; i < e; i += blockDim.x) {
-    const double p[3] = {x[i], y[i], z[i]};
-    const double mi = m[i];
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      bad |= !isfinite(p[d]);
-      lo[d] = fmin(lo[d], p[d]);
-      hi[d] = fmax(hi[d], p[d]);
-    }
-    bad |= !(mi > 0.0) || !isfinite(mi);
-    sysid[i] = s;
-  }
-  if (bad) atomicOr(status, 1);
-  __shared__ double sh[6][kBlock / 32];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    for (int o = 16; o > 0; o >>= 1) {
-      lo[d] = fmin(lo[d], __shfl_xor_sync(0xffffffffu, lo[d], o));
-      hi[d] = fmax(hi[d], __shfl_xor_sync(0xffffffffu, hi[d], o));
-    }
-    if (lane == 0) {
-      sh[d][w] = lo[d];
-      sh[3 + d][w] = hi[d];
-    }
-  }
-  __syncthreads();
-  if (threadIdx.x != 0) return;
-  for (int d = 0; d < 3; ++d)
-    for (int q = 1; q < kBlock / 32; ++q) {
-      sh[d][0] = fmin(sh[d][0], sh[d][q]);
-      sh[3 + d][0] = fmax(sh[3 + d][0], sh[3 + d][q]);
-    }
-  double ext = __dsub_rn(sh[3][0], sh[0][0]);
-  ext = fmax(ext, __dsub_rn(sh[4][0], sh[1][0]));
-  ext = fmax(ext, __dsub_rn(sh[5][0], sh[2][0]));
-  for (int d = 0; d < 3; ++d) sbox[4 * s + d] = sh[d][0];
-  sbox[4 * s + 3] = ext > 0.0 ? __ddiv_rn(2097152.0, ext) : 0.0;
+  const Extremes v = body_extremes(x, y, z, m, b + threadIdx.x, e, blockDim.x, status);
+  for (int64_t i = b + threadIdx.x; i < e; i += blockDim.x) sysid[i] = s;
+  if (threadIdx.x == 0) write_box(v, sbox + 4 * static_cast<int64_t>(s));
 }
 
 __global__ void k_keys_sys(const double *__restrict__ x, const double *__restrict__ y,
@@ -438,9 +428,10 @@ __global__ void k_finish_cells(int64_t n, int n_crit, int nsys, int64_t cap, con
 // Leaves: a warp takes G leaves and 32 of their bodies at a time.  The centre
 // of mass is summed in body order (as its definition here demands), one lane
 // per (leaf, component); then each lane forms its body's offset and the ten
-// products of up to second order, and one lane per (leaf, moment) sums in body
-// order with one FMA per body.  About 17 FP64 warp instructions per leaf at
-// G = 8 against 27 with a thread per leaf (leaves differ in size), and a chain
+// products of up to second order, and one lane per moment sums leaf by leaf in
+// body order with one FMA per body (lanes over all (leaf, moment) instead run as
+// long as the largest leaf of the tile: 178 against 164 us at N = 1M).  About 18 FP64 warp
+// instructions per leaf at G = 8 against 27 with a thread per leaf, and a chain
 // of about 75 instead of 1,100 for a leaf of 25 bodies.
 // A moment as (base product of up to second order) x coordinate: base 0..9 =
 // mu, mx, my, mz, mxx, mxy, mxz, myy, myz, mzz; coordinate 0..2, 3: one.
@@ -455,7 +446,6 @@ __global__ void __launch_bounds__(kUpWarps * 32) k_leaf_upward(
     const double *__restrict__ Zb, const double *__restrict__ Mb, double *__restrict__ S, double *__restrict__ M,
     double *__restrict__ Z, double *__restrict__ invM, double *__restrict__ mom) {
   pdl_wait();
-  constexpr int kRounds = (G * kMomStride + 31) / 32;
   __shared__ double sh[kUpWarps][14][33];  // per body: ten products, x, y, z, 1 (first: mu x, mu y, mu z, mu)
   __shared__ double com[kUpWarps][G][4];
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
@@ -515,9 +505,8 @@ __global__ void __launch_bounds__(kUpWarps * 32) k_leaf_upward(
     }
   }
   __syncwarp();
-  double acc[kRounds];
-#pragma unroll
-  for (int r = 0; r < kRounds; ++r) acc[r] = 0.0;
+  const int base = l < kMomStride ? c_mom_base[l] : 0, coord = l < kMomStride ? c_mom_coord[l] : 0;
+  double acc = 0.0;  // of the leaf that the tiles have reached
   for (int t0 = 0; t0 < total; t0 += 32) {
     int g;
     const int i = locate(t0, g);
@@ -540,21 +529,18 @@ __global__ void __launch_bounds__(kUpWarps * 32) k_leaf_upward(
       sh[w][13][l] = 1.0;
     }
     __syncwarp();
-#pragma unroll
-    for (int r = 0; r < kRounds; ++r) {
-      const int task = l + 32 * r, tg = task / kMomStride, q = task - tg * kMomStride;
-      const int te = __shfl_sync(0xffffffffu, end, tg < G ? tg : 0), tc = __shfl_sync(0xffffffffu, cnt, tg < G ? tg : 0);
-      if (tg < ng) {
-        const double *p = sh[w][c_mom_base[q]], *x = sh[w][10 + c_mom_coord[q]];
-        for (int k = max(te - tc - t0, 0); k < min(te - t0, 32); ++k) acc[r] = fma(p[k], x[k], acc[r]);
+    const double *q = sh[w][base], *xc = sh[w][10 + coord];
+    for (int tg = 0; tg < ng; ++tg) {
+      const int te = __shfl_sync(0xffffffffu, end, tg) - t0, tb = te - __shfl_sync(0xffffffffu, cnt, tg);
+      if (te <= 0 || tb >= 32) continue;
+      for (int k = max(tb, 0); k < min(te, 32); ++k) acc = fma(q[k], xc[k], acc);
+      if (te <= 32) {
+        if (l < kMomStride)
+          mom[static_cast<int64_t>(leaves[q0 + tg]) * kMomStride + l] = l == 0 ? com[w][tg][3] : acc;
+        acc = 0.0;
       }
     }
     __syncwarp();
-  }
-#pragma unroll
-  for (int r = 0; r < kRounds; ++r) {
-    const int task = l + 32 * r, tg = task / kMomStride, q = task - tg * kMomStride;
-    if (tg < ng) mom[static_cast<int64_t>(leaves[q0 + tg]) * kMomStride + q] = q == 0 ? com[w][tg][3] : acc[r];
   }
 }
 
@@ -756,7 +742,7 @@ int ensure_cells(fmm_ctx *c, int64_t need) {
   return FMM_OK;
 }
 
-// device words of the tree stage: [0] bad input, [8, 32) the levels' first
+// device words of the tree stage: [0] bad input, [1] blocks done, [8, 32) the levels' first
 // cell ids, the number of cells and of leaves
 constexpr int kStatusLvl = 8;
 constexpr int kStatusWords = kStatusLvl + kLevels + 2;
@@ -780,19 +766,17 @@ int build_tree(fmm_ctx *c) {
   AMFMM_TRY(ensure<int32_t>(c, c->cell_at, static_cast<size_t>(kMaxLevel + 1) * n));
   AMFMM_TRY(ensure<int>(c, c->status, kStatusWords));
   const int nbb = std::max(1, std::min<int>(c->num_sms * 4, static_cast<int>((n + kBlock - 1) / kBlock)));
-  AMFMM_TRY(ensure<double>(c, c->bbox_part, 6 * nbb));
+  AMFMM_TRY(ensure<long long>(c, c->bbox_part, 6 * nbb));
   AMFMM_TRY(ensure<double>(c, c->bbox, 8));
-  
 
   int *status = ptr<int>(c->status);
   AMFMM_CUDA(c, cudaMemsetAsync(status, 0, sizeof(int) * kStatusWords, st));
   const int nsys = c->sz.nsys;
   int which = 0;
   if (nsys == 1) {
-    launch(c, k_bbox_partial, nbb, kBlock, 0, c->x, c->y, c->z, c->m, n, ptr<double>(c->bbox_part), status);
-    AMFMM_TRY(launched(c, "bbox_partial"));
-    launch(c, k_bbox_final, 1, kBlock, 0, ptr<double>(c->bbox_part), nbb, ptr<double>(c->bbox));
-    AMFMM_TRY(launched(c, "bbox_final"));
+    launch(c, k_bbox, nbb, kBlock, 0, c->x, c->y, c->z, c->m, n, ptr<long long>(c->bbox_part), status,
+           reinterpret_cast<unsigned *>(status + 1), ptr<double>(c->bbox));
+    AMFMM_TRY(launched(c, "bbox"));
     launch(c, k_keys, grid_for(n, kBlock), kBlock, 0, c->x, c->y, c->z, n, ptr<double>(c->bbox),
            ptr<uint64_t>(c->key[0]), ptr<uint32_t>(c->idx[0]));
     AMFMM_TRY(launched(c, "keys"));
