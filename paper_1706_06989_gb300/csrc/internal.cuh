@@ -55,6 +55,7 @@ struct Sizes {
   double lo[3] = {0, 0, 0}, scale = 0;
   int64_t p2p_body_pairs = 0;
   int64_t p2p_items = 0;         // near-field work items (chunks of the leaves' column streams)
+  int64_t p2p_heavy_leaves = 0;  // of the mixed form, see p2p.cu
   std::vector<int64_t> lvl_off;  // cells of level l are [lvl_off[l], lvl_off[l+1])
 };
 
@@ -160,7 +161,7 @@ struct fmm_ctx {
   amfmm::DBuf ekey[2], eval[2], m2l_pos, m2l_off, m2l_slots, cell32, qoh;
   // P2P grouping
   amfmm::DBuf pkey[2], pval[2], p2p_A, p2p_offA, p2p_offB, p2p_pos, p2p_poff, p2p_len,
-      p2p_slots, p2p_colOff, p2p_cols, p2p_nb, p2p_pre, p2p_rec, p2p_items, p2p_itemOff, p2p_extraOff,
+      p2p_slots, p2p_colOff, p2p_cols, p2p_nb, p2p_pre, p2p_rec, p2p_rowpart, p2p_items, p2p_itemOff, p2p_extraOff,
       p2p_extra, p2p_heavy;
   // scan / sort scratch; `totals` holds small device results (1 KiB):
   // [0,16) scan totals, [64,72) near-field body-pair count, [80,88) selector-scored pairs, [88,92) selector candidates, [96,104) slot total,

@@ -96,10 +96,141 @@ __device__ __forceinline__ float3 offset32(const BodyF &b, const float4 zh, cons
                      (b.h.z - zh.z) + (b.l.z - zl.z));
 }
 
-template <int ROWS>
+// Work items: the column stream of a leaf is cut into chunks of at most
+// `chunk` columns (the first chunk also holds all of the leaf's own bodies,
+// so that the one-sided self sums stay in one warp).  One warp per chunk
+// keeps a leaf that the walk paired with millions of bodies (a large sparse
+// leaf next to a dense region) from serialising the kernel.  Leaf order: there
+// neighbouring warps share partner columns in cache.
+//
+// A leaf with a good part of what an average warp gets in all would still be what
+// the kernel ends on, and a chunk cannot be made smaller: every lane's FP32 sum
+// over a chunk's columns is one rounding sequence.  But the A side's rows are
+// independent of one another, and so are the B side's columns: such a heavy
+// leaf's chunks become items of kItemRows rows (A side only) and items of
+// kItemCols columns (B side only), which evaluate its pairs twice, in the same
+// order within every sum.  Near field without and with this rule, and with the
+// line at the average itself and at half of it: N = 65,536 (outlying leaves with
+// up to 65,000 columns) 337, 141, 165, 143 us; a forest of 48 systems 552, 516,
+// 601, 548; 200,000 bodies of two clusters 440, 303, 389, 316; a disc of 262,144
+// 508, 424, 533, 455.  At N = 1M the line is at 4,270 columns and no leaf beyond.
+constexpr int kChunk = 4096;
+constexpr int kItemRows = 4;
+constexpr int kItemCols = 512;
+constexpr int kHeavyMin = 512;
+// items {leaf, first column, end column, -1 or place in `extra`}; an item of a
+// heavy leaf has the complement of the end column, and its first row, or -1 for
+// the B side, in item_rows.  A heavy leaf's places: its self sums, then the
+// A-side sums of every chunk.
+
+__device__ __forceinline__ int chunks_of(int ncol, int nself) {
+  const int first = max(kChunk, nself);
+  return ncol <= first ? 1 : 1 + (ncol - first + kChunk - 1) / kChunk;
+}
+__device__ __forceinline__ int2 chunk_range(int j, int cb, int ce, int nself) {
+  const int first = max(kChunk, nself);
+  if (j == 0) return make_int2(cb, min(ce, cb + first));
+  const int c0 = cb + first + (j - 1) * kChunk;
+  return make_int2(c0, min(ce, c0 + kChunk));
+}
+// more columns than a third of the average of the warps that run at once
+__device__ __forceinline__ bool is_heavy(int ncol, int total, int warps) {
+  return ncol > max(kHeavyMin, total / (3 * warps));
+}
+
+__global__ void k_item_counts(int32_t nleaf, const int32_t *__restrict__ leaves, const int32_t *__restrict__ count,
+                              const int32_t *__restrict__ colOff, const int32_t *__restrict__ total, int warps,
+                              int32_t *__restrict__ nitems, int32_t *__restrict__ nextra, int *__restrict__ nheavy) {
+  pdl_wait();
+  const int q = blockIdx.x * blockDim.x + threadIdx.x;
+  if (q >= nleaf) return;
+  const int L = leaves[q], cb = colOff[L], ce = colOff[L + 1], nA = count[L];
+  const int k = chunks_of(ce - cb, nA);
+  if (!is_heavy(ce - cb, *total, warps)) {
+    nitems[q] = k;
+    nextra[q] = (k - 1) * 3 * nA;
+    return;
+  }
+  int items = 0;
+  for (int j = 0; j < k; ++j) {
+    const int2 c = chunk_range(j, cb, ce, nA);
+    items += (nA + kItemRows - 1) / kItemRows + (c.y - c.x + kItemCols - 1) / kItemCols;
+  }
+  atomicAdd(nheavy, 1);
+  nitems[q] = items;
+  nextra[q] = (k + 1) * 3 * nA;
+}
+
+__global__ void k_item_fill(int32_t nleaf, const int32_t *__restrict__ leaves, const int32_t *__restrict__ count,
+                            const int32_t *__restrict__ colOff, const int32_t *__restrict__ total, int warps,
+                            const int32_t *__restrict__ itemOff, const int32_t *__restrict__ extraOff,
+                            int4 *__restrict__ items, int32_t *__restrict__ item_rows) {
+  pdl_wait();
+  const int q = blockIdx.x * blockDim.x + threadIdx.x;
+  if (q >= nleaf) return;
+  const int L = leaves[q];
+  const int cb = colOff[L], ce = colOff[L + 1], nA = count[L];
+  const int k = chunks_of(ce - cb, nA);
+  const bool heavy = is_heavy(ce - cb, *total, warps);
+  int o = itemOff[q];
+  for (int j = 0; j < k; ++j) {
+    const int2 c = chunk_range(j, cb, ce, nA);
+    if (!heavy) {
+      items[o++] = make_int4(L, c.x, c.y, j == 0 ? -1 : extraOff[q] + (j - 1) * 3 * nA);
+      continue;
+    }
+    for (int r = 0; r < nA; r += kItemRows) {
+      item_rows[o] = r;
+      items[o++] = make_int4(L, c.x, ~c.y, extraOff[q] + (j + 1) * 3 * nA);
+    }
+    for (int b = c.x; b < c.y; b += kItemCols) {
+      item_rows[o] = -1;
+      items[o++] = make_int4(L, b, ~min(c.y, b + kItemCols), extraOff[q]);
+    }
+  }
+}
+
+// A leaf whose column stream was split adds the A-side partials of its later
+// chunks, in chunk order, once every chunk is done (one thread per body); a
+// heavy leaf its self sums and those of all chunks.
+__global__ void k_p2p_chunks(int32_t nleaf, int64_t n, const int32_t *__restrict__ leaves,
+                             const int32_t *__restrict__ begin, const int32_t *__restrict__ count,
+                             const int32_t *__restrict__ colOff, const int32_t *__restrict__ total, int warps,
+                             const int32_t *__restrict__ extraOff, const double *__restrict__ extra,
+                             double *__restrict__ near) {
+  pdl_wait();
+  const int q = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const int l = threadIdx.x & 31;
+  if (q >= nleaf) return;
+  const int e0 = extraOff[q], e1 = extraOff[q + 1];
+  if (e0 == e1) return;
+  const int L = leaves[q];
+  const int bA = begin[L], nA = count[L];
+  const bool heavy = is_heavy(colOff[L + 1] - colOff[L], *total, warps);
+  for (int r = l; r < nA; r += 32) {
+    double a0 = 0.0, a1 = 0.0, a2 = 0.0;
+    if (!heavy) {
+      a0 = near[bA + r];
+      a1 = near[n + bA + r];
+      a2 = near[2 * n + bA + r];
+    }
+    for (int k = e0; k < e1; k += 3 * nA) {
+      const double *e = extra + k + 3 * r;
+      a0 += e[0];
+      a1 += e[1];
+      a2 += e[2];
+    }
+    near[bA + r] = a0;
+    near[n + bA + r] = a1;
+    near[2 * n + bA + r] = a2;
+  }
+}
+
+// HEAVY: there are items of heavy leaves (the test for them costs 1% otherwise).
+template <int ROWS, bool HEAVY>
 __global__ void __launch_bounds__(kWarps * 32) k_p2p(
-    int32_t nitem, int64_t n, const int4 *__restrict__ items, const int32_t *__restrict__ begin,
-    const int32_t *__restrict__ count, const double *__restrict__ Zc, const int2 *__restrict__ cols,
+    int32_t nitem, int64_t n, const int4 *__restrict__ items, const int32_t *__restrict__ item_rows,
+    const int32_t *__restrict__ begin, const int32_t *__restrict__ count, const double *__restrict__ Zc, const int2 *__restrict__ cols,
     double *__restrict__ near, double *__restrict__ extra, float *__restrict__ slots,
     const BodyF *__restrict__ bodyf, float eps2, int *__restrict__ queue) {
   pdl_wait();
@@ -123,11 +254,17 @@ __global__ void __launch_bounds__(kWarps * 32) k_p2p(
   const int L = it.x;
   const bool first = it.w < 0;
   const int bA = begin[L], nA = count[L];
+  // an item of a heavy leaf (see k_item_fill): rows [ra, rb) on the A side, or the
+  // columns' B side
+  const bool heavy = HEAVY && it.z < 0;
+  const int part = heavy ? item_rows[q] : 0;
+  const bool sideA = !heavy || part >= 0, sideB = !heavy || part < 0;
+  const int ra = heavy && sideA ? part : 0, rb = heavy && sideA ? min(nA, part + kItemRows) : nA;
   const double zx = Zc[3 * L], zy = Zc[3 * L + 1], zz = Zc[3 * L + 2];
   const float4 zh = make_float4(static_cast<float>(zx), static_cast<float>(zy), static_cast<float>(zz), 0.f);
   const float4 zl =
       make_float4(static_cast<float>(zx - zh.x), static_cast<float>(zy - zh.y), static_cast<float>(zz - zh.z), 0.f);
-  const int cb = it.y, ce = it.z;
+  const int cb = it.y, ce = heavy ? ~it.z : it.z;
   if (first) {
     for (int t = l; t < nA; t += 32) {
       near[bA + t] = 0.0;
@@ -137,8 +274,8 @@ __global__ void __launch_bounds__(kWarps * 32) k_p2p(
   }
   __syncwarp();
   constexpr int kRows = ROWS;
-  for (int r0 = 0; r0 < nA; r0 += kRows) {
-    const int nr = min(kRows, nA - r0);
+  for (int r0 = ra; r0 < rb; r0 += kRows) {
+    const int nr = min(kRows, rb - r0);
     if (l < nr) {
       const int i = bA + r0 + l;
       const BodyF b = bodyf[i];
@@ -172,7 +309,7 @@ __global__ void __launch_bounds__(kWarps * 32) k_p2p(
         zj = o.z;
         mj = rb.h.w;
       }
-      const bool mutual = col.y >= 0;
+      const bool mutual = col.y >= 0 && sideA;
       float bx = 0.f, by = 0.f, bz = 0.f;
       // eight rows per step, then four and two: independent dependency chains
       // for the pipelines and less loop control per pair
@@ -198,8 +335,8 @@ __global__ void __launch_bounds__(kWarps * 32) k_p2p(
           }
         }
       }
-      if (valid) {
-        if (mutual) {
+      if (valid && sideB) {
+        if (col.y >= 0) {
           float *o = slots + 3 * static_cast<int64_t>(col.y);
           if (r0 == 0) {
             o[0] = bx;
@@ -210,6 +347,12 @@ __global__ void __launch_bounds__(kWarps * 32) k_p2p(
             o[1] += by;
             o[2] += bz;
           }
+        } else if (heavy) {
+          double *o = extra + it.w + 3 * (col.x - bA);
+          const bool set = r0 == 0;
+          o[0] = (set ? 0.0 : o[0]) + static_cast<double>(bx);
+          o[1] = (set ? 0.0 : o[1]) + static_cast<double>(by);
+          o[2] = (set ? 0.0 : o[2]) + static_cast<double>(bz);
         } else {
           near[col.x] += static_cast<double>(bx);
           near[n + col.x] += static_cast<double>(by);
@@ -220,7 +363,7 @@ __global__ void __launch_bounds__(kWarps * 32) k_p2p(
     __syncwarp();
     // A-side: every row's partials summed over the lanes in a fixed order,
     // pairwise in FP32, then one FP64 addition
-    for (int v = l; v < 3 * nr; v += 32) {
+    for (int v = l; sideA && v < 3 * nr; v += 32) {
       float g[4];
 #pragma unroll
       for (int h = 0; h < 4; ++h) {
@@ -235,77 +378,6 @@ __global__ void __launch_bounds__(kWarps * 32) k_p2p(
     }
     __syncwarp();
   }
-  }
-}
-
-// A leaf whose column stream was split adds the A-side partials of its later
-// chunks, in chunk order, once every chunk is done (one thread per body).
-__global__ void k_p2p_chunks(int32_t nleaf, int64_t n, const int32_t *__restrict__ leaves,
-                             const int32_t *__restrict__ begin, const int32_t *__restrict__ count,
-                             const int32_t *__restrict__ itemOff, const int4 *__restrict__ items,
-                             const double *__restrict__ extra, double *__restrict__ near) {
-  pdl_wait();
-  const int q = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int l = threadIdx.x & 31;
-  if (q >= nleaf) return;
-  const int i0 = itemOff[q], i1 = itemOff[q + 1];
-  if (i1 - i0 < 2) return;
-  const int L = leaves[q];
-  const int bA = begin[L], nA = count[L];
-  for (int r = l; r < nA; r += 32) {
-    double a0 = near[bA + r], a1 = near[n + bA + r], a2 = near[2 * n + bA + r];
-    for (int k = i0 + 1; k < i1; ++k) {
-      const double *e = extra + items[k].w + 3 * r;
-      a0 += e[0];
-      a1 += e[1];
-      a2 += e[2];
-    }
-    near[bA + r] = a0;
-    near[n + bA + r] = a1;
-    near[2 * n + bA + r] = a2;
-  }
-}
-
-// Work items: the column stream of a leaf is cut into chunks of at most
-// `chunk` columns (the first chunk also holds all of the leaf's own bodies,
-// so that the one-sided self sums stay in one warp).  One warp per chunk
-// keeps a leaf that the walk paired with millions of bodies (a large sparse
-// leaf next to a dense region) from serialising the kernel.  Leaf order: there
-// neighbouring warps share partner columns in cache.
-constexpr int kChunk = 4096;
-
-__device__ __forceinline__ int chunks_of(int ncol, int nself) {
-  const int first = max(kChunk, nself);
-  return ncol <= first ? 1 : 1 + (ncol - first + kChunk - 1) / kChunk;
-}
-
-__global__ void k_item_counts(int32_t nleaf, const int32_t *__restrict__ leaves, const int32_t *__restrict__ count,
-                              const int32_t *__restrict__ colOff, int32_t *__restrict__ nitems,
-                              int32_t *__restrict__ nextra) {
-  pdl_wait();
-  const int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= nleaf) return;
-  const int L = leaves[q];
-  const int k = chunks_of(colOff[L + 1] - colOff[L], count[L]);
-  nitems[q] = k;
-  nextra[q] = (k - 1) * 3 * count[L];
-}
-
-__global__ void k_item_fill(int32_t nleaf, const int32_t *__restrict__ leaves, const int32_t *__restrict__ count,
-                            const int32_t *__restrict__ colOff, const int32_t *__restrict__ itemOff,
-                            const int32_t *__restrict__ extraOff, int4 *__restrict__ items) {
-  pdl_wait();
-  const int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= nleaf) return;
-  const int L = leaves[q];
-  const int cb = colOff[L], ce = colOff[L + 1], nA = count[L];
-  const int k = chunks_of(ce - cb, nA);
-  const int first = max(kChunk, nA);
-  int o = itemOff[q];
-  items[o] = make_int4(L, cb, min(ce, cb + first), -1);
-  for (int j = 1; j < k; ++j) {
-    const int c0 = cb + first + (j - 1) * kChunk;
-    items[o + j] = make_int4(L, c0, min(ce, c0 + kChunk), extraOff[q] + (j - 1) * 3 * nA);
   }
 }
 
@@ -460,30 +532,34 @@ __global__ void k_cols_pairs(int64_t K, const int2 *__restrict__ pairs, const in
   }
 }
 
-template <int ROWS>
+// the warps that the rule of heavy leaves counts with (16 run per SM at the
+// default tile; the rule must be the same in every stage of a solve)
+int heavy_warps(const fmm_ctx *c) { return 16 * std::max(1, c->num_sms); }
+
+template <int ROWS, bool HEAVY>
 int launch_p2p_rows(fmm_ctx *c) {
   const int64_t n = c->sz.n;
   const int32_t nleaf = static_cast<int32_t>(c->sz.nleaf);
   const size_t shm = kWarps * sizeof(P2PSmem<ROWS>);
   // per function and device, so set on every launch (a host-side call)
-  AMFMM_CUDA(c, cudaFuncSetAttribute(k_p2p<ROWS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  AMFMM_CUDA(c, cudaFuncSetAttribute(k_p2p<ROWS, HEAVY>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      static_cast<int>(shm)));
   const int32_t nitem = static_cast<int32_t>(c->sz.p2p_items);
   int per_sm = 0;
-  AMFMM_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_p2p<ROWS>, kWarps * 32, shm));
+  AMFMM_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_p2p<ROWS, HEAVY>, kWarps * 32, shm));
   const int64_t resident = static_cast<int64_t>(std::max(1, per_sm)) * std::max(1, c->num_sms);
   const unsigned grid = static_cast<unsigned>(std::min<int64_t>(grid_for(nitem, kWarps), resident));
   int *queue = ptr<int32_t>(c->totals) + 40;
   AMFMM_CUDA(c, cudaMemsetAsync(queue, 0, sizeof(int), c->stream));
-  launch(c, k_p2p<ROWS>, grid, kWarps * 32, shm, nitem, n, ptr<int4>(c->p2p_items), ptr<int32_t>(c->begin),
-         ptr<int32_t>(c->count), ptr<double>(c->Z), ptr<int2>(c->p2p_cols), ptr<double>(c->near),
+  launch(c, k_p2p<ROWS, HEAVY>, grid, kWarps * 32, shm, nitem, n, ptr<int4>(c->p2p_items), ptr<int32_t>(c->p2p_rowpart),
+         ptr<int32_t>(c->begin), ptr<int32_t>(c->count), ptr<double>(c->Z), ptr<int2>(c->p2p_cols), ptr<double>(c->near),
          ptr<double>(c->p2p_extra), static_cast<float *>(c->p2p_slots.p), ptr<BodyF>(c->bodyf),
          static_cast<float>(c->eps2), queue);
   AMFMM_TRY(launched(c, "p2p"));
   if (nitem > nleaf) {
     launch(c, k_p2p_chunks, grid_for(static_cast<int64_t>(nleaf) * 32, 256), 256, 0, nleaf, n, ptr<int32_t>(c->leaves),
-           ptr<int32_t>(c->begin), ptr<int32_t>(c->count), ptr<int32_t>(c->p2p_itemOff), ptr<int4>(c->p2p_items),
-           ptr<double>(c->p2p_extra), ptr<double>(c->near));
+           ptr<int32_t>(c->begin), ptr<int32_t>(c->count), ptr<int32_t>(c->p2p_colOff), ptr<int32_t>(c->totals) + 32,
+           heavy_warps(c), ptr<int32_t>(c->p2p_extraOff), ptr<double>(c->p2p_extra), ptr<double>(c->near));
     AMFMM_TRY(launched(c, "p2p_chunks"));
   }
   return FMM_OK;
@@ -548,13 +624,15 @@ int p2p_prepare(fmm_ctx *c) {
   AMFMM_TRY(ensure<int32_t>(c, c->p2p_itemOff, nleaf + 1));
   AMFMM_TRY(ensure<int32_t>(c, c->p2p_extraOff, nleaf + 1));
   int32_t *itemOff = ptr<int32_t>(c->p2p_itemOff), *extraOff = ptr<int32_t>(c->p2p_extraOff);
-  // totals: [32] columns, [33] work items, [34] extra partials (int32 slots)
+  // totals: [32] columns, [33] work items, [34] extra partials, [35] heavy leaves (int32 slots)
   int32_t *itot = ptr<int32_t>(c->totals) + 33, *etot = ptr<int32_t>(c->totals) + 34;
+  int32_t *nheavy = ptr<int32_t>(c->totals) + 35;
+  AMFMM_CUDA(c, cudaMemsetAsync(nheavy, 0, sizeof(int32_t), st));
   int32_t *icnt = cnt, *ecnt = ptr<int32_t>(c->flag);  // free scratch of >= nleaf + 1
   AMFMM_CUDA(c, cudaMemsetAsync(icnt + nleaf, 0, sizeof(int32_t), st));
   AMFMM_CUDA(c, cudaMemsetAsync(ecnt + nleaf, 0, sizeof(int32_t), st));
   launch(c, k_item_counts, grid_for(nleaf, 256), 256, 0, nleaf, ptr<int32_t>(c->leaves), ptr<int32_t>(c->count),
-         colOff, icnt, ecnt);
+         colOff, ctot, heavy_warps(c), icnt, ecnt, nheavy);
   AMFMM_TRY(launched(c, "p2p_item_counts"));
   AMFMM_TRY(exclusive_scan_i32(c, icnt, itemOff, nleaf + 1, itot));
   AMFMM_TRY(exclusive_scan_i32(c, ecnt, extraOff, nleaf + 1, etot));
@@ -565,12 +643,12 @@ int p2p_prepare(fmm_ctx *c) {
     HostRead rb[2];
     int nr = 0;
     if (K > 0) rb[nr++] = HostRead{h, ptot, sizeof(int64_t)};
-    rb[nr++] = HostRead{hc, ctot, 3 * sizeof(int32_t)};
+    rb[nr++] = HostRead{hc, ctot, 4 * sizeof(int32_t)};
     AMFMM_TRY(read_back(c, rb, nr));
     if (capturing(c)) {
       Expect e;
       if (K > 0) e.add64(ptot, static_cast<uint64_t>(h[0]));
-      for (int k = 0; k < 3; ++k) e.add(ctot + k, static_cast<uint32_t>(hc[k]));
+      for (int k = 0; k < 4; ++k) e.add(ctot + k, static_cast<uint32_t>(hc[k]));
       AMFMM_TRY(graph_expect(c, e));
       st = c->stream;
     }
@@ -583,10 +661,12 @@ int p2p_prepare(fmm_ctx *c) {
   if (nslot / 3 + n + 1 > 0x7fffffffLL)
     return set_error(c, FMM_EUNSUPPORTED, "too many near-field slots (%lld values)", (long long)nslot);
   c->sz.p2p_items = nitem;
+  c->sz.p2p_heavy_leaves = hc[3];
   AMFMM_TRY(ensure<int4>(c, c->p2p_items, nitem + 1));
   AMFMM_TRY(ensure<double>(c, c->p2p_extra, nextra + 1));
+  AMFMM_TRY(ensure<int32_t>(c, c->p2p_rowpart, nitem + 1));
   launch(c, k_item_fill, grid_for(nleaf, 256), 256, 0, nleaf, ptr<int32_t>(c->leaves), ptr<int32_t>(c->count), colOff,
-         itemOff, extraOff, ptr<int4>(c->p2p_items));
+         ctot, heavy_warps(c), itemOff, extraOff, ptr<int4>(c->p2p_items), ptr<int32_t>(c->p2p_rowpart));
   AMFMM_TRY(launched(c, "p2p_item_fill"));
   AMFMM_TRY(ensure_bytes(c, c->p2p_slots, static_cast<size_t>(nslot + 3) * sizeof(float)));
   AMFMM_TRY(ensure<int2>(c, c->p2p_cols, ncol + 1));
@@ -603,10 +683,11 @@ int p2p_prepare(fmm_ctx *c) {
 }
 
 int p2p_run(fmm_ctx *c) {
+  const bool heavy = c->sz.p2p_heavy_leaves > 0;
   switch (c->p2p_rows) {
-    case 8: return launch_p2p_rows<8>(c);
-    case 32: return launch_p2p_rows<32>(c);
-    default: return launch_p2p_rows<16>(c);
+    case 8: return heavy ? launch_p2p_rows<8, true>(c) : launch_p2p_rows<8, false>(c);
+    case 32: return heavy ? launch_p2p_rows<32, true>(c) : launch_p2p_rows<32, false>(c);
+    default: return heavy ? launch_p2p_rows<16, true>(c) : launch_p2p_rows<16, false>(c);
   }
 }
 
