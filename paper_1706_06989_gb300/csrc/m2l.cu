@@ -909,9 +909,7 @@ int launch_m2l32_gather(fmm_ctx *c) {
   const uint32_t *partner = ptr<uint32_t>(c->eval[c->m2l_which]);
   const float *c32 = ptr<float>(c->cell32);
   double *loc = ptr<double>(c->loc);
-  cudaStream_t st = c->stream;
   int *queue = ptr<int32_t>(c->totals) + 41;
-  AMFMM_CUDA(c, cudaMemsetAsync(queue, 0, sizeof(int), st));
   const bool tf = cell32_tf(c);
   auto kern = c->opts.variant == FMM_UC   ? (tf ? k_m2l32_gather<FMM_UC, true> : k_m2l32_gather<FMM_UC, false>)
               : c->opts.variant == FMM_TC ? (tf ? k_m2l32_gather<FMM_TC, true> : k_m2l32_gather<FMM_TC, false>)

@@ -144,6 +144,7 @@ __global__ void k_item_counts(int32_t nleaf, const int32_t *__restrict__ leaves,
   pdl_wait();
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= nleaf) return;
+  if (q == 0) nitems[nleaf] = nextra[nleaf] = 0;
   const int L = leaves[q], cb = colOff[L], ce = colOff[L + 1], nA = count[L];
   const int k = chunks_of(ce - cb, nA);
   if (!is_heavy(ce - cb, *total, warps)) {
@@ -419,7 +420,8 @@ __global__ void k_p2p_reduce(int64_t n, const int32_t *__restrict__ leaf_of, con
   near[2 * n + i] = a2;
 }
 
-// the sorted (A, B) as pairs, and every pair's column count n_B
+// the sorted (A, B) as pairs, and every pair's column count n_B (and a zero for
+// the total of the scan)
 __global__ void k_sorted_pairs(int64_t K, const uint32_t *__restrict__ key, const uint32_t *__restrict__ val,
                                const int32_t *__restrict__ count, int2 *__restrict__ out, int32_t *__restrict__ nb) {
   pdl_wait();
@@ -428,6 +430,7 @@ __global__ void k_sorted_pairs(int64_t K, const uint32_t *__restrict__ key, cons
   const int2 p = make_int2(static_cast<int>(key[s]), static_cast<int>(val[s]));
   out[s] = p;
   nb[s] = count[p.y];
+  if (s == 0) nb[K] = 0;
 }
 
 // pos[s] = CSR position of sorted pair s on its B side; len[e] = 3 n_B
@@ -550,7 +553,6 @@ int launch_p2p_rows(fmm_ctx *c) {
   const int64_t resident = static_cast<int64_t>(std::max(1, per_sm)) * std::max(1, c->num_sms);
   const unsigned grid = static_cast<unsigned>(std::min<int64_t>(grid_for(nitem, kWarps), resident));
   int *queue = ptr<int32_t>(c->totals) + 40;
-  AMFMM_CUDA(c, cudaMemsetAsync(queue, 0, sizeof(int), c->stream));
   launch(c, k_p2p<ROWS, HEAVY>, grid, kWarps * 32, shm, nitem, n, ptr<int4>(c->p2p_items), ptr<int32_t>(c->p2p_rowpart),
          ptr<int32_t>(c->begin), ptr<int32_t>(c->count), ptr<double>(c->Z), ptr<int2>(c->p2p_cols), ptr<double>(c->near),
          ptr<double>(c->p2p_extra), static_cast<float *>(c->p2p_slots.p), ptr<BodyF>(c->bodyf),
@@ -584,7 +586,6 @@ int p2p_prepare(fmm_ctx *c) {
   int32_t *colOff = ptr<int32_t>(c->p2p_colOff);
   unsigned long long *stat = ptr<unsigned long long>(c->totals) + 8;
   int32_t *ctot = ptr<int32_t>(c->totals) + 32;
-  AMFMM_CUDA(c, cudaMemsetAsync(stat, 0, sizeof(unsigned long long), st));
   AMFMM_TRY(ensure<int32_t>(c, c->p2p_nb, K + 1));
   AMFMM_TRY(ensure<int32_t>(c, c->p2p_pre, K + 1));
   int32_t *nb = ptr<int32_t>(c->p2p_nb), *pre = ptr<int32_t>(c->p2p_pre);
@@ -612,7 +613,6 @@ int p2p_prepare(fmm_ctx *c) {
   // column stream per leaf: pre = prefix sums of n_B over the A-sorted pairs
   // (K + 1 entries, so pre[K] is the total)
   if (K > 0) {
-    AMFMM_CUDA(c, cudaMemsetAsync(nb + K, 0, sizeof(int32_t), st));
     AMFMM_TRY(exclusive_scan_i32(c, nb, pre, K + 1, nullptr));
   }
   AMFMM_CUDA(c, cudaMemsetAsync(cnt, 0, sizeof(int32_t) * (nc + 1), st));
@@ -627,10 +627,7 @@ int p2p_prepare(fmm_ctx *c) {
   // totals: [32] columns, [33] work items, [34] extra partials, [35] heavy leaves (int32 slots)
   int32_t *itot = ptr<int32_t>(c->totals) + 33, *etot = ptr<int32_t>(c->totals) + 34;
   int32_t *nheavy = ptr<int32_t>(c->totals) + 35;
-  AMFMM_CUDA(c, cudaMemsetAsync(nheavy, 0, sizeof(int32_t), st));
   int32_t *icnt = cnt, *ecnt = ptr<int32_t>(c->flag);  // free scratch of >= nleaf + 1
-  AMFMM_CUDA(c, cudaMemsetAsync(icnt + nleaf, 0, sizeof(int32_t), st));
-  AMFMM_CUDA(c, cudaMemsetAsync(ecnt + nleaf, 0, sizeof(int32_t), st));
   launch(c, k_item_counts, grid_for(nleaf, 256), 256, 0, nleaf, ptr<int32_t>(c->leaves), ptr<int32_t>(c->count),
          colOff, ctot, heavy_warps(c), icnt, ecnt, nheavy);
   AMFMM_TRY(launched(c, "p2p_item_counts"));

@@ -462,8 +462,6 @@ int p2p64_prepare(fmm_ctx *c) {
   unsigned long long *ext64 = ptr<unsigned long long>(c->totals) + 12;
   int32_t *icnt = ptr<int32_t>(c->incl), *ecnt = ptr<int32_t>(c->flag);  // free scratch of >= nleaf + 1
   int32_t *itemOff = ptr<int32_t>(c->p2p_itemOff), *extraOff = ptr<int32_t>(c->p2p_extraOff);
-  AMFMM_CUDA(c, cudaMemsetAsync(stat, 0, sizeof(unsigned long long), st));
-  AMFMM_CUDA(c, cudaMemsetAsync(ext64, 0, sizeof(unsigned long long), st));
   launch(c, k_items64_count, grid_for(32 * (static_cast<int64_t>(nleaf) + 1), 256), 256, 0, nleaf,
          ptr<int32_t>(c->leaves), ptr<int32_t>(c->count), off, K > 0 ? ptr<uint32_t>(c->pval[c->p2p_which]) : nullptr,
          icnt, ecnt, stat, ext64);
@@ -500,7 +498,6 @@ int p2p64_run(fmm_ctx *c) {
   const int64_t resident = static_cast<int64_t>(std::max(1, per_sm)) * std::max(1, c->num_sms);
   const unsigned grid = static_cast<unsigned>(std::min<int64_t>(grid_for(nitem, kWarps), resident));
   int *queue = ptr<int32_t>(c->totals) + 40;
-  AMFMM_CUDA(c, cudaMemsetAsync(queue, 0, sizeof(int), c->stream));
   launch(c, kern, grid, kWarps * 32, 0, nitem, c->sz.n, ptr<int4>(c->p2p_items), ptr<int32_t>(c->begin),
          ptr<int32_t>(c->count), ptr<int32_t>(c->p2p_offA),
          c->sz.n_p2p > 0 ? ptr<uint32_t>(c->pval[c->p2p_which]) : nullptr, ptr<int2>(c->p2p_heavy),

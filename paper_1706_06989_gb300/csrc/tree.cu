@@ -640,11 +640,13 @@ __global__ void __launch_bounds__(kUpWarps * 32) k_internal_upward(
   }
 }
 
-// Centres as hi + lo floats for the filter of R_max.
-__global__ void k_split_centres(int32_t ncell, const double *__restrict__ Z, float4 *__restrict__ zf) {
+// Centres as hi + lo floats for the filter of R_max, whose maxima start at zero.
+__global__ void k_split_centres(int32_t ncell, const double *__restrict__ Z, float4 *__restrict__ zf,
+                                unsigned long long *__restrict__ rmax2) {
   pdl_wait();
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= ncell) return;
+  rmax2[c] = 0;
   const double x = Z[3 * c], y = Z[3 * c + 1], z = Z[3 * c + 2];
   const float hx = static_cast<float>(x), hy = static_cast<float>(y), hz = static_cast<float>(z);
   zf[2 * c] = make_float4(hx, hy, hz, 0.f);
@@ -896,7 +898,6 @@ int build_tree(fmm_ctx *c) {
 
 int upward(fmm_ctx *c) {
   const int64_t n = c->sz.n, nc = c->sz.ncell;
-  cudaStream_t st = c->stream;
   AMFMM_TRY(ensure<double>(c, c->S, 3 * nc));
   AMFMM_TRY(ensure<double>(c, c->M, nc));
   AMFMM_TRY(ensure<double>(c, c->Z, 3 * nc));
@@ -929,10 +930,9 @@ int upward(fmm_ctx *c) {
     AMFMM_TRY(launched(c, "internal_upward"));
   }
   }
-  AMFMM_CUDA(c, cudaMemsetAsync(c->rmax2.p, 0, sizeof(unsigned long long) * nc, st));
   AMFMM_TRY(ensure<float4>(c, c->cellzf, 2 * nc));
   launch(c, k_split_centres, grid_for(nc, kBlock), kBlock, 0, static_cast<int32_t>(nc), ptr<double>(c->Z),
-         ptr<float4>(c->cellzf));
+         ptr<float4>(c->cellzf), ptr<unsigned long long>(c->rmax2));
   AMFMM_TRY(launched(c, "split_centres"));
   launch(c, k_rmax_bodies, grid_for(n, kBlock), kBlock, 0, n, c->sz.depth + 1, ptr<int32_t>(c->cell_at),
          ptr<BodyF>(c->bodyf), ptr<float4>(c->cellzf), ptr<double>(c->X), ptr<double>(c->Y), ptr<double>(c->Zb),

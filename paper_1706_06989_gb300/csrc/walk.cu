@@ -361,11 +361,21 @@ __global__ void __launch_bounds__(kGenBlock, kGenBlocksPerSM) k_walk_gen(
   }
 }
 
-// one self pair per root, and the first generation's inputs
-__global__ void k_roots_front(int32_t nsys, int4 *__restrict__ front, GenState *__restrict__ gs) {
+// One self pair per root; the generation records, zero but for the first
+// generation's inputs; and zero counters for the stages that follow (words of
+// `totals`: body pairs, scored pairs, FP64 near-field partials, heavy leaves,
+// the work queues).
+__global__ void k_roots_front(int32_t nsys, int4 *__restrict__ front, GenState *__restrict__ gs, int nrec,
+                              int32_t *__restrict__ totals) {
   pdl_wait();
   const int s = blockIdx.x * blockDim.x + threadIdx.x;
   if (s < nsys) front[s] = split_record(s, 1, s, false);
+  if (blockIdx.x > 0) return;
+  int *words = reinterpret_cast<int *>(gs);
+  for (int q = threadIdx.x; q < nrec * static_cast<int>(sizeof(GenState) / sizeof(int)); q += blockDim.x) words[q] = 0;
+  const int q = threadIdx.x;
+  if (q == 16 || q == 17 || q == 20 || q == 21 || q == 24 || q == 25 || q == 35 || q == 40 || q == 41) totals[q] = 0;
+  __syncthreads();
   if (s == 0) gs[0].in = GenIn{nsys, 0, 0, 0};
 }
 
@@ -419,7 +429,6 @@ int walk(fmm_ctx *c) {
       return set_error(c, FMM_EUNSUPPORTED, "the learned selector works on one system at a time");
     AMFMM_TRY(cell_features(c));
     if (c->sel_rule == FMM_SEL_RELATIVE) AMFMM_TRY(field_estimate(c));
-    AMFMM_CUDA(c, cudaMemsetAsync(ptr<int64_t>(c->totals) + 10, 0, sizeof(int64_t), st));
   }
   // one self pair per root: systems of a forest never interact
   const int64_t nsys = c->sz.nsys;
@@ -433,9 +442,8 @@ int walk(fmm_ctx *c) {
   if (sizeof(GenState) * (ngen + 1) > 8192) return set_error(c, FMM_EUNSUPPORTED, "tree too deep for the walk state");
   GenState *gs = static_cast<GenState *>(c->walk_state.p);
   const unsigned grid = static_cast<unsigned>(std::max(1, c->num_sms * kGenBlocksPerSM));
-  // generation records: zero, then the first generation's inputs (the roots)
-  AMFMM_CUDA(c, cudaMemsetAsync(gs, 0, sizeof(GenState) * (ngen + 1), st));
-  launch(c, k_roots_front, grid_for(nsys, kBlock), kBlock, 0, static_cast<int32_t>(nsys), ptr<int4>(c->front[0]), gs);
+  launch(c, k_roots_front, grid_for(nsys, kBlock), kBlock, 0, static_cast<int32_t>(nsys), ptr<int4>(c->front[0]), gs,
+         ngen + 1, ptr<int32_t>(c->totals));
   AMFMM_TRY(launched(c, "walk_roots"));
   int gstart = 0;  // first generation to (re)run
   for (int attempt = 0;; ++attempt) {
