@@ -552,18 +552,16 @@ __global__ void __launch_bounds__(kUpWarps * 32) k_leaf_upward(
 // The child dipoles D' (zero about a centre of mass up to rounding, Sec. 2)
 // are left out of the shift; the parent's dipole is the shift of the child
 // monopoles, D_i = Sum M' s_i.
-// A warp takes CELLS parents, eight lanes each, one per child: a lane shifts its
+// A warp takes four parents, eight lanes each, one per child: a lane shifts its
 // child's moments, and one lane per (parent, moment) adds the shifted ones in
-// octant order.  About 120 FP64 warp instructions whatever the number of
-// parents in the warp; a thread per parent had a chain of 600 (52 us per level
-// of 4,000 to 16,000 cells), a warp per parent one of 170 (14 to 21 us).
-template <int CELLS>
+// octant order.  About 120 FP64 warp instructions for four parents; a thread per
+// parent had a chain of 600 (52 us per level of 4,000 to 16,000 cells).
 __global__ void __launch_bounds__(kUpWarps * 32) k_internal_upward(
     int32_t c0, int32_t c1, const int32_t *__restrict__ first_child, const int32_t *__restrict__ nchild,
     double *__restrict__ S, double *__restrict__ M, double *__restrict__ Z, double *__restrict__ invM,
     double *__restrict__ mom) {
   pdl_wait();
-  constexpr int kRounds = (CELLS * kMomStride + 31) / 32;
+  constexpr int CELLS = 4, kRounds = (CELLS * kMomStride + 31) / 32;
   __shared__ double sh[kUpWarps][kMomStride][33];
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
   const int64_t first = c0 + static_cast<int64_t>(blockIdx.x * kUpWarps + w) * CELLS;
@@ -637,6 +635,72 @@ __global__ void __launch_bounds__(kUpWarps * 32) k_internal_upward(
         for (int j = 0; j < n; ++j) a += sh[w][t][8 * tg + j];
       mom[(first + tg) * kMomStride + t] = t == 0 ? total : a;
     }
+  }
+}
+
+// The same with a block per parent, for levels that leave the GPU idle: a thread
+// per (child, moment), and every warp, on its own partition, takes the centre of
+// mass for itself, so that the chain is one division and about 25 more FP64
+// instructions instead of 120: upward pass 66 -> 47 us at N = 2,000, 114 -> 89 at
+// 65,536, 233 -> 197 for a disc of 262,144 with 15 levels.
+__constant__ signed char c_oct[10][3] = {{0, 0, 0}, {0, 0, 1}, {0, 0, 2}, {0, 1, 1}, {0, 1, 2},
+                                         {0, 2, 2}, {1, 1, 1}, {1, 1, 2}, {1, 2, 2}, {2, 2, 2}};
+__constant__ signed char c_quad[3][3] = {{4, 5, 6}, {5, 7, 8}, {6, 8, 9}};
+
+__global__ void __launch_bounds__(128) k_internal_upward_block(
+    int32_t c0, const int32_t *__restrict__ first_child, const int32_t *__restrict__ nchild, double *__restrict__ S,
+    double *__restrict__ M, double *__restrict__ Z, double *__restrict__ invM, double *__restrict__ mom) {
+  pdl_wait();
+  __shared__ double q[8 * kMomStride], sh[kMomStride][9], sv[8][3];
+  const int t = threadIdx.x, l = t & 31;
+  const int c = c0 + blockIdx.x;
+  const int nch = nchild[c];
+  if (nch == 0) return;  // whole block
+  const int f = first_child[c];
+  for (int e = t; e < nch * kMomStride; e += 128) q[e] = mom[static_cast<int64_t>(f) * kMomStride + e];
+  // lane 4 k + d: component d of child k (d = 3: the mass)
+  const int ck = l >> 2, d = l & 3;
+  const bool child = ck < nch;
+  const double v = child ? (d < 3 ? S[3 * (f + ck) + d] : M[f + ck]) : 0.0;
+  const double zk = child && d < 3 ? Z[3 * (f + ck) + d] : 0.0;
+  double s = 0.0;
+  for (int k = 0; k < nch; ++k) s = __dadd_rn(s, __shfl_sync(0xffffffffu, v, 4 * k + d));
+  const double mm = __shfl_sync(0xffffffffu, s, 3);
+  const double z = __ddiv_rn(d == 3 ? 1.0 : s, mm);
+  if (t < 32 && child && d < 3) sv[ck][d] = zk - z;
+  if (t < 3) {
+    S[3 * c + t] = s;
+    Z[3 * c + t] = z;
+  } else if (t == 3) {
+    M[c] = mm;
+    invM[c] = z;
+  }
+  __syncthreads();
+  if (t < 80) {
+    const int k = t / 10, r = t - 10 * k;
+    if (k < nch) {
+      const double *m = q + kMomStride * k;
+      const int a = c_oct[r][0], b = c_oct[r][1], e = c_oct[r][2];
+      const double sa = sv[k][a], sb = sv[k][b], se = sv[k][e];
+      sh[10 + r][k] = m[10 + r] + (m[c_quad[a][b]] * se + m[c_quad[a][e]] * sb + m[c_quad[b][e]] * sa) +
+                      m[0] * sa * sb * se;
+    }
+  } else {
+    const int k = (t - 80) / 6, r = t - 80 - 6 * k;
+    if (k < nch) {
+      const double *m = q + kMomStride * k;
+      const int a = r < 3 ? 0 : r < 5 ? 1 : 2, b = r < 3 ? r : r < 5 ? r - 2 : 2;
+      const double ms = m[0] * sv[k][a];
+      sh[4 + r][k] = m[4 + r] + ms * sv[k][b];
+      if (r < 3) sh[1 + r][k] = m[0] * sv[k][r];
+    }
+  }
+  __syncthreads();
+  if (t < kMomStride) {
+    double a = 0.0;
+    if (t > 0)
+      for (int k = 0; k < nch; ++k) a += sh[t][k];
+    mom[static_cast<int64_t>(c) * kMomStride + t] = t == 0 ? mm : a;
   }
 }
 
@@ -922,11 +986,16 @@ int upward(fmm_ctx *c) {
   AMFMM_TRY(launched(c, "leaf_upward"));
   for (int lev = c->sz.depth - 1; lev >= 0; --lev) {
     const int64_t c0 = c->sz.lvl_off[lev], c1 = c->sz.lvl_off[lev + 1];
-    const bool many = c1 - c0 >= 4 * fill;  // four parents per warp once one each would fill the GPU
-    const auto up = many ? k_internal_upward<4> : k_internal_upward<1>;
-    launch(c, up, grid_for(c1 - c0, many ? 4 * kUpWarps : kUpWarps), kUpWarps * 32, 0, static_cast<int32_t>(c0),
-           static_cast<int32_t>(c1), ptr<int32_t>(c->first_child), ptr<int32_t>(c->nchild), ptr<double>(c->S),
-           ptr<double>(c->M), ptr<double>(c->Z), ptr<double>(c->invM), ptr<double>(c->mom));
+    // four parents per warp once that gives every partition of the GPU two warps
+    // (lines at twice to eight times as many parents measured the same within 1%)
+    if (c1 - c0 >= fill)
+      launch(c, k_internal_upward, grid_for(c1 - c0, 4 * kUpWarps), kUpWarps * 32, 0, static_cast<int32_t>(c0),
+             static_cast<int32_t>(c1), ptr<int32_t>(c->first_child), ptr<int32_t>(c->nchild), ptr<double>(c->S),
+             ptr<double>(c->M), ptr<double>(c->Z), ptr<double>(c->invM), ptr<double>(c->mom));
+    else
+      launch(c, k_internal_upward_block, static_cast<unsigned>(c1 - c0), 128, 0, static_cast<int32_t>(c0),
+             ptr<int32_t>(c->first_child), ptr<int32_t>(c->nchild), ptr<double>(c->S), ptr<double>(c->M),
+             ptr<double>(c->Z), ptr<double>(c->invM), ptr<double>(c->mom));
     AMFMM_TRY(launched(c, "internal_upward"));
   }
   }
