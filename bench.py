@@ -44,20 +44,18 @@ FP32_PEAK = SM_COUNT * SM_MAX_MHZ * 1e6 * 256
 # kernels' expressions: an accepted M2L pair of each variant (unsoftened:
 # trace-free quadrupoles, and for TC trace-free octupoles), a body pair
 M2L_FLOPS = {"UC": 162, "TC": 235, "TCO": 238}
-# of those, the FP64 form's pair kernel leaves the 32 products of the unit
-# tensors U2 and U3 by their scale factors to the per-cell reduction
-M2L_FLOPS_IN_REDUCE_FP64 = 32
+# the FP64 form's pair kernel: unscaled, trace-reduced tensors (the per-cell sums
+# scale them and restore the traces)
+M2L_FLOPS_FP64 = {"UC": 104, "TC": 170, "TCO": 177}
 # the selector experiment's measure of interaction work: a fixed weight per
 # accepted pair (the TC pair's flops written with the trace terms) and per
 # body pair, so that its gains compare interaction sets, not kernel versions
 WORK_PER_M2L_PAIR = 295
 # DRAM traffic of the dominant kernel per unit it processes, from one ncu
-# capture (dram__bytes_read.sum + dram__bytes_write.sum) of k_p2p<double, 16>
-# on a Plummer sphere of N = 262,144 (theta = 0.5, TC): 137,841,920 B read and
-# 215,840,000 B written for 115,126,406 body pairs.  Scaled by the body pairs
-# of the launch timed (the traffic grows with them: column stream, B-side
-# partial slots and near-field sums are all per pair or per body).
-TRAFFIC_PER_UNIT = {("p2p", "fp64"): (137841920 + 215840000) / 115126406}
+# capture (dram__bytes_read.sum + dram__bytes_write.sum) of k_p2p64 on a Plummer
+# sphere of N = 262,144 (theta = 0.5): 23,775,744 B read and 2,304 B written
+# for 115,126,406 body pairs, scaled by the body pairs of the launch timed.
+TRAFFIC_PER_UNIT = {("p2p", "fp64"): (23775744 + 2304) / 115126406}
 P2P_FLOPS_PER_BODY_PAIR = 25
 ORACLE_SAMPLE_N = 131072      # single-core oracle sample (bodies)
 REFERENCE_N = 262144          # bodies per step of the reference arm (all cores)
@@ -320,7 +318,7 @@ def run_ours(a):
     # roofline of the dominant interaction kernel (alu bound, FP64 or FP32)
     m2l_ms = statistics.mean(kern["m2l"])
     p2p_ms = statistics.mean(kern["p2p"])
-    m2l_flops = (M2L_FLOPS[a.variant] - (M2L_FLOPS_IN_REDUCE_FP64 if a.precision == "fp64" else 0)) * st.n_m2l
+    m2l_flops = (M2L_FLOPS_FP64 if a.precision == "fp64" else M2L_FLOPS)[a.variant] * st.n_m2l
     p2p_flops = P2P_FLOPS_PER_BODY_PAIR * st.p2p_body_pairs
     peak = FP64_PEAK if a.precision == "fp64" else FP32_PEAK
     if a.order_p != 3:
@@ -334,6 +332,9 @@ def run_ours(a):
     traffic = tpu * (st.p2p_body_pairs if dom == "p2p" else st.n_m2l) if tpu else None
     roofline = {"bound": "alu", "kernel": dom, "achieved": achieved, "peak": peak / 1e12, "unit": "TFLOP/s",
                 "frac": achieved / (peak / 1e12), "traffic": traffic,
+                "note": ("the FP64 near field is evaluated in fixed point on the integer pipes (two-sided pairs once "
+                         "from each side), so its algorithmic rate may exceed the FP64 pipe's peak"
+                         if (dom, a.precision) == ("p2p", "fp64") else None),
                 "traffic_unit": "bytes per launch (ncu capture scaled by units)" if traffic else None,
                 "peak_source": ("derived: 152 SMs x 2070 MHz x %s flop/clk/SM (FMA = 2)"
                                 % ("4 FP64" if a.precision == "fp64" else "256 FP32")),
@@ -451,6 +452,7 @@ def run_ours(a):
         dev2 = (torch.linalg.norm(got2 - got, dim=1) / torch.linalg.norm(got, dim=1)).cpu().numpy()
         fb2, tb2 = s2.balance(x, y, z, m, *out2)
         m2l2, p2p2 = statistics.mean(k2["m2l"]), statistics.mean(k2["p2p"])
+        m2l_flops = (M2L_FLOPS_FP64 if oprec == "fp64" else M2L_FLOPS)[a.variant] * st.n_m2l
         pk2 = FP64_PEAK if oprec == "fp64" else FP32_PEAK
         other = {"precision": oprec, "value": ws * a.n * len(t2) / (sum(t2) / 1e3) if ws == 1 else None,
                  "ms_per_step": statistics.mean(t2), "rms_force_err": float(np.sqrt(np.mean(rel2 ** 2))),
