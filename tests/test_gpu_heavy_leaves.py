@@ -45,3 +45,16 @@ def test_outlying_leaves():
     ref = oracle.Oracle(p[:, 0].copy(), p[:, 1].copy(), p[:, 2].copy(), m, 0.4, 25).accel("TC")
     dev = np.linalg.norm(a - ref, axis=1) / np.linalg.norm(ref, axis=1)
     assert np.sqrt(np.mean(dev**2)) <= 1e-6
+
+
+def test_partials_at_the_ends_of_the_float_range():
+    """Partners' partials of any size are widened exactly: masses from 1e-30 to
+    1e30 in one system, every pair summed directly."""
+    from paper_1706_06989_gb300 import fmm
+    p = ics.uniform_cube(600, seed=4).pos()
+    m = 10.0 ** np.random.default_rng(4).uniform(-30, 30, 600)
+    d = [torch.from_numpy(np.ascontiguousarray(v)).cuda() for v in (p[:, 0], p[:, 1], p[:, 2], m)]
+    a = torch.stack(fmm.FMM(theta=1e-4, n_crit=4, precision="mixed").solve(*d), 1).cpu().numpy()
+    ref = oracle.direct(p[:, 0].copy(), p[:, 1].copy(), p[:, 2].copy(), m)
+    dev = np.linalg.norm(a - ref, axis=1) / np.linalg.norm(ref, axis=1)
+    assert np.sqrt(np.mean(dev**2)) <= 1e-6
