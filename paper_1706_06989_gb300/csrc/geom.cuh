@@ -1,9 +1,10 @@
-// geom.cuh -- centre of mass of a cell, shared by every expansion order.
+// geom.cuh -- the opening criterion and the records of the walk's frontier, shared
+// by the walk and the learned selector.
 //
-// Sec. 2: the opening criterion compares centres of mass, so Z must come out
-// identical wherever it is computed.  A leaf sums its bodies in sorted order,
-// any other cell sums its children in octant order, Z = S / M, every step an
-// explicitly rounded FP64 operation (no FMA contraction).
+// Sec. 2: the criterion compares centres of mass, so Z must come out identical
+// wherever it is computed.  A leaf sums its bodies in sorted order, any other
+// cell its children in octant order, Z = S / M, every step an explicitly rounded
+// FP64 operation (no FMA contraction).
 #pragma once
 
 namespace amfmm {

@@ -273,7 +273,6 @@ inline unsigned grid_for(int64_t n, int block) {
 // Exclusive prefix sums; `total` (device, 1 element) receives the sum.
 int exclusive_scan_i32(fmm_ctx *c, const int32_t *in, int32_t *out, int64_t n, int32_t *total);
 int exclusive_scan_i64(fmm_ctx *c, const int64_t *in, int64_t *out, int64_t n, int64_t *total);
-int exclusive_scan_i4(fmm_ctx *c, const int4 *in, int4 *out, int64_t n, int4 *total);
 // Stable LSD radix sort of (key, value) pairs on the low `bits` key bits.
 // Sorted data ends in buffer index *which (0 or 1) of the ping-pong pairs.
 int radix_sort_u64(fmm_ctx *c, DBuf key[2], DBuf val[2], int64_t n, int bits, int *which);

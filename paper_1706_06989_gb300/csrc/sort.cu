@@ -16,23 +16,14 @@ constexpr int kRedundantTiles = 4096;  // up to 8M elements: two launches per sc
 // ---- element operations for the scans ----
 __device__ __forceinline__ int32_t vadd(int32_t a, int32_t b) { return a + b; }
 __device__ __forceinline__ int64_t vadd(int64_t a, int64_t b) { return a + b; }
-__device__ __forceinline__ int4 vadd(int4 a, int4 b) {
-  return make_int4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
-}
 template <class T> __device__ __forceinline__ T vzero();
 template <> __device__ __forceinline__ int32_t vzero<int32_t>() { return 0; }
 template <> __device__ __forceinline__ int64_t vzero<int64_t>() { return 0; }
-template <> __device__ __forceinline__ int4 vzero<int4>() { return make_int4(0, 0, 0, 0); }
 
 __device__ __forceinline__ int32_t shfl_up(int32_t v, int d) { return __shfl_up_sync(0xffffffffu, v, d); }
 __device__ __forceinline__ int64_t shfl_up(int64_t v, int d) {
   return static_cast<int64_t>(__shfl_up_sync(0xffffffffu, static_cast<long long>(v), d));
 }
-__device__ __forceinline__ int4 shfl_up(int4 v, int d) {
-  return make_int4(__shfl_up_sync(0xffffffffu, v.x, d), __shfl_up_sync(0xffffffffu, v.y, d),
-                   __shfl_up_sync(0xffffffffu, v.z, d), __shfl_up_sync(0xffffffffu, v.w, d));
-}
-
 // Inclusive scan across the warp.
 template <class T>
 __device__ __forceinline__ T warp_inclusive(T v) {
@@ -695,9 +686,6 @@ int exclusive_scan_i32(fmm_ctx *c, const int32_t *in, int32_t *out, int64_t n, i
 }
 int exclusive_scan_i64(fmm_ctx *c, const int64_t *in, int64_t *out, int64_t n, int64_t *total) {
   return scan_entry<int64_t>(c, in, out, n, total);
-}
-int exclusive_scan_i4(fmm_ctx *c, const int4 *in, int4 *out, int64_t n, int4 *total) {
-  return scan_entry<int4>(c, in, out, n, total);
 }
 int radix_sort_u64(fmm_ctx *c, DBuf key[2], DBuf val[2], int64_t n, int bits, int *which) {
   return sort_arrays<uint64_t>(c, key, val, n, bits, kSpins, which);

@@ -10,7 +10,6 @@
 // order, other cells sum their children in octant order, Z = S / M, and R_max
 // is the exact maximum over the cell's bodies.
 #include "internal.cuh"
-#include "geom.cuh"
 
 namespace amfmm {
 namespace {
