@@ -846,7 +846,10 @@ int walk_scores(fmm_ctx *c, const long long *nf_dev, int64_t cap, const int4 *fr
          ptr<double4_32a>(c->walk_zr), ptr<CellF>(c->walk_zf), ptr<int32_t>(c->count), c->sel_min_work, lo, hi, score,
          ptr<int32_t>(c->sel_cand), ncand);
   AMFMM_TRY(launched(c, "band_select"));
-  const unsigned g = static_cast<unsigned>(c->num_sms * 4);
+  // as many blocks as run at once (229 registers: two per SM): each stages the
+  // network once.  Walk stage of a disc of 262,144: 1.55 ms; one per SM 1.61, four
+  // 1.65, eight 1.74.
+  const unsigned g = static_cast<unsigned>(c->num_sms * 2);
   launch(c, k_walk_scores, g, 128, 0, front, ptr<int32_t>(c->sel_cand), ncand, ptr<float>(c->sel_params),
          ptr<CellF>(c->walk_zf), ptr<float4>(c->sel_cellfeat),
          c->sel_rule == FMM_SEL_RELATIVE ? ptr<float>(c->sel_lga) : nullptr, score,
