@@ -368,12 +368,15 @@ AMFMM_HD void acc_add(Acc &a, const int32_t q[3], const int32_t dH[3], const int
   }
 }
 
-// A unit for sums over windows of exponents gd - kWinSpan to gd + kWinSpan, em
-// the heaviest source's mass exponent: at the window's bound that source gets
-// k = 24 (30 in the widest window) and keeps 61 bits (55), and it fits down to
-// 2^-8 of the window (closer ones, and sources lighter by 2^22: the caller's
-// FP64 path; raising the unit in mid-sum would cost every pair).
-constexpr int kWinSpan = 3;
+// A unit for sums over sources in a window of exponent gd, em the heaviest one's
+// mass exponent: at the window's bound that source gets k = 24 and fits down to
+// 2^-8 of the window (closer ones: the caller's FP64 path).  A unit is kept while
+// it stays within 2^kUnitSpan of the one that the sources at hand ask for (a window
+// wider or narrower by 2^kWinSpan, or other masses): k is 18 to 30 then, and a
+// source lighter by 2^kClassSpan still gets k < kShiftEnd.  A term rounds to
+// 2^(k - 79) of itself at the window's bound (less when it is closer), so all of
+// them to 2^-49 of the heaviest one's term at worst.
+constexpr int kWinSpan = 3, kUnitSpan = 2 * kWinSpan, kClassSpan = 21;
 AMFMM_HD int unit_guess(int gd, int em) { return 24 + em + 9 - (kFieldUp + 238 + 2 * gd); }
 
 // Constant part of k for a batch of window exponent gd: k = base - em - 3 s2

@@ -162,7 +162,7 @@ struct fmm_ctx {
   // P2P grouping
   amfmm::DBuf pkey[2], pval[2], p2p_A, p2p_offA, p2p_offB, p2p_pos, p2p_poff, p2p_len,
       p2p_slots, p2p_colOff, p2p_cols, p2p_nb, p2p_pre, p2p_rec, p2p_rowpart, p2p_items, p2p_itemOff, p2p_extraOff,
-      p2p_extra, p2p_heavy;
+      p2p_extra;
   // scan / sort scratch; `totals` holds small device results (1 KiB):
   // [0,16) scan totals, [64,72) near-field body-pair count, [80,88) selector-scored pairs, [88,92) selector candidates, [96,104) slot total,
   // [128,144) near-field column, work-item, extra-partial and heavy-leaf totals, [160,168) work queues (near field, gathered far field);

@@ -26,6 +26,12 @@
 // source bodies: each lane converts one to the batch's window and leaves its
 // digits in shared memory.
 //
+// The sums' unit follows the heaviest source of what is being summed, a body at
+// the row's own place apart: a unit set by a body that adds no term there would
+// round the others' terms away.  A batch is therefore taken in classes of mass: the sources
+// within 2^kClassSpan of its heaviest, then those of the rest, and so on (one
+// class unless the masses differ by more).
+//
 // Every sum has a fixed order and every result is independent of which warp
 // takes an item.
 #include <limits.h>
@@ -119,7 +125,7 @@ template <bool SOFT>
 __global__ void __launch_bounds__(kWarps * 32, 4) k_p2p64(
     int32_t nitem, int64_t n, const int4 *__restrict__ items, const int32_t *__restrict__ begin,
     const int32_t *__restrict__ count, const int32_t *__restrict__ off, const uint32_t *__restrict__ partner,
-    const int2 *__restrict__ heavy, const Rec *__restrict__ rec, const double *__restrict__ X,
+    const Rec *__restrict__ rec, const double *__restrict__ X,
     const double *__restrict__ Y, const double *__restrict__ Zb, const double *__restrict__ Mb, double eps2, double *__restrict__ near,
     double *__restrict__ extra, int *__restrict__ queue) {
   pdl_wait();
@@ -140,10 +146,11 @@ __global__ void __launch_bounds__(kWarps * 32, 4) k_p2p64(
     const int sub = l / nr, row = l - sub * nr;
     const bool active = sub < nsub;
     const int i = bA + (active ? row : 0);
-    int g0, em;  // unit of the positions; exponent of the heaviest source but the row's own body
+    int g0;  // unit of the positions
     uint32_t rmag;
     {
       fix::W96 o[3];
+      int em;
       offset(rec[i], rec[bA], o, &g0, &em);
       rmag = max(max(fix::top_mag(o[0]), fix::top_mag(o[1])), fix::top_mag(o[2]));
     }
@@ -162,7 +169,7 @@ __global__ void __launch_bounds__(kWarps * 32, 4) k_p2p64(
     int steps = 0, terms = 0;  // since the last carry: steps of the warp, terms of the lane
     // this group's entries, one per lane (entry 0 of group 0: the leaf itself)
     const int e = it.z * kGroup + l - 1, e0 = off[L], e1 = off[L + 1];
-    int pb = 0, pc = 0, pm = INT_MIN;
+    int pb = 0, pc = 0;
     if (e < 0) {
       pb = begin[L];
       pc = nA;
@@ -170,12 +177,6 @@ __global__ void __launch_bounds__(kWarps * 32, 4) k_p2p64(
       const int P = static_cast<int>(partner[e0 + e]);
       pb = begin[P];
       pc = count[P];
-      pm = heavy[P].x;
-    }
-    {
-      const int2 own = heavy[L];
-      const int mine = it.z == 0 ? (em == own.x ? own.y : own.x) : INT_MIN;
-      em = max(max(mine, __reduce_max_sync(kAll, pm)), -4096);  // (a body alone has no source)
     }
     int incl = pc;
 #pragma unroll
@@ -185,7 +186,8 @@ __global__ void __launch_bounds__(kWarps * 32, 4) k_p2p64(
     }
     const int total = __shfl_sync(kAll, incl, 31);
     const int bodyBase = pb - (incl - pc);  // body of column j of this entry: bodyBase + j
-    int shPrev = -1, shUnit = -1000;  // windows of the digits and of the sums' unit
+    int shPrev = -1;       // window of the digits
+    int unit = INT_MIN / 2;  // the sums' unit, less what acc_carry raises it by
     int32_t H[3], Lo[3];
     bool rounded = false;
     for (int j0 = 0; j0 < total; j0 += 32) {
@@ -213,12 +215,6 @@ __global__ void __launch_bounds__(kWarps * 32, 4) k_p2p64(
 #pragma unroll
         for (int c = 0; c < 3; ++c) rounded |= fix::digits(o[c], sh, &H[c], &Lo[c]);
         shPrev = sh;
-        if (abs(sh - shUnit) > fix::kWinSpan) {  // (also the first batch)
-          flush(acc, terms, sm, l);
-          steps = 0;
-          acc.Ua = fix::unit_guess(gd, em);
-          shUnit = sh;
-        }
       }
       int64_t eh = 0;
       uint32_t el = 0;
@@ -228,6 +224,8 @@ __global__ void __launch_bounds__(kWarps * 32, 4) k_p2p64(
         eh = static_cast<int64_t>(es);
         el = static_cast<uint32_t>(scalbn(es - static_cast<double>(eh), 2 * fix::kDig - 32));
       }
+      const int ncol = min(32, total - j0);
+      int4 dh, dl;
       int32_t close;
       {
         int32_t h[3], lo[3];
@@ -236,79 +234,110 @@ __global__ void __launch_bounds__(kWarps * 32, 4) k_p2p64(
         for (int c = 0; c < 3; ++c) r |= fix::digits(s[c], sh, &h[c], &lo[c]);
         close = __any_sync(kAll, r) ? fix::kCloseRounded : fix::kCloseExact;
         if (SOFT && all64) close = 0x7fffffff;
-        __syncwarp();  // every lane is done with the batch before
-        sm.h[l] = make_int4(h[0], h[1], h[2], lo[0]);
-        sm.l[l] = make_int4(lo[1], lo[2], static_cast<int>(rj.c.y), static_cast<int>(rj.c.z));
-        sm.x[l] = make_int2(emj, jb);
+        dh = make_int4(h[0], h[1], h[2], lo[0]);
+        dl = make_int4(lo[1], lo[2], static_cast<int>(rj.c.y), static_cast<int>(rj.c.z));
+      }
+      unsigned rest = 0xffffffffu >> (32 - ncol);
+#pragma unroll 1
+      do {  // classes of mass
+        const bool there = (rest >> l) & 1u;
+        int top = __shfl_sync(kAll, emj, __ffs(static_cast<int>(rest)) - 1);
+        if (__any_sync(kAll, there && emj != top)) top = __reduce_max_sync(kAll, there ? emj : INT_MIN);
+        const bool in = there && emj >= top - fix::kClassSpan;
+        const unsigned cls = __ballot_sync(kAll, in), tops = __ballot_sync(kAll, in && emj == top);
+        const int nc = __popc(cls);
+        rest &= ~cls;
+        __syncwarp();  // every lane is done with the class before
+        if (in) {
+          const int at = __popc(cls & ((1u << l) - 1));
+          sm.h[at] = dh;
+          sm.l[at] = dl;
+          sm.x[at] = make_int2(emj, jb);
+        }
         __syncwarp();
-      }
-      const int ncol = min(32, total - j0);
-      const int kb = fix::k_base(acc.Ua, gd);
-      // The loop has no branch: close pairs, and those whose factor leaves the
-      // sums' range, add nothing here and are marked for the loop below.
-      unsigned mark = 0, bit = 1;
-      for (int c = active ? sub : 32; c < ncol; c += nsub) {
-        const int4 hh = sm.h[c], ll = sm.l[c];
-        const int32_t dH[3] = {H[0] - hh.x, H[1] - hh.y, H[2] - hh.z};
-        const int32_t dL[3] = {Lo[0] - hh.w, Lo[1] - ll.x, Lo[2] - ll.y};
-        int64_t hi;
-        uint32_t rem;
-        fix::square(dH, dL, &hi, &rem);
-        if constexpr (SOFT) {
-          hi += eh;
-          rem += el;
+        int em = top;
+        if ((tops & (tops - 1)) == 0) {
+          // a single heaviest body: not a source of the row where it is (itself,
+          // or a body at its place)
+          const int second = __reduce_max_sync(kAll, in && emj != top ? emj : INT_MIN);
+          const int at = __popc(cls & (tops - 1));
+          const int4 th = sm.h[at], tl = sm.l[at];
+          if (th.x == H[0] && th.y == H[1] && th.z == H[2] && th.w == Lo[0] && tl.x == Lo[1] && tl.y == Lo[2])
+            em = second;
         }
-        int s2;
-        const uint64_t w = fix::inv_cube(hi, rem, &s2);
-        const uint64_t q = fix::times_mass(w, static_cast<uint32_t>(ll.z), static_cast<uint32_t>(ll.w));
-        int k = kb - sm.x[c].x - 3 * s2;
-        if (fix::is_close(hi, close) || static_cast<unsigned>(k) >= fix::kShiftEnd) {
-          k = fix::kNoTerm;
-          mark |= bit;
-        }
-        bit <<= 1;
-        int32_t qd[3];
-        fix::factor_digits(q, k, qd);
-        fix::acc_add(acc, qd, dH, dL);
-      }
-      terms += 31 - __clz(static_cast<int>(bit)) - __popc(mark);
-      for (; mark; mark &= mark - 1) {
-        const int c = sub + nsub * (__ffs(static_cast<int>(mark)) - 1);
-        const int2 xx = sm.x[c];
-        if (xx.y == i) continue;
-        if constexpr (!SOFT) {
-          fix::W96 a[3], b[3];
-          unpack(rec[i], a);
-          unpack(rec[xx.y], b);
-          int32_t dH[3], dL[3], qd[3];
-          const int shc = fix::close_digits(a, b, dH, dL);
-          int64_t hi;
-          uint32_t rem;
-          int s2;
-          fix::square(dH, dL, &hi, &rem);
-          const uint64_t w = fix::inv_cube(hi, rem, &s2);
-          const uint64_t q =
-              fix::times_mass(w, static_cast<uint32_t>(sm.l[c].z), static_cast<uint32_t>(sm.l[c].w));
-          const int k = kb + 2 * (shc - sh) - xx.x - 3 * s2;
-          if (shc != fix::kNoDigits && static_cast<unsigned>(k) < fix::kShiftEnd) {
-            fix::factor_digits(q, k, qd);
-            fix::acc_add(acc, qd, dH, dL);
-            ++terms;
-            continue;
+        if (em != INT_MIN) {  // (else nothing but that body)
+          const int u = fix::unit_guess(gd, em);
+          if (abs(u - unit) > fix::kUnitSpan) {  // (also at the first class)
+            flush(acc, terms, sm, l);
+            acc.Ua = unit = u;
           }
         }
-        const double3 f = pair64(X[i] - X[xx.y], Y[i] - Y[xx.y], Zb[i] - Zb[xx.y], Mb[xx.y], eps2);
-        sm.f[0][l] += f.x;
-        sm.f[1][l] += f.y;
-        sm.f[2][l] += f.z;
-      }
-      // at most kMaxTerms steps between two carries
-      const int per = (32 + nsub - 1) / nsub;
-      steps += per;
-      if (steps + per > fix::kMaxTerms) {
-        fix::acc_carry(acc, terms);
-        steps = terms = 0;
-      }
+        const int kb = fix::k_base(acc.Ua, gd);
+        // The loop has no branch: close pairs, and those whose factor leaves the
+        // sums' range, add nothing here and are marked for the loop below.
+        unsigned mark = 0, bit = 1;
+        for (int c = active ? sub : 32; c < nc; c += nsub) {
+          const int4 hh = sm.h[c], ll = sm.l[c];
+          const int32_t dH[3] = {H[0] - hh.x, H[1] - hh.y, H[2] - hh.z};
+          const int32_t dL[3] = {Lo[0] - hh.w, Lo[1] - ll.x, Lo[2] - ll.y};
+          int64_t hi;
+          uint32_t rem;
+          fix::square(dH, dL, &hi, &rem);
+          if constexpr (SOFT) {
+            hi += eh;
+            rem += el;
+          }
+          int s2;
+          const uint64_t w = fix::inv_cube(hi, rem, &s2);
+          const uint64_t q = fix::times_mass(w, static_cast<uint32_t>(ll.z), static_cast<uint32_t>(ll.w));
+          int k = kb - sm.x[c].x - 3 * s2;
+          if (fix::is_close(hi, close) || static_cast<unsigned>(k) >= fix::kShiftEnd) {
+            k = fix::kNoTerm;
+            mark |= bit;
+          }
+          bit <<= 1;
+          int32_t qd[3];
+          fix::factor_digits(q, k, qd);
+          fix::acc_add(acc, qd, dH, dL);
+        }
+        terms += 31 - __clz(static_cast<int>(bit)) - __popc(mark);
+        for (; mark; mark &= mark - 1) {
+          const int c = sub + nsub * (__ffs(static_cast<int>(mark)) - 1);
+          const int2 xx = sm.x[c];
+          if (xx.y == i) continue;
+          if constexpr (!SOFT) {
+            fix::W96 a[3], b[3];
+            unpack(rec[i], a);
+            unpack(rec[xx.y], b);
+            int32_t dH[3], dL[3], qd[3];
+            const int shc = fix::close_digits(a, b, dH, dL);
+            int64_t hi;
+            uint32_t rem;
+            int s2;
+            fix::square(dH, dL, &hi, &rem);
+            const uint64_t w = fix::inv_cube(hi, rem, &s2);
+            const uint64_t q =
+                fix::times_mass(w, static_cast<uint32_t>(sm.l[c].z), static_cast<uint32_t>(sm.l[c].w));
+            const int k = kb + 2 * (shc - sh) - xx.x - 3 * s2;
+            if (shc != fix::kNoDigits && static_cast<unsigned>(k) < fix::kShiftEnd) {
+              fix::factor_digits(q, k, qd);
+              fix::acc_add(acc, qd, dH, dL);
+              ++terms;
+              continue;
+            }
+          }
+          const double3 f = pair64(X[i] - X[xx.y], Y[i] - Y[xx.y], Zb[i] - Zb[xx.y], Mb[xx.y], eps2);
+          sm.f[0][l] += f.x;
+          sm.f[1][l] += f.y;
+          sm.f[2][l] += f.z;
+        }
+        // at most kMaxTerms steps between two carries
+        steps += (nc + nsub - 1) / nsub;
+        if (steps + (32 + nsub - 1) / nsub > fix::kMaxTerms) {
+          fix::acc_carry(acc, terms);
+          steps = terms = 0;
+        }
+      } while (rest);
     }
     flush(acc, terms, sm, l);
     double v[3] = {sm.f[0][l], sm.f[1][l], sm.f[2][l]};
@@ -333,28 +362,6 @@ __global__ void __launch_bounds__(kWarps * 32, 4) k_p2p64(
       }
     }
   }
-}
-
-// The two largest mass exponents of every leaf's bodies (INT_MIN without a
-// second one): they set the unit of the sums.
-__global__ void k_leaf_heavy(int32_t nleaf, const int32_t *__restrict__ leaves, const int32_t *__restrict__ begin,
-                             const int32_t *__restrict__ count, const Rec *__restrict__ rec,
-                             int2 *__restrict__ heavy) {
-  pdl_wait();
-  const int q = static_cast<int>((blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x) >> 5);
-  const int l = threadIdx.x & 31;
-  if (q >= nleaf) return;  // a warp per leaf
-  const int L = leaves[q], b = begin[L], n = count[L];
-  int a = INT_MIN, s = INT_MIN;
-  for (int t = l; t < n; t += 32) {
-    const int v = static_cast<int16_t>(rec[b + t].c.w & 0xffffu);
-    s = max(s, min(a, v));
-    a = max(a, v);
-  }
-  const int m = __reduce_max_sync(0xffffffffu, a);
-  const unsigned top = __ballot_sync(0xffffffffu, a == m);
-  const int m2 = __reduce_max_sync(0xffffffffu, a == m ? s : a);
-  if (l == 0) heavy[L] = make_int2(m, (top & (top - 1)) ? m : m2);
 }
 
 // Entry groups of a leaf (its own entry and ne partners)
@@ -449,10 +456,6 @@ int p2p64_prepare(fmm_ctx *c) {
          ptr<double>(c->Mb), forest ? ptr<double>(c->sbox) : ptr<double>(c->bbox), ptr<int32_t>(c->order),
          forest ? ptr<int32_t>(c->sysid) : nullptr, ptr<Rec>(c->p2p_rec));
   AMFMM_TRY(launched(c, "p2p_body_fixed"));
-  AMFMM_TRY(ensure<int2>(c, c->p2p_heavy, nc));
-  launch(c, k_leaf_heavy, grid_for(32 * static_cast<int64_t>(nleaf), 256), 256, 0, nleaf, ptr<int32_t>(c->leaves),
-         ptr<int32_t>(c->begin), ptr<int32_t>(c->count), ptr<Rec>(c->p2p_rec), ptr<int2>(c->p2p_heavy));
-  AMFMM_TRY(launched(c, "p2p_leaf_heavy"));
   // every leaf's partners, in the stable order of the pair list
   int32_t *off = ptr<int32_t>(c->p2p_offA);
   AMFMM_TRY(partner_lists(c, ptr<int2>(c->p2p), K, c->pkey, c->pval, off, &c->p2p_which));
@@ -500,8 +503,7 @@ int p2p64_run(fmm_ctx *c) {
   int *queue = ptr<int32_t>(c->totals) + 40;
   launch(c, kern, grid, kWarps * 32, 0, nitem, c->sz.n, ptr<int4>(c->p2p_items), ptr<int32_t>(c->begin),
          ptr<int32_t>(c->count), ptr<int32_t>(c->p2p_offA),
-         c->sz.n_p2p > 0 ? ptr<uint32_t>(c->pval[c->p2p_which]) : nullptr, ptr<int2>(c->p2p_heavy),
-         ptr<Rec>(c->p2p_rec), ptr<double>(c->X), ptr<double>(c->Y), ptr<double>(c->Zb), ptr<double>(c->Mb), c->eps2,
+         c->sz.n_p2p > 0 ? ptr<uint32_t>(c->pval[c->p2p_which]) : nullptr, ptr<Rec>(c->p2p_rec), ptr<double>(c->X), ptr<double>(c->Y), ptr<double>(c->Zb), ptr<double>(c->Mb), c->eps2,
          ptr<double>(c->near), ptr<double>(c->p2p_extra), queue);
   AMFMM_TRY(launched(c, "p2p"));
   if (c->sz.n_p2p == 0) return FMM_OK;
