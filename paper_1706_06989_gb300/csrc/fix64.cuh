@@ -25,8 +25,11 @@
 // A close pair takes a window of its own from the 96-bit positions
 // (close_digits): closer than 2^-7 of the window when the window rounds a
 // position (coordinates within 2^-4 of the window from zero), else closer than
-// 2^-10, the least the digits' normalisation takes.
+// 2^-10, the least the digits' normalisation takes.  Softened pairs closer than
+// 2^-5, by r^2 without eps^2, are left to FP64: their terms m d / (r^2 + eps^2)^(3/2)
+// shrink with d, and with it the bits that d's digits and the sums' unit leave them.
 #pragma once
+#include <math.h>
 #include <stdint.h>
 
 #ifdef __CUDACC__
@@ -44,6 +47,7 @@ constexpr int kWin = 57;  // |difference| <= 2^kWin
 // r^2 / 2^58, high word, below which a pair is close: 2^42 and 2^36 (signed:
 // hi is -1 for the closest pairs, whose rem makes up for it)
 constexpr int32_t kCloseRounded = 1 << (42 - 32), kCloseExact = 1 << (36 - 32);
+constexpr int32_t kCloseSoft = 1 << (46 - 32);
 AMFMM_HD bool is_close(int64_t hi, int32_t bound) { return static_cast<int32_t>(hi >> 32) < bound; }
 constexpr int kFieldUp = 26;   // fraction bits a factor keeps below its mantissa
 constexpr int kMaxTerms = 32;  // terms before the carries are propagated (a term adds below 2^58 to a1, 2^26 to a0)
@@ -108,6 +112,26 @@ AMFMM_HD uint64_t mul_wide_u(uint32_t a, uint32_t b) {
 // move more.)
 AMFMM_HD int32_t mul_hi(int32_t a, int32_t b) { return static_cast<int32_t>(mul_wide(a, b) >> 32); }
 AMFMM_HD uint32_t mul_hi_u(uint32_t a, uint32_t b) { return static_cast<uint32_t>(mul_wide_u(a, b) >> 32); }
+
+// 64-bit shifts by 0 .. 64 and beyond: what is shifted out is zero.
+AMFMM_HD uint64_t shr64(uint64_t v, unsigned s) {
+#ifdef __CUDA_ARCH__
+  uint64_t d;
+  asm("shr.u64 %0, %1, %2;" : "=l"(d) : "l"(v), "r"(s));
+  return d;
+#else
+  return s < 64 ? v >> s : 0;
+#endif
+}
+AMFMM_HD uint64_t shl64(uint64_t v, unsigned s) {
+#ifdef __CUDA_ARCH__
+  uint64_t d;
+  asm("shl.b64 %0, %1, %2;" : "=l"(d) : "l"(v), "r"(s));
+  return d;
+#else
+  return s < 64 ? v << s : 0;
+#endif
+}
 
 // ---- conversion of the inputs ------------------------------------------
 struct W96 {
@@ -255,6 +279,42 @@ AMFMM_HD void square(const int32_t dH[3], const int32_t dL[3], int64_t *hi, uint
   *rem = ((static_cast<uint32_t>(S1) & 0xfffffffu) >> 2) + static_cast<uint32_t>(S0);
 }
 
+// Softening, for digits in units of 2^gd.  The window is that of the positions
+// alone, so that a length far above the separations takes no bits from the
+// differences: eps^2 = eh 2^58 + el 2^32, like r^2, in units of 2^(2 (gd + t)), t = 0
+// while eps^2 fits.
+struct Soft {
+  int t, s2, room;  // s2 (of inv_cube) at the window's bound; 3 x what it grows by down to the closest pairs
+  int64_t eh;
+  uint32_t el;
+};
+AMFMM_HD int soft_s2(const Soft &s, int bits) {  // at r^2 = 2^bits in units of 2^(2 gd + 58)
+  const int64_t v = s.eh + (bits >= 2 * s.t ? 1ll << (bits - 2 * s.t) : 0);
+  return (clz32(static_cast<uint32_t>(v >> 32)) - 1) >> 1;
+}
+AMFMM_HD Soft soft_window(double eps2, int gd) {
+  Soft s;
+  const int up = ilogb(eps2) - 2 * gd - 2 * kDig - 59;  // eh stays below 2^60
+  s.t = up > 0 ? (up + 1) / 2 : 0;
+  const double e = scalbn(eps2, -2 * (gd + s.t) - 2 * kDig);
+  s.eh = static_cast<int64_t>(e);
+  s.el = static_cast<uint32_t>(scalbn(e - static_cast<double>(s.eh), 2 * kDig - 32));
+  s.s2 = soft_s2(s, 56);
+  s.room = 3 * (soft_s2(s, 46) - s.s2);
+  return s;
+}
+// r^2 + eps^2 from r^2 of the digits' difference
+AMFMM_HD void soften(const Soft &s, int64_t *hi, uint32_t *rem) {
+  if (s.t) {  // the same for a whole batch
+    const unsigned d = 2 * static_cast<unsigned>(s.t);
+    const uint64_t h = static_cast<uint64_t>(*hi);
+    *rem = (d < 26 ? static_cast<uint32_t>(h << (26 - d)) : static_cast<uint32_t>(shr64(h, d - 26))) & 0x3ffffffu;
+    *hi = static_cast<int64_t>(shr64(h, d));
+  }
+  *hi += s.eh;
+  *rem += s.el;
+}
+
 // r^-3 = w 2^-58 2^(-3 (60 - s2 + gd)) for r^2 = (hi 2^58 + rem 2^32) 2^(2 gd),
 // hi >= 2^36; w in [2^56, 2^60).
 AMFMM_HD uint64_t inv_cube(int64_t hi, uint32_t rem, int *s2out) {
@@ -323,26 +383,6 @@ AMFMM_HD void acc_carry(Acc &a, int terms) {
   }
 }
 
-// 64-bit shifts by 0 .. 64 and beyond: what is shifted out is zero.
-AMFMM_HD uint64_t shr64(uint64_t v, unsigned s) {
-#ifdef __CUDA_ARCH__
-  uint64_t d;
-  asm("shr.u64 %0, %1, %2;" : "=l"(d) : "l"(v), "r"(s));
-  return d;
-#else
-  return s < 64 ? v >> s : 0;
-#endif
-}
-AMFMM_HD uint64_t shl64(uint64_t v, unsigned s) {
-#ifdef __CUDA_ARCH__
-  uint64_t d;
-  asm("shl.b64 %0, %1, %2;" : "=l"(d) : "l"(v), "r"(s));
-  return d;
-#else
-  return s < 64 ? v << s : 0;
-#endif
-}
-
 // Digits (weights 2^58, 2^29, 1) of a factor q 2^eq in the sums' unit, where
 // k = Ua + 26 - eq - gd in [0, kShiftEnd) places it; kNoTerm gives zeros.
 constexpr unsigned kShiftEnd = 52;  // (the middle digit of a term is then never zero)
@@ -379,8 +419,16 @@ AMFMM_HD void acc_add(Acc &a, const int32_t q[3], const int32_t dH[3], const int
 constexpr int kWinSpan = 3, kUnitSpan = 2 * kWinSpan, kClassSpan = 21;
 AMFMM_HD int unit_guess(int gd, int em) { return 24 + em + 9 - (kFieldUp + 238 + 2 * gd); }
 
+// Softened, a heavy source next to the row adds little, so every term keeps its own
+// bits: classes span 2^kSoftClassSpan, and the unit gives the heaviest source k = 2
+// at the closest.  The lightest has at most 2^(28 - 79) of its term rounded away.
+constexpr int kSoftUnitSpan = 2, kSoftClassSpan = 9;
+AMFMM_HD int unit_soft(int gd, int em, const Soft &s) {
+  return s.room + 2 + em + 3 * (s.s2 - s.t) - (kFieldUp + 238 + 2 * gd);
+}
+
 // Constant part of k for a batch of window exponent gd: k = base - em - 3 s2
-// with em the source mass's exponent (eq = em - 238 + 3 s2 - 3 gd).
+// with em the source mass's exponent (eq = em - 238 + 3 s2 - 3 gd; softened, gd + t).
 AMFMM_HD int k_base(int Ua, int gd) { return Ua + kFieldUp + 238 + 2 * gd; }
 
 }  // namespace fix

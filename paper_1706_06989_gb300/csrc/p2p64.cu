@@ -91,8 +91,8 @@ __device__ __forceinline__ void offset(const Rec &r, const Rec &origin, fix::W96
 }
 
 // Pairs without digits (positions that agree to 2^-71 of the system's extent,
-// close softened pairs, any pair when the softening length exceeds the
-// system): the direct sum's formula in FP64.
+// close softened pairs, any pair when eps^2 overflows): the direct sum's formula
+// in FP64.
 __device__ __forceinline__ double3 pair64(double dx, double dy, double dz, double m, double eps2) {
   const double d2 = fma(dz, dz, fma(dy, dy, dx * dx));
   if (d2 == 0.0) return make_double3(0.0, 0.0, 0.0);
@@ -119,8 +119,7 @@ __device__ __forceinline__ void flush(fix::Acc &acc, int &terms, WarpSmem &sm, i
   terms = 0;
 }
 
-// SOFT: softening added to r^2 in fixed point; a length beyond the system's
-// extent leaves no digits for the separations, and every pair goes to FP64.
+// SOFT: softening added to r^2 in fixed point.
 template <bool SOFT>
 __global__ void __launch_bounds__(kWarps * 32, 4) k_p2p64(
     int32_t nitem, int64_t n, const int4 *__restrict__ items, const int32_t *__restrict__ begin,
@@ -156,13 +155,7 @@ __global__ void __launch_bounds__(kWarps * 32, 4) k_p2p64(
     }
 #pragma unroll
     for (int c = 0; c < 3; ++c) sm.f[c][l] = 0.0;
-    bool all64 = false;
-    if constexpr (SOFT) {
-      // the window also holds the softening length
-      const double e = scalbn(sqrt(eps2), -(g0 + 64));
-      all64 = !(e < 1073741824.0);
-      if (!all64) rmag = max(rmag, static_cast<uint32_t>(e) + 1u);
-    }
+    const bool all64 = SOFT && !isfinite(eps2);
     rmag = __reduce_max_sync(kAll, rmag);
     fix::Acc acc;
     fix::acc_clear(acc);
@@ -190,6 +183,7 @@ __global__ void __launch_bounds__(kWarps * 32, 4) k_p2p64(
     int unit = INT_MIN / 2;  // the sums' unit, less what acc_carry raises it by
     int32_t H[3], Lo[3];
     bool rounded = false;
+    fix::Soft soft{};
     for (int j0 = 0; j0 < total; j0 += 32) {
       const int j = min(j0 + l, total - 1);
       int own = 0;  // entry of column j: the number of entries that end at or before it
@@ -215,14 +209,7 @@ __global__ void __launch_bounds__(kWarps * 32, 4) k_p2p64(
 #pragma unroll
         for (int c = 0; c < 3; ++c) rounded |= fix::digits(o[c], sh, &H[c], &Lo[c]);
         shPrev = sh;
-      }
-      int64_t eh = 0;
-      uint32_t el = 0;
-      if (SOFT && !all64) {
-        // eps^2 in units of 2^(2 gd + 58), and the rest in units of 2^(2 gd + 32)
-        const double es = scalbn(eps2, -2 * gd - 2 * fix::kDig);
-        eh = static_cast<int64_t>(es);
-        el = static_cast<uint32_t>(scalbn(es - static_cast<double>(eh), 2 * fix::kDig - 32));
+        if (SOFT && !all64) soft = fix::soft_window(eps2, gd);
       }
       const int ncol = min(32, total - j0);
       int4 dh, dl;
@@ -233,7 +220,7 @@ __global__ void __launch_bounds__(kWarps * 32, 4) k_p2p64(
 #pragma unroll
         for (int c = 0; c < 3; ++c) r |= fix::digits(s[c], sh, &h[c], &lo[c]);
         close = __any_sync(kAll, r) ? fix::kCloseRounded : fix::kCloseExact;
-        if (SOFT && all64) close = 0x7fffffff;
+        if (SOFT) close = all64 ? 0x7fffffff : fix::kCloseSoft;
         dh = make_int4(h[0], h[1], h[2], lo[0]);
         dl = make_int4(lo[1], lo[2], static_cast<int>(rj.c.y), static_cast<int>(rj.c.z));
       }
@@ -243,7 +230,7 @@ __global__ void __launch_bounds__(kWarps * 32, 4) k_p2p64(
         const bool there = (rest >> l) & 1u;
         int top = __shfl_sync(kAll, emj, __ffs(static_cast<int>(rest)) - 1);
         if (__any_sync(kAll, there && emj != top)) top = __reduce_max_sync(kAll, there ? emj : INT_MIN);
-        const bool in = there && emj >= top - fix::kClassSpan;
+        const bool in = there && emj >= top - (SOFT ? fix::kSoftClassSpan : fix::kClassSpan);
         const unsigned cls = __ballot_sync(kAll, in), tops = __ballot_sync(kAll, in && emj == top);
         const int nc = __popc(cls);
         rest &= ~cls;
@@ -256,7 +243,7 @@ __global__ void __launch_bounds__(kWarps * 32, 4) k_p2p64(
         }
         __syncwarp();
         int em = top;
-        if ((tops & (tops - 1)) == 0) {
+        if (!SOFT && (tops & (tops - 1)) == 0) {
           // a single heaviest body: not a source of the row where it is (itself,
           // or a body at its place)
           const int second = __reduce_max_sync(kAll, in && emj != top ? emj : INT_MIN);
@@ -266,13 +253,13 @@ __global__ void __launch_bounds__(kWarps * 32, 4) k_p2p64(
             em = second;
         }
         if (em != INT_MIN) {  // (else nothing but that body)
-          const int u = fix::unit_guess(gd, em);
-          if (abs(u - unit) > fix::kUnitSpan) {  // (also at the first class)
+          const int u = SOFT ? fix::unit_soft(gd, em, soft) : fix::unit_guess(gd, em);
+          if (abs(u - unit) > (SOFT ? fix::kSoftUnitSpan : fix::kUnitSpan)) {  // (also at the first class)
             flush(acc, terms, sm, l);
             acc.Ua = unit = u;
           }
         }
-        const int kb = fix::k_base(acc.Ua, gd);
+        const int kb = fix::k_base(acc.Ua, gd) + 3 * soft.t;
         // The loop has no branch: close pairs, and those whose factor leaves the
         // sums' range, add nothing here and are marked for the loop below.
         unsigned mark = 0, bit = 1;
@@ -283,15 +270,13 @@ __global__ void __launch_bounds__(kWarps * 32, 4) k_p2p64(
           int64_t hi;
           uint32_t rem;
           fix::square(dH, dL, &hi, &rem);
-          if constexpr (SOFT) {
-            hi += eh;
-            rem += el;
-          }
+          const bool apart = !fix::is_close(hi, close);
+          if constexpr (SOFT) fix::soften(soft, &hi, &rem);
           int s2;
           const uint64_t w = fix::inv_cube(hi, rem, &s2);
           const uint64_t q = fix::times_mass(w, static_cast<uint32_t>(ll.z), static_cast<uint32_t>(ll.w));
           int k = kb - sm.x[c].x - 3 * s2;
-          if (fix::is_close(hi, close) || static_cast<unsigned>(k) >= fix::kShiftEnd) {
+          if (!apart || static_cast<unsigned>(k) >= fix::kShiftEnd) {
             k = fix::kNoTerm;
             mark |= bit;
           }

@@ -17,18 +17,19 @@ SOURCE = r"""
 namespace amfmm { namespace fix { float seed_error = 0; } }
 using namespace amfmm::fix;
 namespace {
-void pair64(const double *t, const double *s, double m, double f[3]) {
+void pair64(const double *t, const double *s, double m, double eps2, double f[3]) {
   const double d[3] = {t[0] - s[0], t[1] - s[1], t[2] - s[2]};
   const double d2 = std::fma(d[2], d[2], std::fma(d[1], d[1], d[0] * d[0]));
-  const double ri = d2 == 0 ? 0 : 1 / std::sqrt(d2), q = m * (ri * ri * ri);
+  const double ri = d2 == 0 ? 0 : 1 / std::sqrt(d2 + eps2), q = m * (ri * ri * ri);
   for (int c = 0; c < 3; ++c) f[c] += q * d[c];
 }
 }  // namespace
 // own: the target's place among the sources, -1 if it is none.  how[j]: 0
 // integers, 1 integers in a window of the pair's own, 2 FP64.
-extern "C" void near_sum(int ns, const double *t, const double *s, const double *m, int own, double scale, float err,
-                         double *out, unsigned char *how) {
+extern "C" void near_sum(int ns, const double *t, const double *s, const double *m, int own, double scale, double eps2,
+                         float err, double *out, unsigned char *how) {
   seed_error = err;
+  const bool soft = eps2 > 0;
   const int g0 = extent_exponent(scale) - 95;
   W96 pt[3], o[3], ref[3];
   uint32_t rmag = 0;
@@ -69,7 +70,10 @@ extern "C" void near_sum(int ns, const double *t, const double *s, const double 
     for (int c = 0; c < 3; ++c) rounded |= digits(o[c], sh, &H[c], &L[c]);
     for (int j = 0; j < n; ++j)
       for (int c = 0; c < 3; ++c) rounded |= digits(sub96(ps[j][c], ref[c]), sh, &h[j][c], &lo[j][c]);
-    const int32_t bound = rounded ? kCloseRounded : kCloseExact;
+    const int32_t bound = soft ? kCloseSoft : rounded ? kCloseRounded : kCloseExact;
+    const int class_span = soft ? kSoftClassSpan : kClassSpan, unit_span = soft ? kSoftUnitSpan : kUnitSpan;
+    Soft sw{};
+    if (soft) sw = soft_window(eps2, gd);
     bool todo[32];
     for (int j = 0; j < n; ++j) todo[j] = true;
     for (;;) {
@@ -85,18 +89,19 @@ extern "C" void near_sum(int ns, const double *t, const double *s, const double 
       heavy = top;
       bool here = true;
       for (int c = 0; c < 3; ++c) here = here && h[at][c] == H[c] && lo[at][c] == L[c];
-      if (tops == 1 && here) {
+      if (!soft && tops == 1 && here) {
         heavy = none;
         for (int j = 0; j < n; ++j)
           if (todo[j] && em[j] != top) heavy = std::max(heavy, em[j]);
       }
-      if (heavy >= top - kClassSpan && std::abs(unit_guess(gd, heavy) - unit) > kUnitSpan) {
+      const int u = soft ? unit_soft(gd, heavy, sw) : unit_guess(gd, heavy);
+      if (heavy >= top - class_span && std::abs(u - unit) > unit_span) {
         flush();
-        a.Ua = unit = unit_guess(gd, heavy);
+        a.Ua = unit = u;
       }
-      const int kb = k_base(a.Ua, gd);
+      const int kb = k_base(a.Ua, gd) + 3 * sw.t;
       for (int j = 0; j < n; ++j) {
-        if (!todo[j] || em[j] < top - kClassSpan) continue;
+        if (!todo[j] || em[j] < top - class_span) continue;
         todo[j] = false;
         how[j0 + j] = 2;
         if (j0 + j == own) continue;
@@ -108,10 +113,11 @@ extern "C" void near_sum(int ns, const double *t, const double *s, const double 
         const bool close = is_close(hi, bound);
         int shc = sh, s2;
         if (close) {
-          shc = close_digits(pt, ps[j], dH, dL);
+          shc = soft ? kNoDigits : close_digits(pt, ps[j], dH, dL);
           square(dH, dL, &hi, &rem);
         }
         if (shc != kNoDigits) {
+          if (soft) soften(sw, &hi, &rem);
           const uint64_t w = inv_cube(hi, rem, &s2);
           const uint64_t q = times_mass(w, static_cast<uint32_t>(M[j] >> 32), static_cast<uint32_t>(M[j]));
           const int k = kb + 2 * (shc - sh) - em[j] - 3 * s2;
@@ -122,7 +128,7 @@ extern "C" void near_sum(int ns, const double *t, const double *s, const double 
             how[j0 + j] = close;
           }
         }
-        if (how[j0 + j] == 2) pair64(t, s + 3 * (j0 + j), m[j0 + j], out);
+        if (how[j0 + j] == 2) pair64(t, s + 3 * (j0 + j), m[j0 + j], eps2, out);
       }
       acc_carry(a, terms);
       terms = 0;
@@ -135,33 +141,34 @@ extern "C" void near_sum(int ns, const double *t, const double *s, const double 
 
 def build(directory):
     """near_sum as a Python function: (target, sources, masses, own=place of the
-    target among them) -> (sum of m (t - s) / r^3, how[])."""
+    target among them) -> (sum of m (t - s) / (r^2 + eps^2)^(3/2), how[])."""
     src, so = os.path.join(directory, "near.cpp"), os.path.join(directory, "near.so")
     with open(src, "w") as f:
         f.write(SOURCE)
     subprocess.run(["g++", "-O2", "-std=gnu++17", "-shared", "-fPIC", "-I", CSRC, "-o", so, src], check=True)
     f = ctypes.CDLL(so).near_sum
     P, D = ctypes.c_void_p, ctypes.c_double
-    f.argtypes = [ctypes.c_int, P, P, P, ctypes.c_int, D, ctypes.c_float, P, P]
+    f.argtypes = [ctypes.c_int, P, P, P, ctypes.c_int, D, D, ctypes.c_float, P, P]
     f.restype = None
 
-    def near_sum(t, s, m, own=-1, err=0.0, extent=None):
+    def near_sum(t, s, m, eps=0.0, own=-1, err=0.0, extent=None):
         t, s, m = (np.ascontiguousarray(v, dtype=np.float64) for v in (t, s, m))
         p = np.vstack([t[None], s])
         ext = (p.max(0) - p.min(0)).max() if extent is None else extent
         out, how = np.zeros(3), np.zeros(len(s), dtype=np.uint8)
-        f(len(s), t.ctypes.data, s.ctypes.data, m.ctypes.data, own, 2.0 ** 21 / ext, err, out.ctypes.data,
+        f(len(s), t.ctypes.data, s.ctypes.data, m.ctypes.data, own, 2.0 ** 21 / ext, eps * eps, err, out.ctypes.data,
           how.ctypes.data)
         return out, how
 
     return near_sum
 
 
-def exact(t, s, m):
+def exact(t, s, m, eps=0.0):
     """The sum in extended precision, and the sum of its terms' magnitudes."""
     L = np.longdouble
     d = t.astype(L) - s.astype(L)
     r2 = (d * d).sum(1)
-    q = np.where(r2 > 0, m.astype(L) / np.where(r2 > 0, r2 * np.sqrt(r2), 1), 0)
+    e2 = r2 + L(eps * eps)
+    q = np.where(r2 > 0, m.astype(L) / np.where(r2 > 0, e2 * np.sqrt(e2), 1), 0)
     term = q[:, None] * d
     return term.sum(0), float(np.sqrt((term ** 2).sum(1)).sum())
