@@ -23,11 +23,12 @@
 //              first term: a sum rounds nothing but its terms, to 2^-79 of
 //              the largest factor the unit allows.
 // A close pair takes a window of its own from the 96-bit positions
-// (close_digits): closer than 2^-7 of the window when the window rounds a
-// position (coordinates within 2^-4 of the window from zero), else closer than
-// 2^-10, the least the digits' normalisation takes.  Softened pairs closer than
-// 2^-5, by r^2 without eps^2, are left to FP64: their terms m d / (r^2 + eps^2)^(3/2)
-// shrink with d, and with it the bits that d's digits and the sums' unit leave them.
+// (close_digits): closer than 2^-5 of the window when the window rounds a
+// position (coordinates within 2^-4 of the window from zero; a difference there is
+// good to 2^-52 of itself), else closer than 2^-10, the least the digits'
+// normalisation takes.  Softened pairs closer than 2^-5, by r^2 without eps^2, are
+// left to FP64: their terms m d / (r^2 + eps^2)^(3/2) shrink with d, and with it the
+// bits that d's digits and the sums' unit leave them.
 #pragma once
 #include <math.h>
 #include <stdint.h>
@@ -44,10 +45,9 @@ namespace fix {
 constexpr int kDig = 29;  // bits of a digit
 constexpr uint32_t kDigMask = (1u << kDig) - 1;
 constexpr int kWin = 57;  // |difference| <= 2^kWin
-// r^2 / 2^58, high word, below which a pair is close: 2^42 and 2^36 (signed:
+// r^2 / 2^58, high word, below which a pair is close: 2^46 and 2^36 (signed:
 // hi is -1 for the closest pairs, whose rem makes up for it)
-constexpr int32_t kCloseRounded = 1 << (42 - 32), kCloseExact = 1 << (36 - 32);
-constexpr int32_t kCloseSoft = 1 << (46 - 32);
+constexpr int32_t kCloseRounded = 1 << (46 - 32), kCloseExact = 1 << (36 - 32);
 AMFMM_HD bool is_close(int64_t hi, int32_t bound) { return static_cast<int32_t>(hi >> 32) < bound; }
 constexpr int kFieldUp = 26;   // fraction bits a factor keeps below its mantissa
 constexpr int kMaxTerms = 32;  // terms before the carries are propagated (a term adds below 2^58 to a1, 2^26 to a0)
@@ -245,8 +245,8 @@ AMFMM_HD bool digits(const W96 &o, int sh, int32_t *H, int32_t *L) {
 // ---- the pair ----------------------------------------------------------
 // Digits of a close pair's difference d = a - b at the finest window that
 // holds it: the largest component lies in [2^(kWin - 1), 2^kWin).  Returns
-// the window's shift, or kNoDigits when the positions agree to 2^24 units
-// (2^-71 of the system's extent), where their rounding shows.
+// the window's shift, or kNoDigits when the positions agree to 2^53 units
+// (2^-42 of the system's extent), where their rounding shows.
 constexpr int kNoDigits = -1000;
 AMFMM_HD int close_digits(const W96 a[3], const W96 b[3], int32_t H[3], int32_t L[3]) {
   __int128 d[3];
@@ -259,7 +259,7 @@ AMFMM_HD int close_digits(const W96 a[3], const W96 b[3], int32_t H[3], int32_t 
   }
   const uint32_t m2 = static_cast<uint32_t>(m >> 64), m1 = static_cast<uint32_t>(m >> 32), m0 = static_cast<uint32_t>(m);
   const int bits = m2 ? 95 - clz32(m2) : m1 ? 63 - clz32(m1) : 31 - clz32(m0);
-  if (bits < 24) return kNoDigits;
+  if (bits < 53) return kNoDigits;
   const int sh = bits - (kWin - 1);
   for (int c = 0; c < 3; ++c) {
     const __int128 v = sh > 0 ? (d[c] + (static_cast<__int128>(1) << (sh - 1))) >> sh : d[c] << -sh;

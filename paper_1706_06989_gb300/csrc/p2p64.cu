@@ -90,7 +90,7 @@ __device__ __forceinline__ void offset(const Rec &r, const Rec &origin, fix::W96
   *em = static_cast<int16_t>(r.c.w & 0xffffu);
 }
 
-// Pairs without digits (positions that agree to 2^-71 of the system's extent,
+// Pairs without digits (positions that agree to 2^-42 of the system's extent,
 // close softened pairs, any pair when eps^2 overflows): the direct sum's formula
 // in FP64.
 __device__ __forceinline__ double3 pair64(double dx, double dy, double dz, double m, double eps2) {
@@ -220,7 +220,7 @@ __global__ void __launch_bounds__(kWarps * 32, 4) k_p2p64(
 #pragma unroll
         for (int c = 0; c < 3; ++c) r |= fix::digits(s[c], sh, &h[c], &lo[c]);
         close = __any_sync(kAll, r) ? fix::kCloseRounded : fix::kCloseExact;
-        if (SOFT) close = all64 ? 0x7fffffff : fix::kCloseSoft;
+        if (SOFT) close = all64 ? 0x7fffffff : fix::kCloseRounded;
         dh = make_int4(h[0], h[1], h[2], lo[0]);
         dl = make_int4(lo[1], lo[2], static_cast<int>(rj.c.y), static_cast<int>(rj.c.z));
       }

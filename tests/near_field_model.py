@@ -70,7 +70,7 @@ extern "C" void near_sum(int ns, const double *t, const double *s, const double 
     for (int c = 0; c < 3; ++c) rounded |= digits(o[c], sh, &H[c], &L[c]);
     for (int j = 0; j < n; ++j)
       for (int c = 0; c < 3; ++c) rounded |= digits(sub96(ps[j][c], ref[c]), sh, &h[j][c], &lo[j][c]);
-    const int32_t bound = soft ? kCloseSoft : rounded ? kCloseRounded : kCloseExact;
+    const int32_t bound = soft || rounded ? kCloseRounded : kCloseExact;
     const int class_span = soft ? kSoftClassSpan : kClassSpan, unit_span = soft ? kSoftUnitSpan : kUnitSpan;
     Soft sw{};
     if (soft) sw = soft_window(eps2, gd);
