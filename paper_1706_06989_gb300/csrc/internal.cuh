@@ -164,7 +164,7 @@ struct fmm_ctx {
       p2p_slots, p2p_colOff, p2p_cols, p2p_nb, p2p_pre, p2p_rec, p2p_rowpart, p2p_items, p2p_itemOff, p2p_extraOff,
       p2p_extra;
   // scan / sort scratch; `totals` holds small device results (1 KiB):
-  // [0,16) scan totals, [64,72) near-field body-pair count, [80,88) selector-scored pairs, [88,92) selector candidates, [96,104) slot total,
+  // [0,16) scan totals, [64,72) near-field body-pair count, [80,88) selector-scored pairs, [88,92) selector candidates, [96,104) slot total or FP64 partial sums, [104,120) near-field work items and extra partials,
   // [128,144) near-field column, work-item, extra-partial and heavy-leaf totals, [160,168) work queues (near field, gathered far field);
   // the walk clears the counters among them
   amfmm::DBuf scan_tmp, sort_hist, totals, diag;

@@ -143,6 +143,7 @@ __device__ __forceinline__ int2 chunk_range(int j, int cb, int ce, int nself) {
   const int c0 = cb + first + (j - 1) * kChunk;
   return make_int2(c0, min(ce, c0 + kChunk));
 }
+// (counts of places and items in 64 bits: both are refused beyond 2^31 - 1)
 // more columns than a third of the average of the warps that run at once
 __device__ __forceinline__ bool is_heavy(int ncol, int total, int warps) {
   return ncol > max(kHeavyMin, total / (3 * warps));
@@ -150,26 +151,39 @@ __device__ __forceinline__ bool is_heavy(int ncol, int total, int warps) {
 
 __global__ void k_item_counts(int32_t nleaf, const int32_t *__restrict__ leaves, const int32_t *__restrict__ count,
                               const int32_t *__restrict__ colOff, const int32_t *__restrict__ total, int warps,
-                              int32_t *__restrict__ nitems, int32_t *__restrict__ nextra, int *__restrict__ nheavy) {
+                              int32_t *__restrict__ nitems, int32_t *__restrict__ nextra, int *__restrict__ nheavy,
+                              unsigned long long *__restrict__ wide) {
   pdl_wait();
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= nleaf) return;
-  if (q == 0) nitems[nleaf] = nextra[nleaf] = 0;
-  const int L = leaves[q], cb = colOff[L], ce = colOff[L + 1], nA = count[L];
-  const int k = chunks_of(ce - cb, nA);
-  if (!is_heavy(ce - cb, *total, warps)) {
-    nitems[q] = k;
-    nextra[q] = (k - 1) * 3 * nA;
-    return;
+  unsigned long long items = 0, places = 0;
+  if (q < nleaf) {
+    if (q == 0) nitems[nleaf] = nextra[nleaf] = 0;
+    const int L = leaves[q], cb = colOff[L], ce = colOff[L + 1], nA = count[L];
+    const int k = chunks_of(ce - cb, nA);
+    if (!is_heavy(ce - cb, *total, warps)) {
+      items = k;
+      places = (k - 1) * 3ull * nA;
+    } else {
+      for (int j = 0; j < k; ++j) {
+        const int2 c = chunk_range(j, cb, ce, nA);
+        items += (nA + kItemRows - 1) / kItemRows + (c.y - c.x + kItemCols - 1) / kItemCols;
+      }
+      atomicAdd(nheavy, 1);
+      places = (k + 1) * 3ull * nA;
+    }
+    nitems[q] = static_cast<int32_t>(items);
+    nextra[q] = static_cast<int32_t>(places);
   }
-  int items = 0;
-  for (int j = 0; j < k; ++j) {
-    const int2 c = chunk_range(j, cb, ce, nA);
-    items += (nA + kItemRows - 1) / kItemRows + (c.y - c.x + kItemCols - 1) / kItemCols;
+  // the totals: one addition per warp, exact in any order
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    items += __shfl_xor_sync(0xffffffffu, items, o);
+    places += __shfl_xor_sync(0xffffffffu, places, o);
   }
-  atomicAdd(nheavy, 1);
-  nitems[q] = items;
-  nextra[q] = (k + 1) * 3 * nA;
+  if ((threadIdx.x & 31) == 0) {
+    if (items) atomicAdd(wide, items);
+    if (places) atomicAdd(wide + 1, places);
+  }
 }
 
 __global__ void k_item_fill(int32_t nleaf, const int32_t *__restrict__ leaves, const int32_t *__restrict__ count,
@@ -634,27 +648,32 @@ int p2p_prepare(fmm_ctx *c) {
   AMFMM_TRY(ensure<int32_t>(c, c->p2p_itemOff, nleaf + 1));
   AMFMM_TRY(ensure<int32_t>(c, c->p2p_extraOff, nleaf + 1));
   int32_t *itemOff = ptr<int32_t>(c->p2p_itemOff), *extraOff = ptr<int32_t>(c->p2p_extraOff);
-  // totals: [32] columns, [33] work items, [34] extra partials, [35] heavy leaves (int32 slots)
+  // totals: [32] columns, [33] work items, [34] extra partials, [35] heavy leaves (int32 slots), and
+  // [13] work items, [14] extra partials in 64 bits
   int32_t *itot = ptr<int32_t>(c->totals) + 33, *etot = ptr<int32_t>(c->totals) + 34;
   int32_t *nheavy = ptr<int32_t>(c->totals) + 35;
+  unsigned long long *wide = ptr<unsigned long long>(c->totals) + 13;
   int32_t *icnt = cnt, *ecnt = ptr<int32_t>(c->flag);  // free scratch of >= nleaf + 1
   launch(c, k_item_counts, grid_for(nleaf, 256), 256, 0, nleaf, ptr<int32_t>(c->leaves), ptr<int32_t>(c->count),
-         colOff, ctot, heavy_warps(c), icnt, ecnt, nheavy);
+         colOff, ctot, heavy_warps(c), icnt, ecnt, nheavy, wide);
   AMFMM_TRY(launched(c, "p2p_item_counts"));
   AMFMM_TRY(exclusive_scan_i32(c, icnt, itemOff, nleaf + 1, itot));
   AMFMM_TRY(exclusive_scan_i32(c, ecnt, extraOff, nleaf + 1, etot));
-  int32_t *hc = reinterpret_cast<int32_t *>(h + 1);
+  int64_t *hw = h + 1;
+  int32_t *hc = reinterpret_cast<int32_t *>(h + 3);
   {
     // (totals[12], the slot total, is not written after its scan)
     const int64_t *ptot = ptr<int64_t>(c->totals) + 12;
-    HostRead rb[2];
+    HostRead rb[3];
     int nr = 0;
     if (K > 0) rb[nr++] = HostRead{h, ptot, sizeof(int64_t)};
+    rb[nr++] = HostRead{hw, wide, 2 * sizeof(int64_t)};
     rb[nr++] = HostRead{hc, ctot, 4 * sizeof(int32_t)};
     AMFMM_TRY(read_back(c, rb, nr));
     if (capturing(c)) {
       Expect e;
       if (K > 0) e.add64(ptot, static_cast<uint64_t>(h[0]));
+      for (int k = 0; k < 2; ++k) e.add64(wide + k, static_cast<uint64_t>(hw[k]));
       for (int k = 0; k < 4; ++k) e.add(ctot + k, static_cast<uint32_t>(hc[k]));
       AMFMM_TRY(graph_expect(c, e));
       st = c->stream;
@@ -667,6 +686,9 @@ int p2p_prepare(fmm_ctx *c) {
   // anything is sized or launched from these totals
   if (nslot / 3 + n + 1 > 0x7fffffffLL)
     return set_error(c, FMM_EUNSUPPORTED, "too many near-field slots (%lld values)", (long long)nslot);
+  if (hw[0] > 0x7fffffffLL || hw[1] > 0x7fffffffLL)
+    return set_error(c, FMM_EUNSUPPORTED, "too many near-field work items (%lld) or partial sums (%lld)",
+                     (long long)hw[0], (long long)hw[1]);
   c->sz.p2p_items = nitem;
   c->sz.p2p_heavy_leaves = hc[3];
   AMFMM_TRY(ensure<int4>(c, c->p2p_items, nitem + 1));

@@ -353,36 +353,50 @@ __global__ void __launch_bounds__(kWarps * 32, 4) k_p2p64(
 __device__ __forceinline__ int groups_of(int ne) { return (ne + kGroup) / kGroup; }
 
 // Work items and partial sums of every leaf; the near-field work, n_A n_B per
-// leaf pair plus n (n - 1) / 2 per leaf, and the total of the partial sums
-// (one atomic per warp each, integer: exact).
+// leaf pair plus n (n - 1) / 2 per leaf, and the totals of the work items and of
+// the partial sums in 64 bits (one atomic per block each, integer: exact).
+constexpr int kCountBlock = 256;
 __global__ void k_items64_count(int32_t nleaf, const int32_t *__restrict__ leaves, const int32_t *__restrict__ count,
                                 const int32_t *__restrict__ off, const uint32_t *__restrict__ partner,
                                 int32_t *__restrict__ nitems, int32_t *__restrict__ nextra,
-                                unsigned long long *__restrict__ work, unsigned long long *__restrict__ extot) {
+                                unsigned long long *__restrict__ work, unsigned long long *__restrict__ extot,
+                                unsigned long long *__restrict__ ittot) {
   pdl_wait();
   // one warp per leaf
+  __shared__ unsigned long long sum[3][kCountBlock / 32];
   const int q = static_cast<int>((blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x) >> 5);
-  const int l = threadIdx.x & 31;
-  if (q > nleaf) return;
-  if (q == nleaf) {  // closes the scans
-    if (l == 0) nitems[q] = nextra[q] = 0;
-    return;
-  }
-  const int L = leaves[q], a = count[L];
-  const int e0 = off[L], e1 = off[L + 1];
-  unsigned long long cols = 0;
-  for (int e = e0 + l; e < e1; e += 32) {
-    const int P = static_cast<int>(partner[e]);
-    if (P > L) cols += static_cast<unsigned long long>(count[P]);  // each pair once
-  }
+  const int l = threadIdx.x & 31, w = threadIdx.x >> 5;
+  unsigned long long pairs = 0, parts = 0, items = 0;
+  if (q == nleaf && l == 0) nitems[q] = nextra[q] = 0;  // closes the scans
+  if (q < nleaf) {
+    const int L = leaves[q], a = count[L];
+    const int e0 = off[L], e1 = off[L + 1];
+    unsigned long long cols = 0;
+    for (int e = e0 + l; e < e1; e += 32) {
+      const int P = static_cast<int>(partner[e]);
+      if (P > L) cols += static_cast<unsigned long long>(count[P]);  // each pair once
+    }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) cols += __shfl_xor_sync(0xffffffffu, cols, o);
-  if (l == 0) {
+    for (int o = 16; o > 0; o >>= 1) cols += __shfl_xor_sync(0xffffffffu, cols, o);
     const int g = groups_of(e1 - e0), nb = (a + kRows - 1) / kRows;
-    nitems[q] = g * nb;
-    nextra[q] = (g - 1) * 3 * a;
-    atomicAdd(work, a * cols + static_cast<unsigned long long>(a) * (a - 1) / 2);
-    if (g > 1) atomicAdd(extot, static_cast<unsigned long long>(g - 1) * 3 * a);
+    pairs = a * cols + static_cast<unsigned long long>(a) * (a - 1) / 2;
+    parts = static_cast<unsigned long long>(g - 1) * 3 * a;
+    items = static_cast<unsigned long long>(g) * nb;
+    if (l == 0) {
+      nitems[q] = static_cast<int32_t>(items);
+      nextra[q] = static_cast<int32_t>(parts);
+    }
+  }
+  if (l == 0) {
+    sum[0][w] = pairs;
+    sum[1][w] = parts;
+    sum[2][w] = items;
+  }
+  __syncthreads();
+  if (threadIdx.x < 3) {
+    unsigned long long v = 0;
+    for (int k = 0; k < kCountBlock / 32; ++k) v += sum[threadIdx.x][k];
+    if (v) atomicAdd(threadIdx.x == 0 ? work : threadIdx.x == 1 ? extot : ittot, v);
   }
 }
 
@@ -444,32 +458,31 @@ int p2p64_prepare(fmm_ctx *c) {
   // every leaf's partners, in the stable order of the pair list
   int32_t *off = ptr<int32_t>(c->p2p_offA);
   AMFMM_TRY(partner_lists(c, ptr<int2>(c->p2p), K, c->pkey, c->pval, off, &c->p2p_which));
-  // work items; totals: [33] items, [34] partial sums, stat: body pairs, [12] partial sums in 64 bits
+  // work items; totals: [33] items, [34] partial sums, stat: body pairs, [12] partial sums and [13] items in 64 bits
   int32_t *itot = ptr<int32_t>(c->totals) + 33, *etot = ptr<int32_t>(c->totals) + 34;
   unsigned long long *stat = ptr<unsigned long long>(c->totals) + 8;
-  unsigned long long *ext64 = ptr<unsigned long long>(c->totals) + 12;
+  unsigned long long *ext64 = ptr<unsigned long long>(c->totals) + 12, *it64 = ext64 + 1;
   int32_t *icnt = ptr<int32_t>(c->incl), *ecnt = ptr<int32_t>(c->flag);  // free scratch of >= nleaf + 1
   int32_t *itemOff = ptr<int32_t>(c->p2p_itemOff), *extraOff = ptr<int32_t>(c->p2p_extraOff);
-  launch(c, k_items64_count, grid_for(32 * (static_cast<int64_t>(nleaf) + 1), 256), 256, 0, nleaf,
+  launch(c, k_items64_count, grid_for(32 * (static_cast<int64_t>(nleaf) + 1), kCountBlock), kCountBlock, 0, nleaf,
          ptr<int32_t>(c->leaves), ptr<int32_t>(c->count), off, K > 0 ? ptr<uint32_t>(c->pval[c->p2p_which]) : nullptr,
-         icnt, ecnt, stat, ext64);
+         icnt, ecnt, stat, ext64, it64);
   AMFMM_TRY(launched(c, "p2p64_item_counts"));
   AMFMM_TRY(exclusive_scan_i32(c, icnt, itemOff, nleaf + 1, itot));
   AMFMM_TRY(exclusive_scan_i32(c, ecnt, extraOff, nleaf + 1, etot));
   int64_t *h = static_cast<int64_t *>(c->hpin);
-  int32_t *hc = reinterpret_cast<int32_t *>(h + 1);
-  const HostRead rb[2] = {{h, ext64, sizeof(int64_t)}, {hc, itot, sizeof(int32_t)}};
-  AMFMM_TRY(read_back(c, rb, 2));
+  const HostRead rb{h, ext64, 2 * sizeof(int64_t)};
+  AMFMM_TRY(read_back(c, &rb, 1));
   if (capturing(c)) {
     Expect e;
-    e.add64(ext64, static_cast<uint64_t>(h[0]));
-    e.add(itot, static_cast<uint32_t>(hc[0]));
+    for (int k = 0; k < 2; ++k) e.add64(ext64 + k, static_cast<uint64_t>(h[k]));
     AMFMM_TRY(graph_expect(c, e));
     st = c->stream;
   }
-  const int64_t nextra = h[0], nitem = hc[0];
-  if (nextra > 0x7fffffffLL)
-    return set_error(c, FMM_EUNSUPPORTED, "too many near-field partial sums (%lld)", (long long)nextra);
+  const int64_t nextra = h[0], nitem = h[1];
+  if (nextra > 0x7fffffffLL || nitem > 0x7fffffffLL)
+    return set_error(c, FMM_EUNSUPPORTED, "too many near-field work items (%lld) or partial sums (%lld)",
+                     (long long)nitem, (long long)nextra);
   c->sz.p2p_items = nitem;
   AMFMM_TRY(ensure<int4>(c, c->p2p_items, nitem + 1));
   AMFMM_TRY(ensure<double>(c, c->p2p_extra, nextra + 1));

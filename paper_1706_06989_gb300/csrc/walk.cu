@@ -363,7 +363,7 @@ __global__ void __launch_bounds__(kGenBlock, kGenBlocksPerSM) k_walk_gen(
 
 // One self pair per root; the generation records, zero but for the first
 // generation's inputs; and zero counters for the stages that follow (words of
-// `totals`: body pairs, scored pairs, FP64 near-field partials, heavy leaves,
+// `totals`: body pairs, scored pairs, the near field's 64-bit counts, heavy leaves,
 // the work queues).
 __global__ void k_roots_front(int32_t nsys, int4 *__restrict__ front, GenState *__restrict__ gs, int nrec,
                               int32_t *__restrict__ totals) {
@@ -374,7 +374,7 @@ __global__ void k_roots_front(int32_t nsys, int4 *__restrict__ front, GenState *
   int *words = reinterpret_cast<int *>(gs);
   for (int q = threadIdx.x; q < nrec * static_cast<int>(sizeof(GenState) / sizeof(int)); q += blockDim.x) words[q] = 0;
   const int q = threadIdx.x;
-  if (q == 16 || q == 17 || q == 20 || q == 21 || q == 24 || q == 25 || q == 35 || q == 40 || q == 41) totals[q] = 0;
+  if (q == 16 || q == 17 || q == 20 || q == 21 || (q >= 24 && q < 30) || q == 35 || q == 40 || q == 41) totals[q] = 0;
   __syncthreads();
   if (s == 0) gs[0].in = GenIn{nsys, 0, 0, 0};
 }
