@@ -40,8 +40,8 @@ __device__ __forceinline__ int i3(int i, int j, int k) {
 // children.  An FP64 instruction holds its pipe for 64 cycles whatever number
 // of lanes work, so on a small level those 58 are a chain of 2 us; there a
 // warp takes one child, a lane per coefficient, with a chain of 9.
-__global__ void k_l2l(int32_t c0, int32_t c1, const int32_t *__restrict__ parent,
-                      const double *__restrict__ Z, double *__restrict__ loc) {
+__global__ void k_l2l(int32_t c0, int32_t c1, const int32_t *parent,
+                      const double *Z, double *__restrict__ loc) {
   pdl_wait();
   const int c = c0 + blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= c1) return;
@@ -70,8 +70,8 @@ __global__ void k_l2l(int32_t c0, int32_t c1, const int32_t *__restrict__ parent
 constexpr int kL2LWarps = 4;
 
 __global__ void __launch_bounds__(kL2LWarps * 32) k_l2l_warp(int32_t c0, int32_t c1,
-                                                             const int32_t *__restrict__ parent,
-                                                             const double *__restrict__ Z, double *__restrict__ loc) {
+                                                             const int32_t *parent,
+                                                             const double *Z, double *__restrict__ loc) {
   pdl_wait();
   __shared__ double sp[kL2LWarps][kLocStride], sh[kL2LWarps][6];
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
@@ -103,10 +103,10 @@ __global__ void __launch_bounds__(kL2LWarps * 32) k_l2l_warp(int32_t c0, int32_t
 
 // (39 FP64 operations per body through the contraction with x / 2, 68 us at N =
 // 1M; 127 us with every product x_j x_k x_ijk formed on its own)
-__global__ void k_l2p(int64_t n, const int32_t *__restrict__ leaf_of, const double *__restrict__ Z,
-                      const double *__restrict__ loc, const double *__restrict__ X,
-                      const double *__restrict__ Y, const double *__restrict__ Zb,
-                      const double *__restrict__ near, double *__restrict__ acc) {
+__global__ void k_l2p(int64_t n, const int32_t *leaf_of, const double *Z,
+                      const double *loc, const double *X,
+                      const double *Y, const double *Zb,
+                      const double *near, double *__restrict__ acc) {
   pdl_wait();
   const int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (i >= n) return;
@@ -141,7 +141,7 @@ __global__ void k_l2p(int64_t n, const int32_t *__restrict__ leaf_of, const doub
   }
 }
 
-__global__ void k_unpermute(int64_t n, const int32_t *__restrict__ order, const double *__restrict__ acc,
+__global__ void k_unpermute(int64_t n, const int32_t *order, const double *acc,
                             double G, double *__restrict__ ax, double *__restrict__ ay,
                             double *__restrict__ az) {
   pdl_wait();

@@ -35,9 +35,9 @@ constexpr int kP2MRows = P + 1 + (P + 1) * (P + 2) / 2;
 
 template <int P>
 __global__ void __launch_bounds__(kWarps * 32) k_p2m(
-    int32_t nleaf, const int32_t *__restrict__ leaves, const int32_t *__restrict__ begin,
-    const int32_t *__restrict__ count, const double *__restrict__ X, const double *__restrict__ Y,
-    const double *__restrict__ Zb, const double *__restrict__ Mb, double *__restrict__ S, double *__restrict__ M,
+    int32_t nleaf, const int32_t *leaves, const int32_t *begin,
+    const int32_t *count, const double *X, const double *Y,
+    const double *Zb, const double *Mb, double *__restrict__ S, double *__restrict__ M,
     double *__restrict__ Z, double *__restrict__ invM, double *__restrict__ mom) {
   pdl_wait();
   constexpr int NM = mi_off(P + 1), kRounds = (NM + 31) / 32, kRows = kP2MRows<P>;
@@ -122,8 +122,8 @@ __global__ void __launch_bounds__(kWarps * 32) k_p2m(
 // side by side, their moments over a! shifted axis by axis, then added in octant
 // order.  Every warp takes the centre of mass for itself.
 template <int P>
-__global__ void __launch_bounds__(kWarps * 32) k_m2m(int32_t c0, const int32_t *__restrict__ first_child,
-                                                     const int32_t *__restrict__ nchild, double *__restrict__ S,
+__global__ void __launch_bounds__(kWarps * 32) k_m2m(int32_t c0, const int32_t *first_child,
+                                                     const int32_t *nchild, double *__restrict__ S,
                                                      double *__restrict__ M, double *__restrict__ Z,
                                                      double *__restrict__ invM, double *__restrict__ mom) {
   pdl_wait();
@@ -190,8 +190,8 @@ __global__ void __launch_bounds__(kWarps * 32) k_m2m(int32_t c0, const int32_t *
 // One warp per child, axis by axis.
 template <int P>
 __global__ void __launch_bounds__(kWarps * 32) k_l2l_general(int32_t c0, int32_t c1,
-                                                             const int32_t *__restrict__ parent,
-                                                             const double *__restrict__ Z, double *__restrict__ loc) {
+                                                             const int32_t *parent,
+                                                             const double *Z, double *__restrict__ loc) {
   pdl_wait();
   constexpr int NM = mi_off(P + 1), NL = NM - 1;
   __shared__ double buf_all[kWarps][2][NM], sf_all[kWarps][3][P + 1];
@@ -230,10 +230,10 @@ __global__ void __launch_bounds__(kWarps * 32) k_l2l_general(int32_t c0, int32_t
 }
 
 template <int P>
-__global__ void k_l2p_general(int64_t n, const int32_t *__restrict__ leaf_of, const double *__restrict__ Z,
-                              const double *__restrict__ loc, const double *__restrict__ X,
-                              const double *__restrict__ Y, const double *__restrict__ Zb,
-                              const double *__restrict__ near, double *__restrict__ acc) {
+__global__ void k_l2p_general(int64_t n, const int32_t *leaf_of, const double *Z,
+                              const double *loc, const double *X,
+                              const double *Y, const double *Zb,
+                              const double *near, double *__restrict__ acc) {
   pdl_wait();
   const int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (i >= n) return;

@@ -114,7 +114,7 @@ struct UnitDerivs {
 
 // moments folded onto the reduced indices, divided by b!
 template <int P>
-__global__ void __launch_bounds__(128) k_fold_moments(int32_t ncell, const double *__restrict__ mom,
+__global__ void __launch_bounds__(128) k_fold_moments(int32_t ncell, const double *mom,
                                                       double *__restrict__ out) {
   pdl_wait();
   constexpr int NM = mi_off(P + 1), NR = (P + 1) * (P + 1), NS = red_mom_stride(P);
@@ -142,10 +142,10 @@ __global__ void __launch_bounds__(128) k_fold_moments(int32_t ncell, const doubl
 }
 
 template <int P>
-__global__ void __launch_bounds__(128, 2) k_m2l_general(int64_t K, int variant, const int2 *__restrict__ pairs,
-                                                        const double *__restrict__ Z, const double *__restrict__ invM,
-                                                        const double *__restrict__ fold,
-                                                        const int32_t *__restrict__ pos, double *__restrict__ slots) {
+__global__ void __launch_bounds__(128, 2) k_m2l_general(int64_t K, int variant, const int2 *pairs,
+                                                        const double *Z, const double *invM,
+                                                        const double *fold,
+                                                        const int32_t *pos, double *__restrict__ slots) {
   pdl_wait();
   constexpr int NR = (P + 1) * (P + 1), NL = red_loc_stride(P), NS = red_mom_stride(P);
   const int64_t k = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
@@ -239,8 +239,8 @@ __global__ void __launch_bounds__(128, 2) k_m2l_general(int64_t K, int variant, 
 constexpr int kSumBlock = 128;
 
 template <int P>
-__global__ void __launch_bounds__(kSumBlock) k_reduce_general(const int32_t *__restrict__ off,
-                                                              const double *__restrict__ slots,
+__global__ void __launch_bounds__(kSumBlock) k_reduce_general(const int32_t *off,
+                                                              const double *slots,
                                                               double *__restrict__ loc) {
   pdl_wait();
   constexpr int NS = red_loc_stride(P), NR = (P + 1) * (P + 1) - 1, NL = mi_off(P + 1) - 1;

@@ -246,6 +246,12 @@ int launched(fmm_ctx *c, const char *what);
 // blocks come when the running ones have ended, not as soon as all have started
 // (an explicit trigger at the top): then they crowd on the SMs that are free
 // first (1.93 and 4.49 ms; 18.1 against 17.7 at 4M).
+// What a kernel reads may still be written while it is being set up.  It relies on
+// ordinary loads after the wait, which returns once the kernels before have ended
+// and what they wrote is visible.  So no pointer that such a kernel reads is
+// `const T *__restrict__`, which lets loads take the read-only path, defined for
+// data that is constant for the kernel's whole life, and move above the wait.  (The
+// times are within 0.2% of each other, at order 5 0.7% apart.)
 __device__ __forceinline__ void pdl_wait() { cudaGridDependencySynchronize(); }
 template <class... P, class... A>
 inline void launch(fmm_ctx *c, void (*kernel)(P...), dim3 grid, dim3 block, size_t shared, A &&...args) {

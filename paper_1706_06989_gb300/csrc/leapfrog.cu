@@ -15,8 +15,8 @@ namespace {
 
 constexpr int kBlock = 256;
 
-__global__ void k_kick(int64_t n, double h, const double *__restrict__ ax, const double *__restrict__ ay,
-                       const double *__restrict__ az, double *__restrict__ vx, double *__restrict__ vy,
+__global__ void k_kick(int64_t n, double h, const double *ax, const double *ay,
+                       const double *az, double *__restrict__ vx, double *__restrict__ vy,
                        double *__restrict__ vz) {
   pdl_wait();
   const int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
@@ -26,8 +26,8 @@ __global__ void k_kick(int64_t n, double h, const double *__restrict__ ax, const
   vz[i] += h * az[i];
 }
 
-__global__ void k_drift(int64_t n, double dt, const double *__restrict__ vx, const double *__restrict__ vy,
-                        const double *__restrict__ vz, double *__restrict__ x, double *__restrict__ y,
+__global__ void k_drift(int64_t n, double dt, const double *vx, const double *vy,
+                        const double *vz, double *__restrict__ x, double *__restrict__ y,
                         double *__restrict__ z) {
   pdl_wait();
   const int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
@@ -48,13 +48,13 @@ __device__ __forceinline__ void nadd(Comp &a, double v) {
 }
 
 // per-block compensated partials of P = sum m V and L = sum m X x V
-__global__ void __launch_bounds__(kBlock) k_momentum_partial(int64_t n, const double *__restrict__ x,
-                                                             const double *__restrict__ y,
-                                                             const double *__restrict__ z,
-                                                             const double *__restrict__ vx,
-                                                             const double *__restrict__ vy,
-                                                             const double *__restrict__ vz,
-                                                             const double *__restrict__ m,
+__global__ void __launch_bounds__(kBlock) k_momentum_partial(int64_t n, const double *x,
+                                                             const double *y,
+                                                             const double *z,
+                                                             const double *vx,
+                                                             const double *vy,
+                                                             const double *vz,
+                                                             const double *m,
                                                              double *__restrict__ part) {
   pdl_wait();
   Comp v[6];
@@ -90,7 +90,7 @@ __global__ void __launch_bounds__(kBlock) k_momentum_partial(int64_t n, const do
   }
 }
 
-__global__ void k_momentum_final(int nb, const double *__restrict__ part, double *__restrict__ out) {
+__global__ void k_momentum_final(int nb, const double *part, double *__restrict__ out) {
   pdl_wait();
   if (threadIdx.x >= 6 || blockIdx.x != 0) return;
   const int k = threadIdx.x;

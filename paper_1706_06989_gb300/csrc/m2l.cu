@@ -285,11 +285,11 @@ __device__ __forceinline__ void m2l_slot_tf(const double r[3], double MA, double
 // octupole per unit mass (10), trace-free where the slot form takes them so
 // (k_qoh).
 template <int VARIANT, bool TF>
-__global__ void __launch_bounds__(kBlock) k_m2l64(int64_t K, const int2 *__restrict__ pairs,
-                                                   const double *__restrict__ Z,
-                                                   const double *__restrict__ M,
-                                                   const double *__restrict__ qoh,
-                                                   const int32_t *__restrict__ pos, double eps2,
+__global__ void __launch_bounds__(kBlock) k_m2l64(int64_t K, const int2 *pairs,
+                                                   const double *Z,
+                                                   const double *M,
+                                                   const double *qoh,
+                                                   const int32_t *pos, double eps2,
                                                    double *__restrict__ slots) {
   pdl_wait();
   constexpr int kSlot = TF ? kSlotTF : kSlot64;
@@ -475,9 +475,9 @@ __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
 // TF: records of kCell32TF floats with trace-free moments (m2l_one_tf),
 // else kCell32 floats with the raw ones.
 template <int VARIANT, bool TF>
-__global__ void __launch_bounds__(kGatherWarps * 32) k_m2l32_gather(int32_t ncell, const int32_t *__restrict__ off,
-                                                                    const uint32_t *__restrict__ partner,
-                                                                    const float *__restrict__ cell32,
+__global__ void __launch_bounds__(kGatherWarps * 32) k_m2l32_gather(int32_t ncell, const int32_t *off,
+                                                                    const uint32_t *partner,
+                                                                    const float *cell32,
                                                                     double *__restrict__ loc, float eps2,
                                                                     int *__restrict__ queue) {
   pdl_wait();
@@ -560,7 +560,7 @@ __global__ void __launch_bounds__(kGatherWarps * 32) k_m2l32_gather(int32_t ncel
 // per unit mass Oh = O / M (10; xxx xxy xxz xyy xyz xzz yyy yyz yzz zzz).
 // tf_q: Q - (tr Q / 3) I; tf_o: Oh - (1/5)(d_ij t_k + d_ik t_j + d_jk t_i),
 // t_i = Oh_ijj (both trace-free).
-__global__ void k_qoh(int32_t ncell, const double *__restrict__ invM, const double *__restrict__ mom, int tf_q,
+__global__ void k_qoh(int32_t ncell, const double *invM, const double *mom, int tf_q,
                       int tf_o, double *__restrict__ qoh) {
   pdl_wait();
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
@@ -599,8 +599,8 @@ __global__ void k_qoh(int32_t ncell, const double *__restrict__ invM, const doub
 }
 
 // FP32 copy of the cell data for the mixed form
-__global__ void k_cell32(int32_t ncell, const double *__restrict__ Z, const double *__restrict__ M,
-                         const double *__restrict__ invM, const double *__restrict__ mom,
+__global__ void k_cell32(int32_t ncell, const double *Z, const double *M,
+                         const double *invM, const double *mom,
                          float *__restrict__ cell32) {
   pdl_wait();
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
@@ -623,8 +623,8 @@ __global__ void k_cell32(int32_t ncell, const double *__restrict__ Z, const doub
 // The same with trace-free moments, kCell32TF floats: Z hi (3), Z lo (3), M,
 // Q - tr Q / 3 I (xx xy xz yy yz), Oh = O / M less its trace part (xxx xxy
 // xxz xyy xyz yyy yyz), one pad; the traces are removed in FP64.
-__global__ void k_cell32_tf(int32_t ncell, const double *__restrict__ Z, const double *__restrict__ M,
-                            const double *__restrict__ invM, const double *__restrict__ mom,
+__global__ void k_cell32_tf(int32_t ncell, const double *Z, const double *M,
+                            const double *invM, const double *mom,
                             float *__restrict__ cell32) {
   pdl_wait();
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
@@ -662,9 +662,9 @@ __global__ void k_cell32_tf(int32_t ncell, const double *__restrict__ Z, const d
 
 // The two order-3 TC locals of given pairs, [k][side][20] (labels of the
 // learned selector)
-__global__ void k_pair_locals(int64_t K, const int2 *__restrict__ pairs, const double *__restrict__ Z,
-                              const double *__restrict__ M, const double *__restrict__ invM,
-                              const double *__restrict__ mom, double *__restrict__ out) {
+__global__ void k_pair_locals(int64_t K, const int2 *pairs, const double *Z,
+                              const double *M, const double *invM,
+                              const double *mom, double *__restrict__ out) {
   pdl_wait();
   const int64_t k = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (k >= K) return;
@@ -693,7 +693,7 @@ __global__ void k_pair_locals(int64_t K, const int2 *__restrict__ pairs, const d
 // position of the next cell): every position s starts the cells
 // (key[s-1], key[s]], and the last entry closes the cells after it.
 // Four positions per thread, read as one 16-byte load (key is 16-byte aligned).
-__global__ void k_segment_offsets(int64_t E, int32_t ncell, const uint32_t *__restrict__ key,
+__global__ void k_segment_offsets(int64_t E, int32_t ncell, const uint32_t *key,
                                   int32_t *__restrict__ off) {
   pdl_wait();
   const int64_t s0 = 4 * (blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x);
@@ -720,7 +720,7 @@ __global__ void k_segment_offsets(int64_t E, int32_t ncell, const uint32_t *__re
   }
 }
 
-__global__ void k_inverse(int64_t E, const uint32_t *__restrict__ sval, int32_t *__restrict__ pos) {
+__global__ void k_inverse(int64_t E, const uint32_t *sval, int32_t *__restrict__ pos) {
   pdl_wait();
   const int64_t s = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (s < E) pos[sval[s]] = static_cast<int32_t>(s);
@@ -767,8 +767,8 @@ constexpr bool red_plan_ok() {
 static_assert(red_plan_ok(), "one shuffle per phase must carry every scale factor");
 static_assert((kRedPhases * 32) % kSlot64 == 0, "a period of loads covers whole slots");
 
-__global__ void __launch_bounds__(kRedWarps * 32) k_m2l_reduce(int32_t ncell, const int32_t *__restrict__ off,
-                                                               const double *__restrict__ slots,
+__global__ void __launch_bounds__(kRedWarps * 32) k_m2l_reduce(int32_t ncell, const int32_t *off,
+                                                               const double *slots,
                                                                double *__restrict__ loc) {
   pdl_wait();
   __shared__ double part[kRedWarps][kRedPhases][32];
@@ -796,7 +796,7 @@ __global__ void __launch_bounds__(kRedWarps * 32) k_m2l_reduce(int32_t ncell, co
 #pragma unroll
       for (int u = 0; u < kRedPhases; ++u) {
         const int64_t e = b + l + 32 * (h * kRedPhases + u);
-        v[h][u] = e < e1 ? __ldg(&slots[e]) : 0.0;
+        v[h][u] = e < e1 ? slots[e] : 0.0;
       }
 #pragma unroll
     for (int h = 0; h < kRedPeriods; ++h)
@@ -833,8 +833,8 @@ __global__ void __launch_bounds__(kRedWarps * 32) k_m2l_reduce(int32_t ncell, co
 // needs, one FMA each; the FP64 pipe bounds it (50M slots of N = 1M: 1.38 ms
 // against 2.18 with 24 values on 32 lanes).  The halves' sums are added, and the
 // trace relations give the components that the slots leave out.
-__global__ void __launch_bounds__(kRedWarps * 32) k_m2l_reduce_tf(int32_t ncell, const int32_t *__restrict__ off,
-                                                                  const double *__restrict__ slots,
+__global__ void __launch_bounds__(kRedWarps * 32) k_m2l_reduce_tf(int32_t ncell, const int32_t *off,
+                                                                  const double *slots,
                                                                   double *__restrict__ loc) {
   pdl_wait();
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31, q = l & 15;

@@ -149,8 +149,8 @@ __device__ __forceinline__ bool is_heavy(int ncol, int total, int warps) {
   return ncol > max(kHeavyMin, total / (3 * warps));
 }
 
-__global__ void k_item_counts(int32_t nleaf, const int32_t *__restrict__ leaves, const int32_t *__restrict__ count,
-                              const int32_t *__restrict__ colOff, const int32_t *__restrict__ total, int warps,
+__global__ void k_item_counts(int32_t nleaf, const int32_t *leaves, const int32_t *count,
+                              const int32_t *colOff, const int32_t *total, int warps,
                               int32_t *__restrict__ nitems, int32_t *__restrict__ nextra, int *__restrict__ nheavy,
                               unsigned long long *__restrict__ wide) {
   pdl_wait();
@@ -186,9 +186,9 @@ __global__ void k_item_counts(int32_t nleaf, const int32_t *__restrict__ leaves,
   }
 }
 
-__global__ void k_item_fill(int32_t nleaf, const int32_t *__restrict__ leaves, const int32_t *__restrict__ count,
-                            const int32_t *__restrict__ colOff, const int32_t *__restrict__ total, int warps,
-                            const int32_t *__restrict__ itemOff, const int32_t *__restrict__ extraOff,
+__global__ void k_item_fill(int32_t nleaf, const int32_t *leaves, const int32_t *count,
+                            const int32_t *colOff, const int32_t *total, int warps,
+                            const int32_t *itemOff, const int32_t *extraOff,
                             int4 *__restrict__ items, int32_t *__restrict__ item_rows) {
   pdl_wait();
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
@@ -218,10 +218,10 @@ __global__ void k_item_fill(int32_t nleaf, const int32_t *__restrict__ leaves, c
 // A leaf whose column stream was split adds the A-side partials of its later
 // chunks, in chunk order, once every chunk is done (one thread per body); a
 // heavy leaf its self sums and those of all chunks.
-__global__ void k_p2p_chunks(int32_t nleaf, int64_t n, const int32_t *__restrict__ leaves,
-                             const int32_t *__restrict__ begin, const int32_t *__restrict__ count,
-                             const int32_t *__restrict__ colOff, const int32_t *__restrict__ total, int warps,
-                             const int32_t *__restrict__ extraOff, const double *__restrict__ extra,
+__global__ void k_p2p_chunks(int32_t nleaf, int64_t n, const int32_t *leaves,
+                             const int32_t *begin, const int32_t *count,
+                             const int32_t *colOff, const int32_t *total, int warps,
+                             const int32_t *extraOff, const double *extra,
                              double *__restrict__ near) {
   pdl_wait();
   const int q = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -254,10 +254,10 @@ __global__ void k_p2p_chunks(int32_t nleaf, int64_t n, const int32_t *__restrict
 // HEAVY: there are items of heavy leaves (the test for them costs 1% otherwise).
 template <int ROWS, bool HEAVY>
 __global__ void __launch_bounds__(kWarps * 32) k_p2p(
-    int32_t nitem, int64_t n, const int4 *__restrict__ items, const int32_t *__restrict__ item_rows,
-    const int32_t *__restrict__ begin, const int32_t *__restrict__ count, const double *__restrict__ Zc, const int2 *__restrict__ cols,
+    int32_t nitem, int64_t n, const int4 *items, const int32_t *item_rows,
+    const int32_t *begin, const int32_t *count, const double *Zc, const int2 *cols,
     double *__restrict__ near, double *__restrict__ extra, float *__restrict__ slots,
-    const BodyF *__restrict__ bodyf, float eps2, int *__restrict__ queue) {
+    const BodyF *bodyf, float eps2, int *__restrict__ queue) {
   pdl_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
@@ -408,9 +408,9 @@ __global__ void __launch_bounds__(kWarps * 32) k_p2p(
 
 // Each body adds, in sorted order, the partials that the pairs in which its
 // leaf is the larger id left for it.
-__global__ void k_p2p_reduce(int64_t n, const int32_t *__restrict__ leaf_of, const int32_t *__restrict__ begin,
-                             const int32_t *__restrict__ offB, const int64_t *__restrict__ poff,
-                             const float *__restrict__ slots, double *__restrict__ near) {
+__global__ void k_p2p_reduce(int64_t n, const int32_t *leaf_of, const int32_t *begin,
+                             const int32_t *offB, const int64_t *poff,
+                             const float *slots, double *__restrict__ near) {
   pdl_wait();
   const int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (i >= n) return;
@@ -446,8 +446,8 @@ __global__ void k_p2p_reduce(int64_t n, const int32_t *__restrict__ leaf_of, con
 
 // the sorted (A, B) as pairs, and every pair's column count n_B (and a zero for
 // the total of the scan)
-__global__ void k_sorted_pairs(int64_t K, const uint32_t *__restrict__ key, const uint32_t *__restrict__ val,
-                               const int32_t *__restrict__ count, int2 *__restrict__ out, int32_t *__restrict__ nb) {
+__global__ void k_sorted_pairs(int64_t K, const uint32_t *key, const uint32_t *val,
+                               const int32_t *count, int2 *__restrict__ out, int32_t *__restrict__ nb) {
   pdl_wait();
   const int64_t s = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (s >= K) return;
@@ -458,8 +458,8 @@ __global__ void k_sorted_pairs(int64_t K, const uint32_t *__restrict__ key, cons
 }
 
 // pos[s] = CSR position of sorted pair s on its B side; len[e] = 3 n_B
-__global__ void k_b_positions(int64_t K, const uint32_t *__restrict__ key, const uint32_t *__restrict__ sval,
-                              const int32_t *__restrict__ count, int32_t *__restrict__ pos,
+__global__ void k_b_positions(int64_t K, const uint32_t *key, const uint32_t *sval,
+                              const int32_t *count, int32_t *__restrict__ pos,
                               int64_t *__restrict__ len) {
   pdl_wait();
   const int64_t e = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
@@ -481,8 +481,8 @@ int bits_for(int64_t v) {
 // pre of the partners' sizes over the A-sorted pairs, the bodies of its
 // partners.  Also the near-field work: n_A n_B per leaf pair plus
 // n (n - 1) / 2 per leaf (one atomic per warp, integer: exact).
-__global__ void k_leaf_cols(int32_t nleaf, const int32_t *__restrict__ leaves, const int32_t *__restrict__ count,
-                            const int32_t *__restrict__ offA, const int32_t *__restrict__ pre,
+__global__ void k_leaf_cols(int32_t nleaf, const int32_t *leaves, const int32_t *count,
+                            const int32_t *offA, const int32_t *pre,
                             int32_t *__restrict__ ccount, unsigned long long *__restrict__ work) {
   pdl_wait();
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
@@ -499,8 +499,8 @@ __global__ void k_leaf_cols(int32_t nleaf, const int32_t *__restrict__ leaves, c
   if ((threadIdx.x & 31) == 0 && v) atomicAdd(work, v);
 }
 
-__global__ void k_cols_self(int32_t nleaf, const int32_t *__restrict__ leaves, const int32_t *__restrict__ begin,
-                            const int32_t *__restrict__ count, const int32_t *__restrict__ colOff,
+__global__ void k_cols_self(int32_t nleaf, const int32_t *leaves, const int32_t *begin,
+                            const int32_t *count, const int32_t *colOff,
                             int2 *__restrict__ cols) {
   pdl_wait();
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
@@ -510,10 +510,10 @@ __global__ void k_cols_self(int32_t nleaf, const int32_t *__restrict__ leaves, c
   for (int t = 0; t < count[L]; ++t) cols[c0 + t] = make_int2(b + t, -1);
 }
 
-__global__ void k_cols_pairs(int64_t K, const int2 *__restrict__ pairs, const int32_t *__restrict__ begin,
-                             const int32_t *__restrict__ count, const int32_t *__restrict__ colOff,
-                             const int32_t *__restrict__ offA, const int32_t *__restrict__ pre,
-                             const int32_t *__restrict__ pos, const int64_t *__restrict__ poff,
+__global__ void k_cols_pairs(int64_t K, const int2 *pairs, const int32_t *begin,
+                             const int32_t *count, const int32_t *colOff,
+                             const int32_t *offA, const int32_t *pre,
+                             const int32_t *pos, const int64_t *poff,
                              int2 *__restrict__ cols) {
   pdl_wait();
   // A warp writes the runs of its 32 pairs together: entry j of the warp's

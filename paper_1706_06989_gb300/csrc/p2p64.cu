@@ -52,10 +52,10 @@ struct Rec {
   uint4 a, b, c;  // x0 x1 x2 y0 | y1 y2 z0 z1 | z2 m1 m0 (mass exponent, extent exponent << 16)
 };
 
-__global__ void k_body_fixed(int64_t n, const double *__restrict__ X, const double *__restrict__ Y,
-                             const double *__restrict__ Zb, const double *__restrict__ Mb,
-                             const double *__restrict__ box, const int32_t *__restrict__ order,
-                             const int32_t *__restrict__ sysid, Rec *__restrict__ rec) {
+__global__ void k_body_fixed(int64_t n, const double *X, const double *Y,
+                             const double *Zb, const double *Mb,
+                             const double *box, const int32_t *order,
+                             const int32_t *sysid, Rec *__restrict__ rec) {
   pdl_wait();
   const int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (i >= n) return;
@@ -122,10 +122,10 @@ __device__ __forceinline__ void flush(fix::Acc &acc, int &terms, WarpSmem &sm, i
 // SOFT: softening added to r^2 in fixed point.
 template <bool SOFT>
 __global__ void __launch_bounds__(kWarps * 32, 4) k_p2p64(
-    int32_t nitem, int64_t n, const int4 *__restrict__ items, const int32_t *__restrict__ begin,
-    const int32_t *__restrict__ count, const int32_t *__restrict__ off, const uint32_t *__restrict__ partner,
-    const Rec *__restrict__ rec, const double *__restrict__ X,
-    const double *__restrict__ Y, const double *__restrict__ Zb, const double *__restrict__ Mb, double eps2, double *__restrict__ near,
+    int32_t nitem, int64_t n, const int4 *items, const int32_t *begin,
+    const int32_t *count, const int32_t *off, const uint32_t *partner,
+    const Rec *rec, const double *X,
+    const double *Y, const double *Zb, const double *Mb, double eps2, double *__restrict__ near,
     double *__restrict__ extra, int *__restrict__ queue) {
   pdl_wait();
   __shared__ WarpSmem smem[kWarps];
@@ -356,8 +356,8 @@ __device__ __forceinline__ int groups_of(int ne) { return (ne + kGroup) / kGroup
 // leaf pair plus n (n - 1) / 2 per leaf, and the totals of the work items and of
 // the partial sums in 64 bits (one atomic per block each, integer: exact).
 constexpr int kCountBlock = 256;
-__global__ void k_items64_count(int32_t nleaf, const int32_t *__restrict__ leaves, const int32_t *__restrict__ count,
-                                const int32_t *__restrict__ off, const uint32_t *__restrict__ partner,
+__global__ void k_items64_count(int32_t nleaf, const int32_t *leaves, const int32_t *count,
+                                const int32_t *off, const uint32_t *partner,
                                 int32_t *__restrict__ nitems, int32_t *__restrict__ nextra,
                                 unsigned long long *__restrict__ work, unsigned long long *__restrict__ extot,
                                 unsigned long long *__restrict__ ittot) {
@@ -400,9 +400,9 @@ __global__ void k_items64_count(int32_t nleaf, const int32_t *__restrict__ leave
   }
 }
 
-__global__ void k_items64_fill(int32_t nleaf, const int32_t *__restrict__ leaves, const int32_t *__restrict__ count,
-                               const int32_t *__restrict__ off, const int32_t *__restrict__ itemOff,
-                               const int32_t *__restrict__ extraOff, int4 *__restrict__ items) {
+__global__ void k_items64_fill(int32_t nleaf, const int32_t *leaves, const int32_t *count,
+                               const int32_t *off, const int32_t *itemOff,
+                               const int32_t *extraOff, int4 *__restrict__ items) {
   pdl_wait();
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= nleaf) return;
@@ -416,10 +416,10 @@ __global__ void k_items64_fill(int32_t nleaf, const int32_t *__restrict__ leaves
 
 // Adds the partial sums of a leaf's later entry groups, in group order (one
 // warp per leaf).
-__global__ void k_p2p64_groups(int32_t nleaf, int64_t n, const int32_t *__restrict__ leaves,
-                               const int32_t *__restrict__ begin, const int32_t *__restrict__ count,
-                               const int32_t *__restrict__ off, const int32_t *__restrict__ extraOff,
-                               const double *__restrict__ extra, double *__restrict__ near) {
+__global__ void k_p2p64_groups(int32_t nleaf, int64_t n, const int32_t *leaves,
+                               const int32_t *begin, const int32_t *count,
+                               const int32_t *off, const int32_t *extraOff,
+                               const double *extra, double *__restrict__ near) {
   pdl_wait();
   const int q = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int l = threadIdx.x & 31;

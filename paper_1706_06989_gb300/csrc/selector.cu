@@ -54,8 +54,8 @@ namespace {
 // this GPU, and the features only need BF16 accuracy).
 __device__ __forceinline__ float lg(float v) { return __log2f(v) * 0.30102999566f; }
 
-__global__ void k_cell_features(int32_t ncell, const double *__restrict__ Rmax, const double *__restrict__ M,
-                                const double *__restrict__ mom, int mstride, const int32_t *__restrict__ count,
+__global__ void k_cell_features(int32_t ncell, const double *Rmax, const double *M,
+                                const double *mom, int mstride, const int32_t *count,
                                 float4 *__restrict__ cf) {
   pdl_wait();
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
@@ -74,8 +74,8 @@ __global__ void k_cell_features(int32_t ncell, const double *__restrict__ Rmax, 
 // N_A + N_B, with the pair ordered by R_max (FP32, descending), then by id,
 // so that (A, B) and (B, A) give the same features and decision.  |r| comes
 // from the hi + lo float centres.
-__device__ __forceinline__ void pair_features(int A, int B, const CellF *__restrict__ zf,
-                                              const float4 *__restrict__ cf, float f[kF]) {
+__device__ __forceinline__ void pair_features(int A, int B, const CellF *zf,
+                                              const float4 *cf, float f[kF]) {
   CellF a = zf[A], b = zf[B];
   if (b.h.w > a.h.w || (b.h.w == a.h.w && B < A)) {
     const int t = A;
@@ -100,8 +100,8 @@ __device__ __forceinline__ void pair_features(int A, int B, const CellF *__restr
   f[7] = lg(fa.w + fb.w);
 }
 
-__global__ void k_features(int64_t K, const int2 *__restrict__ pairs, const CellF *__restrict__ zf,
-                           const float4 *__restrict__ cf, float *__restrict__ feat) {
+__global__ void k_features(int64_t K, const int2 *pairs, const CellF *zf,
+                           const float4 *cf, float *__restrict__ feat) {
   pdl_wait();
   const int64_t k = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (k >= K) return;
@@ -118,8 +118,8 @@ __global__ void k_features(int64_t K, const int2 *__restrict__ pairs, const Cell
 // Stored as log10 |a|.
 constexpr int kFieldTile = 256;
 
-__global__ void __launch_bounds__(kFieldTile) k_field_estimate(int32_t ncell, const CellF *__restrict__ zf,
-                                                              const double *__restrict__ M, int32_t k0,
+__global__ void __launch_bounds__(kFieldTile) k_field_estimate(int32_t ncell, const CellF *zf,
+                                                              const double *M, int32_t k0,
                                                               int32_t k1, float *__restrict__ lga) {
   pdl_wait();
   __shared__ float4 src[kFieldTile];
@@ -170,11 +170,11 @@ constexpr int kLabelTargets = 128;
 __device__ __forceinline__ int label_target(int t, int n) {
   return n <= kLabelTargets ? t : static_cast<int>((static_cast<int64_t>(t) * n) / kLabelTargets);
 }
-__global__ void __launch_bounds__(128) k_labels(int64_t K, const int2 *__restrict__ pairs,
-                                                const int32_t *__restrict__ begin, const int32_t *__restrict__ count,
-                                                const double *__restrict__ X, const double *__restrict__ Y,
-                                                const double *__restrict__ Zb, const double *__restrict__ Mb,
-                                                const double *__restrict__ Z, const double *__restrict__ loc_pair,
+__global__ void __launch_bounds__(128) k_labels(int64_t K, const int2 *pairs,
+                                                const int32_t *begin, const int32_t *count,
+                                                const double *X, const double *Y,
+                                                const double *Zb, const double *Mb,
+                                                const double *Z, const double *loc_pair,
                                                 float *__restrict__ label) {
   pdl_wait();
   const int64_t k = blockIdx.x;
@@ -284,7 +284,7 @@ struct NetSmem {
   float b1[kH], b2[kH], b3[kH], w4[kH], b4, mean[kF], scale[kF];
 };
 
-__device__ void load_net(NetSmem &s, const float *__restrict__ p) {
+__device__ void load_net(NetSmem &s, const float *p) {
   for (int q = threadIdx.x; q < kH * 16; q += blockDim.x) {
     const int o = q / 16, i = q % 16;
     s.W1[o][i] = __float2bfloat16_rn(i < kF ? p[kOffW1 + o * kF + i] : 0.f);
@@ -476,8 +476,8 @@ __device__ __forceinline__ void infer16(const NetSmem &s, const NetRegs &r, cons
 }
 
 // inference over K samples of raw features
-__global__ void __launch_bounds__(128) k_mlp_infer(int64_t K, const float *__restrict__ params,
-                                                   const float *__restrict__ feat, float *__restrict__ out) {
+__global__ void __launch_bounds__(128) k_mlp_infer(int64_t K, const float *params,
+                                                   const float *feat, float *__restrict__ out) {
   pdl_wait();
   __shared__ NetSmem s;
   __shared__ float xs[4][16][kF];
@@ -510,8 +510,8 @@ struct TrainSmem {
   float hin[64][kH];  // the BF16-rounded input of the current layer (as FP32)
 };
 
-__global__ void __launch_bounds__(128) k_mlp_grad(int64_t B, const float *__restrict__ params,
-                                                  const float *__restrict__ feat, const float *__restrict__ lab,
+__global__ void __launch_bounds__(128) k_mlp_grad(int64_t B, const float *params,
+                                                  const float *feat, const float *lab,
                                                   float *__restrict__ part, float *__restrict__ loss_part) {
   pdl_wait();
   extern __shared__ __align__(16) unsigned char raw[];
@@ -652,7 +652,7 @@ __global__ void __launch_bounds__(128) k_mlp_grad(int64_t B, const float *__rest
 }
 
 // gradient = sum of the block partials in block order; loss likewise
-__global__ void k_grad_reduce(int nblk, const float *__restrict__ part, const float *__restrict__ loss_part,
+__global__ void k_grad_reduce(int nblk, const float *part, const float *loss_part,
                               int64_t B, float *__restrict__ grad, float *__restrict__ loss) {
   pdl_wait();
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
@@ -669,7 +669,7 @@ __global__ void k_grad_reduce(int nblk, const float *__restrict__ part, const fl
 }
 
 __global__ void k_adam(float *__restrict__ p, float *__restrict__ m, float *__restrict__ v,
-                       const float *__restrict__ g, float lr, float b1, float b2, float eps, int step) {
+                       const float *g, float lr, float b1, float b2, float eps, int step) {
   pdl_wait();
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= kNWeights) return;
@@ -695,9 +695,9 @@ __global__ void k_adam(float *__restrict__ p, float *__restrict__ m, float *__re
 // list's order varies from run to run, but a pair's score depends only on the
 // pair (the rows of a tensor-core product are independent), so the walk does
 // not.  k_walk_scores then runs the network on the candidates only.
-__global__ void k_band_select(const long long *__restrict__ nf_dev, int64_t cap, const int4 *__restrict__ front,
-                              const double4_32a *__restrict__ zr, const CellF *__restrict__ zf,
-                              const int32_t *__restrict__ count, int64_t min_work, double th_lo, double th_hi,
+__global__ void k_band_select(const long long *nf_dev, int64_t cap, const int4 *front,
+                              const double4_32a *zr, const CellF *zf,
+                              const int32_t *count, int64_t min_work, double th_lo, double th_hi,
                               float *__restrict__ score, int32_t *__restrict__ cand, unsigned *__restrict__ ncand) {
   pdl_wait();
   // the frontier size comes from the walk's generation record; a frontier
@@ -745,12 +745,12 @@ __global__ void k_band_select(const long long *__restrict__ nf_dev, int64_t cap,
 // side A's error is at most 10^pred M_B/r^2, side B's 10^pred M_A/r^2, and
 //   score = pred + log10 max(M_B / (r^2 |a_A|), M_A / (r^2 |a_B|)),
 // compared by the walk with log10 of the relative target.
-__global__ void __launch_bounds__(128) k_walk_scores(const int4 *__restrict__ front,
-                                                     const int32_t *__restrict__ cand,
-                                                     const unsigned *__restrict__ ncand,
-                                                     const float *__restrict__ params,
-                                                     const CellF *__restrict__ zf, const float4 *__restrict__ cf,
-                                                     const float *__restrict__ lga, float *__restrict__ score,
+__global__ void __launch_bounds__(128) k_walk_scores(const int4 *front,
+                                                     const int32_t *cand,
+                                                     const unsigned *ncand,
+                                                     const float *params,
+                                                     const CellF *zf, const float4 *cf,
+                                                     const float *lga, float *__restrict__ score,
                                                      unsigned long long *__restrict__ scored) {
   pdl_wait();
   __shared__ NetSmem s;
@@ -797,8 +797,8 @@ __global__ void __launch_bounds__(128) k_walk_scores(const int4 *__restrict__ fr
   }
 }
 
-__global__ void k_gather_batch(int64_t B, const int64_t *__restrict__ perm, int64_t start, int64_t n,
-                               const float *__restrict__ X, const float *__restrict__ y, float *__restrict__ xb,
+__global__ void k_gather_batch(int64_t B, const int64_t *perm, int64_t start, int64_t n,
+                               const float *X, const float *y, float *__restrict__ xb,
                                float *__restrict__ yb) {
   pdl_wait();
   const int64_t b = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;

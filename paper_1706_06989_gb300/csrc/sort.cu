@@ -60,7 +60,7 @@ __device__ __forceinline__ T block_exclusive(T v, T *excl) {
 }
 
 template <class T>
-__global__ void k_tile_reduce(const T *__restrict__ in, int64_t n, T *__restrict__ sums) {
+__global__ void k_tile_reduce(const T *in, int64_t n, T *__restrict__ sums) {
   pdl_wait();
   const int64_t base = static_cast<int64_t>(blockIdx.x) * kScanTile;
   T s = vzero<T>();
@@ -79,9 +79,9 @@ __global__ void k_tile_reduce(const T *__restrict__ in, int64_t n, T *__restrict
 // (integer addition: exact in any order), else zero.  The last tile writes
 // the grand total.
 template <class T>
-__global__ void k_tile_scan(const T *__restrict__ in, T *__restrict__ out, int64_t n,
-                            const T *__restrict__ offs, T *__restrict__ total,
-                            const T *__restrict__ sums) {
+__global__ void k_tile_scan(const T *in, T *__restrict__ out, int64_t n,
+                            const T *offs, T *__restrict__ total,
+                            const T *sums) {
   pdl_wait();
   const int64_t base = static_cast<int64_t>(blockIdx.x) * kScanTile;
   T pre = vzero<T>();
@@ -199,7 +199,7 @@ enum SortSource {
   kSecondSide = 4  // key: pairs[i].y, value i
 };
 template <class K>
-__device__ __forceinline__ K sort_key(const K *__restrict__ key, int src, int64_t i) {
+__device__ __forceinline__ K sort_key(const K *key, int src, int64_t i) {
   return src == kFirstSide ? key[2 * i] : src == kSecondSide ? key[2 * i + 1] : key[i];
 }
 
@@ -224,7 +224,7 @@ constexpr int kHistLoads = 8;  // keys in flight per thread
 
 // Adds the digits of keys [i0, i1) to cnt[p * R + digit], p < passes.
 template <class K, int R>
-__device__ __forceinline__ void count_digits(const K *__restrict__ key, int src, int64_t i0, int64_t i1, int shift0,
+__device__ __forceinline__ void count_digits(const K *key, int src, int64_t i0, int64_t i1, int shift0,
                                              int passes, int width, int *cnt) {
   const int t = threadIdx.x, lane = t & 31;
   const unsigned dmask = (1u << width) - 1;
@@ -255,7 +255,7 @@ __device__ __forceinline__ void count_digits(const K *__restrict__ key, int src,
 
 // One wave: digits of all passes.
 template <class K, int R>
-__global__ void __launch_bounds__(kHistBlock) k_sort_hist(const K *__restrict__ key, int src, int64_t n, int passes,
+__global__ void __launch_bounds__(kHistBlock) k_sort_hist(const K *key, int src, int64_t n, int passes,
                                                           int width, SortCtl<R> *__restrict__ ctl) {
   pdl_wait();
   extern __shared__ int cnt[];  // [passes][R]
@@ -291,7 +291,7 @@ __global__ void __launch_bounds__(kHistBlock) k_sort_hist(const K *__restrict__ 
 // Many keys: digits of one pass per group, a block per tile (added up in the
 // group's row), and their totals; clears the tile's row.
 template <class K, int R>
-__global__ void __launch_bounds__(kHistBlock) k_group_hist(const K *__restrict__ key, int src, int64_t n, int ktile,
+__global__ void __launch_bounds__(kHistBlock) k_group_hist(const K *key, int src, int64_t n, int ktile,
                                                            int tiles, int pass, int width, SortCtl<R> *__restrict__ ctl,
                                                            WaveRows wave, int64_t ntiles) {
   pdl_wait();
@@ -336,7 +336,7 @@ __global__ void __launch_bounds__(kHistBlock) k_group_hist(const K *__restrict__
 
 // rows[group][digit]: counts -> first positions.  A block takes 32 digits.
 template <int R>
-__global__ void __launch_bounds__(1024) k_group_scan(int ngroup, int pass, const SortCtl<R> *__restrict__ ctl,
+__global__ void __launch_bounds__(1024) k_group_scan(int ngroup, int pass, const SortCtl<R> *ctl,
                                                      int32_t *__restrict__ rows) {
   pdl_wait();
   __shared__ int part[32][33], wsum[32];
@@ -391,8 +391,8 @@ constexpr int kSpins = 1 << 16;
 
 template <class K, int THREADS, int ITEMS, int RB, bool WAVE>
 __global__ void __launch_bounds__(THREADS, 1024 / THREADS) k_radix_pass(
-    const K *__restrict__ key, const uint32_t *__restrict__ val, int src, int64_t n, int pass, int width,
-    SortCtl<(1 << RB)> *__restrict__ ctl, const int32_t *__restrict__ rows, WaveRows wave, int spins,
+    const K *key, const uint32_t *val, int src, int64_t n, int pass, int width,
+    SortCtl<(1 << RB)> *__restrict__ ctl, const int32_t *rows, WaveRows wave, int spins,
     K *__restrict__ okey, uint32_t *__restrict__ oval) {
   pdl_wait();
   constexpr int kGroup = ::amfmm::kGroup<WAVE>;

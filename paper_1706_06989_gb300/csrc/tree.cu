@@ -65,8 +65,8 @@ __device__ __forceinline__ Extremes no_extremes() {
   }
   return v;
 }
-__device__ __forceinline__ Extremes body_extremes(const double *__restrict__ x, const double *__restrict__ y,
-                                                  const double *__restrict__ z, const double *__restrict__ m,
+__device__ __forceinline__ Extremes body_extremes(const double *x, const double *y,
+                                                  const double *z, const double *m,
                                                   int64_t first, int64_t end, int64_t stride, int *status) {
   Extremes v = no_extremes();
   bool bad = false;
@@ -97,8 +97,8 @@ __device__ __forceinline__ void write_box(const Extremes &v, double *__restrict_
 // Bounding cube: every block its part, the last one to finish the whole (minima
 // and maxima are exact, so their order does not matter).  14 us at N = 1M; two
 // launches with FP64 comparisons took 45.6 + 10.1.
-__global__ void k_bbox(const double *__restrict__ x, const double *__restrict__ y, const double *__restrict__ z,
-                       const double *__restrict__ m, int64_t n, long long *__restrict__ part,
+__global__ void k_bbox(const double *x, const double *y, const double *z,
+                       const double *m, int64_t n, long long *__restrict__ part,
                        int *__restrict__ status, unsigned *__restrict__ done, double *__restrict__ bbox) {
   pdl_wait();
   __shared__ bool last;
@@ -139,8 +139,8 @@ __device__ __forceinline__ uint64_t spread3(uint64_t q) {
   return q;
 }
 
-__global__ void k_keys(const double *__restrict__ x, const double *__restrict__ y,
-                       const double *__restrict__ z, int64_t n, const double *__restrict__ bbox,
+__global__ void k_keys(const double *x, const double *y,
+                       const double *z, int64_t n, const double *bbox,
                        uint64_t *__restrict__ key, uint32_t *__restrict__ idx) {
   pdl_wait();
   int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
@@ -160,9 +160,9 @@ __global__ void k_keys(const double *__restrict__ x, const double *__restrict__ 
 // ---------------------------------------------------------------------------
 // one block per system: its cube (lo, scale), the system id of its bodies and
 // the bad-data flag
-__global__ void k_bbox_sys(const double *__restrict__ x, const double *__restrict__ y,
-                           const double *__restrict__ z, const double *__restrict__ m,
-                           const int64_t *__restrict__ off, double *__restrict__ sbox,
+__global__ void k_bbox_sys(const double *x, const double *y,
+                           const double *z, const double *m,
+                           const int64_t *off, double *__restrict__ sbox,
                            int32_t *__restrict__ sysid, int *__restrict__ status) {
   pdl_wait();
   const int s = blockIdx.x;
@@ -172,9 +172,9 @@ __global__ void k_bbox_sys(const double *__restrict__ x, const double *__restric
   if (threadIdx.x == 0) write_box(v, sbox + 4 * static_cast<int64_t>(s));
 }
 
-__global__ void k_keys_sys(const double *__restrict__ x, const double *__restrict__ y,
-                           const double *__restrict__ z, int64_t n, const double *__restrict__ sbox,
-                           const int32_t *__restrict__ sysid, uint64_t *__restrict__ key,
+__global__ void k_keys_sys(const double *x, const double *y,
+                           const double *z, int64_t n, const double *sbox,
+                           const int32_t *sysid, uint64_t *__restrict__ key,
                            uint32_t *__restrict__ idx) {
   pdl_wait();
   int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
@@ -186,7 +186,7 @@ __global__ void k_keys_sys(const double *__restrict__ x, const double *__restric
 }
 
 // second pass: (system of the body at sorted position s, s)
-__global__ void k_sys_keys(int64_t n, const uint32_t *__restrict__ idx, const int32_t *__restrict__ sysid,
+__global__ void k_sys_keys(int64_t n, const uint32_t *idx, const int32_t *sysid,
                            uint32_t *__restrict__ skey, uint32_t *__restrict__ sval) {
   pdl_wait();
   int64_t s = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
@@ -195,8 +195,8 @@ __global__ void k_sys_keys(int64_t n, const uint32_t *__restrict__ idx, const in
   sval[s] = static_cast<uint32_t>(s);
 }
 
-__global__ void k_gather_sorted(int64_t n, const uint32_t *__restrict__ perm, const uint64_t *__restrict__ k1,
-                                const uint32_t *__restrict__ i1, uint64_t *__restrict__ k2,
+__global__ void k_gather_sorted(int64_t n, const uint32_t *perm, const uint64_t *k1,
+                                const uint32_t *i1, uint64_t *__restrict__ k2,
                                 uint32_t *__restrict__ i2) {
   pdl_wait();
   int64_t t = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
@@ -207,9 +207,9 @@ __global__ void k_gather_sorted(int64_t n, const uint32_t *__restrict__ perm, co
 
 // Gather the bodies into key order, also as hi + lo floats (R_max, and the
 // mixed form's near field).
-__global__ void k_permute(const double *__restrict__ x, const double *__restrict__ y,
-                          const double *__restrict__ z, const double *__restrict__ m,
-                          const uint32_t *__restrict__ idx, int64_t n, double *__restrict__ X,
+__global__ void k_permute(const double *x, const double *y,
+                          const double *z, const double *m,
+                          const uint32_t *idx, int64_t n, double *__restrict__ X,
                           double *__restrict__ Y, double *__restrict__ Zb, double *__restrict__ Mb,
                           int32_t *__restrict__ order, BodyF *__restrict__ bodyf) {
   pdl_wait();
@@ -252,13 +252,13 @@ __device__ __forceinline__ int shared_digits(uint64_t a, uint64_t b) {
   return d == 0 ? kMaxLevel : (__clzll(static_cast<long long>(d)) - 1) / 3;
 }
 // system of the body at sorted position s
-__device__ __forceinline__ int system_of(const int32_t *__restrict__ sysid, const uint32_t *__restrict__ idx,
+__device__ __forceinline__ int system_of(const int32_t *sysid, const uint32_t *idx,
                                          int64_t s) {
   return sysid ? sysid[idx[s]] : 0;
 }
 // digits shared by the ends of the window [j, j + w], -1 if there is none
-__device__ __forceinline__ int window_digits(const uint64_t *__restrict__ key, const uint32_t *__restrict__ idx,
-                                             const int32_t *__restrict__ sysid, int64_t n, int64_t j, int w) {
+__device__ __forceinline__ int window_digits(const uint64_t *key, const uint32_t *idx,
+                                             const int32_t *sysid, int64_t n, int64_t j, int w) {
   if (j < 0 || j + w >= n || system_of(sysid, idx, j) != system_of(sysid, idx, j + w)) return -1;
   return shared_digits(key[j], key[j + w]);
 }
@@ -266,13 +266,13 @@ __device__ __forceinline__ int window_digits(const uint64_t *__restrict__ key, c
 // For n_crit beyond kWindowMax: the windows' digits, and their running maximum
 // over the last 2^k window starts by doubling (out = max of in at j and at
 // j - step).
-__global__ void k_window_digits(const uint64_t *__restrict__ key, const uint32_t *__restrict__ idx,
-                                const int32_t *__restrict__ sysid, int64_t n, int w, int8_t *__restrict__ out) {
+__global__ void k_window_digits(const uint64_t *key, const uint32_t *idx,
+                                const int32_t *sysid, int64_t n, int w, int8_t *__restrict__ out) {
   pdl_wait();
   const int64_t j = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (j < n) out[j] = static_cast<int8_t>(window_digits(key, idx, sysid, n, j, w));
 }
-__global__ void k_window_max(int64_t n, int64_t step, const int8_t *__restrict__ in, int8_t *__restrict__ out) {
+__global__ void k_window_max(int64_t n, int64_t step, const int8_t *in, int8_t *__restrict__ out) {
   pdl_wait();
   const int64_t j = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (j < n) out[j] = j >= step ? max(in[j], in[j - step]) : in[j];
@@ -282,9 +282,9 @@ __global__ void k_window_max(int64_t n, int64_t step, const int8_t *__restrict__
 // system) and its leaf's level; per block and level: cells and leaves that
 // start there.  wmax (n_crit > kWindowMax): the maximum over the body's
 // windows.
-__global__ void k_cell_levels(const uint64_t *__restrict__ key, const uint32_t *__restrict__ idx,
-                              const int32_t *__restrict__ sysid, int64_t n, int n_crit,
-                              const int8_t *__restrict__ wmax, char2 *__restrict__ lv, int32_t *__restrict__ cnt) {
+__global__ void k_cell_levels(const uint64_t *key, const uint32_t *idx,
+                              const int32_t *sysid, int64_t n, int n_crit,
+                              const int8_t *wmax, char2 *__restrict__ lv, int32_t *__restrict__ cnt) {
   pdl_wait();
   extern __shared__ int8_t win[];  // kBlock + n_crit window starts
   __shared__ int32_t tot[2][kLevels];
@@ -320,7 +320,7 @@ __global__ void k_cell_levels(const uint64_t *__restrict__ key, const uint32_t *
 // Emits the cells: begin, level, parent; every body's cell per level (-1 below
 // its leaf), its leaf, and the leaves in id order.  lvl: first id of every
 // level (23 entries) and the number of leaves.
-__global__ void k_emit_cells(int64_t n, const char2 *__restrict__ lv, const int32_t *__restrict__ offs, int64_t cap,
+__global__ void k_emit_cells(int64_t n, const char2 *lv, const int32_t *offs, int64_t cap,
                              int32_t *__restrict__ begin, int32_t *__restrict__ level, int32_t *__restrict__ parent,
                              int32_t *__restrict__ cell_at, int32_t *__restrict__ leaf_of,
                              int32_t *__restrict__ leaves, int32_t *__restrict__ lvl) {
@@ -384,10 +384,10 @@ __global__ void k_emit_cells(int64_t n, const char2 *__restrict__ lv, const int3
 // Ends and children of the cells.  A cell ends where its next sibling begins,
 // or with its parent; the children of a split cell are the cells of its first
 // to its last body on the next level.
-__global__ void k_finish_cells(int64_t n, int n_crit, int nsys, int64_t cap, const int64_t *__restrict__ sys_off,
-                               const int32_t *__restrict__ lvl, const int32_t *__restrict__ begin,
-                               const int32_t *__restrict__ level, const int32_t *__restrict__ parent,
-                               const int32_t *__restrict__ cell_at, int32_t *__restrict__ count,
+__global__ void k_finish_cells(int64_t n, int n_crit, int nsys, int64_t cap, const int64_t *sys_off,
+                               const int32_t *lvl, const int32_t *begin,
+                               const int32_t *level, const int32_t *parent,
+                               const int32_t *cell_at, int32_t *__restrict__ count,
                                int32_t *__restrict__ first_child, int32_t *__restrict__ nchild) {
   pdl_wait();
   const int ncell = lvl[kLevels];
@@ -440,9 +440,9 @@ constexpr int kUpWarps = 4;
 
 template <int G>
 __global__ void __launch_bounds__(kUpWarps * 32) k_leaf_upward(
-    int32_t nleaf, const int32_t *__restrict__ leaves, const int32_t *__restrict__ begin,
-    const int32_t *__restrict__ count, const double *__restrict__ X, const double *__restrict__ Y,
-    const double *__restrict__ Zb, const double *__restrict__ Mb, double *__restrict__ S, double *__restrict__ M,
+    int32_t nleaf, const int32_t *leaves, const int32_t *begin,
+    const int32_t *count, const double *X, const double *Y,
+    const double *Zb, const double *Mb, double *__restrict__ S, double *__restrict__ M,
     double *__restrict__ Z, double *__restrict__ invM, double *__restrict__ mom) {
   pdl_wait();
   __shared__ double sh[kUpWarps][14][33];  // per body: ten products, x, y, z, 1 (first: mu x, mu y, mu z, mu)
@@ -556,7 +556,7 @@ __global__ void __launch_bounds__(kUpWarps * 32) k_leaf_upward(
 // octant order.  About 120 FP64 warp instructions for four parents; a thread per
 // parent had a chain of 600 (52 us per level of 4,000 to 16,000 cells).
 __global__ void __launch_bounds__(kUpWarps * 32) k_internal_upward(
-    int32_t c0, int32_t c1, const int32_t *__restrict__ first_child, const int32_t *__restrict__ nchild,
+    int32_t c0, int32_t c1, const int32_t *first_child, const int32_t *nchild,
     double *__restrict__ S, double *__restrict__ M, double *__restrict__ Z, double *__restrict__ invM,
     double *__restrict__ mom) {
   pdl_wait();
@@ -647,7 +647,7 @@ __constant__ signed char c_oct[10][3] = {{0, 0, 0}, {0, 0, 1}, {0, 0, 2}, {0, 1,
 __constant__ signed char c_quad[3][3] = {{4, 5, 6}, {5, 7, 8}, {6, 8, 9}};
 
 __global__ void __launch_bounds__(128) k_internal_upward_block(
-    int32_t c0, const int32_t *__restrict__ first_child, const int32_t *__restrict__ nchild, double *__restrict__ S,
+    int32_t c0, const int32_t *first_child, const int32_t *nchild, double *__restrict__ S,
     double *__restrict__ M, double *__restrict__ Z, double *__restrict__ invM, double *__restrict__ mom) {
   pdl_wait();
   __shared__ double q[8 * kMomStride], sh[kMomStride][9], sv[8][3];
@@ -704,7 +704,7 @@ __global__ void __launch_bounds__(128) k_internal_upward_block(
 }
 
 // Centres as hi + lo floats for the filter of R_max, whose maxima start at zero.
-__global__ void k_split_centres(int32_t ncell, const double *__restrict__ Z, float4 *__restrict__ zf,
+__global__ void k_split_centres(int32_t ncell, const double *Z, float4 *__restrict__ zf,
                                 unsigned long long *__restrict__ rmax2) {
   pdl_wait();
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
@@ -729,9 +729,9 @@ __global__ void k_split_centres(int32_t ncell, const double *__restrict__ Z, flo
 // 1,048,576).  The maximum is taken on the bit pattern (monotone for
 // non-negative doubles); it is exact, so its order does not matter.
 __global__ void __launch_bounds__(kBlock) k_rmax_bodies(
-    int64_t n, int nlev, const int32_t *__restrict__ cell_at, const BodyF *__restrict__ bodyf,
-    const float4 *__restrict__ zf, const double *__restrict__ X, const double *__restrict__ Y,
-    const double *__restrict__ Zb, const double *__restrict__ Z, unsigned long long *__restrict__ rmax2) {
+    int64_t n, int nlev, const int32_t *cell_at, const BodyF *bodyf,
+    const float4 *zf, const double *X, const double *Y,
+    const double *Zb, const double *Z, unsigned long long *__restrict__ rmax2) {
   pdl_wait();
   __shared__ int2 todo[kBlock / 32][64];  // (body, cell) still to be evaluated
   const int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
@@ -794,7 +794,7 @@ __global__ void __launch_bounds__(kBlock) k_rmax_bodies(
   evaluate(0, have);
 }
 
-__global__ void k_rmax_final(int32_t ncell, const unsigned long long *__restrict__ rmax2,
+__global__ void k_rmax_final(int32_t ncell, const unsigned long long *rmax2,
                              double *__restrict__ Rmax) {
   pdl_wait();
   int c = blockIdx.x * blockDim.x + threadIdx.x;

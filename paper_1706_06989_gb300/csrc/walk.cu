@@ -33,9 +33,9 @@ enum Action : int32_t { kSelfLeaf = 0, kSelfSplit = 1, kAccept = 2, kNear = 3, k
 
 // packs the walk's per-cell inputs: {Z, R_max} (FP64 and the FP32 filter's
 // copy, with nchild | level << 8) and {first child, nchild}
-__global__ void k_pack_cells(int32_t ncell, const double *__restrict__ Z, const double *__restrict__ Rmax,
-                             const int32_t *__restrict__ nchild, const int32_t *__restrict__ level,
-                             const int32_t *__restrict__ first_child, double4_32a *__restrict__ zr, CellF *__restrict__ zf, int2 *__restrict__ nl) {
+__global__ void k_pack_cells(int32_t ncell, const double *Z, const double *Rmax,
+                             const int32_t *nchild, const int32_t *level,
+                             const int32_t *first_child, double4_32a *__restrict__ zr, CellF *__restrict__ zf, int2 *__restrict__ nl) {
   pdl_wait();
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= ncell) return;
@@ -54,8 +54,8 @@ __global__ void k_pack_cells(int32_t ncell, const double *__restrict__ Z, const 
 // the pair (then the criterion is a floor on the accepted set, which bounds the
 // work of a strict target).  Everything a decision usually needs is loaded
 // before the first branch.
-__device__ __forceinline__ int classify(int A, int B, const double4_32a *__restrict__ zr,
-                                        const CellF *__restrict__ zf, double theta, float th2f, bool accept_hint,
+__device__ __forceinline__ int classify(int A, int B, const double4_32a *zr,
+                                        const CellF *zf, double theta, float th2f, bool accept_hint,
                                         int &children) {
   const CellF fA = zf[A], fB = zf[B];
   const int nlA = __float_as_int(fA.l.w), nlB = __float_as_int(fB.l.w), ka = nlA & 255, kb = nlB & 255;
@@ -157,8 +157,8 @@ __device__ __forceinline__ void st_volatile4(int4 *p, int4 v) {
 // walk and flags it, and the host grows the buffers (keeping what earlier
 // generations wrote) and resumes the walk at the flagged generation.
 __global__ void __launch_bounds__(kGenBlock, kGenBlocksPerSM) k_walk_gen(
-    GenState *__restrict__ gs, int g, const int4 *__restrict__ front, const int2 *__restrict__ nl,
-    const double4_32a *__restrict__ zr, const CellF *__restrict__ zf, double theta, const float *__restrict__ score,
+    GenState *__restrict__ gs, int g, const int4 *front, const int2 *nl,
+    const double4_32a *zr, const CellF *zf, double theta, const float *score,
     float target, int4 *__restrict__ next, int64_t cap_next,
     int2 *__restrict__ m2l, int64_t cap_m2l, int2 *__restrict__ p2p, int64_t cap_p2p, int32_t *__restrict__ self,
     int64_t cap_self, unsigned epoch, int64_t max_places, int *__restrict__ flag, int4 *__restrict__ agg,
