@@ -251,12 +251,17 @@ __global__ void k_p2p_chunks(int32_t nleaf, int64_t n, const int32_t *leaves,
   }
 }
 
+// The FP64 sums of a body have one order, however its leaf is worked on (the line
+// of heavy leaves depends on the whole call, and a system solved alone and in a
+// forest must agree): the self sums of all passes over the leaf's rows, then the A
+// side of its chunks in order.  A leaf of several passes keeps the first chunk's
+// A-side sums in `late` until the last.
 // HEAVY: there are items of heavy leaves (the test for them costs 1% otherwise).
 template <int ROWS, bool HEAVY>
 __global__ void __launch_bounds__(kWarps * 32) k_p2p(
     int32_t nitem, int64_t n, const int4 *items, const int32_t *item_rows,
     const int32_t *begin, const int32_t *count, const double *Zc, const int2 *cols,
-    double *__restrict__ near, double *__restrict__ extra, float *__restrict__ slots,
+    double *__restrict__ near, double *__restrict__ late, double *__restrict__ extra, float *__restrict__ slots,
     const BodyF *bodyf, float eps2, int *__restrict__ queue) {
   pdl_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -398,11 +403,17 @@ __global__ void __launch_bounds__(kWarps * 32) k_p2p(
         g[h] = ((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7]));
       }
       const double s = static_cast<double>((g[0] + g[1]) + (g[2] + g[3]));
-      if (first) near[static_cast<int64_t>(v % 3) * n + bA + r0 + v / 3] += s;
+      const int64_t body = static_cast<int64_t>(v % 3) * n + bA + r0 + v / 3;
+      if (first && nA <= kRows) near[body] += s;
+      else if (first) late[body] = s;
       else extra[it.w + 3 * (r0 + v / 3) + v % 3] = s;
     }
     __syncwarp();
   }
+  if (first && nA > kRows)
+    for (int t = l; t < nA; t += 32)
+#pragma unroll
+      for (int d = 0; d < 3; ++d) near[d * n + bA + t] += late[d * n + bA + t];
   }
 }
 
@@ -579,7 +590,7 @@ int launch_p2p_rows(fmm_ctx *c) {
   int *queue = ptr<int32_t>(c->totals) + 40;
   launch(c, k_p2p<ROWS, HEAVY>, grid, kWarps * 32, shm, nitem, n, ptr<int4>(c->p2p_items), ptr<int32_t>(c->p2p_rowpart),
          ptr<int32_t>(c->begin), ptr<int32_t>(c->count), ptr<double>(c->Z), ptr<int2>(c->p2p_cols), ptr<double>(c->near),
-         ptr<double>(c->p2p_extra), static_cast<float *>(c->p2p_slots.p), ptr<BodyF>(c->bodyf),
+         ptr<double>(c->acc), ptr<double>(c->p2p_extra), static_cast<float *>(c->p2p_slots.p), ptr<BodyF>(c->bodyf),
          static_cast<float>(c->eps2), queue);
   AMFMM_TRY(launched(c, "p2p"));
   if (nitem > nleaf) {
@@ -598,6 +609,7 @@ int p2p_prepare(fmm_ctx *c) {
   const int64_t K = c->sz.n_p2p, nc = c->sz.ncell, n = c->sz.n;
   const int32_t nleaf = static_cast<int32_t>(c->sz.nleaf);
   AMFMM_TRY(ensure<double>(c, c->near, 3 * n));
+  AMFMM_TRY(ensure<double>(c, c->acc, 3 * n));  // A-side sums of leaves of several passes; the downward pass writes it
   AMFMM_TRY(ensure<int32_t>(c, c->p2p_offA, nc + 1));
   AMFMM_TRY(ensure<int32_t>(c, c->p2p_offB, nc + 1));
   AMFMM_TRY(ensure<int32_t>(c, c->p2p_colOff, nc + 1));
