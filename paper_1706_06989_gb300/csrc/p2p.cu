@@ -119,15 +119,23 @@ __device__ __forceinline__ float3 offset32(const BodyF &b, const float4 zh, cons
 // independent of one another, and so are the B side's columns: such a heavy
 // leaf's chunks become items of kItemRows rows (A side only) and items of
 // kItemCols columns (B side only), which evaluate its pairs twice, in the same
-// order within every sum.  Near field without and with this rule, and with the
-// line at the average itself and at half of it: N = 65,536 (outlying leaves with
-// up to 65,000 columns) 337, 141, 165, 143 us; a forest of 48 systems 552, 516,
-// 601, 548; 200,000 bodies of two clusters 440, 303, 389, 316; a disc of 262,144
-// 508, 424, 533, 455.  At N = 1M the line is at 4,270 columns and no leaf beyond.
+// order within every sum.  The line is half of the average work of the warps that run
+// at once, in body pairs of a chunk, and at least 512 columns; and where not even a
+// whole chunk of a whole leaf exceeds the average, no leaf is what the kernel ends on
+// (262,144 bodies in leaves of up to 256: 5.4 ms, with half of the work in parts 6.3).
+// Near field (us) without the rule, and with the line at the average itself, half, a
+// third and a sixth of it: N = 65,536 (outlying leaves with up to 65,000 columns) 350,
+// 141, 132, 136, 136;
+// a forest of 48 systems 547, 543, 490, 496, 513; 200,000 bodies of two clusters 460,
+// 292, 294, 290, 306; a disc of 262,144 518, 452, 377, 374, 395; N = 1M 803, 794, 773,
+// 771, 802; leaves of up to 128 bodies at 1M 5,043, 5,154, 5,058, 5,276, 6,519, of up to
+// 512 34,516, 34,442, 34,471, 34,560, 37,427 (54,362 with a line in columns, which
+// made every large leaf heavy).
 constexpr int kChunk = 4096;
 constexpr int kItemRows = 4;
 constexpr int kItemCols = 512;
 constexpr int kHeavyMin = 512;
+constexpr int kHeavyPart = 2;
 // items {leaf, first column, end column, -1 or place in `extra`}; an item of a
 // heavy leaf has the complement of the end column, and its first row, or -1 for
 // the B side, in item_rows.  A heavy leaf's places: its self sums, then the
@@ -144,13 +152,17 @@ __device__ __forceinline__ int2 chunk_range(int j, int cb, int ce, int nself) {
   return make_int2(c0, min(ce, c0 + kChunk));
 }
 // (counts of places and items in 64 bits: both are refused beyond 2^31 - 1)
-// more columns than a third of the average of the warps that run at once
-__device__ __forceinline__ bool is_heavy(int ncol, int total, int warps) {
-  return ncol > max(kHeavyMin, total / (3 * warps));
+// `pairs`: body pairs of all leaves; `warps`: that run at once; `full`: body pairs of
+// a whole chunk of a whole leaf
+__device__ __forceinline__ bool is_heavy(int ncol, int nA, const unsigned long long *pairs, int warps,
+                                         long long full) {
+  const long long chunk = static_cast<long long>(min(ncol, max(kChunk, nA))) * nA;
+  const long long average = static_cast<long long>(*pairs) / warps;
+  return ncol > kHeavyMin && chunk > average / kHeavyPart && max(chunk, full) > average;
 }
 
 __global__ void k_item_counts(int32_t nleaf, const int32_t *leaves, const int32_t *count,
-                              const int32_t *colOff, const int32_t *total, int warps,
+                              const int32_t *colOff, const unsigned long long *pairs, int warps, long long full,
                               int32_t *__restrict__ nitems, int32_t *__restrict__ nextra, int *__restrict__ nheavy,
                               unsigned long long *__restrict__ wide) {
   pdl_wait();
@@ -160,7 +172,7 @@ __global__ void k_item_counts(int32_t nleaf, const int32_t *leaves, const int32_
     if (q == 0) nitems[nleaf] = nextra[nleaf] = 0;
     const int L = leaves[q], cb = colOff[L], ce = colOff[L + 1], nA = count[L];
     const int k = chunks_of(ce - cb, nA);
-    if (!is_heavy(ce - cb, *total, warps)) {
+    if (!is_heavy(ce - cb, nA, pairs, warps, full)) {
       items = k;
       places = (k - 1) * 3ull * nA;
     } else {
@@ -187,7 +199,7 @@ __global__ void k_item_counts(int32_t nleaf, const int32_t *leaves, const int32_
 }
 
 __global__ void k_item_fill(int32_t nleaf, const int32_t *leaves, const int32_t *count,
-                            const int32_t *colOff, const int32_t *total, int warps,
+                            const int32_t *colOff, const unsigned long long *pairs, int warps, long long full,
                             const int32_t *itemOff, const int32_t *extraOff,
                             int4 *__restrict__ items, int32_t *__restrict__ item_rows) {
   pdl_wait();
@@ -196,7 +208,7 @@ __global__ void k_item_fill(int32_t nleaf, const int32_t *leaves, const int32_t 
   const int L = leaves[q];
   const int cb = colOff[L], ce = colOff[L + 1], nA = count[L];
   const int k = chunks_of(ce - cb, nA);
-  const bool heavy = is_heavy(ce - cb, *total, warps);
+  const bool heavy = is_heavy(ce - cb, nA, pairs, warps, full);
   int o = itemOff[q];
   for (int j = 0; j < k; ++j) {
     const int2 c = chunk_range(j, cb, ce, nA);
@@ -220,7 +232,7 @@ __global__ void k_item_fill(int32_t nleaf, const int32_t *leaves, const int32_t 
 // heavy leaf its self sums and those of all chunks.
 __global__ void k_p2p_chunks(int32_t nleaf, int64_t n, const int32_t *leaves,
                              const int32_t *begin, const int32_t *count,
-                             const int32_t *colOff, const int32_t *total, int warps,
+                             const int32_t *colOff, const unsigned long long *pairs, int warps, long long full,
                              const int32_t *extraOff, const double *extra,
                              double *__restrict__ near) {
   pdl_wait();
@@ -231,7 +243,7 @@ __global__ void k_p2p_chunks(int32_t nleaf, int64_t n, const int32_t *leaves,
   if (e0 == e1) return;
   const int L = leaves[q];
   const int bA = begin[L], nA = count[L];
-  const bool heavy = is_heavy(colOff[L + 1] - colOff[L], *total, warps);
+  const bool heavy = is_heavy(colOff[L + 1] - colOff[L], nA, pairs, warps, full);
   for (int r = l; r < nA; r += 32) {
     double a0 = 0.0, a1 = 0.0, a2 = 0.0;
     if (!heavy) {
@@ -573,6 +585,10 @@ __global__ void k_cols_pairs(int64_t K, const int2 *pairs, const int32_t *begin,
 // the warps that the rule of heavy leaves counts with (16 run per SM at the
 // default tile; the rule must be the same in every stage of a solve)
 int heavy_warps(const fmm_ctx *c) { return 16 * std::max(1, c->num_sms); }
+long long full_chunk(const fmm_ctx *c) {
+  const long long rows = std::min<int64_t>(c->opts.n_crit, c->sz.n);
+  return std::max<long long>(kChunk, rows) * rows;
+}
 
 template <int ROWS, bool HEAVY>
 int launch_p2p_rows(fmm_ctx *c) {
@@ -595,8 +611,9 @@ int launch_p2p_rows(fmm_ctx *c) {
   AMFMM_TRY(launched(c, "p2p"));
   if (nitem > nleaf) {
     launch(c, k_p2p_chunks, grid_for(static_cast<int64_t>(nleaf) * 32, 256), 256, 0, nleaf, n, ptr<int32_t>(c->leaves),
-           ptr<int32_t>(c->begin), ptr<int32_t>(c->count), ptr<int32_t>(c->p2p_colOff), ptr<int32_t>(c->totals) + 32,
-           heavy_warps(c), ptr<int32_t>(c->p2p_extraOff), ptr<double>(c->p2p_extra), ptr<double>(c->near));
+           ptr<int32_t>(c->begin), ptr<int32_t>(c->count), ptr<int32_t>(c->p2p_colOff),
+           ptr<unsigned long long>(c->totals) + 8, heavy_warps(c), full_chunk(c), ptr<int32_t>(c->p2p_extraOff),
+           ptr<double>(c->p2p_extra), ptr<double>(c->near));
     AMFMM_TRY(launched(c, "p2p_chunks"));
   }
   return FMM_OK;
@@ -667,7 +684,7 @@ int p2p_prepare(fmm_ctx *c) {
   unsigned long long *wide = ptr<unsigned long long>(c->totals) + 13;
   int32_t *icnt = cnt, *ecnt = ptr<int32_t>(c->flag);  // free scratch of >= nleaf + 1
   launch(c, k_item_counts, grid_for(nleaf, 256), 256, 0, nleaf, ptr<int32_t>(c->leaves), ptr<int32_t>(c->count),
-         colOff, ctot, heavy_warps(c), icnt, ecnt, nheavy, wide);
+         colOff, stat, heavy_warps(c), full_chunk(c), icnt, ecnt, nheavy, wide);
   AMFMM_TRY(launched(c, "p2p_item_counts"));
   AMFMM_TRY(exclusive_scan_i32(c, icnt, itemOff, nleaf + 1, itot));
   AMFMM_TRY(exclusive_scan_i32(c, ecnt, extraOff, nleaf + 1, etot));
@@ -707,7 +724,7 @@ int p2p_prepare(fmm_ctx *c) {
   AMFMM_TRY(ensure<double>(c, c->p2p_extra, nextra + 1));
   AMFMM_TRY(ensure<int32_t>(c, c->p2p_rowpart, nitem + 1));
   launch(c, k_item_fill, grid_for(nleaf, 256), 256, 0, nleaf, ptr<int32_t>(c->leaves), ptr<int32_t>(c->count), colOff,
-         ctot, heavy_warps(c), itemOff, extraOff, ptr<int4>(c->p2p_items), ptr<int32_t>(c->p2p_rowpart));
+         stat, heavy_warps(c), full_chunk(c), itemOff, extraOff, ptr<int4>(c->p2p_items), ptr<int32_t>(c->p2p_rowpart));
   AMFMM_TRY(launched(c, "p2p_item_fill"));
   AMFMM_TRY(ensure_bytes(c, c->p2p_slots, static_cast<size_t>(nslot + 3) * sizeof(float)));
   AMFMM_TRY(ensure<int2>(c, c->p2p_cols, ncol + 1));
