@@ -214,7 +214,8 @@ int fmm_autotune_ncrit(fmm_ctx *ctx, const double *x, const double *y, const dou
 /* a13: picks the leaf size and the leaf tile together: every pair
  * (ncrit[a], tiles[b]) is timed as above; ms_out (HOST, nn x nt floats, row
  * a = ncrit[a], may be NULL) receives the mean ms of each pair, *best_ncrit
- * and *best_tile (HOST) the fastest.  Tiles are 8, 16 or 32 (fmm_set_tile).
+ * and *best_tile (HOST) the fastest.  Tiles are 8, 16 or 32 (fmm_set_tile);
+ * in the FP64 form, which has none, each leaf size is timed once.
  * The context's options and tile are restored afterwards.  Synchronises the
  * stream. */
 int fmm_autotune(fmm_ctx *ctx, const double *x, const double *y, const double *z, const double *m,

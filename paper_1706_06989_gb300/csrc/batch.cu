@@ -5,7 +5,8 @@
 // at most n_crit bodies, Sec. 2) and leaf tile (the rows of a leaf the near
 // field stages per pass); the fastest pair is returned.  Every candidate
 // gives a valid solve of the same method: n_crit changes the tree, the tile
-// only the order of the near field's work.
+// only the order of the near field's work.  The FP64 form's near field has no
+// tile: one time stands for all of a leaf size, and the first tile is returned.
 #include "internal.cuh"
 
 using namespace amfmm;
@@ -60,12 +61,13 @@ extern "C" int fmm_autotune(fmm_ctx *c, const double *x, const double *y, const 
   float best_ms = 0.f;
   *best_ncrit = ncrit[0];
   *best_tile = tiles[0];
-  for (int a = 0; a < nn && rc == FMM_OK; ++a)
+  for (int a = 0; a < nn && rc == FMM_OK; ++a) {
+    float ms = 0.f;
     for (int b = 0; b < nt && rc == FMM_OK; ++b) {
       c->opts.n_crit = ncrit[a];
       c->p2p_rows = tiles[b];
-      float ms = 0.f;
-      rc = time_batch(c, e0, e1, x, y, z, m, offsets, nsys, reps, ax, ay, az, &ms);
+      if (b == 0 || c->opts.precision == FMM_MIXED)
+        rc = time_batch(c, e0, e1, x, y, z, m, offsets, nsys, reps, ax, ay, az, &ms);
       if (ms_out) ms_out[a * nt + b] = ms;
       if (rc == FMM_OK && ((a == 0 && b == 0) || ms < best_ms)) {
         best_ms = ms;
@@ -73,6 +75,7 @@ extern "C" int fmm_autotune(fmm_ctx *c, const double *x, const double *y, const 
         *best_tile = tiles[b];
       }
     }
+  }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   c->opts = saved;

@@ -63,7 +63,7 @@ GraphKey key_of(const fmm_ctx *c, const double *ax, const double *ay, const doub
   k.order_P = c->opts.order_P;
   k.variant = c->opts.variant;
   k.precision = c->opts.precision;
-  k.rows = c->p2p_rows;
+  k.rows = c->opts.precision == FMM_MIXED ? c->p2p_rows : 0;  // the FP64 form has no tile
   k.alloc_gen = c->alloc_gen;
   return k;
 }
