@@ -319,7 +319,7 @@ int fmm_selector_train(fmm_ctx *ctx, float *params, float *adam, const float *X,
 int fmm_debug_walk_wait_timeout(fmm_ctx *ctx);
 /* Test hook: the radix sort of n (key, value) pairs on the device (keys of 4 or
  * 8 bytes, their low `bits` bits), with at most `spins` polls per wait of a tile
- * for the tiles before it. */
+ * for the tiles before it (0: no tile waits, each counts the keys before it). */
 int fmm_debug_sort(fmm_ctx *ctx, int key_bytes, const void *key, const uint32_t *val, int64_t n, int bits, int spins,
                    void *okey, uint32_t *oval);
 

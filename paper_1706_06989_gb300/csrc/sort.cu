@@ -507,9 +507,9 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) k_radix_pass(
       if (w * kWarpKeys + r * 32 + lane < nvalid) sv[at(r)] = v[r];
     // first position of the thread's digits: all tiles before this one
     const int grp = static_cast<int>(tile / kGroup), g0 = grp * kGroup;
-    bool failed = false;
+    bool failed = spins == 0;  // (tests: every tile counts for itself)
     if (WAVE) {
-      for (int g = t; g < grp; g += THREADS) {
+      for (int g = failed ? grp : t; g < grp; g += THREADS) {
         int polls = 0;
         while (*reinterpret_cast<volatile unsigned *>(&wave.arrived[g]) < kGroup)
           if (++polls > spins) {
@@ -710,8 +710,8 @@ int sort_pairs(fmm_ctx *c, const int2 *pairs, int64_t K, bool second, DBuf key[2
 using namespace amfmm;
 
 // Test hook of the sort (no counterpart in the paper): sorts n (key, value)
-// pairs given on the device with at most `spins` polls per look-back wait (0:
-// every wait that is not served at once counts the earlier keys itself).
+// pairs given on the device with at most `spins` polls per look-back wait (0: no
+// tile waits, each counts the keys before it itself).
 extern "C" int fmm_debug_sort(fmm_ctx *c, int key_bytes, const void *key, const uint32_t *val, int64_t n, int bits,
                               int spins, void *okey, uint32_t *oval) {
   if (!c || (key_bytes != 4 && key_bytes != 8) || n < 1 || bits < 1 || bits > 8 * key_bytes - 1 || spins < 0)
