@@ -327,6 +327,8 @@ int reduce_general(fmm_ctx *c);
 int downward_general(fmm_ctx *c);
 
 // learned selector (selector.cu, m2l.cu)
+constexpr int64_t kSelMaxRecords = int64_t(1) << 29;  // of a frontier that it scores
+static_assert(8 * kSelMaxRecords <= int64_t(1) << 32, "candidates are places of records, eight each, in 32 bits");
 int cell_features(fmm_ctx *c);  // per-cell parts of the selector's features
 int field_estimate(fmm_ctx *c);  // per-cell log10 |a| estimate of the selector's relative rule
 int walk_scores(fmm_ctx *c, const long long *nf_dev, int64_t cap, const int4 *front, float *score);

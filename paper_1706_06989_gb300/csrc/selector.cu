@@ -698,7 +698,7 @@ __global__ void k_adam(float *__restrict__ p, float *__restrict__ m, float *__re
 __global__ void k_band_select(const long long *nf_dev, int64_t cap, const int4 *front,
                               const double4_32a *zr, const CellF *zf,
                               const int32_t *count, int64_t min_work, double th_lo, double th_hi,
-                              float *__restrict__ score, int32_t *__restrict__ cand, unsigned *__restrict__ ncand) {
+                              float *__restrict__ score, uint32_t *__restrict__ cand, unsigned *__restrict__ ncand) {
   pdl_wait();
   // the frontier size comes from the walk's generation record; a frontier
   // beyond the buffers (the walk then stops and runs again) is not scored
@@ -732,7 +732,7 @@ __global__ void k_band_select(const long long *nf_dev, int64_t cap, const int4 *
     unsigned at = 0;
     if (lane == 0) at = atomicAdd(ncand, static_cast<unsigned>(__popc(m)));
     at = __shfl_sync(0xffffffffu, at, 0);
-    if (ok) cand[at + __popc(m & ((1u << lane) - 1u))] = static_cast<int32_t>(t);
+    if (ok) cand[at + __popc(m & ((1u << lane) - 1u))] = static_cast<uint32_t>(t);
   }
   }
 }
@@ -746,7 +746,7 @@ __global__ void k_band_select(const long long *nf_dev, int64_t cap, const int4 *
 //   score = pred + log10 max(M_B / (r^2 |a_A|), M_A / (r^2 |a_B|)),
 // compared by the walk with log10 of the relative target.
 __global__ void __launch_bounds__(128) k_walk_scores(const int4 *front,
-                                                     const int32_t *cand,
+                                                     const uint32_t *cand,
                                                      const unsigned *ncand,
                                                      const float *params,
                                                      const CellF *zf, const float4 *cf,
@@ -774,9 +774,9 @@ __global__ void __launch_bounds__(128) k_walk_scores(const int4 *front,
       float f[kF] = {0, 0, 0, 0, 0, 0, 0, 0};
       float ad = 0.f;
       if (base + lane < K) {
-        const int slot = cand[base + lane];
+        const uint32_t slot = cand[base + lane];
         int2 pr = make_int2(0, 0);
-        front_pair(front[slot >> 3], slot & 7, pr);
+        front_pair(front[slot >> 3], static_cast<int>(slot & 7), pr);
         pair_features(pr.x, pr.y, zf, cf, f);
         const float l2r = 2.f * f[0];
         ad = lga ? fmaxf(cf[pr.y].y - l2r - lga[pr.x], cf[pr.x].y - l2r - lga[pr.y])
@@ -844,13 +844,13 @@ int walk_scores(fmm_ctx *c, const long long *nf_dev, int64_t cap, const int4 *fr
   // persistent grids: the frontier size is only known on the device
   launch(c, k_band_select, static_cast<unsigned>(c->num_sms * 8), 256, 0, nf_dev, cap, front,
          ptr<double4_32a>(c->walk_zr), ptr<CellF>(c->walk_zf), ptr<int32_t>(c->count), c->sel_min_work, lo, hi, score,
-         ptr<int32_t>(c->sel_cand), ncand);
+         ptr<uint32_t>(c->sel_cand), ncand);
   AMFMM_TRY(launched(c, "band_select"));
   // as many blocks as run at once (229 registers: two per SM): each stages the
   // network once.  Walk stage of a disc of 262,144: 1.55 ms; one per SM 1.61, four
   // 1.65, eight 1.74.
   const unsigned g = static_cast<unsigned>(c->num_sms * 2);
-  launch(c, k_walk_scores, g, 128, 0, front, ptr<int32_t>(c->sel_cand), ncand, ptr<float>(c->sel_params),
+  launch(c, k_walk_scores, g, 128, 0, front, ptr<uint32_t>(c->sel_cand), ncand, ptr<float>(c->sel_params),
          ptr<CellF>(c->walk_zf), ptr<float4>(c->sel_cellfeat),
          c->sel_rule == FMM_SEL_RELATIVE ? ptr<float>(c->sel_lga) : nullptr, score,
          ptr<unsigned long long>(c->totals) + 10);

@@ -448,11 +448,13 @@ int walk(fmm_ctx *c) {
   int gstart = 0;  // first generation to (re)run
   for (int attempt = 0;; ++attempt) {
     if (attempt > 16) return set_error(c, FMM_EINVAL, "walk: outputs still overflow after growing the buffers");
-    const int64_t cap_next = std::min(c->front[0].cap, c->front[1].cap) / sizeof(int4);
+    int64_t cap_next = std::min(c->front[0].cap, c->front[1].cap) / sizeof(int4);
+    // the selector names a place of a record by 32 bits; a larger frontier ends the walk
+    if (c->sel_enabled) cap_next = std::min(cap_next, kSelMaxRecords);
     cap_front = cap_next;
     if (c->sel_enabled) {  // one score and one candidate slot per place of a record
       AMFMM_TRY(ensure<float>(c, c->sel_score, 8 * cap_front));
-      AMFMM_TRY(ensure<int32_t>(c, c->sel_cand, 8 * cap_front));
+      AMFMM_TRY(ensure<uint32_t>(c, c->sel_cand, 8 * cap_front));
     }
     // tiles are full-sized as soon as there are more of them than blocks
     const int64_t max_places = std::max<int64_t>(grid, (cap_next + kGenTile - 1) / kGenTile) + 1;
