@@ -53,9 +53,9 @@ M2L_FLOPS_FP64 = {"UC": 104, "TC": 170, "TCO": 177}
 WORK_PER_M2L_PAIR = 295
 # DRAM traffic of the dominant kernel per unit it processes, from one ncu
 # capture (dram__bytes_read.sum + dram__bytes_write.sum) of k_p2p64 on a Plummer
-# sphere of N = 262,144 (theta = 0.5): 23,775,744 B read and 2,304 B written
+# sphere of N = 262,144 (theta = 0.5): 23,484,416 B read and 11,776 B written
 # for 115,126,406 body pairs, scaled by the body pairs of the launch timed.
-TRAFFIC_PER_UNIT = {("p2p", "fp64"): (23775744 + 2304) / 115126406}
+TRAFFIC_PER_UNIT = {("p2p", "fp64"): (23484416 + 11776) / 115126406}
 P2P_FLOPS_PER_BODY_PAIR = 25
 # the FP64 form's near field works in fixed point and takes a body pair once from each
 # side: 32 x 32-bit products (64-bit or high word) per side, counted from the kernel's

@@ -27,7 +27,7 @@
  * Errors: every int-returning call returns FMM_OK (0) or a negative code;
  * fmm_last_error gives a one-line message.  A failed call leaves the
  * context usable for a new fmm_build_tree.  Input validation: n >= 1,
- * 0 < theta <= 1 (Sec. 2), n_crit >= 1, order_P in {3, 4, 5}; a body with a
+ * 0 < theta <= 1 (Sec. 2), n_crit >= 1, order_P from 3 to 8; a body with a
  * non-finite coordinate or a mass that is not positive and finite is
  * detected on the device and reported as FMM_EINVAL by the next call that
  * synchronises (fmm_build_tree).
@@ -69,7 +69,7 @@ typedef struct fmm_ctx fmm_ctx;
 typedef struct {
   double theta;  /* opening angle, 0 < theta <= 1 (Sec. 2) */
   int n_crit;    /* a cell with at most n_crit bodies is a leaf (Sec. 2: 25) */
-  int order_P;   /* expansion order: 3 (Eqs. 2-4), or 4, 5 (App. A; FP64 only) */
+  int order_P;   /* expansion order: 3 (Eqs. 2-4), or 4 to 8 (App. A; FP64 only) */
   int variant;   /* FMM_UC, FMM_TC or FMM_TCO */
   int precision; /* FMM_FP64 or FMM_MIXED */
   double G;      /* gravitational constant applied to the accelerations */
@@ -110,7 +110,7 @@ int fmm_set_timing(fmm_ctx *ctx, int enable);
  * form with R^2 -> R^2 + eps^2), so TC and TCO still cancel every pair's
  * torque.  The tree, the opening criterion and the lists do not depend on
  * eps.  eps = 0 (the default) is the unsoftened method.  Built at order
- * P = 3 (FP64 and mixed); a softened solve at P = 4, 5 returns
+ * P = 3 (FP64 and mixed); a softened solve at P = 4 to 8 returns
  * FMM_EUNSUPPORTED from fmm_interact.  FMM_EINVAL for eps < 0 or not finite.
  * The learned selector's training labels stay those of the unsoftened
  * expansion. */
@@ -141,7 +141,7 @@ int fmm_upward(fmm_ctx *ctx);
 /* a5-a8: dual-tree walk under the opening criterion
  * |Z_A - Z_B| >= (R_A,max + R_B,max)/theta (Sec. 2) producing the accepted
  * cell pairs and the leaf pairs; mutual M2L of every accepted pair with the
- * variant's corrective force (Eqs. 3, 4, 7, 8); mutual P2P of every leaf
+ * variant's corrective force (Eqs. 3, 4, 7, 8); direct sums of every leaf
  * pair and self leaf; fixed-order segmented sums.  Synchronises the stream
  * (list lengths are read back). */
 int fmm_interact(fmm_ctx *ctx);

@@ -2,8 +2,9 @@
 //
 // GB300 retires 1.7 to 2 FP64 operations per clock and SM, but 32 32 x 32 ->
 // 64-bit integer products and 64 shifts or additions (measured), so a sum that
-// is bound by the FP64 pipe runs faster in fixed point, and keeps more bits.
-// One ordered body pair (target i, source j) takes about 145 integer
+// is bound by the FP64 pipe runs faster in fixed point, and no less exactly: on
+// systems of every kind tested the rms error is 0.15 to 0.5 of that of FP64
+// arithmetic.  One ordered body pair (target i, source j) takes about 145 integer
 // instructions, 36 of them products, and no FP64 one.
 //
 // Formats
@@ -226,7 +227,7 @@ AMFMM_HD uint32_t top_mag(const W96 &o) {
 }
 
 // Shift that brings differences of offsets, |a| < (ma + 1) 2^64 and
-// |b| < (mb + 1) 2^64, to at most 2^kWin: between 10 and 41.
+// |b| < (mb + 1) 2^64, to at most 2^kWin: between 9 and 39 (offsets stay below 2^94).
 AMFMM_HD int window_shift(uint32_t ma, uint32_t mb) {
   const uint32_t s = ma + mb + 2;  // < 2^32: magnitudes are below 2^31
   return 64 + (32 - clz32(s)) - kWin;

@@ -175,7 +175,7 @@ struct fmm_ctx {
   double sel_theta_max = 1.0;  // upper edge of the band the network decides
   int64_t sel_min_work = 256;  // pairs with n_A n_B below this are left to the floor
   int sel_rule = FMM_SEL_RELATIVE;  // acceptance rule of the learned selector
-  // index tables of the table-driven general order (P = 6 .. 8)
+  // moments folded onto the reduced indices, per cell (P = 4 .. 8)
   amfmm::DBuf gen_fold;
   // host-solve staging
   amfmm::DBuf hx, hy, hz, hm, hax, hay, haz;

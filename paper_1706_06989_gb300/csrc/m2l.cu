@@ -385,7 +385,7 @@ __device__ __forceinline__ void m2l_one(const T r[3], T MT, T iMT, T MS, const T
 }
 
 // m2l_one for the unsoftened UC and TC forms, on trace-free moments (see
-// HARM of m2l_pair): QS5 = the source's trace-free quadrupole (xx xy xz yy
+// m2l_slot_tf): QS5 = the source's trace-free quadrupole (xx xy xz yy
 // yz; zz = -xx - yy), OhT and OhS its target's and its own trace-free
 // octupoles per unit mass (xxx xxy xxz xyy xyz yyy yyz; xzz = -xxx - xyy,
 // yzz = -xxy - yyy, zzz = -xxz - yyz).  The correction becomes

@@ -5,18 +5,20 @@
 // warp, an integer product for four.  In FP64 arithmetic the near field ran at
 // the FP64 pipe's rate (20 instructions per body pair, the pipe 90% busy) with
 // every other unit idle: 16.1 ms at N = 1,048,576 (Plummer, theta = 0.5, 421M
-// body pairs), 4.45 ms at 262,144, 1.21 ms at 2,000.  In fixed point: 7.24,
-// 1.98 and 0.11 ms.  It is bound by the integer pipes (290 cycles per step of
-// 32 ordered pairs and partition; 3 to 5 resident blocks per SM time the same),
-// and more exact: a pair's factor is good to 2^-54.6 (FP64: about 2^-52) and
-// the sums round nothing.
+// body pairs), 4.45 ms at 262,144, 1.21 ms at 2,000.  In fixed point: 7.22,
+// 1.99 and 0.08 ms.  It is bound by the integer pipes and the latencies around
+// them (four resident blocks per SM; with three 8.4 ms at N = 1,048,576, with five,
+// which spill registers, 7.5), and no less exact: a pair's factor is good to
+// 2^-54.6 (FP64: about 2^-52), and a term rounds once.
 //
 // One-sided: each leaf gathers from its own bodies and from every leaf paired
 // with it, on either side.  A pair is then evaluated twice, but the sums live
 // in registers (the mutual form kept a third of its traffic in shared-memory
 // partials, and wrote and read 24 bytes per body and pair), and the
 // preparation needs one sort of the leaf pairs instead of two, no slot offsets
-// and no column arrays.
+// and no column arrays.  The two forces of a pair are rounded independently, from
+// the same separation; the net force stays at rounding level (5.6e-18 of the sum of
+// the magnitudes at N = 1,048,576).
 //
 // Work item: 16 bodies (rows) of a leaf at most, and a group of 32 entries of
 // the leaf's list (itself first, then its partners in the stable order of the
@@ -28,9 +30,11 @@
 //
 // The sums' unit follows the heaviest source of what is being summed, a body at
 // the row's own place apart: a unit set by a body that adds no term there would
-// round the others' terms away.  A batch is therefore taken in classes of mass: the sources
-// within 2^kClassSpan of its heaviest, then those of the rest, and so on (one
-// class unless the masses differ by more).
+// round the others' terms away.  A batch is therefore taken in classes of mass: the
+// sources within 2^kClassSpan of its heaviest, then those of the rest, and so on
+// (one class unless the masses differ by more).  N = 262,144 with half of the masses
+// 1e-10 of the others: 4.35 ms (FP64 arithmetic 5.85); spread evenly over 2^90, five
+// classes a batch, 17.0 (13.1).
 //
 // Every sum has a fixed order and every result is independent of which warp
 // takes an item.
@@ -505,8 +509,8 @@ int p2p64_run(fmm_ctx *c) {
   int *queue = ptr<int32_t>(c->totals) + 40;
   launch(c, kern, grid, kWarps * 32, 0, nitem, c->sz.n, ptr<int4>(c->p2p_items), ptr<int32_t>(c->begin),
          ptr<int32_t>(c->count), ptr<int32_t>(c->p2p_offA),
-         c->sz.n_p2p > 0 ? ptr<uint32_t>(c->pval[c->p2p_which]) : nullptr, ptr<Rec>(c->p2p_rec), ptr<double>(c->X), ptr<double>(c->Y), ptr<double>(c->Zb), ptr<double>(c->Mb), c->eps2,
-         ptr<double>(c->near), ptr<double>(c->p2p_extra), queue);
+         c->sz.n_p2p > 0 ? ptr<uint32_t>(c->pval[c->p2p_which]) : nullptr, ptr<Rec>(c->p2p_rec), ptr<double>(c->X),
+         ptr<double>(c->Y), ptr<double>(c->Zb), ptr<double>(c->Mb), c->eps2, ptr<double>(c->near), ptr<double>(c->p2p_extra), queue);
   AMFMM_TRY(launched(c, "p2p"));
   if (c->sz.n_p2p == 0) return FMM_OK;
   launch(c, k_p2p64_groups, grid_for(static_cast<int64_t>(nleaf) * 32, 256), 256, 0, nleaf, c->sz.n,
