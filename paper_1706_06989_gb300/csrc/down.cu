@@ -34,8 +34,13 @@ __device__ __forceinline__ int i3(int i, int j, int k) {
   return 9;                               // zzz
 }
 
-// With h_ij = C_ijk s_k:  C_i' = C_i + (C_ij + h_ij / 2) s_j.
-//
+// With h_ij = C_ijk s_k:  C_i' = C_i + (C_ij + h_ij / 2) s_j.  Both kernels spell out
+// every operation, so that it makes no difference which of them takes a level (it
+// follows from the number of cells, in a forest of all systems).
+__device__ __forceinline__ double dot3(double a0, double a1, double a2, double s0, double s1, double s2) {
+  return fma(a2, s2, fma(a1, s1, __dmul_rn(a0, s0)));
+}
+
 // A thread per child where a level fills the GPU: 58 FP64 instructions for 32
 // children.  An FP64 instruction holds its pipe for 64 cycles whatever number
 // of lanes work, so on a small level those 58 are a chain of 2 us; there a
@@ -59,12 +64,13 @@ __global__ void k_l2l(int32_t c0, int32_t c1, const int32_t *parent,
 #pragma unroll
     for (int j = i; j < 3; ++j) {
       const int q = i2(i, j);
-      h[q] = Pl[9 + i3(i, j, 0)] * s[0] + Pl[9 + i3(i, j, 1)] * s[1] + Pl[9 + i3(i, j, 2)] * s[2];
-      C[3 + q] += Pl[3 + q] + h[q];
+      h[q] = dot3(Pl[9 + i3(i, j, 0)], Pl[9 + i3(i, j, 1)], Pl[9 + i3(i, j, 2)], s[0], s[1], s[2]);
+      C[3 + q] = __dadd_rn(C[3 + q], __dadd_rn(Pl[3 + q], h[q]));
       h[q] = fma(0.5, h[q], Pl[3 + q]);
     }
 #pragma unroll
-  for (int i = 0; i < 3; ++i) C[i] += Pl[i] + (h[i2(i, 0)] * s[0] + h[i2(i, 1)] * s[1] + h[i2(i, 2)] * s[2]);
+  for (int i = 0; i < 3; ++i)
+    C[i] = __dadd_rn(C[i], __dadd_rn(Pl[i], dot3(h[i2(i, 0)], h[i2(i, 1)], h[i2(i, 2)], s[0], s[1], s[2])));
 }
 
 constexpr int kL2LWarps = 4;
@@ -92,13 +98,13 @@ __global__ void __launch_bounds__(kL2LWarps * 32) k_l2l_warp(int32_t c0, int32_t
   const int i = q < 3 ? 0 : q < 5 ? 1 : 2;
   const int j = q < 3 ? q : q < 5 ? q - 2 : 2;
   if (q >= 0 && q < 6) {
-    const double h = sp[w][9 + i3(i, j, 0)] * s0 + sp[w][9 + i3(i, j, 1)] * s1 + sp[w][9 + i3(i, j, 2)] * s2;
+    const double h = dot3(sp[w][9 + i3(i, j, 0)], sp[w][9 + i3(i, j, 1)], sp[w][9 + i3(i, j, 2)], s0, s1, s2);
     sh[w][q] = fma(0.5, h, up);
-    up += h;
+    up = __dadd_rn(up, h);
   }
   __syncwarp();
-  if (l < 3) up += sh[w][i2(l, 0)] * s0 + sh[w][i2(l, 1)] * s1 + sh[w][i2(l, 2)] * s2;
-  if (l < 19) loc[static_cast<int64_t>(c) * kLocStride + l] = own + up;
+  if (l < 3) up = __dadd_rn(up, dot3(sh[w][i2(l, 0)], sh[w][i2(l, 1)], sh[w][i2(l, 2)], s0, s1, s2));
+  if (l < 19) loc[static_cast<int64_t>(c) * kLocStride + l] = __dadd_rn(own, up);
 }
 
 // (39 FP64 operations per body through the contraction with x / 2, 68 us at N =

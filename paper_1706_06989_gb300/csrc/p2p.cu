@@ -61,9 +61,9 @@ __device__ __forceinline__ void acc_zero(P2PSmem<ROWS> &sm, int nr, int l) {
 // these three scalar updates.)
 template <int ROWS>
 __device__ __forceinline__ void acc_sub(P2PSmem<ROWS> &sm, int i, int l, float s, float dx, float dy, float dz) {
-  sm.acc[3 * i][l] -= s * dx;
-  sm.acc[3 * i + 1][l] -= s * dy;
-  sm.acc[3 * i + 2][l] -= s * dz;
+  sm.acc[3 * i][l] = fmaf(-s, dx, sm.acc[3 * i][l]);
+  sm.acc[3 * i + 1][l] = fmaf(-s, dy, sm.acc[3 * i + 1][l]);
+  sm.acc[3 * i + 2][l] = fmaf(-s, dz, sm.acc[3 * i + 2][l]);
 }
 
 // below this squared separation two bodies count as coincident (their 1/r^3
@@ -88,9 +88,9 @@ __device__ __forceinline__ void rows32(P2PSmem<ROWS> &sm, int i, int l, bool val
     const float ri = ok ? rsqrtf(r2) : 0.f;
     r3[u] = ri * ri * ri;
     const float si = rw.w * r3[u];
-    bx += si * dx[u];
-    by += si * dy[u];
-    bz += si * dz[u];
+    bx = fmaf(si, dx[u], bx);
+    by = fmaf(si, dy[u], by);
+    bz = fmaf(si, dz[u], bz);
   }
   if (mutual) {
 #pragma unroll
@@ -368,9 +368,9 @@ __global__ void __launch_bounds__(kWarps * 32) k_p2p(
           const float ri = rsqrtf(r2);
           const float r3 = ri * ri * ri;
           const float si = sm.row[i][3] * r3;
-          bx += si * dx;
-          by += si * dy;
-          bz += si * dz;
+          bx = fmaf(si, dx, bx);
+          by = fmaf(si, dy, by);
+          bz = fmaf(si, dz, bz);
           if (mutual) {
             const float sj = mj * r3;
             acc_sub(sm, i, l, sj, dx, dy, dz);

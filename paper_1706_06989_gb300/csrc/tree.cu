@@ -551,6 +551,16 @@ __global__ void __launch_bounds__(kUpWarps * 32) k_leaf_upward(
 // The child dipoles D' (zero about a centre of mass up to rounding, Sec. 2)
 // are left out of the shift; the parent's dipole is the shift of the child
 // monopoles, D_i = Sum M' s_i.
+// Two kernels do this, by the number of cells of the level, which in a forest is that
+// of all systems; every operation is spelled out, so that a system's moments have the
+// same bits alone and in a forest.
+__device__ __forceinline__ double shift_quad(double q, double Ms_i, double s_j) { return fma(Ms_i, s_j, q); }
+__device__ __forceinline__ double shift_oct(double o, double Qij, double Qik, double Qjk, double Ms_i, double si,
+                                            double sj, double sk) {
+  const double t = fma(Qjk, si, fma(Qik, sj, __dmul_rn(Qij, sk)));
+  return fma(__dmul_rn(Ms_i, sj), sk, __dadd_rn(o, t));
+}
+
 // A warp takes four parents, eight lanes each, one per child: a lane shifts its
 // child's moments, and one lane per (parent, moment) adds the shifted ones in
 // octant order.  About 120 FP64 warp instructions for four parents; a thread per
@@ -606,20 +616,20 @@ __global__ void __launch_bounds__(kUpWarps * 32) k_internal_upward(
   for (int d = 0; d < 3; ++d) sv[d] = zk[d] - __shfl_sync(0xffffffffu, z, 8 * g + d);
   __syncwarp();
   if (child) {
-    const double Ms[3] = {q[0] * sv[0], q[0] * sv[1], q[0] * sv[2]};
+    const double Ms[3] = {__dmul_rn(q[0], sv[0]), __dmul_rn(q[0], sv[1]), __dmul_rn(q[0], sv[2])};
     const double Q[3][3] = {{q[4], q[5], q[6]}, {q[5], q[7], q[8]}, {q[6], q[8], q[9]}};
 #pragma unroll
     for (int d = 0; d < 3; ++d) sh[w][1 + d][l] = Ms[d];
     const int qi[6] = {0, 0, 0, 1, 1, 2}, qj[6] = {0, 1, 2, 1, 2, 2};
 #pragma unroll
-    for (int t = 0; t < 6; ++t) sh[w][4 + t][l] = q[4 + t] + Ms[qi[t]] * sv[qj[t]];
+    for (int t = 0; t < 6; ++t) sh[w][4 + t][l] = shift_quad(q[4 + t], Ms[qi[t]], sv[qj[t]]);
     const int oi[10] = {0, 0, 0, 0, 0, 0, 1, 1, 1, 2};
     const int oj[10] = {0, 0, 0, 1, 1, 2, 1, 1, 2, 2};
     const int ok[10] = {0, 1, 2, 1, 2, 2, 1, 2, 2, 2};
 #pragma unroll
     for (int t = 0; t < 10; ++t) {
       const int a = oi[t], b = oj[t], e = ok[t];
-      sh[w][10 + t][l] = q[10 + t] + (Q[a][b] * sv[e] + Q[a][e] * sv[b] + Q[b][e] * sv[a]) + Ms[a] * sv[b] * sv[e];
+      sh[w][10 + t][l] = shift_oct(q[10 + t], Q[a][b], Q[a][e], Q[b][e], Ms[a], sv[a], sv[b], sv[e]);
     }
   }
   __syncwarp();
@@ -681,17 +691,16 @@ __global__ void __launch_bounds__(128) k_internal_upward_block(
       const double *m = q + kMomStride * k;
       const int a = c_oct[r][0], b = c_oct[r][1], e = c_oct[r][2];
       const double sa = sv[k][a], sb = sv[k][b], se = sv[k][e];
-      sh[10 + r][k] = m[10 + r] + (m[c_quad[a][b]] * se + m[c_quad[a][e]] * sb + m[c_quad[b][e]] * sa) +
-                      m[0] * sa * sb * se;
+      sh[10 + r][k] = shift_oct(m[10 + r], m[c_quad[a][b]], m[c_quad[a][e]], m[c_quad[b][e]], __dmul_rn(m[0], sa),
+                                sa, sb, se);
     }
   } else {
     const int k = (t - 80) / 6, r = t - 80 - 6 * k;
     if (k < nch) {
       const double *m = q + kMomStride * k;
       const int a = r < 3 ? 0 : r < 5 ? 1 : 2, b = r < 3 ? r : r < 5 ? r - 2 : 2;
-      const double ms = m[0] * sv[k][a];
-      sh[4 + r][k] = m[4 + r] + ms * sv[k][b];
-      if (r < 3) sh[1 + r][k] = m[0] * sv[k][r];
+      sh[4 + r][k] = shift_quad(m[4 + r], __dmul_rn(m[0], sv[k][a]), sv[k][b]);
+      if (r < 3) sh[1 + r][k] = __dmul_rn(m[0], sv[k][r]);
     }
   }
   __syncthreads();
