@@ -448,7 +448,6 @@ __global__ void k_p2p64_groups(int32_t nleaf, int64_t n, const int32_t *leaves,
 }  // namespace
 
 int p2p64_prepare(fmm_ctx *c) {
-  cudaStream_t st = c->stream;
   const int64_t K = c->sz.n_p2p, nc = c->sz.ncell, n = c->sz.n;
   const int32_t nleaf = static_cast<int32_t>(c->sz.nleaf);
   if (2 * K > 0x7fffffffLL) return set_error(c, FMM_EUNSUPPORTED, "too many leaf pairs (%lld)", (long long)K);
@@ -485,7 +484,6 @@ int p2p64_prepare(fmm_ctx *c) {
     Expect e;
     for (int k = 0; k < 2; ++k) e.add64(ext64 + k, static_cast<uint64_t>(h[k]));
     AMFMM_TRY(graph_expect(c, e));
-    st = c->stream;
   }
   const int64_t nextra = h[0], nitem = h[1];
   if (nextra > 0x7fffffffLL || nitem > 0x7fffffffLL)
